@@ -78,7 +78,10 @@ typedef struct {
 } ptadd_material;
 
 typedef enum {
-    PTADD_FP64 = 0, /* every pair interaction in FP64                                  */
+    PTADD_FP64 = 0, /* FP64 results: pairs nearer than 32a (or 1/16 of a segment's     *
+                     * length) in FP64, the others in double-float arithmetic (two     *
+                     * FP32 parts, ~48 bits) on the FP32 pipe, whose error is far      *
+                     * below the rounding error that the close pairs leave             */
     PTADD_MIXED = 1 /* pairs farther than 10a in FP32 (compensated), nearer in FP64;   *
                      * positions, forces and averages always FP64                      */
 } ptadd_precision;
@@ -603,7 +606,7 @@ ptadd_status ptadd_fma_peak(int device, int fp64, double seconds, double* flops)
  * Call it with the device that owns `stream` and the arrays current
  * (cudaSetDevice): the scratch used is that device's.
  *
- * Scratch: one fixed array of about 7 MB in the library's device memory.
+ * Scratch: one fixed array of about 10 MB in the library's device memory.
  * With lazy module loading (the CUDA default) the library's module, and with
  * it the array, is loaded on a device at the first call there: that first
  * call allocates device memory outside the caller's pool and may

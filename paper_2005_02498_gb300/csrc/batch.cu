@@ -50,8 +50,9 @@ struct WorkItem {
 };
 
 struct BatchConfig {
-    int tpb = 128;         // targets per tile (threads per block)
+    int tpb = 128;         // targets per tile (threads per block) of the mixed kernel
     int chunk_len = 2048;  // sources per chunk
+    bool by_hand = false;  // set by ptadd_batch_configure: chunk_len holds for FP64 as it is
 };
 
 struct DevBatch {
@@ -64,6 +65,7 @@ struct DevBatch {
     uint8_t* pinned = nullptr;
     double* src = nullptr;
     float* src32 = nullptr;
+    float* srcdf = nullptr;
     double *fpart = nullptr, *vel = nullptr, *force = nullptr, *partial = nullptr, *acc = nullptr;
     std::vector<double> last_LV;  // [3R] (1/|B|) sum L vbar of the last burst, time-averaged, SI
     int64_t fpart_cap = 0;  // doubles
@@ -89,6 +91,7 @@ struct DevBatch {
     std::vector<int64_t> node_off, tgt_off;
     std::vector<double> volume, origin, sh;
     BatchConfig cfg;
+    int items_prec = -1;  // precision the work list was built for
     int tuned = 0;
     // graph of two steps
     cudaGraphExec_t graph = nullptr;
@@ -108,7 +111,6 @@ struct DevBatch {
 namespace {
 
 constexpr int BRED = 256;   // nodes per reduction block
-constexpr int TILE_FP64 = 128;
 // sources per staged tile of the mixed kernel: 192 at 128 threads (3 blocks
 // of 66.5 KB fit one SM's shared memory), 128 at 64 threads
 template <int TPB>
@@ -118,38 +120,19 @@ constexpr int tile_mix() { return TPB >= 128 ? 192 : 128; }
 __global__ void batch_prep_kernel(int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt,
                                   const int32_t* __restrict__ loop_of, const int32_t* __restrict__ real_of,
                                   const double* __restrict__ loop_b, const double* __restrict__ origin,
-                                  double* __restrict__ src, float* __restrict__ src32)
+                                  double* __restrict__ src, float* __restrict__ src32, float* __restrict__ srcdf,
+                                  double a2)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t j = nxt[i];
-    const double x1 = pos[i], y1 = pos[n + i], z1 = pos[2 * n + i];
-    const double dx = pos[j] - x1, dy = pos[n + j] - y1, dz = pos[2 * n + j] - z1;
-    const double L = sqrt(dx * dx + dy * dy + dz * dz);
-    const int k = loop_of[i];
-    const double bx = loop_b[3 * k], by = loop_b[3 * k + 1], bz = loop_b[3 * k + 2];
-    double tx = 1.0, ty = 0.0, tz = 0.0;
-    if (L > 0.0) {
-        tx = dx / L;
-        ty = dy / L;
-        tz = dz / L;
-    }
-    const double qx = by * tz - bz * ty, qy = bz * tx - bx * tz, qz = bx * ty - by * tx;
-    double* r = src + (int64_t)SRC_STRIDE * i;
-    r[0] = x1; r[1] = y1; r[2] = z1; r[3] = L;
-    r[4] = tx; r[5] = ty; r[6] = tz; r[7] = 0.0;
-    r[8] = bx; r[9] = by; r[10] = bz; r[11] = 0.0;
-    r[12] = qx; r[13] = qy; r[14] = qz; r[15] = 0.0;
-    const int rr = real_of[i];
-    const double rx = x1 - origin[3 * rr], ry = y1 - origin[3 * rr + 1], rz = z1 - origin[3 * rr + 2];
-    const double hx = rint(rx), hy = rint(ry), hz = rint(rz);
-    float* f = src32 + (int64_t)SRC32_STRIDE * i;
-    f[0] = (float)hx; f[1] = (float)hy; f[2] = (float)hz;
-    f[3] = (float)(rx - hx); f[4] = (float)(ry - hy); f[5] = (float)(rz - hz);
-    f[6] = (float)L;
-    f[7] = (float)tx; f[8] = (float)ty; f[9] = (float)tz;
-    f[10] = (float)bx; f[11] = (float)by; f[12] = (float)bz;
-    f[13] = (float)qx; f[14] = (float)qy; f[15] = (float)qz;
+    const int k = loop_of[i], rr = real_of[i];
+    const double x1[3] = {pos[i], pos[n + i], pos[2 * n + i]};
+    const double x2[3] = {pos[j], pos[n + j], pos[2 * n + j]};
+    const double b[3] = {loop_b[3 * k], loop_b[3 * k + 1], loop_b[3 * k + 2]};
+    const double o[3] = {origin[3 * rr], origin[3 * rr + 1], origin[3 * rr + 2]};
+    seg_records(x1, x2, b, o, a2, src + (int64_t)SRC_STRIDE * i, src32 ? src32 + (int64_t)SRC32_STRIDE * i : nullptr,
+                srcdf ? srcdf + (int64_t)SRCDF_STRIDE * i : nullptr);
 }
 
 struct BatchPairArgs {
@@ -158,6 +141,7 @@ struct BatchPairArgs {
     const int32_t* nxt;
     const double* src;
     const float* src32;
+    const float* srcdf;
     const int32_t* tgt;
     const int64_t* node_off;
     const int64_t* fp_base;
@@ -179,6 +163,7 @@ __device__ __forceinline__ TileArgs tile_from_item(const BatchPairArgs& b, const
     a.nxt = b.nxt;
     a.src = b.src;
     a.src32 = b.src32;
+    a.srcdf = b.srcdf;
     a.tgt = b.tgt;
     a.t_begin = w.t_begin;
     a.t_count = w.t_count;
@@ -196,14 +181,14 @@ __device__ __forceinline__ TileArgs tile_from_item(const BatchPairArgs& b, const
     return a;
 }
 
-// Persistent pair kernel: each block pulls work items until the list is
-// exhausted (the counter only grows, so the loop always ends).
-template <int TPB, int MINB, bool MIXED>
-__global__ void __launch_bounds__(TPB, MINB) batch_pair_kernel(BatchPairArgs b, Consts c, float near2)
+// Persistent pair kernels: each block pulls work items until the list is
+// exhausted (the counter only grows, so the loop always ends).  Mixed: blocks
+// of the configured tile; FP64: blocks of one warp.
+template <int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB) batch_pair_mixed_kernel(BatchPairArgs b, Consts c, float near2)
 {
     constexpr int TILE_MIX = tile_mix<TPB>();
-    constexpr int SM_BYTES = MIXED ? (int)sizeof(MixSmem<TILE_MIX, TPB>) : TILE_FP64 * SRC_STRIDE * 8;
-    __shared__ __align__(16) unsigned char smem[SM_BYTES];
+    __shared__ MixSmem<TILE_MIX, TPB> sm;
     __shared__ int item;
     for (;;) {
         if (threadIdx.x == 0) item = (int)atomicAdd(b.counter, 1u);
@@ -212,11 +197,26 @@ __global__ void __launch_bounds__(TPB, MINB) batch_pair_kernel(BatchPairArgs b, 
         __syncthreads();
         if (it >= b.n_items) break;
         const WorkItem w = b.items[it];
-        const TileArgs a = tile_from_item(b, w);
-        if (MIXED)
-            pair_tile_mixed<TILE_MIX, TPB>(a, c, near2, *reinterpret_cast<MixSmem<TILE_MIX, TPB>*>(smem));
-        else
-            pair_tile_fp64<TILE_FP64>(a, c, reinterpret_cast<double2*>(smem));
+        pair_tile_mixed<TILE_MIX, TPB>(tile_from_item(b, w), c, near2, sm);
+    }
+}
+
+__global__ void __launch_bounds__(32, 16) batch_pair_fp64_kernel(BatchPairArgs b, Consts c)
+{
+    __shared__ DFSmem sm;
+    for (;;) {
+        int it = 0;
+        if (threadIdx.x == 0) it = (int)atomicAdd(b.counter, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= b.n_items) break;
+        const WorkItem w = b.items[it];
+        TileArgs a = tile_from_item(b, w);
+        for (int t = 0; t < w.t_count; t += 32) {  // (more than 32 targets only where set by hand)
+            a.t_begin = w.t_begin + t;
+            a.t_count = min(32, w.t_count - t);
+            pair_tile_fp64(a, c, sm);
+            __syncwarp();
+        }
     }
 }
 
@@ -385,30 +385,49 @@ ptadd_status bd_alloc(T** p, size_t count)
     return PTADD_OK;
 }
 
-// Work list and fpart layout for a configuration; returns the fpart size needed.
-int64_t build_items(const DevBatch& B, const BatchConfig& cfg, std::vector<WorkItem>& items,
+// Targets per tile and sources per chunk of the work list.  FP64 tiles are one
+// warp's and, where the configured chunks would not fill the GPU, cut finer by
+// the rule of the single network (for the mean realisation), unless the
+// configuration was set by hand.
+void item_shape(const DevBatch& B, const BatchConfig& cfg, int prec, int64_t& tpb, int64_t& chunk_len)
+{
+    tpb = cfg.tpb;
+    chunk_len = cfg.chunk_len;
+    if (prec != (int)PTADD_MIXED && !cfg.by_hand) {
+        tpb = 32;
+        int64_t tiles = 0;
+        for (int r = 0; r < B.R; ++r) tiles += (B.tgt_off[r + 1] - B.tgt_off[r] + 31) / 32;
+        chunk_len = std::min(chunk_len, fp64_chunk_len(tiles, B.n / B.R));
+    }
+}
+
+// Work list and fpart layout for a configuration and precision; returns the
+// fpart size needed.
+int64_t build_items(const DevBatch& B, const BatchConfig& cfg, int prec, std::vector<WorkItem>& items,
                     std::vector<int64_t>& fp_base, std::vector<int32_t>& chunks)
 {
+    int64_t tpb, chunk_len;
+    item_shape(B, cfg, prec, tpb, chunk_len);
     items.clear();
     fp_base.assign(B.R, 0);
     chunks.assign(B.R, 0);
     int64_t off = 0;
     for (int r = 0; r < B.R; ++r) {
         const int64_t s0 = B.node_off[r], nr = B.node_off[r + 1] - s0;
-        const int32_t nch = (int32_t)((nr + cfg.chunk_len - 1) / cfg.chunk_len);
+        const int32_t nch = (int32_t)((nr + chunk_len - 1) / chunk_len);
         chunks[r] = nch;
         fp_base[r] = off;
         off += (int64_t)nch * 6 * nr;
         const int64_t t0 = B.tgt_off[r], t1 = B.tgt_off[r + 1];
-        for (int64_t tb = t0; tb < t1; tb += cfg.tpb)
+        for (int64_t tb = t0; tb < t1; tb += tpb)
             for (int32_t ch = 0; ch < nch; ++ch) {
                 WorkItem w;
                 w.r = r;
                 w.chunk = ch;
                 w.t_begin = (int32_t)tb;
-                w.t_count = (int32_t)std::min<int64_t>(cfg.tpb, t1 - tb);
-                w.js = (int32_t)(s0 + (int64_t)ch * cfg.chunk_len);
-                w.je = (int32_t)std::min<int64_t>(s0 + nr, w.js + (int64_t)cfg.chunk_len);
+                w.t_count = (int32_t)std::min<int64_t>(tpb, t1 - tb);
+                w.js = (int32_t)(s0 + (int64_t)ch * chunk_len);
+                w.je = (int32_t)std::min<int64_t>(s0 + nr, w.js + chunk_len);
                 items.push_back(w);
             }
     }
@@ -419,12 +438,12 @@ int64_t build_items(const DevBatch& B, const BatchConfig& cfg, std::vector<WorkI
     return off;
 }
 
-ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, cudaStream_t s)
+ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStream_t s)
 {
     std::vector<WorkItem> items;
     std::vector<int64_t> fp_base;
     std::vector<int32_t> chunks;
-    const int64_t need = build_items(B, cfg, items, fp_base, chunks);
+    const int64_t need = build_items(B, cfg, prec, items, fp_base, chunks);
     if (need > B.fpart_cap) {
         set_error("internal: partial-force buffer too small for the configuration");
         return PTADD_ERR_STATE;
@@ -441,6 +460,7 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, cudaStream_t s)
     PTADD_CUDA(cudaStreamSynchronize(s));
     B.n_items = (int)items.size();
     B.cfg = cfg;
+    B.items_prec = prec;
     if (B.graph) {
         cudaGraphExecDestroy(B.graph);
         B.graph = nullptr;
@@ -456,6 +476,7 @@ BatchPairArgs pair_args(const DevBatch& B)
     a.nxt = B.nxt;
     a.src = B.src;
     a.src32 = B.src32;
+    a.srcdf = B.srcdf;
     a.tgt = B.tgt;
     a.node_off = B.d_node_off;
     a.fp_base = B.d_fp_base;
@@ -470,35 +491,42 @@ BatchPairArgs pair_args(const DevBatch& B)
     return a;
 }
 
-template <int TPB, int MINB, bool MIXED>
-cudaError_t launch_batch_pair_t(const DevBatch& B, const Consts& c, float near2, cudaStream_t s)
+// Source records of the step (src32 is also what the junction search reads).
+void launch_batch_prep(const DevBatch& B, int prec, const Consts& c, cudaStream_t s)
+{
+    const bool mixed = prec == (int)PTADD_MIXED;
+    batch_prep_kernel<<<(unsigned)((B.n + 63) / 64), 64, 0, s>>>(
+        B.n, B.pos[B.cur], B.nxt, B.loop_of, B.real_of, B.loop_b, B.d_origin, B.src,
+        mixed || B.junc ? B.src32 : nullptr, mixed ? nullptr : B.srcdf, c.a2);
+}
+
+template <typename Kernel, typename... Args>
+cudaError_t launch_persistent(Kernel k, int tpb, int n_items, cudaStream_t s, Args... args)
 {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_pair_kernel<TPB, MINB, MIXED>, TPB, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, tpb, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    const int grid = std::min(sms * per_sm, std::max(1, B.n_items));
-    batch_pair_kernel<TPB, MINB, MIXED><<<grid, TPB, 0, s>>>(pair_args(B), c, near2);
+    k<<<std::min(sms * per_sm, std::max(1, n_items)), tpb, 0, s>>>(args...);
     return cudaGetLastError();
 }
 
 cudaError_t launch_batch_pair(const DevBatch& B, int prec, const Consts& c, cudaStream_t s)
 {
+    if (prec != (int)PTADD_MIXED) return launch_persistent(batch_pair_fp64_kernel, 32, B.n_items, s, pair_args(B), c);
     const float near2 = (float)((NEAR_FACTOR * NEAR_FACTOR + 1.0) * c.a2);
-    const bool mixed = prec == (int)PTADD_MIXED;
     if (B.cfg.tpb == 64)
-        return mixed ? launch_batch_pair_t<64, 6, true>(B, c, near2, s) : launch_batch_pair_t<64, 6, false>(B, c, near2, s);
-    return mixed ? launch_batch_pair_t<128, 3, true>(B, c, near2, s) : launch_batch_pair_t<128, 3, false>(B, c, near2, s);
+        return launch_persistent(batch_pair_mixed_kernel<64, 6>, 64, B.n_items, s, pair_args(B), c, near2);
+    return launch_persistent(batch_pair_mixed_kernel<128, 3>, 128, B.n_items, s, pair_args(B), c, near2);
 }
 
 // One DD step of the whole batch on stream s (pos[cur] -> pos[1-cur]).
 cudaError_t batch_step(DevBatch& B, int prec, const Consts& c, double dt_hat, cudaStream_t s)
 {
     const unsigned nb = (unsigned)((B.n + 255) / 256);
-    batch_prep_kernel<<<nb, 256, 0, s>>>(B.n, B.pos[B.cur], B.nxt, B.loop_of, B.real_of, B.loop_b, B.d_origin, B.src,
-                                         B.src32);
+    launch_batch_prep(B, prec, c, s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s);
@@ -544,7 +572,7 @@ void free_batch(DevBatch& B)
     if (B.d_loop_off) cudaFree(B.d_loop_off);
     if (B.cm_scratch) cudaFree(B.cm_scratch);
     void* ptrs[] = {B.pos[0],   B.pos[1],    B.nxt,       B.prv,        B.loop_of,  B.real_of, B.tgt,
-                    B.loop_b,   B.loop_n,    B.pinned,    B.src,        B.src32,    B.fpart,   B.vel,
+                    B.loop_b,   B.loop_n,    B.pinned,    B.src,        B.src32,    B.srcdf,   B.fpart,   B.vel,
                     B.force,    B.partial,   B.acc,       B.d_node_off, B.d_fp_base, B.d_chunks, B.d_origin,
                     B.d_sh,     B.d_blk_real, B.d_blk_start, B.d_real_blk, B.d_items, B.counter, B.flag,
                     B.near_count, B.staging, B.k64};
@@ -553,15 +581,7 @@ void free_batch(DevBatch& B)
     B = DevBatch{};
 }
 
-Consts batch_consts(const ptadd_ctx* ctx)
-{
-    Consts c;
-    const double r = ctx->mat.a / ctx->len_unit;
-    c.a2 = r * r;
-    c.c1 = 1.0 / (8.0 * M_PI);
-    c.c2 = 1.0 / (4.0 * M_PI * (1.0 - ctx->mat.nu));
-    return c;
-}
+Consts batch_consts(const ptadd_ctx* ctx) { return make_consts(ctx->mat.a / ctx->len_unit, ctx->mat.nu); }
 
 // ----------------------------------------------------------- tune cache
 #ifndef PTADD_BUILD_HASH
@@ -773,7 +793,8 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
         std::vector<int32_t> ch;
         BatchConfig smallest;
         smallest.chunk_len = 1024;
-        B.fpart_cap = build_items(B, smallest, items, fb, ch);
+        for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
+            B.fpart_cap = std::max(B.fpart_cap, build_items(B, smallest, prec, items, fb, ch));
     }
 
     ptadd_status st = PTADD_OK;
@@ -791,6 +812,7 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     BALLOC(B.pinned, n);
     BALLOC(B.src, SRC_STRIDE * n);
     BALLOC(B.src32, SRC32_STRIDE * n);
+    BALLOC(B.srcdf, SRCDF_STRIDE * n);
     BALLOC(B.fpart, B.fpart_cap);
     BALLOC(B.vel, 3 * n);
     BALLOC(B.force, 3 * n);
@@ -849,7 +871,7 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     PTADD_CUDA(cudaStreamSynchronize(s));
     BatchConfig cfg;
     B.tuned = tune_lookup(tune_path(nullptr), tune_key(ctx, B, (int)ctx->prec), cfg) ? 1 : 0;
-    return apply_config(B, cfg, s);
+    return apply_config(B, cfg, (int)ctx->prec, s);
 }
 
 ptadd_status ptadd_batch_set_stress(ptadd_ctx* ctx, const double* sig6)
@@ -885,6 +907,10 @@ ptadd_status ptadd_batch_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, dou
     const Consts c = batch_consts(ctx);
     const double dt_hat = dt * ctx->mat.mu / ctx->mat.B;
     const int prec = (int)ctx->prec;
+    if (B.items_prec != prec) {  // the precision was switched since the work list was built
+        ptadd_status st = apply_config(B, B.cfg, prec, s);
+        if (st != PTADD_OK) return st;
+    }
     PTADD_CUDA(cudaMemsetAsync(B.acc, 0, 16 * (size_t)B.R * sizeof(double), s));
     PTADD_CUDA(cudaMemsetAsync(B.flag, 0, sizeof(int), s));
     B.dt_s = dt;
@@ -1088,7 +1114,8 @@ ptadd_status ptadd_batch_configure(ptadd_ctx* ctx, int32_t tile_targets, int32_t
     BatchConfig cfg;
     cfg.tpb = tile_targets;
     cfg.chunk_len = chunk_sources;
-    ptadd_status st = apply_config(*ctx->batch, cfg, ctx->own_stream);
+    cfg.by_hand = true;
+    ptadd_status st = apply_config(*ctx->batch, cfg, (int)ctx->prec, ctx->own_stream);
     if (st == PTADD_OK) ctx->batch->tuned = 0;
     return st;
 }
@@ -1105,9 +1132,12 @@ ptadd_status ptadd_batch_get_forces(ptadd_ctx* ctx, double* F)
     cudaStream_t s = ctx->own_stream;
     PTADD_CUDA(cudaStreamSynchronize(ctx->stream));
     const Consts c = batch_consts(ctx);
+    if (B.items_prec != (int)ctx->prec) {
+        ptadd_status st = apply_config(B, B.cfg, (int)ctx->prec, s);
+        if (st != PTADD_OK) return st;
+    }
     const unsigned nb = (unsigned)((B.n + 255) / 256);
-    batch_prep_kernel<<<nb, 256, 0, s>>>(B.n, B.pos[B.cur], B.nxt, B.loop_of, B.real_of, B.loop_b, B.d_origin, B.src,
-                                         B.src32);
+    launch_batch_prep(B, (int)ctx->prec, c, s);
     PTADD_CUDA(cudaGetLastError());
     PTADD_CUDA(cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s));
     if (B.n_items > 0) PTADD_CUDA(launch_batch_pair(B, (int)ctx->prec, c, s));
@@ -1157,7 +1187,7 @@ ptadd_status ptadd_batch_autotune(ptadd_ctx* ctx, const char* cache_path, int fo
     BatchConfig cached;
     if (!force && tune_lookup(path, key, cached)) {
         B.tuned = 1;
-        return apply_config(B, cached, ctx->own_stream);
+        return apply_config(B, cached, prec, ctx->own_stream);
     }
     cudaStream_t s = ctx->own_stream;
     PTADD_CUDA(cudaStreamSynchronize(ctx->stream));
@@ -1170,18 +1200,16 @@ ptadd_status ptadd_batch_autotune(ptadd_ctx* ctx, const char* cache_path, int fo
     BatchConfig best;
     double best_ms = INFINITY;
     ptadd_status st = PTADD_OK;
-    const unsigned nb = (unsigned)((B.n + 255) / 256);
     for (int ti = 0; ti < 2 && st == PTADD_OK; ++ti)
         for (int ci = 0; ci < 3 && st == PTADD_OK; ++ci) {
             BatchConfig cfg;
             cfg.tpb = tpbs[ti];
             cfg.chunk_len = chunks[ci];
-            st = apply_config(B, cfg, s);
+            st = apply_config(B, cfg, prec, s);
             if (st != PTADD_OK) break;
             float best_rep = INFINITY;
             for (int rep = 0; rep < 3; ++rep) {  // first repetition is a warm-up
-                batch_prep_kernel<<<nb, 256, 0, s>>>(B.n, B.pos[B.cur], B.nxt, B.loop_of, B.real_of, B.loop_b,
-                                                     B.d_origin, B.src, B.src32);
+                launch_batch_prep(B, prec, c, s);
                 cudaError_t e = cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s);
                 if (e == cudaSuccess) e = cudaEventRecord(e0, s);
                 if (e == cudaSuccess && B.n_items > 0) e = launch_batch_pair(B, prec, c, s);
@@ -1206,7 +1234,7 @@ ptadd_status ptadd_batch_autotune(ptadd_ctx* ctx, const char* cache_path, int fo
     if (st != PTADD_OK) return st;
     tune_store(path, key, best, best_ms);
     B.tuned = 1;
-    return apply_config(B, best, s);
+    return apply_config(B, best, prec, s);
 }
 
 ptadd_status ptadd_batch_run(ptadd_ctx* ctx, int32_t R, const int64_t* node_off, int64_t n_loops,

@@ -1,6 +1,6 @@
 // dd_kernels.cu -- one explicit DD step on the GPU (Sec. 2.1 of the paper):
 //   seg_prep      : per-segment source records from the current positions
-//   pair_fp64     : O(N^2) stress at the 4 Gauss points of every target
+//   pair_fp64 / pair_mixed : O(N^2) stress at the 4 Gauss points of every target
 //                   segment, contracted with its Burgers vector, folded into
 //                   the two nodal force parts of the segment (PK force, linear
 //                   shape functions)
@@ -25,76 +25,69 @@ namespace ptadd {
 // ----------------------------------------------------------- seg_prep
 __global__ void seg_prep_kernel(int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt,
                                 const int32_t* __restrict__ loop_of, const double* __restrict__ loop_b,
-                                double* __restrict__ src, float* __restrict__ src32, double ox, double oy, double oz)
+                                double* __restrict__ src, float* __restrict__ src32, float* __restrict__ srcdf,
+                                double ox, double oy, double oz, int origin_node0, double a2)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t j = nxt[i];
-    const double x1 = pos[i], y1 = pos[n + i], z1 = pos[2 * n + i];
-    const double dx = pos[j] - x1, dy = pos[n + j] - y1, dz = pos[2 * n + j] - z1;
-    const double L = sqrt(dx * dx + dy * dy + dz * dz);
     const int k = loop_of[i];
-    double bx = loop_b[3 * k], by = loop_b[3 * k + 1], bz = loop_b[3 * k + 2];
-    double tx = 1.0, ty = 0.0, tz = 0.0;
-    if (L > 0.0) {
-        tx = dx / L;
-        ty = dy / L;
-        tz = dz / L;
-    }
-    double* r = src + (int64_t)SRC_STRIDE * i;
-    r[0] = x1; r[1] = y1; r[2] = z1; r[3] = L;
-    r[4] = tx; r[5] = ty; r[6] = tz; r[7] = 0.0;
-    r[8] = bx; r[9] = by; r[10] = bz; r[11] = 0.0;
-    r[12] = by * tz - bz * ty;
-    r[13] = bz * tx - bx * tz;
-    r[14] = bx * ty - by * tx;
-    r[15] = 0.0;
-    if (src32) {
-        float* f = src32 + (int64_t)SRC32_STRIDE * i;
-        const double rx = x1 - ox, ry = y1 - oy, rz = z1 - oz;
-        const double hx = rint(rx), hy = rint(ry), hz = rint(rz);
-        f[0] = (float)hx; f[1] = (float)hy; f[2] = (float)hz;
-        f[3] = (float)(rx - hx); f[4] = (float)(ry - hy); f[5] = (float)(rz - hz);
-        f[6] = (float)L;
-        f[7] = (float)tx; f[8] = (float)ty; f[9] = (float)tz;
-        f[10] = (float)bx; f[11] = (float)by; f[12] = (float)bz;
-        f[13] = (float)r[12]; f[14] = (float)r[13]; f[15] = (float)r[14];
-    }
+    const double x1[3] = {pos[i], pos[n + i], pos[2 * n + i]};
+    const double x2[3] = {pos[j], pos[n + j], pos[2 * n + j]};
+    const double b[3] = {loop_b[3 * k], loop_b[3 * k + 1], loop_b[3 * k + 2]};
+    double o[3] = {ox, oy, oz};
+    if (origin_node0)
+        for (int e = 0; e < 3; ++e) o[e] = rint(pos[e * n]);
+    seg_records(x1, x2, b, o, a2, src + (int64_t)SRC_STRIDE * i, src32 ? src32 + (int64_t)SRC32_STRIDE * i : nullptr,
+                srcdf ? srcdf + (int64_t)SRCDF_STRIDE * i : nullptr);
 }
 
-cudaError_t launch_seg_prep(const DevNetwork& net, cudaStream_t st)
+cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& c, cudaStream_t st)
 {
     const int64_t n = net.n_nodes;
     if (n == 0) return cudaSuccess;
-    seg_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, net.pos[net.cur], net.nxt, net.loop_of,
-                                                                  net.loop_b, net.src, net.src32, net.origin[0],
-                                                                  net.origin[1], net.origin[2]);
+    const bool mixed = precision == (int)PTADD_MIXED;
+    seg_prep_kernel<<<(unsigned)((n + 63) / 64), 64, 0, st>>>(n, net.pos[net.cur], net.nxt, net.loop_of, net.loop_b,
+                                                              net.src, mixed ? net.src32 : nullptr,
+                                                              mixed ? nullptr : net.srcdf, net.origin[0],
+                                                              net.origin[1], net.origin[2], net.origin_node0 ? 1 : 0,
+                                                              c.a2);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ pair stage
-// Grid: x = target tiles of PAIR_TPB threads (one target segment each),
-//       y = source chunks.  Each block runs one tile (pair_tile.cuh): it
+// Grid: x = target tiles of one segment per thread (mixed: MIX_TPB, FP64: a
+// warp), y = source chunks.  Each block runs one tile (pair_tile.cuh): it
 // stages source records through shared memory; every thread walks them in the
 // same order (broadcast reads) and accumulates (sigma b') at its 4 Gauss points.
-constexpr int PAIR_TPB = 128;
-constexpr int PAIR_TILE = 128;
 constexpr int MIX_TPB = 128;
+constexpr int MIX_MAX_CHUNKS = 64;
 constexpr int MIX_TILE = 192;  // sources per staged tile: 3 blocks of 66.5 KB fit one SM's shared memory
 constexpr int MIX_MINB = 3;  // resident blocks per SM the register budget is sized for
 
-__global__ void __launch_bounds__(PAIR_TPB) pair_fp64_kernel(TileArgs base, int64_t n_tgt, int64_t chunk_len,
-                                                             Consts c)
+// FP64 path.  Bound by the FP32 pipe: about 1550 packed FP32 instructions per
+// source and warp, two pipe cycles each (3100 of the 3650 cycles that a source
+// takes on a full scheduler).  32 768 segments: 96.5 ms per evaluation (1.11e10
+// pairs/s), 826 ms when every pair ran on the FP64 pipe; 512 segments: 56
+// against 560 us per launch.  One-warp blocks: 16 at 128 registers per thread
+// run 8192 segments in 6.15 ms, 12 at 168 in 6.19, 8 in 6.35; blocks of four
+// warps the same.  The points of a pair go through one copy of the code two at
+// a time: with all four unrolled the loop (62 KB) missed the instruction cache
+// (9.8 ms).
+constexpr int DF_MINB = 16;
+
+__global__ void __launch_bounds__(32, DF_MINB) pair_fp64_kernel(TileArgs base, int64_t n_tgt, int64_t chunk_len,
+                                                                Consts c)
 {
-    __shared__ double2 tile[PAIR_TILE * SRC_STRIDE / 2];
+    __shared__ DFSmem sm;
     TileArgs a = base;
-    a.t_begin = (int64_t)blockIdx.x * PAIR_TPB;
-    a.t_count = min((int64_t)PAIR_TPB, n_tgt - a.t_begin);
+    a.t_begin = (int64_t)blockIdx.x * 32;
+    a.t_count = min((int64_t)32, n_tgt - a.t_begin);
     a.js = (int64_t)blockIdx.y * chunk_len;
     a.je = min(a.n, a.js + chunk_len);
     a.add_app = blockIdx.y == 0;
     a.fp = base.fp + (int64_t)blockIdx.y * 6 * a.n;
-    pair_tile_fp64<PAIR_TILE>(a, c, tile);
+    pair_tile_fp64(a, c, sm);
 }
 
 __global__ void __launch_bounds__(MIX_TPB, MIX_MINB) pair_mixed_kernel(TileArgs base, int64_t n_tgt, int64_t chunk_len,
@@ -111,37 +104,70 @@ __global__ void __launch_bounds__(MIX_TPB, MIX_MINB) pair_mixed_kernel(TileArgs 
     pair_tile_mixed<MIX_TILE, MIX_TPB>(a, c, near2, sm);
 }
 
-int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
+// SMs and resident pair blocks per SM, queried once per device and precision.
+static void pair_slots(int mixed, int& sms, int& per_sm)
 {
-    // About 16 waves of resident blocks, so that the blocks still running
-    // when the others have finished (the tail) cost a few per cent; chunks of
-    // at least two source tiles, so the per-block set-up and the nodal
-    // output stay small next to the pair work, unless that leaves less than
-    // one wave (a small network): then chunks down to 32 sources, so that the
-    // few targets' work (and their FP64 near pairs) spreads over more SMs.
-    // The device queries are made once per device and precision.
     static std::atomic<int> cached[64][2][2];  // [device][mixed] -> {sms, blocks per SM}; 0: not yet
-    int dev = 0, sms = 152, per_sm = 2;
-    const int mixed = precision == (int)PTADD_MIXED ? 1 : 0;
+    int dev = 0;
+    sms = 152;
+    per_sm = 2;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
         cached[dev][mixed][0].load(std::memory_order_acquire) > 0) {
         sms = cached[dev][mixed][0].load(std::memory_order_relaxed);
         per_sm = cached[dev][mixed][1].load(std::memory_order_relaxed);
-    } else {
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (mixed)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_mixed_kernel, MIX_TPB, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_fp64_kernel, PAIR_TPB, 0);
-        if (per_sm < 1) per_sm = 1;
-        if (dev >= 0 && dev < 64) {
-            cached[dev][mixed][1].store(per_sm, std::memory_order_relaxed);
-            cached[dev][mixed][0].store(sms, std::memory_order_release);
-        }
+        return;
     }
-    const int64_t tiles_t = (n_tgt + PAIR_TPB - 1) / PAIR_TPB;
-    int64_t cap = n_src / (2 * PAIR_TILE);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (mixed)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_mixed_kernel, MIX_TPB, 0);
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_fp64_kernel, 32, 0);
+    if (per_sm < 1) per_sm = 1;
+    if (dev >= 0 && dev < 64) {
+        cached[dev][mixed][1].store(per_sm, std::memory_order_relaxed);
+        cached[dev][mixed][0].store(sms, std::memory_order_release);
+    }
+}
+
+int64_t fp64_chunk_len(int64_t tiles, int64_t n_src)
+{
+    // Resident one-warp tiles: 16 per SM.  Up to 16 waves of them in chunks of
+    // at least 64 sources (one group of sums), so that the tail costs a few per
+    // cent.  Where that leaves fewer than four waves the chunks shrink, down to
+    // 4 sources: a lone warp spends 3.3 us on a source, and the FP64 near pairs
+    // of a loop (5 us per 32) sit in few chunks.  Measured, us per launch: 512
+    // segments 93 / 68 / 56 / 65 in chunks of 16 / 8 / 4 / 2, 64 targets x 1280
+    // sources 101 / 57 / 35 in 20 / 10 / 5, 1041 x 1485 244 / 220 / 190 in 23 / 12
+    // / 6, 8192 segments 6330 / 6163 / 6155 in 128 / 64 / 32.
+    int sms, per_sm;
+    pair_slots(0, sms, per_sm);
+    const int64_t slots = (int64_t)sms * per_sm;
+    tiles = std::max<int64_t>(tiles, 1);
+    int64_t ch = std::min((16 * slots + tiles - 1) / tiles, n_src / 64);
+    if (tiles * ch < 4 * slots) ch = std::min((4 * slots + tiles - 1) / tiles, n_src / 4);
+    ch = std::max<int64_t>(ch, 1);
+    return (n_src + ch - 1) / ch;
+}
+
+int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
+{
+    if (precision != (int)PTADD_MIXED) {
+        int64_t len = fp64_chunk_len((n_tgt + 31) / 32, n_src);
+        len = std::max(len, (n_src + max_chunks - 1) / max_chunks);
+        return (int)((n_src + len - 1) / len);
+    }
+    // About 16 waves of resident blocks, so that the blocks still running
+    // when the others have finished (the tail) cost a few per cent; chunks of
+    // at least 256 sources, so the per-block set-up and the nodal
+    // output stay small next to the pair work, unless that leaves less than
+    // one wave (a small network): then chunks down to 32 sources, so that the
+    // few targets' work (and their FP64 near pairs) spreads over more SMs.
+    int sms, per_sm;
+    pair_slots(1, sms, per_sm);
+    const int64_t tiles_t = (n_tgt + MIX_TPB - 1) / MIX_TPB;
+    int64_t cap = n_src / 256;
     if (tiles_t * cap < (int64_t)sms * per_sm) cap = std::max<int64_t>(cap, n_src / 32);
+    if (cap > MIX_MAX_CHUNKS) cap = MIX_MAX_CHUNKS;
     if (cap > max_chunks) cap = max_chunks;
     if (cap < 1) cap = 1;
     const int64_t want_blocks = (int64_t)sms * per_sm * 16;
@@ -163,6 +189,7 @@ cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt
     a.nxt = net.nxt;
     a.src = net.src;
     a.src32 = net.src32;
+    a.srcdf = net.srcdf;
     a.tgt = tgt;
     for (int k = 0; k < 6; ++k) a.sh[k] = sh[k];
     for (int k = 0; k < 3; ++k) a.origin[k] = net.origin[k];
@@ -177,28 +204,43 @@ cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt
         pair_mixed_kernel<<<grid, MIX_TPB, 0, st>>>(a, n_tgt, chunk_len, c, near2);
         return cudaGetLastError();
     }
-    dim3 grid((unsigned)((n_tgt + PAIR_TPB - 1) / PAIR_TPB), (unsigned)chunks);
-    pair_fp64_kernel<<<grid, PAIR_TPB, 0, st>>>(a, n_tgt, chunk_len, c);
+    const dim3 grid((unsigned)((n_tgt + 31) / 32), (unsigned)chunks);
+    pair_fp64_kernel<<<grid, 32, 0, st>>>(a, n_tgt, chunk_len, c);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------- node_velocity
-__global__ void node_velocity_kernel(int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt,
-                                     const int32_t* __restrict__ prv, const int32_t* __restrict__ loop_of,
-                                     const double* __restrict__ loop_n, const uint8_t* __restrict__ pinned,
-                                     const double* __restrict__ fpart, int chunks, double* __restrict__ force,
-                                     double* __restrict__ vel)
+// Block: 32 nodes x NV_ROWS rows.  Row y sums the chunks y, y + NV_ROWS, ... of
+// its 32 nodes (coalesced), the rows are added in order: a fixed summation
+// order whatever the schedule.  (A thread per node would walk up to 500 chunks
+// of a small network one after another.)
+constexpr int NV_ROWS = 8;
+
+__global__ void __launch_bounds__(32 * NV_ROWS) node_velocity_kernel(
+    int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt, const int32_t* __restrict__ prv,
+    const int32_t* __restrict__ loop_of, const double* __restrict__ loop_n, const uint8_t* __restrict__ pinned,
+    const double* __restrict__ fpart, int chunks, double* __restrict__ force, double* __restrict__ vel)
 {
-    const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (a >= n) return;
-    const int64_t p = prv[a], nx = nxt[a];
+    __shared__ double red[NV_ROWS][3][32];
+    const int64_t a = blockIdx.x * (int64_t)32 + threadIdx.x;
+    const int64_t p = a < n ? prv[a] : 0;
     double F[3] = {0, 0, 0};
-    for (int ch = 0; ch < chunks; ++ch) {
-        const double* fp = fpart + (int64_t)ch * 6 * n;
-        F[0] += fp[0 * n + a] + fp[3 * n + p];
-        F[1] += fp[1 * n + a] + fp[4 * n + p];
-        F[2] += fp[2 * n + a] + fp[5 * n + p];
-    }
+    if (a < n)
+        for (int ch = threadIdx.y; ch < chunks; ch += NV_ROWS) {
+            const double* fp = fpart + (int64_t)ch * 6 * n;
+            F[0] += fp[0 * n + a] + fp[3 * n + p];
+            F[1] += fp[1 * n + a] + fp[4 * n + p];
+            F[2] += fp[2 * n + a] + fp[5 * n + p];
+        }
+#pragma unroll
+    for (int e = 0; e < 3; ++e) red[threadIdx.y][e][threadIdx.x] = F[e];
+    __syncthreads();
+    if (threadIdx.y != 0 || a >= n) return;
+#pragma unroll
+    for (int y = 1; y < NV_ROWS; ++y)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) F[e] += red[y][e][threadIdx.x];
+    const int64_t nx = nxt[a];
     const double xa = pos[a], ya = pos[n + a], za = pos[2 * n + a];
     const double px = xa - pos[p], py = ya - pos[n + p], pz = za - pos[2 * n + p];
     const double qx = pos[nx] - xa, qy = pos[n + nx] - ya, qz = pos[2 * n + nx] - za;
@@ -220,9 +262,8 @@ cudaError_t launch_node_velocity(const DevNetwork& net, int chunks, cudaStream_t
 {
     const int64_t n = net.n_nodes;
     if (n == 0) return cudaSuccess;
-    node_velocity_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, net.pos[net.cur], net.nxt, net.prv,
-                                                                       net.loop_of, net.loop_n, net.pinned,
-                                                                       net.fpart, chunks, net.force, net.vel);
+    node_velocity_kernel<<<(unsigned)((n + 31) / 32), dim3(32, NV_ROWS), 0, st>>>(
+        n, net.pos[net.cur], net.nxt, net.prv, net.loop_of, net.loop_n, net.pinned, net.fpart, chunks, net.force, net.vel);
     return cudaGetLastError();
 }
 

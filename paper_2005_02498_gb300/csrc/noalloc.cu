@@ -5,7 +5,7 @@
 // records, per-chunk partial nodal forces, ...) lives in one file-scope
 // __device__ array sized for at most PTADD_NOALLOC_MAX_SEGMENTS segments.
 // Every GPU on which the library's module is loaded holds that array (about
-// 7 MB) until the process exits; with lazy module loading (the CUDA default)
+// 10 MB) until the process exits; with lazy module loading (the CUDA default)
 // that happens at the first call on the device.  Host code cannot use the
 // array's name as a device address: every call made outside stream capture
 // looks the address up with cudaGetSymbolAddress (with the caller's device
@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "ptadd_internal.cuh"
@@ -28,12 +29,12 @@ namespace ptadd {
 namespace {
 
 constexpr int64_t NA_MAX = PTADD_NOALLOC_MAX_SEGMENTS;
-constexpr int NA_CHUNKS = 4;
-// doubles per segment: positions 3, source record 16, partial forces 6 per
-// chunk, force 3, velocity 3, Burgers vector 3, normal 3; then four int32
+constexpr int NA_CHUNKS = 4;  // source chunks at NA_MAX segments (smaller networks: more, in the same space)
+// doubles per segment: positions 3, source record 16, double-float record 18
+// (36 floats), partial forces 6 per chunk, force 3, velocity 3, Burgers vector 3, normal 3; then four int32
 // tables (loop index, target list, checked nxt and prv copies) and the error
 // word packed into the same array.
-constexpr int64_t NA_DOUBLES_PER_SEG = 3 + SRC_STRIDE + 6 * NA_CHUNKS + 3 + 3 + 3 + 3;
+constexpr int64_t NA_DOUBLES_PER_SEG = 3 + SRC_STRIDE + SRCDF_STRIDE / 2 + 6 * NA_CHUNKS + 3 + 3 + 3 + 3;
 // + 4*NA_MAX int32 (= 2*NA_MAX doubles) + slack for the 256-byte alignment of
 // the regions (each pad < 32 doubles) and the error word
 constexpr int64_t NA_DOUBLES = NA_DOUBLES_PER_SEG * NA_MAX + 2 * NA_MAX + 512;
@@ -158,7 +159,8 @@ extern "C" ptadd_status ptadd_forces_noalloc(const ptadd_material* mat, int64_t 
     net.n_loops = n;
     net.pos[0] = base + off; off = align32(off + 3 * n);
     net.src = base + off;    off = align32(off + SRC_STRIDE * n);
-    net.fpart = base + off;  off = align32(off + 6 * NA_CHUNKS * n);
+    net.srcdf = reinterpret_cast<float*>(base + off); off = align32(off + SRCDF_STRIDE / 2 * n);
+    net.fpart = base + off;  off = align32(off + 6 * NA_CHUNKS * NA_MAX);
     net.force = base + off;  off = align32(off + 3 * n);
     net.vel = base + off;    off = align32(off + 3 * n);
     net.loop_b = base + off; off = align32(off + 3 * n);
@@ -170,23 +172,20 @@ extern "C" ptadd_status ptadd_forces_noalloc(const ptadd_material* mat, int64_t 
     net.prv = net.nxt + align32(n);
     int* err = reinterpret_cast<int*>(net.prv + align32(n));
     net.pinned = nullptr;
+    net.origin_node0 = true;
     net.cur = 0;
-    net.max_chunks = NA_CHUNKS;
+    net.max_chunks = (int)std::min<int64_t>(512, NA_CHUNKS * NA_MAX / n);  // what the partial-force region holds
 
     const unsigned blk = (unsigned)((n + 255) / 256);
     PTADD_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     na_prepare<<<blk, 256, 0, s>>>(n, xyz_dev, burgers_dev, nxt_dev, prv_dev, ldexp(1.0, -len_exp), len_unit,
                                    net.pos[0], net.loop_b, net.loop_n, net.loop_of, tgt, net.nxt, net.prv, err);
     PTADD_CUDA(cudaGetLastError());
-    Consts c;
-    const double r = mat->a / len_unit;
-    c.a2 = r * r;
-    c.c1 = 1.0 / (8.0 * M_PI);
-    c.c2 = 1.0 / (4.0 * M_PI * (1.0 - mat->nu));
+    const Consts c = make_consts(mat->a / len_unit, mat->nu);
     double sh[6];
     for (int k = 0; k < 6; ++k) sh[k] = sig_app[k] / mat->mu;
-    const int chunks = choose_chunks(n, n, NA_CHUNKS, (int)PTADD_FP64);
-    PTADD_CUDA(launch_seg_prep(net, s));
+    const int chunks = choose_chunks(n, n, net.max_chunks, (int)PTADD_FP64);
+    PTADD_CUDA(launch_seg_prep(net, (int)PTADD_FP64, c, s));
     PTADD_CUDA(launch_pair(net, tgt, n, chunks, (int)PTADD_FP64, c, sh, s));
     PTADD_CUDA(launch_node_velocity(net, chunks, s));
     na_finish<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(n, net.force, mat->mu * len_unit * len_unit, err,

@@ -13,6 +13,7 @@
 
 #include <cuda_runtime.h>
 
+#include "df_field.cuh"
 #include "ptadd_internal.cuh"
 #include "seg_field.cuh"
 
@@ -24,6 +25,7 @@ struct TileArgs {
     const int32_t* nxt;
     const double* src;      // FP64 source records
     const float* src32;     // FP32 source records (mixed)
+    const float* srcdf;     // double-float source records (FP64)
     const int32_t* tgt;     // target segment list
     int64_t t_begin;        // first entry of tgt for thread 0
     int64_t t_count;        // targets in this tile (<= blockDim.x)
@@ -37,6 +39,124 @@ struct TileArgs {
     unsigned long long* near_count;
     const double* k64;      // device copy of {a2, c1, c2} for the near-field path (mixed)
 };
+
+// ---------------------------------------------------------------- records
+constexpr double DF_NEAR = 32.0;      // in core widths a
+constexpr double DF_FAR = 2097152.0;  // 2^21 units
+// The two FP32 parts of an FP64 value in FP32's normal range (or 0), the first
+// by truncation: the mantissa fields are moved on the integer pipe, because the
+// hardware conversions and every FP64 operation run on the 1/64-rate FP64 pipe
+// (one FP64 subtraction is left; h + l differs from x by less than 2^-46 |x|).
+__device__ __forceinline__ DF1 df_split(double x)
+{
+    const float h = d2f_seed0(x);
+    return DF1{h, d2f_seed0(x - f2d_seed0(h))};
+}
+
+// The three FP32 parts of x - o (o an integer), scaled; NaN outside their range.
+__device__ __forceinline__ void df_parts(double x, double o, float* f)
+{
+    constexpr float sc = 1.0f / (1 << -DF_SCALE);
+    const double h = rint(x), r = x - h, ho = h - o;
+    const float m = rintf((float)r * 8388608.0f) * (1.0f / 8388608.0f);
+    f[0] = fabs(ho) < 8388608.0 ? (float)ho * sc : __int_as_float(0x7fffffff);
+    f[1] = m * sc;
+    f[2] = (float)(r - (double)m) * sc;
+}
+
+// The records of segment i, from its end nodes and its Burgers vector: src
+// always, src32 and srcdf where given; o the integer-valued origin of both.
+__device__ __forceinline__ void seg_records(const double x1[3], const double x2[3], const double b[3],
+                                            const double o[3], double a2, double* r, float* f32, float* fdf)
+{
+    const double dx = x2[0] - x1[0], dy = x2[1] - x1[1], dz = x2[2] - x1[2];
+    const double LL = dx * dx + dy * dy + dz * dz, L = sqrt(LL);
+    double t[3] = {1.0, 0.0, 0.0};
+    if (L > 0.0) {
+        t[0] = dx / L;
+        t[1] = dy / L;
+        t[2] = dz / L;
+    }
+    const double q[3] = {b[1] * t[2] - b[2] * t[1], b[2] * t[0] - b[0] * t[2], b[0] * t[1] - b[1] * t[0]};
+    double2* r2 = reinterpret_cast<double2*>(r);
+    r2[0] = make_double2(x1[0], x1[1]);
+    r2[1] = make_double2(x1[2], L);
+    r2[2] = make_double2(t[0], t[1]);
+    r2[3] = make_double2(t[2], 0.0);
+    r2[4] = make_double2(b[0], b[1]);
+    r2[5] = make_double2(b[2], 0.0);
+    r2[6] = make_double2(q[0], q[1]);
+    r2[7] = make_double2(q[2], 0.0);
+    if (f32) {
+        float v[SRC32_STRIDE];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double rx = x1[k] - o[k], hx = rint(rx);
+            v[k] = (float)hx;
+            v[3 + k] = (float)(rx - hx);
+            v[7 + k] = (float)t[k];
+            v[10 + k] = (float)b[k];
+            v[13 + k] = (float)q[k];
+        }
+        v[6] = (float)L;
+        float4* d = reinterpret_cast<float4*>(f32);
+#pragma unroll
+        for (int e = 0; e < SRC32_STRIDE / 4; ++e) d[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+    }
+    if (fdf) {
+        constexpr double SC = 1.0 / (1 << -DF_SCALE);
+        // the source's frame: e along the part of b normal to t (any normal if
+        // there is none), made orthogonal to t a second time because b - (b.t) t
+        // loses digits when b is nearly along t
+        const double bt = fma(b[0], t[0], fma(b[1], t[1], b[2] * t[2]));
+        double v[3] = {fma(-bt, t[0], b[0]), fma(-bt, t[1], b[1]), fma(-bt, t[2], b[2])};
+        const double c0 = fma(v[0], t[0], fma(v[1], t[1], v[2] * t[2]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = fma(-c0, t[k], v[k]);
+        double vv = fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+        double ie = vv > 0.0 ? 1.0 / sqrt(vv) : 0.0;
+        const double be = vv * ie;
+        if (!(vv > 0.0)) {
+            const double ax = fabs(t[0]), ay = fabs(t[1]), az = fabs(t[2]);
+            const int m = ax <= ay && ax <= az ? 0 : (ay <= az ? 1 : 2);
+            const double tm = m == 0 ? t[0] : (m == 1 ? t[1] : t[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] = fma(-tm, t[k], k == m ? 1.0 : 0.0);
+            vv = fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+            ie = 1.0 / sqrt(vv);
+        }
+        double e[3] = {v[0] * ie, v[1] * ie, v[2] * ie};
+        const double c1 = fma(e[0], t[0], fma(e[1], t[1], e[2] * t[2]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) e[k] = fma(-c1, t[k], e[k]);
+        float f[SRCDF_STRIDE];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int i = (k + 1) % 3, j = (k + 2) % 3;
+            df_parts(x1[k], o[k], f + 3 * k);
+            const DF1 ft = df_split(t[k]), fe = df_split(e[k]), fn = df_split(fma(t[i], e[j], -(t[j] * e[i])));
+            f[9 + k] = ft.h;
+            f[12 + k] = ft.l;
+            f[15 + k] = fe.h;
+            f[18 + k] = fe.l;
+            f[21 + k] = fn.h;
+            f[24 + k] = fn.l;
+        }
+        const DF1 l = df_split(L * SC), ll = df_split(LL * (SC * SC)), fb = df_split(bt), fe = df_split(be);
+        f[27] = l.h;
+        f[28] = l.l;
+        f[29] = ll.h;
+        f[30] = ll.l;
+        f[31] = fb.h;
+        f[32] = fb.l;
+        f[33] = fe.h;
+        f[34] = fe.l;
+        f[35] = fmaxf((float)(DF_NEAR * DF_NEAR * SC * SC * a2), ll.h * (1.0f / 256.0f));
+        float4* d = reinterpret_cast<float4*>(fdf);
+#pragma unroll
+        for (int k = 0; k < SRCDF_STRIDE / 4; ++k) d[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+    }
+}
 
 __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, double Dx, double Dy, double Dz,
                                            const double bt[3], double acc[4][3])
@@ -73,69 +193,297 @@ __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, doubl
     fp[5 * st] = Fe[2];
 }
 
-// ------------------------------------------------------------------ FP64
-// smem: TILE * SRC_STRIDE doubles (as double2).
-template <int TILE>
-__device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& c, double2* tile)
+// ------------------------------------------------------------ near field
+// One near-field (Gauss point, source) pair in FP64: (sigma b') of source js
+// at Gauss point qp of target seg, from the FP64 records.
+__device__ __forceinline__ double3 near_field_fp64(const double* __restrict__ pos, int64_t n,
+                                                   const int32_t* __restrict__ nxt, const double* __restrict__ src,
+                                                   int64_t seg, int64_t js, int qp, const double* __restrict__ k64)
 {
+    const double a2 = k64[0], c1 = k64[1], c2 = k64[2];
+    const double* tr = src + (int64_t)SRC_STRIDE * seg;
+    const int64_t sb = nxt[seg];
+    const double xa = pos[seg], ya = pos[n + seg], za = pos[2 * n + seg];
+    const double Dx = pos[sb] - xa, Dy = pos[n + sb] - ya, Dz = pos[2 * n + sb] - za;
+    const double bt[3] = {tr[8], tr[9], tr[10]};
+    const double* r64 = src + (int64_t)SRC_STRIDE * js;
+    const double x1d[3] = {r64[0], r64[1], r64[2]};
+    const double td[3] = {r64[4], r64[5], r64[6]};
+    const double bd[3] = {r64[8], r64[9], r64[10]};
+    const double qd[3] = {r64[12], r64[13], r64[14]};
+    const double nr = -c1 / c2;
+    PairK kd;
+    pair_constants(td, qd, bt, nr, kd);
+    const double xi = gl4_xi(qp);
+    const double xq0 = __dadd_rn(xa, __dmul_rn(xi, Dx));
+    const double xq1 = __dadd_rn(ya, __dmul_rn(xi, Dy));
+    const double xq2 = __dadd_rn(za, __dmul_rn(xi, Dz));
+    double vd[3] = {0.0, 0.0, 0.0};
+    seg_sigma_b(xq0 - x1d[0], xq1 - x1d[1], xq2 - x1d[2], td, r64[3], bd, qd, bt, kd, a2, nr, vd);
+    return make_double3(c2 * vd[0], c2 * vd[1], c2 * vd[2]);
+}
+
+// Near pairs found by a warp wait in a per-warp queue of (source index,
+// owner lane << 2 | Gauss point) entries; a full queue is evaluated 32 at a
+// time, one entry per lane, so the FP64 work runs with every lane busy.
+// Each result goes to its owner's FP64 near sums in queue order, so the
+// summation order (and the result) does not depend on scheduling.
+constexpr int NEAR_Q = 160;  // <= 31 waiting + 128 added by one source (4 Gauss points x 32 lanes)
+
+// Evaluate the first cnt (<= 32) entries of a warp queue; warp-uniform call.
+static __device__ __noinline__ void near_flush(const double* __restrict__ pos, int64_t n,
+                                               const int32_t* __restrict__ nxt, const double* __restrict__ src,
+                                               const double* __restrict__ k64, int64_t seg,
+                                               const uint2* __restrict__ q, int cnt, double* __restrict__ nacc,
+                                               int tpb)
+{
+    const int lane = threadIdx.x & 31;
+    const uint2 e = lane < cnt ? q[lane] : make_uint2(0u, 0u);
+    const int64_t seg_o = __shfl_sync(0xffffffffu, (long long)seg, (int)((e.y >> 2) & 31u));
+    double3 d = make_double3(0.0, 0.0, 0.0);
+    if (lane < cnt) d = near_field_fp64(pos, n, nxt, src, seg_o, (int64_t)e.x, (int)(e.y & 3u), k64);
+    for (int k = 0; k < cnt; ++k) {
+        const double dx = __shfl_sync(0xffffffffu, d.x, k);
+        const double dy = __shfl_sync(0xffffffffu, d.y, k);
+        const double dz = __shfl_sync(0xffffffffu, d.z, k);
+        const unsigned tag = __shfl_sync(0xffffffffu, e.y, k);
+        if ((int)((tag >> 2) & 31u) == lane) {
+            double* acc = nacc + 3 * (int)(tag & 3u) * tpb + threadIdx.x;
+            acc[0] += dx;
+            acc[tpb] += dy;
+            acc[2 * tpb] += dz;
+        }
+    }
+}
+
+// Drop the first 32 entries of a warp queue holding cnt (32 < cnt <= NEAR_Q)
+// of them: chunk by chunk, each read before the chunk below it is overwritten.
+__device__ __forceinline__ void near_shift(uint2* q, int cnt)
+{
+    const int lane = threadIdx.x & 31;
+    for (int base = 32; base < cnt; base += 32) {
+        const uint2 u = base + lane < cnt ? q[base + lane] : make_uint2(0u, 0u);
+        __syncwarp();
+        if (base + lane < cnt) q[base - 32 + lane] = u;
+        __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------ FP64
+// FP64 results.  A (Gauss point, source) pair nearer than DF_NEAR a, or than
+// 1/16 of either segment's length, is evaluated in FP64 (near_flush); every
+// other pair in double-float arithmetic on the FP32 pipe (df_field.cuh).  The
+// rounding error of the nodal forces comes from the close pairs, whose field
+// is the largest and whose geometry cancels: against an 80-bit reference the
+// relative error of the forces (1e-12 to 3e-12 over the loop networks of 42 to
+// 1500 nodes) is the same to 0.1 % with every pair in FP64 and with the pairs
+// beyond 20 a, 32 a, 64 a or 256 a in double-float; a pair beyond 32 a errs by
+// 2e-14 of itself in the median.
+//
+// The sums over DF_GROUP tiles' sources are kept in double-float per Gauss
+// point (in shared memory: they are touched once per source, and the two
+// chains of Gauss points then share one copy of the code, which must fit the
+// instruction cache) and are added to FP64 sums when the group closes.
+// Coordinates enter as three FP32 parts (srcdf records), so that x_a - x1 is
+// exact to 2^-48 units; a pair outside their range, or with a distance or a
+// length of DF_FAR or more, is evaluated in FP64.  A tile is one warp's: no lane waits for
+// another warp, and a small network gives as many tiles as it has warps.
+constexpr int DF_REC = 64;            // floats of a staged source record
+constexpr int DF_TILE = 16;           // sources per staged tile
+constexpr int DF_GROUP = 4;           // staged tiles per group of double-float sums
+
+struct DFSmem {
+    // per source: t, e, n (h x 3, l x 3 each), L, L^2, bt, be (h, l each), every
+    // value in both lanes (26 float2), then x (9), the squared near limit
+    float4 rec[DF_TILE * DF_REC / 4];
+    float2 sum[16 * 32];  // double-float sums: [chain * 8 + 2 * e + part][thread], e = 3: along b'
+    double nacc[12 * 32];  // FP64 sums: [qp * 3 + e][thread]
+    double k64[3];          // {a2, c1, c2} for the near field
+    uint2 queue[NEAR_Q];
+};
+
+__device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& c, DFSmem& sm)
+{
+    constexpr double SC = 1.0 / (1 << -DF_SCALE);
+    constexpr float far2 = (float)(DF_FAR * DF_FAR * SC * SC);
     const int64_t n = a.n;
     const bool active = threadIdx.x < a.t_count;
     const int64_t seg = active ? a.tgt[a.t_begin + threadIdx.x] : a.tgt[a.t_begin];
-    const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
     const int64_t sb = a.nxt[seg];
-    const double xa = a.pos[seg], ya = a.pos[n + seg], za = a.pos[2 * n + seg];
-    const double Dx = a.pos[sb] - xa, Dy = a.pos[n + sb] - ya, Dz = a.pos[2 * n + sb] - za;
-    const double bt[3] = {tr[8], tr[9], tr[10]};
-    double xq[4][3];
+    float xt[9], lim_t;
+    DF1 D[3];
+    DF2 bt[3];
+    bool wide = false;  // a target too long for the double-float range
+    {
+        const float* fr = a.srcdf + (int64_t)SRCDF_STRIDE * seg;
 #pragma unroll
-    for (int qp = 0; qp < 4; ++qp) {
-        // x_q = x_a + xi_q (x_b - x_a), rounded as written (no contraction)
-        const double xi = gl4_xi(qp);
-        xq[qp][0] = __dadd_rn(xa, __dmul_rn(xi, Dx));
-        xq[qp][1] = __dadd_rn(ya, __dmul_rn(xi, Dy));
-        xq[qp][2] = __dadd_rn(za, __dmul_rn(xi, Dz));
+        for (int k = 0; k < 9; ++k) xt[k] = fr[k];
+        lim_t = fr[35];
+        const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            D[k] = df_split((a.pos[k * n + sb] - a.pos[k * n + seg]) * SC);
+            wide = wide || !(fabsf(D[k].h) < (float)(DF_FAR * SC));
+            bt[k] = df_all(df_split(tr[8 + k]));
+        }
     }
-    double acc[4][3];  // (sigma b') / c2 at the Gauss points, without the term along b'
-    double accb[4];    // coefficient sums of the term along b'
+    const DFConst K = c.df;
 #pragma unroll
-    for (int qp = 0; qp < 4; ++qp) acc[qp][0] = acc[qp][1] = acc[qp][2] = accb[qp] = 0.0;
-    const double nr = -c.c1 / c.c2, nra2 = nr * c.a2, kn = 1.0 - 2.0 * c.c1 / c.c2;
+    for (int k = 0; k < 12; ++k) sm.nacc[k * 32 + threadIdx.x] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) sm.sum[k * 32 + threadIdx.x] = p_all(0.0f);
+    if (threadIdx.x == 0) {
+        sm.k64[0] = c.a2;
+        sm.k64[1] = c.c1;
+        sm.k64[2] = c.c2;
+    }
+    const int lane = threadIdx.x;
+    const unsigned lt = (1u << lane) - 1u;
+    uint2* wq = sm.queue;
+    int qn = 0;  // entries waiting in this warp's queue (warp-uniform)
+    int open = 0;  // tiles in the open group
 
-    for (int64_t j0 = a.js; j0 < a.je; j0 += TILE) {
-        const int cnt = (int)min((int64_t)TILE, a.je - j0);
-        __syncthreads();
-        const double2* g = reinterpret_cast<const double2*>(a.src + (int64_t)SRC_STRIDE * j0);
-        for (int e = threadIdx.x; e < cnt * (SRC_STRIDE / 2); e += blockDim.x) tile[e] = g[e];
-        __syncthreads();
-        for (int jj = 0; jj < cnt; ++jj) {
-            const double* r = reinterpret_cast<const double*>(tile + jj * (SRC_STRIDE / 2));
-            const double L = r[3];
-            if (!(L > 0.0)) continue;  // zero-length source: no field (uniform branch)
-            const double x1[3] = {r[0], r[1], r[2]};
-            const double t[3] = {r[4], r[5], r[6]};
-            const double b[3] = {r[8], r[9], r[10]};
-            const double q[3] = {r[12], r[13], r[14]};
-            PairK k;
-            pair_constants(t, q, bt, nr, k);
-            // per Gauss point the geometry, then a vote: where every pair of
-            // the warp is one-sided the straddling forms are not evaluated
-            // (the FP64 pipe is the bound, so the branches cost nothing there)
+    for (int64_t j0 = a.js; j0 < a.je; j0 += DF_TILE) {
+        const int cnt = (int)min((int64_t)DF_TILE, a.je - j0);
+        __syncwarp();
+        // 9 float4 per source: x y z of 9, then the 26 values that go to both lanes, the limit
+        for (int e = threadIdx.x; e < cnt * 9; e += 32) {
+            const int js = e / 9, k = e - 9 * js;
+            const float4 u = reinterpret_cast<const float4*>(a.srcdf + (int64_t)SRCDF_STRIDE * (j0 + js))[k];
+            const float v[4] = {u.x, u.y, u.z, u.w};
+            float* d = reinterpret_cast<float*>(sm.rec + js * (DF_REC / 4));
 #pragma unroll
-            for (int qp = 0; qp < 4; ++qp) {
-                SegGeo G;
-                seg_geo(xq[qp][0] - x1[0], xq[qp][1] - x1[1], xq[qp][2] - x1[2], t, L, c.a2, G);
-                if (__all_sync(0xffffffffu, seg_one_side(G, L)))
-                    seg_sigma_b_geo<1>(G, t, L, b, q, bt, k, c.a2, nr, nra2, kn, acc[qp], accb[qp]);
+            for (int i = 0; i < 4; ++i) {
+                const int f = 4 * k + i;
+                if (f < 9)
+                    d[52 + f] = v[i];
+                else if (f < 35)
+                    reinterpret_cast<float2*>(d)[f - 9] = p_all(v[i]);
                 else
-                    seg_sigma_b_geo<0>(G, t, L, b, q, bt, k, c.a2, nr, nra2, kn, acc[qp], accb[qp]);
+                    d[61] = v[i];
+            }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int jj = 0; jj < cnt; ++jj) {
+            const float4* r4 = sm.rec + jj * (DF_REC / 4);
+            const float2* r2 = reinterpret_cast<const float2*>(r4);
+            if (!(r2[18].x > 0.0f)) continue;  // zero-length source: no field (uniform branch)
+            DFPair P;
+            float near2;
+            unsigned nr = 0u;  // Gauss points of this thread that go to FP64
+            bool out;
+            {
+                const float* x = reinterpret_cast<const float*>(r4 + 13);
+                DF2 RD[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) RD[k] = df_pair2(df_diff(xt + 3 * k, x + 3 * k), D[k]);
+                near2 = fmaxf(lim_t, x[9]);
+                out = wide || !(r2[18].x < (float)(DF_FAR * SC)) ||
+                      !(RD[0].h.x * RD[0].h.x + RD[1].h.x * RD[1].h.x + RD[2].h.x * RD[2].h.x < far2);
+                const DF2 t[3] = {{r2[0], r2[3]}, {r2[1], r2[4]}, {r2[2], r2[5]}};
+                const DF2 e[3] = {{r2[6], r2[9]}, {r2[7], r2[10]}, {r2[8], r2[11]}};
+                const DF2 m[3] = {{r2[12], r2[15]}, {r2[13], r2[16]}, {r2[14], r2[17]}};
+                P.y = df_dot(RD, t);
+                P.al = df_dot(RD, e);
+                P.be = df_dot(RD, m);
+                DF2 te[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    te[k] = DF2{make_float2(t[k].h.x, e[k].h.x), make_float2(t[k].l.x, e[k].l.x)};
+                const DF2 w = df_dot(te, bt);
+                P.tb = DF1{w.h.x, w.l.x};
+                P.eb = DF1{w.h.y, w.l.y};
+                const DF2 u = df_dot(m, bt);
+                P.nb = DF1{u.h.x, u.l.x};
+            }
+            if (__any_sync(0xffffffffu, out)) {
+                nr = 15u;
+            } else {
+#pragma unroll 1
+                for (int ch = 0; ch < 2; ++ch) {
+                    constexpr DF1 x0 = df_from(gl4_xi(0)), x1 = df_from(gl4_xi(1)), x2 = df_from(gl4_xi(2)),
+                                  x3 = df_from(gl4_xi(3));
+                    const DF2 xi = ch ? df_pair2(x2, x3) : df_pair2(x0, x1);
+                    const DF2 L = {r2[18], r2[19]}, LL = {r2[20], r2[21]}, sbt = {r2[22], r2[23]}, sbe = {r2[24], r2[25]};
+                    DFGeo G;
+                    df_geo(P, xi, L, K, G);
+                    const float ddx = G.y.h.x < 0.0f ? G.r1s.h.x : (G.u2.h.x < 0.0f ? G.r2s.h.x : G.d2.h.x);
+                    const float ddy = G.y.h.y < 0.0f ? G.r1s.h.y : (G.u2.h.y < 0.0f ? G.r2s.h.y : G.d2.h.y);
+                    const Lanes far = {!(ddx < near2), !(ddy < near2)};
+                    nr |= ((far.x ? 0u : 1u) | (far.y ? 0u : 2u)) << (2 * ch);
+                    DF2 St, Se, Sn, cb;
+                    df_field(G, P, L, LL, sbt, sbe, K, far, St, Se, Sn, cb);
+                    float2* acc = sm.sum + (ch * 8) * 32 + threadIdx.x;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        DF2 s = {acc[2 * k * 32], acc[(2 * k + 1) * 32]};
+                        s = df_fma(St, DF2{r2[k], r2[3 + k]}, s);
+                        s = df_fma(Se, DF2{r2[6 + k], r2[9 + k]}, s);
+                        s = df_fma(Sn, DF2{r2[12 + k], r2[15 + k]}, s);
+                        acc[2 * k * 32] = s.h;
+                        acc[(2 * k + 1) * 32] = s.l;
+                    }
+                    const DF2 s = df_add(DF2{acc[6 * 32], acc[7 * 32]}, cb);
+                    acc[6 * 32] = s.h;
+                    acc[7 * 32] = s.l;
+                }
+            }
+            if (__any_sync(0xffffffffu, active && nr != 0u)) {
+                const unsigned js = (unsigned)(j0 + jj);
+#pragma unroll 1
+                for (int qp = 0; qp < 4; ++qp) {
+                    const bool mine = active && ((nr >> qp) & 1u);
+                    const unsigned bal = __ballot_sync(0xffffffffu, mine);
+                    if (mine) wq[qn + __popc(bal & lt)] = make_uint2(js, ((unsigned)lane << 2) | (unsigned)qp);
+                    qn += __popc(bal);
+                }
+                while (qn >= 32) {
+                    __syncwarp();
+                    near_flush(a.pos, n, a.nxt, a.src, sm.k64, seg, wq, 32, sm.nacc, 32);
+                    near_shift(wq, qn);
+                    qn -= 32;
+                }
+            }
+        }
+        if (++open == DF_GROUP || j0 + DF_TILE >= a.je) {
+            // the group's sums to FP64, restoring the factor c2 and the unit of length
+            open = 0;
+            const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
+            const double k2 = c.c2 * SC;
+#pragma unroll 1
+            for (int ch = 0; ch < 2; ++ch) {
+                float2* q = sm.sum + (ch * 8) * 32 + threadIdx.x;
+                const double bx = (double)q[6 * 32].x + (double)q[7 * 32].x;
+                const double by = (double)q[6 * 32].y + (double)q[7 * 32].y;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    double* acc = sm.nacc + (6 * ch + e) * 32 + threadIdx.x;
+                    const float2 h = q[2 * e * 32], l = q[(2 * e + 1) * 32];
+                    acc[0] = fma(k2, fma(bx, tr[8 + e], (double)h.x + (double)l.x), acc[0]);
+                    acc[3 * 32] = fma(k2, fma(by, tr[8 + e], (double)h.y + (double)l.y), acc[3 * 32]);
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) q[k * 32] = p_all(0.0f);
             }
         }
     }
+    if (qn > 0) {
+        __syncwarp();
+        near_flush(a.pos, n, a.nxt, a.src, sm.k64, seg, wq, qn, sm.nacc, 32);
+    }
+    __syncwarp();
+    if (!active) return;
+    const double xa = a.pos[seg], ya = a.pos[n + seg], za = a.pos[2 * n + seg];
+    const double Dx = a.pos[sb] - xa, Dy = a.pos[n + sb] - ya, Dz = a.pos[2 * n + sb] - za;
+    const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
+    const double b64[3] = {tr[8], tr[9], tr[10]};
+    double acc[4][3];
 #pragma unroll
     for (int qp = 0; qp < 4; ++qp)
 #pragma unroll
-        for (int e = 0; e < 3; ++e) acc[qp][e] = c.c2 * fma(accb[qp], bt[e], acc[qp][e]);
-    if (active) tile_store(a, seg, Dx, Dy, Dz, bt, acc);
+        for (int e = 0; e < 3; ++e) acc[qp][e] = sm.nacc[(3 * qp + e) * 32 + threadIdx.x];
+    tile_store(a, seg, Dx, Dy, Dz, b64, acc);
 }
 
 // ----------------------------------------------------------------- mixed
@@ -315,42 +663,6 @@ __device__ __forceinline__ void seg_coef2(const Geo2& G, const Src2& S, const fl
     C.cb = mul2(qR, B0);
 }
 
-// One near-field (Gauss point, source) pair in FP64: (sigma b') of source js
-// at Gauss point qp of target seg, from the FP64 records.
-__device__ __forceinline__ double3 near_field_fp64(const double* __restrict__ pos, int64_t n,
-                                                   const int32_t* __restrict__ nxt, const double* __restrict__ src,
-                                                   int64_t seg, int64_t js, int qp, const double* __restrict__ k64)
-{
-    const double a2 = k64[0], c1 = k64[1], c2 = k64[2];
-    const double* tr = src + (int64_t)SRC_STRIDE * seg;
-    const int64_t sb = nxt[seg];
-    const double xa = pos[seg], ya = pos[n + seg], za = pos[2 * n + seg];
-    const double Dx = pos[sb] - xa, Dy = pos[n + sb] - ya, Dz = pos[2 * n + sb] - za;
-    const double bt[3] = {tr[8], tr[9], tr[10]};
-    const double* r64 = src + (int64_t)SRC_STRIDE * js;
-    const double x1d[3] = {r64[0], r64[1], r64[2]};
-    const double td[3] = {r64[4], r64[5], r64[6]};
-    const double bd[3] = {r64[8], r64[9], r64[10]};
-    const double qd[3] = {r64[12], r64[13], r64[14]};
-    const double nr = -c1 / c2;
-    PairK kd;
-    pair_constants(td, qd, bt, nr, kd);
-    const double xi = gl4_xi(qp);
-    const double xq0 = __dadd_rn(xa, __dmul_rn(xi, Dx));
-    const double xq1 = __dadd_rn(ya, __dmul_rn(xi, Dy));
-    const double xq2 = __dadd_rn(za, __dmul_rn(xi, Dz));
-    double vd[3] = {0.0, 0.0, 0.0};
-    seg_sigma_b(xq0 - x1d[0], xq1 - x1d[1], xq2 - x1d[2], td, r64[3], bd, qd, bt, kd, a2, nr, vd);
-    return make_double3(c2 * vd[0], c2 * vd[1], c2 * vd[2]);
-}
-
-// Near pairs found by a warp wait in a per-warp queue of (source index,
-// owner lane << 2 | Gauss point) entries; a full queue is evaluated 32 at a
-// time, one entry per lane, so the FP64 work runs with every lane busy.
-// Each result goes to its owner's FP64 near sums in queue order, so the
-// summation order (and the result) does not depend on scheduling.
-constexpr int NEAR_Q = 160;  // <= 31 waiting + 128 added by one source (4 Gauss points x 32 lanes)
-
 template <int TILE, int TPB>
 struct MixSmem {
     float2 tile[TILE * MIX_REC];  // source records (MIX_REC float2 each)
@@ -358,45 +670,6 @@ struct MixSmem {
     float2 ksum[12 * TPB];             // Kahan sums of the work item: [p * 3 + e][thread], then compensations
     uint2 queue[TPB / 32][NEAR_Q];
 };
-
-// Evaluate the first cnt (<= 32) entries of a warp queue; warp-uniform call.
-static __device__ __noinline__ void near_flush(const double* __restrict__ pos, int64_t n,
-                                               const int32_t* __restrict__ nxt, const double* __restrict__ src,
-                                               const double* __restrict__ k64, int64_t seg,
-                                               const uint2* __restrict__ q, int cnt, double* __restrict__ nacc,
-                                               int tpb)
-{
-    const int lane = threadIdx.x & 31;
-    const uint2 e = lane < cnt ? q[lane] : make_uint2(0u, 0u);
-    const int64_t seg_o = __shfl_sync(0xffffffffu, (long long)seg, (int)((e.y >> 2) & 31u));
-    double3 d = make_double3(0.0, 0.0, 0.0);
-    if (lane < cnt) d = near_field_fp64(pos, n, nxt, src, seg_o, (int64_t)e.x, (int)(e.y & 3u), k64);
-    for (int k = 0; k < cnt; ++k) {
-        const double dx = __shfl_sync(0xffffffffu, d.x, k);
-        const double dy = __shfl_sync(0xffffffffu, d.y, k);
-        const double dz = __shfl_sync(0xffffffffu, d.z, k);
-        const unsigned tag = __shfl_sync(0xffffffffu, e.y, k);
-        if ((int)((tag >> 2) & 31u) == lane) {
-            double* acc = nacc + 3 * (int)(tag & 3u) * tpb + threadIdx.x;
-            acc[0] += dx;
-            acc[tpb] += dy;
-            acc[2 * tpb] += dz;
-        }
-    }
-}
-
-// Drop the first 32 entries of a warp queue holding cnt (32 < cnt <= NEAR_Q)
-// of them: chunk by chunk, each read before the chunk below it is overwritten.
-__device__ __forceinline__ void near_shift(uint2* q, int cnt)
-{
-    const int lane = threadIdx.x & 31;
-    for (int base = 32; base < cnt; base += 32) {
-        const uint2 u = base + lane < cnt ? q[base + lane] : make_uint2(0u, 0u);
-        __syncwarp();
-        if (base + lane < cnt) q[base - 32 + lane] = u;
-        __syncwarp();
-    }
-}
 
 template <int TILE, int TPB>
 __device__ __forceinline__ void pair_tile_mixed(const TileArgs& a, const Consts& c, float near2,

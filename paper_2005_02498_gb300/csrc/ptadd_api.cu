@@ -6,12 +6,15 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
 #include "ptadd_internal.cuh"
 
 namespace ptadd {
+
+constexpr int FPART_MAX_CHUNKS = 512;
 
 static thread_local char g_err[1024] = "no error";
 
@@ -47,22 +50,13 @@ static void free_network(DevNetwork& n)
 {
     void* ptrs[] = {n.pos[0], n.pos[1], n.nxt,   n.prv,   n.loop_of, n.loop_b,  n.loop_n, n.pinned, n.tgt_burst,
                     n.tgt_all, n.src,    n.fpart, n.vel,   n.force,   n.partial, n.acc,    n.flag,   n.staging,
-                    n.src32,   n.near_count, n.k64, n.loop_off, n.cm_scratch};
+                    n.src32,   n.srcdf, n.near_count, n.k64, n.loop_off, n.cm_scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     n = DevNetwork{};
 }
 
-static Consts make_consts(const ptadd_ctx* ctx)
-{
-    const ptadd_material& m = ctx->mat;
-    Consts c;
-    const double r = m.a / ctx->len_unit;
-    c.a2 = r * r;
-    c.c1 = 1.0 / (8.0 * M_PI);
-    c.c2 = 1.0 / (4.0 * M_PI * (1.0 - m.nu));
-    return c;
-}
+static Consts make_consts(const ptadd_ctx* ctx) { return make_consts(ctx->mat.a / ctx->len_unit, ctx->mat.nu); }
 
 }  // namespace ptadd
 
@@ -213,7 +207,11 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
         if (!(pinned && pinned[i] && pinned[nxt[i]])) tb.push_back((int32_t)i);
     }
     net.n_tgt_burst = (int64_t)tb.size();
-    net.max_chunks = 64;
+    // the most chunks any evaluation of this network splits its sources into
+    net.max_chunks = 1;
+    for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
+        for (int64_t nt : {net.n_tgt_burst, n})
+            net.max_chunks = std::max(net.max_chunks, choose_chunks(nt, n, FPART_MAX_CHUNKS, prec));
     net.max_red_blocks = (int)((n + 255) / 256);
 
     ptadd_status st = PTADD_OK;
@@ -238,6 +236,7 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     ALLOC(net.flag, 1);
     ALLOC(net.staging, 3 * n);
     ALLOC(net.src32, SRC32_STRIDE * n);
+    ALLOC(net.srcdf, SRCDF_STRIDE * n);
     ALLOC(net.near_count, 1);
     ALLOC(net.k64, 4);
     ALLOC(net.loop_off, n_loops + 1);
@@ -329,7 +328,7 @@ static ptadd_status eval_forces(ptadd_ctx* ctx, const int32_t* tgt, int64_t n_tg
     cudaStream_t s = ctx->stream;
     if (n_tgt < net.n_nodes)
         PTADD_CUDA(cudaMemsetAsync(net.fpart, 0, (size_t)chunks * 6 * net.n_nodes * sizeof(double), s));
-    PTADD_CUDA(launch_seg_prep(net, s));
+    PTADD_CUDA(launch_seg_prep(net, (int)ctx->prec, c, s));
     std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
     if (ctx->timing && n_tgt > 0) {
         ptadd_status st = take_events(ctx, ev);

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/ptadd.h"
+#include "df_field.cuh"
 
 struct ptadd_ctx;
 
@@ -48,6 +49,12 @@ constexpr int SRC_STRIDE = 16;
 // own (integer origin Ot nearby) as (x1_hi - Ot) + x1_lo with one rounding,
 // and R0 = x - x1 keeps ~1e-7 relative accuracy for every pair.
 constexpr int SRC32_STRIDE = 16;
+// Double-float record of the FP64 path (36 floats, lengths scaled by 2^DF_SCALE):
+//   [0..8] x1 - origin per coordinate as an integer, a multiple of 2^-23 below
+//   1/2 and the rest   [9..11] t high parts [12..14] t low parts   [15..20] e, the
+//   same   [21..26] n = t x e   [27..28] L   [29..30] L^2   [31..32] b.t   [33..34] b.e
+//   [35] squared near limit of the segment (df_field.cuh has the frame t, e, n)
+constexpr int SRCDF_STRIDE = 36;
 // Near field of the mixed path: point-to-segment distance below 10 a, with a
 // 1 % margin in favour of FP64 on the FP32 estimate of that distance.
 constexpr double NEAR_FACTOR = 10.1;
@@ -68,7 +75,9 @@ struct DevNetwork {
     int32_t* tgt_all = nullptr;    // every segment
     double* src = nullptr;         // [n*SRC_STRIDE]
     float* src32 = nullptr;        // [n*SRC32_STRIDE] FP32 records of the mixed path
-    double origin[3] = {0, 0, 0};  // integer-valued origin of the FP32 hi/lo split
+    float* srcdf = nullptr;        // [n*SRCDF_STRIDE] double-float records of the FP64 path
+    double origin[3] = {0, 0, 0};  // integer-valued origin of the FP32 records
+    bool origin_node0 = false;     // instead: node 0's position rounded (read on the device)
     unsigned long long* near_count = nullptr;  // FP64 point-pairs of the mixed path
     double* k64 = nullptr;         // {a2, c1, c2} for the near-field path of the mixed kernel
     double* fpart = nullptr;       // [max_chunks*6*n] partial nodal-force parts
@@ -91,11 +100,22 @@ struct Consts {
     double a2;   // (a/l)^2
     double c1;   // 1/(8 pi)
     double c2;   // 1/(4 pi (1 - nu))
+    DFConst df;  // the FP64 path's far field
 };
+inline Consts make_consts(double a_internal, double nu)
+{
+    Consts c;
+    c.a2 = a_internal * a_internal;
+    c.c1 = 1.0 / (8.0 * 3.14159265358979323846);
+    c.c2 = 1.0 / (4.0 * 3.14159265358979323846 * (1.0 - nu));
+    const double sc = 1.0 / (1 << -DF_SCALE), r = -c.c1 / c.c2;
+    c.df = DFConst{df_from(c.a2 * (sc * sc)), df_from(r), df_from(r * c.a2 * (sc * sc)), df_from(1.0 + 2.0 * r)};
+    return c;
+}
 
 // ------------------------------------------------------------ launchers
 // All return cudaGetLastError() of their launches.
-cudaError_t launch_seg_prep(const DevNetwork& net, cudaStream_t st);
+cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& c, cudaStream_t st);
 // pair stage: writes fpart[chunk][6][seg] for the listed targets
 cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt, int chunks,
                         int precision, const Consts& c, const double sig_hat[6], cudaStream_t st);
@@ -112,6 +132,8 @@ cudaError_t launch_consistent_velocity_raw(int64_t n_loops, const int64_t* loop_
 // Lp/rho sample of the step-start state, Euler update into the other buffer,
 // and the fixed-order reduction into net.acc (weighted by dt_hat)
 cudaError_t launch_lp_euler(DevNetwork& net, double dt_hat, cudaStream_t st);
+// sources per FP64 work item for a number of one-warp target tiles
+int64_t fp64_chunk_len(int64_t tiles, int64_t n_src);
 int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision);
 
 // peak microbenchmark

@@ -70,6 +70,13 @@ __device__ __forceinline__ double f2d_seed(float y)
     const unsigned hi = (u & 0x80000000u) | ((((u >> 23) & 0xFFu) + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
     return __hiloint2double((int)hi, (int)(u << 29));
 }
+// The same for any finite value: 0 below FP32's normal range (an underflow
+// the callers can leave out), saturated above it.
+__device__ __forceinline__ float d2f_seed0(double x)
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) > 896u ? d2f_seed(x) : 0.0f;
+}
+__device__ __forceinline__ double f2d_seed0(float y) { return y != 0.0f ? f2d_seed(y) : 0.0; }
 __device__ __forceinline__ double rcp_nr(double x)
 {
     const double y = f2d_seed(rcp_approx(d2f_seed(x)));
@@ -132,15 +139,8 @@ __device__ __forceinline__ bool seg_one_side(const SegGeo& G, double L) { return
 //   c_Rp = (q.Rp)(K2 (Rp.b') - K3 t.b') - J0 q.b',
 //   c_t = r A0 (Rp.(b x b')) + C1 q.b' + (q.Rp)(K4 t.b' - K3 (Rp.b')),
 //   c_b = (q.Rp) B0,
-// with Rp.(b x b') evaluated as b'.(Rp x b), reusing Rp x b.  SAME = 1: the
-// caller knows the pair is one-sided; the one-side integrals then come from
-// the single reciprocal rr = 1 / ((p + m)(1 + pm)(1/rho1 + 1/rho2)) through
-// Q = Li rr: J0 = Li / (p + m) = Q (1 + pm) isum, J1 = Li / isum =
-// Q (p + m)(1 + pm), K2 = J0 W = Q (isum Aw + (1 + pm) isum ssum), where
-// W = Aw / (1 + pm) + ssum and Aw = ssum - d^2 / (rho1^2 rho2^2) =
-// (u1^2 + u2^2 + d^2) / (rho1^2 rho2^2) >= ssum / 2.  SAME = 0: either form,
-// chosen per pair.
-template <int SAME>
+// with Rp.(b x b') evaluated as b'.(Rp x b), reusing Rp x b.  The FP64 kernels
+// evaluate only close pairs with it (df_field.cuh has the others').
 __device__ __forceinline__ void seg_sigma_b_geo(const SegGeo& G, const double t[3], double L, const double b[3],
                                                 const double q[3], const double bt[3], const PairK& k, double a2,
                                                 double nr, double nra2, double kn, double s[3], double& sb)
@@ -155,25 +155,14 @@ __device__ __forceinline__ void seg_sigma_b_geo(const SegGeo& G, const double t[
     const double isum = i1 + i2, ssum = i1s + i2s;
     const double pps = p + m, one_pm = 1.0 + pm;
     const double Li = L * (u2 - y) * i12;  // L (u1 + u2) / (rho1^2 rho2^2)
-    double J0, J1, K2;
-    if (SAME) {
-        const double T = one_pm * isum, den = pps * one_pm;
-        const double rr = rcp_nr(pps * T);
-        const double Z = fma(isum, fma(-d2, i12, ssum), T * ssum);
-        const double Q = Li * rr;
-        J0 = Q * T;
-        J1 = Q * den;
-        K2 = Q * Z;
-    } else {
-        const bool same = seg_one_side(G, L);
-        const double den = same ? pps * one_pm : d2;
-        const double rr = rcp_nr(den * isum);
-        const double rden = rr * isum;  // 1/den
-        J1 = Li * (rr * den);
-        J0 = same ? (Li * rden) * one_pm : (p - m) * rden;
-        const double Wt = same ? fma((r1s + u2 * u2) * i12 * rden, pps, ssum) : (3.0 - S) * rden;
-        K2 = J0 * Wt;
-    }
+    const bool same = seg_one_side(G, L);
+    const double den = same ? pps * one_pm : d2;
+    const double rr = rcp_nr(den * isum);
+    const double rden = rr * isum;  // 1/den
+    const double J1 = Li * (rr * den);
+    const double J0 = same ? (Li * rden) * one_pm : (p - m) * rden;
+    const double Wt = same ? fma((r1s + u2 * u2) * i12 * rden, pps, ssum) : (3.0 - S) * rden;
+    const double K2 = J0 * Wt;
     const double K3 = J1 * fma(i1, i2, ssum);
     const double K4 = J0 * S;
     const double B0 = fma(a2, K2, J0);
@@ -205,7 +194,7 @@ __device__ __forceinline__ void seg_sigma_b(double R0x, double R0y, double R0z, 
     SegGeo G;
     seg_geo(R0x, R0y, R0z, t, L, a2, G);
     double sb = 0.0;
-    seg_sigma_b_geo<0>(G, t, L, b, q, bt, k, a2, nr, nr * a2, 1.0 + 2.0 * nr, s, sb);
+    seg_sigma_b_geo(G, t, L, b, q, bt, k, a2, nr, nr * a2, 1.0 + 2.0 * nr, s, sb);
     s[0] = fma(sb, bt[0], s[0]);
     s[1] = fma(sb, bt[1], s[1]);
     s[2] = fma(sb, bt[2], s[2]);
@@ -213,12 +202,12 @@ __device__ __forceinline__ void seg_sigma_b(double R0x, double R0y, double R0z, 
 
 // Gauss-Legendre rule on [0,1]: the textbook 4-point abscissae z and
 // weights W on [-1,1] mapped by xi = (1 + z)/2, w = W/2.
-__device__ __forceinline__ double gl4_xi(int qp)
+__host__ __device__ __forceinline__ constexpr double gl4_xi(int qp)
 {
     constexpr double z0 = 0.8611363115940526, z1 = 0.3399810435848563;
     return qp == 0 ? 0.5 * (1.0 - z0) : qp == 1 ? 0.5 * (1.0 - z1) : qp == 2 ? 0.5 * (1.0 + z1) : 0.5 * (1.0 + z0);
 }
-__device__ __forceinline__ double gl4_w(int qp)
+__host__ __device__ __forceinline__ constexpr double gl4_w(int qp)
 {
     constexpr double W0 = 0.3478548451374538, W1 = 0.6521451548625461;
     return (qp == 0 || qp == 3) ? 0.5 * W0 : 0.5 * W1;
