@@ -4,17 +4,15 @@
 //
 // Layout: the realisations' nodes are concatenated (realisation r owns nodes
 // [node_off[r], node_off[r+1])); every per-node table is indexed globally.
-// One DD step is five phases, each one launch (nine with junctions: release,
-// capture search and hold after the node phase, the clock event at the end):
-//   prep     : source records (FP64 + FP32 hi/lo about the realisation's origin)
-//   pair     : PERSISTENT kernel (one block per SM slot) that pulls work tiles
-//              (realisation, <= TPB targets, source chunk) from a list sorted
-//              by cost, largest first, through one atomic counter, so the
-//              256x spread of N_r^2 does not leave SMs idle;
-//   node     : nodal force = sum of the chunk parts, glide mobility;
-//   lp_euler : per-block partial Lp/rho sums (a block never spans two
-//              realisations) and the Euler update;
-//   finish   : one block per realisation sums its partials in a fixed order.
+// One DD step is two launches (more with junctions: release, capture search and
+// hold act on the velocities between the halves of the second, the clock event
+// follows):
+//   pair : PERSISTENT kernel (one block per SM slot) that pulls work tiles
+//          (realisation, targets, source chunk) from a list sorted by cost,
+//          largest first, through one atomic counter, so the 256x spread of N_r^2
+//          does not leave SMs idle;
+//   step : nodal forces = sums of the chunk parts, mobility, Lp/rho sums, the Euler
+//          update, the next step's source records (step.cu).
 // Kernel boundaries order the phases (no device-side barrier, nothing to spin
 // on).  Two steps (position buffers 0->1->0) are captured once into a CUDA
 // graph and replayed, so a 2000-step burst costs 1000 graph launches.
@@ -38,6 +36,7 @@
 
 #include "pair_tile.cuh"
 #include "ptadd_internal.cuh"
+#include "step.cuh"
 
 namespace ptadd {
 
@@ -66,7 +65,7 @@ struct DevBatch {
     double* src = nullptr;
     float* src32 = nullptr;
     float* srcdf = nullptr;
-    double *fpart = nullptr, *vel = nullptr, *force = nullptr, *partial = nullptr, *acc = nullptr;
+    double *fpart = nullptr, *vel = nullptr, *force = nullptr, *part = nullptr, *acc = nullptr;
     std::vector<double> last_LV;  // [3R] (1/|B|) sum L vbar of the last burst, time-averaged, SI
     int64_t fpart_cap = 0;  // doubles
     // per realisation (device)
@@ -75,11 +74,11 @@ struct DevBatch {
     int32_t* d_chunks = nullptr;
     double* d_origin = nullptr;  // 3R
     double* d_sh = nullptr;      // 6R
-    // lp reduction: block b covers nodes [blk_start[b], blk_start[b] + RED) of realisation blk_real[b]
-    int32_t* d_blk_real = nullptr;
-    int64_t* d_blk_start = nullptr;
-    int32_t* d_real_blk = nullptr;  // R+1
-    int nblk = 0;
+    int32_t* grp_off = nullptr;   // node groups of the step kernels (step.cuh)
+    int32_t* real_grp = nullptr;  // [R+1] first group of each realisation
+    int n_grp = 0;
+    bool grp_whole = true;
+    int max_chunks = 1;           // of the current work list
     WorkItem* d_items = nullptr;
     int n_items = 0;
     unsigned* counter = nullptr;
@@ -95,6 +94,7 @@ struct DevBatch {
     int tuned = 0;
     // graph of two steps
     cudaGraphExec_t graph = nullptr;
+    int64_t graph_launches = 0;  // kernels it holds
     double graph_dt = 0.0;
     int graph_prec = -1;
     int graph_cur = -1;
@@ -102,7 +102,7 @@ struct DevBatch {
     bool graph_cons = false;
     bool consistent = false;          // consistent mobility in this burst (the context's setting)
     int64_t* d_loop_off = nullptr;    // [n_loops + 1] (consistent mobility)
-    double* cm_scratch = nullptr;     // [5 n] (consistent mobility)
+    double* cm_scratch = nullptr;     // [10 n] (consistent mobility)
     DevBatchJunctions* junc = nullptr;  // junctions (ptadd_batch_set_junctions), NULL: off
     double dt_s = 0.0;                  // the step of the current burst, s (the junction clock)
     double time_scale = 0.0;            // mu / B: internal time -> s
@@ -110,7 +110,6 @@ struct DevBatch {
 
 namespace {
 
-constexpr int BRED = 256;   // nodes per reduction block
 // sources per staged tile of the mixed kernel: 192 at 128 threads (3 blocks
 // of 66.5 KB fit one SM's shared memory), 128 at 64 threads
 template <int TPB>
@@ -218,132 +217,6 @@ __global__ void __launch_bounds__(32, 16) batch_pair_fp64_kernel(BatchPairArgs b
             __syncwarp();
         }
     }
-}
-
-__global__ void batch_node_kernel(int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt,
-                                  const int32_t* __restrict__ prv, const int32_t* __restrict__ loop_of,
-                                  const int32_t* __restrict__ real_of, const double* __restrict__ loop_n,
-                                  const uint8_t* __restrict__ pinned, const int64_t* __restrict__ node_off,
-                                  const int64_t* __restrict__ fp_base, const int32_t* __restrict__ chunks,
-                                  const double* __restrict__ fpart, double* __restrict__ force,
-                                  double* __restrict__ vel)
-{
-    const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (a >= n) return;
-    const int r = real_of[a];
-    const int64_t base = node_off[r], nr = node_off[r + 1] - base;
-    const int64_t la = a - base, lp = prv[a] - base;
-    const double* fp0 = fpart + fp_base[r];
-    double F[3] = {0, 0, 0};
-    const int nch = chunks[r];
-    for (int ch = 0; ch < nch; ++ch) {
-        const double* fp = fp0 + (int64_t)ch * 6 * nr;
-        F[0] += fp[0 * nr + la] + fp[3 * nr + lp];
-        F[1] += fp[1 * nr + la] + fp[4 * nr + lp];
-        F[2] += fp[2 * nr + la] + fp[5 * nr + lp];
-    }
-    const int64_t p = prv[a], nx = nxt[a];
-    const double xa = pos[a], ya = pos[n + a], za = pos[2 * n + a];
-    const double px = xa - pos[p], py = ya - pos[n + p], pz = za - pos[2 * n + p];
-    const double qx = pos[nx] - xa, qy = pos[n + nx] - ya, qz = pos[2 * n + nx] - za;
-    const double M = 0.5 * (sqrt(px * px + py * py + pz * pz) + sqrt(qx * qx + qy * qy + qz * qz));
-    const int k = loop_of[a];
-    const double nn[3] = {loop_n[3 * k], loop_n[3 * k + 1], loop_n[3 * k + 2]};
-    double v[3] = {0, 0, 0};
-    if (!pinned[a] && M > 0.0) {
-        const double nF = nn[0] * F[0] + nn[1] * F[1] + nn[2] * F[2];
-        v[0] = (F[0] - nn[0] * nF) / M;
-        v[1] = (F[1] - nn[1] * nF) / M;
-        v[2] = (F[2] - nn[2] * nF) / M;
-    }
-    force[a] = F[0]; force[n + a] = F[1]; force[2 * n + a] = F[2];
-    vel[a] = v[0]; vel[n + a] = v[1]; vel[2 * n + a] = v[2];
-}
-
-// per-segment sums of the step-start state: L b (x) (t x vbar) (9), L (1), L vbar (3)
-constexpr int BSUM = 13;
-
-__global__ void __launch_bounds__(BRED) batch_lp_euler_kernel(
-    int64_t n, const double* __restrict__ pos, double* __restrict__ pos_next, const int32_t* __restrict__ nxt,
-    const int32_t* __restrict__ loop_of, const double* __restrict__ loop_b, const double* __restrict__ vel,
-    const int32_t* __restrict__ blk_real, const int64_t* __restrict__ blk_start,
-    const int64_t* __restrict__ node_off, double dt, double* __restrict__ partial, int* __restrict__ flag)
-{
-    __shared__ double red[BRED / 32][BSUM];
-    const int r = blk_real[blockIdx.x];
-    const int64_t i = blk_start[blockIdx.x] + threadIdx.x;
-    const bool in = i < node_off[r + 1];
-    double v13[BSUM];
-#pragma unroll
-    for (int m = 0; m < BSUM; ++m) v13[m] = 0.0;
-    if (in) {
-        const int64_t j = nxt[i];
-        const double dx = pos[j] - pos[i], dy = pos[n + j] - pos[n + i], dz = pos[2 * n + j] - pos[2 * n + i];
-        const double vx = 0.5 * (vel[i] + vel[j]);
-        const double vy = 0.5 * (vel[n + i] + vel[n + j]);
-        const double vz = 0.5 * (vel[2 * n + i] + vel[2 * n + j]);
-        const double cx = dy * vz - dz * vy, cy = dz * vx - dx * vz, cz = dx * vy - dy * vx;
-        const int k = loop_of[i];
-        const double b0 = loop_b[3 * k], b1 = loop_b[3 * k + 1], b2 = loop_b[3 * k + 2];
-        const double L = sqrt(dx * dx + dy * dy + dz * dz);
-        v13[0] = b0 * cx; v13[1] = b0 * cy; v13[2] = b0 * cz;
-        v13[3] = b1 * cx; v13[4] = b1 * cy; v13[5] = b1 * cz;
-        v13[6] = b2 * cx; v13[7] = b2 * cy; v13[8] = b2 * cz;
-        v13[9] = L;
-        v13[10] = L * vx; v13[11] = L * vy; v13[12] = L * vz;
-        const double nxp = __dadd_rn(pos[i], __dmul_rn(vel[i], dt));
-        const double nyp = __dadd_rn(pos[n + i], __dmul_rn(vel[n + i], dt));
-        const double nzp = __dadd_rn(pos[2 * n + i], __dmul_rn(vel[2 * n + i], dt));
-        pos_next[i] = nxp;
-        pos_next[n + i] = nyp;
-        pos_next[2 * n + i] = nzp;
-        if (!isfinite(nxp) || !isfinite(nyp) || !isfinite(nzp)) atomicOr(flag, 1);
-    }
-#pragma unroll
-    for (int m = 0; m < BSUM; ++m) {
-        double v = v13[m];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][m] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < BSUM) {
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < BRED / 32; ++w) s += red[w][threadIdx.x];
-        partial[(int64_t)blockIdx.x * BSUM + threadIdx.x] = s;
-    }
-}
-
-// One block per realisation: its partials in order, weighted by dt, into
-// acc[16 r + 0..9] (Lp, rho) and acc[16 r + 13..15] (polar velocity); the
-// unweighted line length into acc[16 r + 11].
-__global__ void batch_finish_kernel(const int32_t* __restrict__ real_blk, const double* __restrict__ partial,
-                                    double dt, double* __restrict__ acc)
-{
-    __shared__ double red[128][BSUM];
-    const int r = blockIdx.x;
-    const int b0 = real_blk[r], b1 = real_blk[r + 1];
-    double s[BSUM];
-#pragma unroll
-    for (int m = 0; m < BSUM; ++m) s[m] = 0.0;
-    for (int b = b0 + threadIdx.x; b < b1; b += 128)
-#pragma unroll
-        for (int m = 0; m < BSUM; ++m) s[m] += partial[(int64_t)b * BSUM + m];
-#pragma unroll
-    for (int m = 0; m < BSUM; ++m) red[threadIdx.x][m] = s[m];
-    __syncthreads();
-    for (int h = 64; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-#pragma unroll
-            for (int m = 0; m < BSUM; ++m) red[threadIdx.x][m] += red[threadIdx.x + h][m];
-        __syncthreads();
-    }
-    if (threadIdx.x < BSUM) {
-        const int slot = threadIdx.x < 10 ? threadIdx.x : threadIdx.x + 3;
-        acc[16 * r + slot] = fma(red[0][threadIdx.x], dt, acc[16 * r + slot]);
-    }
-    if (threadIdx.x == 9) acc[16 * r + 11] = red[0][9];  // the step's line length (junction jumps weight it)
 }
 
 __global__ void batch_soa_to_aos(int64_t n, const double* __restrict__ soa, double scale, double* __restrict__ aos)
@@ -455,12 +328,11 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStr
     PTADD_CUDA(cudaMemcpyAsync(B.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, s));
     PTADD_CUDA(cudaMemcpyAsync(B.d_fp_base, fp_base.data(), B.R * sizeof(int64_t), cudaMemcpyHostToDevice, s));
     PTADD_CUDA(cudaMemcpyAsync(B.d_chunks, chunks.data(), B.R * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    // non-target entries must read as zero
-    PTADD_CUDA(cudaMemsetAsync(B.fpart, 0, (size_t)need * sizeof(double), s));
     PTADD_CUDA(cudaStreamSynchronize(s));
     B.n_items = (int)items.size();
     B.cfg = cfg;
     B.items_prec = prec;
+    B.max_chunks = *std::max_element(chunks.begin(), chunks.end());
     if (B.graph) {
         cudaGraphExecDestroy(B.graph);
         B.graph = nullptr;
@@ -522,45 +394,68 @@ cudaError_t launch_batch_pair(const DevBatch& B, int prec, const Consts& c, cuda
     return launch_persistent(batch_pair_mixed_kernel<128, 3>, 128, B.n_items, s, pair_args(B), c, near2);
 }
 
-// One DD step of the whole batch on stream s (pos[cur] -> pos[1-cur]).
-cudaError_t batch_step(DevBatch& B, int prec, const Consts& c, double dt_hat, cudaStream_t s)
+StepArgs batch_step_args(const DevBatch& B, int prec, const Consts& c, double dt_hat)
 {
-    const unsigned nb = (unsigned)((B.n + 255) / 256);
-    launch_batch_prep(B, prec, c, s);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
+    const bool mixed = prec == (int)PTADD_MIXED;
+    StepArgs a;
+    a.n = B.n;
+    a.pos = B.pos[B.cur];
+    a.pos_next = B.pos[1 - B.cur];
+    a.nxt = B.nxt;
+    a.prv = B.prv;
+    a.loop_of = B.loop_of;
+    a.loop_b = B.loop_b;
+    a.loop_n = B.loop_n;
+    a.loop_off = B.d_loop_off;
+    a.pinned = B.pinned;
+    a.grp_off = B.grp_off;
+    a.real_of = B.real_of;
+    a.node_off = B.d_node_off;
+    a.fp_base = B.d_fp_base;
+    a.chunks_of = B.d_chunks;
+    a.fpart = B.fpart;
+    a.vel = B.vel;
+    a.scr = B.cm_scratch;
+    a.src = B.src;
+    a.src32 = mixed || B.junc ? B.src32 : nullptr;  // (the junction search reads it too)
+    a.srcdf = mixed ? nullptr : B.srcdf;
+    a.origin = B.d_origin;
+    a.a2 = c.a2;
+    a.dt = dt_hat;
+    a.part = B.part;
+    a.flag = B.flag;
+    a.counter = B.counter;
+    return a;
+}
+
+// One DD step of the whole batch on stream s (pos[cur] -> pos[1-cur]); the
+// records are those of pos[cur] and the work counter is 0.
+cudaError_t batch_step(DevBatch& B, int prec, const Consts& c, double dt_hat, cudaStream_t s, int64_t* launches)
+{
+    cudaError_t e;
     if (B.n_items > 0) {
         e = launch_batch_pair(B, prec, c, s);
         if (e != cudaSuccess) return e;
+        *launches += 1;
     }
-    batch_node_kernel<<<nb, 256, 0, s>>>(B.n, B.pos[B.cur], B.nxt, B.prv, B.loop_of, B.real_of, B.loop_n, B.pinned,
-                                         B.d_node_off, B.d_fp_base, B.d_chunks, B.fpart, B.force, B.vel);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (B.consistent) {
-        e = launch_consistent_velocity_raw(B.n_loops, B.d_loop_off, B.pos[B.cur], B.n, B.force, B.pinned, B.loop_n,
-                                           B.vel, B.cm_scratch, s);
-        if (e != cudaSuccess) return e;
-    }
+    const StepArgs a = batch_step_args(B, prec, c, dt_hat);
+    const int mob = STEP_NODE | (B.consistent ? STEP_CONSISTENT : 0), move = STEP_EULER | STEP_PREP;
     if (B.junc) {
+        e = launch_step(a, B.n_grp, B.grp_whole, B.max_chunks, mob, s, launches);
+        if (e != cudaSuccess) return e;
         e = launch_batch_junction_update(B.junc, B.pos[B.cur], B.src32, B.nxt, B.loop_of, B.real_of, B.d_node_off,
                                          B.pinned, B.vel, s);
         if (e != cudaSuccess) return e;
-    }
-    batch_lp_euler_kernel<<<B.nblk, BRED, 0, s>>>(B.n, B.pos[B.cur], B.pos[1 - B.cur], B.nxt, B.loop_of, B.loop_b,
-                                                  B.vel, B.d_blk_real, B.d_blk_start, B.d_node_off, dt_hat, B.partial,
-                                                  B.flag);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    batch_finish_kernel<<<B.R, 128, 0, s>>>(B.d_real_blk, B.partial, dt_hat, B.acc);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (B.junc) {
-        e = launch_batch_junction_event(B.junc, B.acc, B.dt_s, dt_hat, B.time_scale, s);
+        e = launch_step(a, B.n_grp, B.grp_whole, B.max_chunks, move, s, launches);
         if (e != cudaSuccess) return e;
+        e = launch_step_finish(B.R, B.real_grp, B.part, true, B.acc, s);
+        if (e != cudaSuccess) return e;
+        e = launch_batch_junction_event(B.junc, B.acc, B.dt_s, dt_hat, B.time_scale, s);
+        *launches += 5;
+    } else {
+        e = launch_step(a, B.n_grp, B.grp_whole, B.max_chunks, mob | move, s, launches);
     }
+    if (e != cudaSuccess) return e;
     B.cur = 1 - B.cur;
     return cudaSuccess;
 }
@@ -573,8 +468,8 @@ void free_batch(DevBatch& B)
     if (B.cm_scratch) cudaFree(B.cm_scratch);
     void* ptrs[] = {B.pos[0],   B.pos[1],    B.nxt,       B.prv,        B.loop_of,  B.real_of, B.tgt,
                     B.loop_b,   B.loop_n,    B.pinned,    B.src,        B.src32,    B.srcdf,   B.fpart,   B.vel,
-                    B.force,    B.partial,   B.acc,       B.d_node_off, B.d_fp_base, B.d_chunks, B.d_origin,
-                    B.d_sh,     B.d_blk_real, B.d_blk_start, B.d_real_blk, B.d_items, B.counter, B.flag,
+                    B.force,    B.part,      B.acc,       B.d_node_off, B.d_fp_base, B.d_chunks, B.d_origin,
+                    B.d_sh,     B.grp_off,   B.real_grp,  B.d_items, B.counter, B.flag,
                     B.near_count, B.staging, B.k64};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -763,9 +658,9 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
         }
     }
     B.tgt_off.assign(R + 1, 0);
-    std::vector<int32_t> blk_real;
-    std::vector<int64_t> blk_start;
-    std::vector<int32_t> real_blk(R + 1, 0);
+    const StepGroups grp = step_groups(n_loops, loop_off, R, node_off);
+    B.n_grp = grp.real_grp[R];
+    B.grp_whole = grp.whole;
     B.pairs = 0;
     for (int r = 0; r < R; ++r) {
         const int64_t a = node_off[r], b = node_off[r + 1];
@@ -775,16 +670,9 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
             if (!(pin[i] && pin[nxt[i]])) tgt.push_back((int32_t)i);
         }
         B.pairs += ((int64_t)tgt.size() - B.tgt_off[r]) * (b - a);
-        real_blk[r] = (int32_t)blk_real.size();
-        for (int64_t s0 = a; s0 < b; s0 += BRED) {
-            blk_real.push_back(r);
-            blk_start.push_back(s0);
-        }
     }
     B.tgt_off[R] = (int64_t)tgt.size();
-    real_blk[R] = (int32_t)blk_real.size();
     B.n_tgt = (int64_t)tgt.size();
-    B.nblk = (int)blk_real.size();
 
     // partial-force capacity: the smallest chunk length any configuration uses
     {
@@ -816,23 +704,22 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     BALLOC(B.fpart, B.fpart_cap);
     BALLOC(B.vel, 3 * n);
     BALLOC(B.force, 3 * n);
-    BALLOC(B.partial, (int64_t)BSUM * B.nblk);
+    BALLOC(B.part, 16 * (int64_t)B.n_grp);
     BALLOC(B.acc, 16 * (int64_t)R);
     BALLOC(B.d_node_off, R + 1);
     BALLOC(B.d_fp_base, R);
     BALLOC(B.d_chunks, R);
     BALLOC(B.d_origin, 3 * R);
     BALLOC(B.d_sh, 6 * R);
-    BALLOC(B.d_blk_real, B.nblk);
-    BALLOC(B.d_blk_start, B.nblk);
-    BALLOC(B.d_real_blk, R + 1);
+    BALLOC(B.grp_off, grp.off.size());
+    BALLOC(B.real_grp, R + 1);
     BALLOC(B.counter, 1);
     BALLOC(B.flag, 1);
     BALLOC(B.near_count, 1);
     BALLOC(B.staging, 3 * n);
     BALLOC(B.k64, 4);
     BALLOC(B.d_loop_off, n_loops + 1);
-    BALLOC(B.cm_scratch, 5 * n);
+    BALLOC(B.cm_scratch, 10 * n);
 #undef BALLOC
     if (st != PTADD_OK) {
         free_batch(B);
@@ -856,9 +743,8 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     H2D(B.d_loop_off, loop_off, n_loops + 1);
     H2D(B.d_origin, origin.data(), 3 * R);
     H2D(B.d_sh, sh.data(), 6 * R);
-    H2D(B.d_blk_real, blk_real.data(), B.nblk);
-    H2D(B.d_blk_start, blk_start.data(), B.nblk);
-    H2D(B.d_real_blk, real_blk.data(), R + 1);
+    H2D(B.grp_off, grp.off.data(), grp.off.size());
+    H2D(B.real_grp, grp.real_grp.data(), R + 1);
 #undef H2D
     PTADD_CUDA(cudaMemsetAsync(B.acc, 0, 16 * (size_t)R * sizeof(double), s));
     PTADD_CUDA(cudaMemsetAsync(B.flag, 0, sizeof(int), s));
@@ -917,8 +803,14 @@ ptadd_status ptadd_batch_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, dou
     B.time_scale = ctx->mat.mu / ctx->mat.B;
     const bool junc = B.junc != nullptr;
     B.consistent = ctx->consistent_mass;
-    const int per_step = (junc ? 9 : 5) + (B.consistent ? 1 : 0);
     int64_t left = n_steps;
+    if (n_steps > 0) {
+        launch_batch_prep(B, prec, c, s);
+        PTADD_CUDA(cudaGetLastError());
+        PTADD_CUDA(cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s));
+        PTADD_CUDA(cudaMemsetAsync(B.part, 0, 16 * (size_t)B.n_grp * sizeof(double), s));
+        ctx->kernel_launches += 1;
+    }
     if (left >= 2) {
         if (!B.graph || B.graph_dt != dt_hat || B.graph_prec != prec || B.graph_cur != B.cur || B.graph_junc != junc ||
             B.graph_cons != B.consistent) {
@@ -927,8 +819,9 @@ ptadd_status ptadd_batch_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, dou
             const int cur0 = B.cur;
             cudaGraph_t g = nullptr;
             PTADD_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-            cudaError_t e = batch_step(B, prec, c, dt_hat, s);
-            if (e == cudaSuccess) e = batch_step(B, prec, c, dt_hat, s);
+            B.graph_launches = 0;
+            cudaError_t e = batch_step(B, prec, c, dt_hat, s, &B.graph_launches);
+            if (e == cudaSuccess) e = batch_step(B, prec, c, dt_hat, s, &B.graph_launches);
             cudaError_t e2 = cudaStreamEndCapture(s, &g);
             B.cur = cur0;
             if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -953,12 +846,15 @@ ptadd_status ptadd_batch_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, dou
         while (left >= 2) {
             PTADD_CUDA(cudaGraphLaunch(B.graph, s));
             left -= 2;
-            ctx->kernel_launches += 2 * per_step;
+            ctx->kernel_launches += B.graph_launches;
         }
     }
     if (left == 1) {
-        PTADD_CUDA(batch_step(B, prec, c, dt_hat, s));
-        ctx->kernel_launches += per_step;
+        PTADD_CUDA(batch_step(B, prec, c, dt_hat, s, &ctx->kernel_launches));
+    }
+    if (n_steps > 0) {
+        PTADD_CUDA(launch_step_finish(B.R, B.real_grp, B.part, false, B.acc, s));
+        ctx->kernel_launches += 1;
     }
     std::vector<double> acc(16 * (size_t)B.R);
     int flag = 0;
@@ -1136,14 +1032,11 @@ ptadd_status ptadd_batch_get_forces(ptadd_ctx* ctx, double* F)
         ptadd_status st = apply_config(B, B.cfg, (int)ctx->prec, s);
         if (st != PTADD_OK) return st;
     }
-    const unsigned nb = (unsigned)((B.n + 255) / 256);
     launch_batch_prep(B, (int)ctx->prec, c, s);
     PTADD_CUDA(cudaGetLastError());
     PTADD_CUDA(cudaMemsetAsync(B.counter, 0, sizeof(unsigned), s));
     if (B.n_items > 0) PTADD_CUDA(launch_batch_pair(B, (int)ctx->prec, c, s));
-    batch_node_kernel<<<nb, 256, 0, s>>>(B.n, B.pos[B.cur], B.nxt, B.prv, B.loop_of, B.real_of, B.loop_n, B.pinned,
-                                         B.d_node_off, B.d_fp_base, B.d_chunks, B.fpart, B.force, B.vel);
-    PTADD_CUDA(cudaGetLastError());
+    PTADD_CUDA(launch_node_force(batch_step_args(B, (int)ctx->prec, c, 0.0), B.force, s));
     batch_forces_out<<<(unsigned)((3 * B.n + 255) / 256), 256, 0, s>>>(
         B.n, B.force, B.pinned, ctx->mat.mu * ctx->len_unit * ctx->len_unit, B.staging);
     PTADD_CUDA(cudaGetLastError());

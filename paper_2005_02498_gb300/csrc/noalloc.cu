@@ -24,17 +24,18 @@
 #include <mutex>
 
 #include "ptadd_internal.cuh"
+#include "step.cuh"
 
 namespace ptadd {
 namespace {
 
 constexpr int64_t NA_MAX = PTADD_NOALLOC_MAX_SEGMENTS;
 constexpr int NA_CHUNKS = 4;  // source chunks at NA_MAX segments (smaller networks: more, in the same space)
-// doubles per segment: positions 3, source record 16, double-float record 18
-// (36 floats), partial forces 6 per chunk, force 3, velocity 3, Burgers vector 3, normal 3; then four int32
+// doubles per segment: positions 3, source record 16, double-float record 24
+// (48 floats), partial forces 6 per chunk, force 3, velocity 3, Burgers vector 3, normal 3; then four int32
 // tables (loop index, target list, checked nxt and prv copies) and the error
 // word packed into the same array.
-constexpr int64_t NA_DOUBLES_PER_SEG = 3 + SRC_STRIDE + SRCDF_STRIDE / 2 + 6 * NA_CHUNKS + 3 + 3 + 3 + 3;
+constexpr int64_t NA_DOUBLES_PER_SEG = 3 + SRC_STRIDE + SRCDF_STRIDE / 2 + 6 * NA_CHUNKS + 3 + 3;
 // + 4*NA_MAX int32 (= 2*NA_MAX doubles) + slack for the 256-byte alignment of
 // the regions (each pad < 32 doubles) and the error word
 constexpr int64_t NA_DOUBLES = NA_DOUBLES_PER_SEG * NA_MAX + 2 * NA_MAX + 512;
@@ -85,7 +86,7 @@ ptadd_status scratch_for_current_device(cudaStream_t s, double** out)
 __global__ void na_prepare(int64_t n, const double* __restrict__ xyz, const double* __restrict__ burgers,
                            const int32_t* __restrict__ nxt_in, const int32_t* __restrict__ prv_in,
                            double pos_scale, double len_unit, double* __restrict__ pos, double* __restrict__ bseg,
-                           double* __restrict__ nseg, int32_t* __restrict__ loop_of, int32_t* __restrict__ tgt,
+                           int32_t* __restrict__ loop_of, int32_t* __restrict__ tgt,
                            int32_t* __restrict__ nxt, int32_t* __restrict__ prv, int* __restrict__ err)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -99,7 +100,6 @@ __global__ void na_prepare(int64_t n, const double* __restrict__ xyz, const doub
     for (int c = 0; c < 3; ++c) {
         pos[c * n + i] = xyz[3 * i + c] * pos_scale;  // power of two: exact
         bseg[3 * i + c] = burgers[3 * i + c] / len_unit;
-        nseg[3 * i + c] = 0.0;
     }
     loop_of[i] = (int32_t)i;  // one Burgers vector per segment
     tgt[i] = (int32_t)i;
@@ -162,9 +162,7 @@ extern "C" ptadd_status ptadd_forces_noalloc(const ptadd_material* mat, int64_t 
     net.srcdf = reinterpret_cast<float*>(base + off); off = align32(off + SRCDF_STRIDE / 2 * n);
     net.fpart = base + off;  off = align32(off + 6 * NA_CHUNKS * NA_MAX);
     net.force = base + off;  off = align32(off + 3 * n);
-    net.vel = base + off;    off = align32(off + 3 * n);
     net.loop_b = base + off; off = align32(off + 3 * n);
-    net.loop_n = base + off; off = align32(off + 3 * n);
     int32_t* ints = reinterpret_cast<int32_t*>(base + off);
     net.loop_of = ints;
     int32_t* tgt = ints + align32(n);
@@ -179,7 +177,7 @@ extern "C" ptadd_status ptadd_forces_noalloc(const ptadd_material* mat, int64_t 
     const unsigned blk = (unsigned)((n + 255) / 256);
     PTADD_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     na_prepare<<<blk, 256, 0, s>>>(n, xyz_dev, burgers_dev, nxt_dev, prv_dev, ldexp(1.0, -len_exp), len_unit,
-                                   net.pos[0], net.loop_b, net.loop_n, net.loop_of, tgt, net.nxt, net.prv, err);
+                                   net.pos[0], net.loop_b, net.loop_of, tgt, net.nxt, net.prv, err);
     PTADD_CUDA(cudaGetLastError());
     const Consts c = make_consts(mat->a / len_unit, mat->nu);
     double sh[6];
@@ -187,7 +185,12 @@ extern "C" ptadd_status ptadd_forces_noalloc(const ptadd_material* mat, int64_t 
     const int chunks = choose_chunks(n, n, net.max_chunks, (int)PTADD_FP64);
     PTADD_CUDA(launch_seg_prep(net, (int)PTADD_FP64, c, s));
     PTADD_CUDA(launch_pair(net, tgt, n, chunks, (int)PTADD_FP64, c, sh, s));
-    PTADD_CUDA(launch_node_velocity(net, chunks, s));
+    StepArgs na;
+    na.n = n;
+    na.prv = net.prv;
+    na.chunks = chunks;
+    na.fpart = net.fpart;
+    PTADD_CUDA(launch_node_force(na, net.force, s));
     na_finish<<<(unsigned)((3 * n + 255) / 256), 256, 0, s>>>(n, net.force, mat->mu * len_unit * len_unit, err,
                                                               F_dev);
     PTADD_CUDA(cudaGetLastError());

@@ -69,7 +69,7 @@ __device__ __forceinline__ void df_parts(double x, double o, float* f)
 __device__ __forceinline__ void seg_records(const double x1[3], const double x2[3], const double b[3],
                                             const double o[3], double a2, double* r, float* f32, float* fdf)
 {
-    const double dx = x2[0] - x1[0], dy = x2[1] - x1[1], dz = x2[2] - x1[2];
+    const double dx = x2[0] - x1[0], dy = x2[1] - x1[1], dz = x2[2] - x1[2], d[3] = {dx, dy, dz};
     const double LL = dx * dx + dy * dy + dz * dz, L = sqrt(LL);
     double t[3] = {1.0, 0.0, 0.0};
     if (L > 0.0) {
@@ -99,9 +99,9 @@ __device__ __forceinline__ void seg_records(const double x1[3], const double x2[
             v[13 + k] = (float)q[k];
         }
         v[6] = (float)L;
-        float4* d = reinterpret_cast<float4*>(f32);
+        float4* out = reinterpret_cast<float4*>(f32);
 #pragma unroll
-        for (int e = 0; e < SRC32_STRIDE / 4; ++e) d[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+        for (int e = 0; e < SRC32_STRIDE / 4; ++e) out[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
     }
     if (fdf) {
         constexpr double SC = 1.0 / (1 << -DF_SCALE);
@@ -135,6 +135,11 @@ __device__ __forceinline__ void seg_records(const double x1[3], const double x2[
             const int i = (k + 1) % 3, j = (k + 2) % 3;
             df_parts(x1[k], o[k], f + 3 * k);
             const DF1 ft = df_split(t[k]), fe = df_split(e[k]), fn = df_split(fma(t[i], e[j], -(t[j] * e[i])));
+            const DF1 fd = df_split(d[k] * SC), fb = df_split(b[k]);
+            f[36 + k] = fd.h;
+            f[39 + k] = fd.l;
+            f[42 + k] = fb.h;
+            f[45 + k] = fb.l;
             f[9 + k] = ft.h;
             f[12 + k] = ft.l;
             f[15 + k] = fe.h;
@@ -152,14 +157,16 @@ __device__ __forceinline__ void seg_records(const double x1[3], const double x2[
         f[33] = fe.h;
         f[34] = fe.l;
         f[35] = fmaxf((float)(DF_NEAR * DF_NEAR * SC * SC * a2), ll.h * (1.0f / 256.0f));
-        float4* d = reinterpret_cast<float4*>(fdf);
+        float4* out = reinterpret_cast<float4*>(fdf);
 #pragma unroll
-        for (int k = 0; k < SRCDF_STRIDE / 4; ++k) d[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+        for (int k = 0; k < SRCDF_STRIDE / 4; ++k) out[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
     }
 }
 
-__device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, double Dx, double Dy, double Dz,
-                                           const double bt[3], double acc[4][3])
+// Adds sigma_app b' (where the tile has it) to the four sums of sigma b', and the
+// nodal force parts of the sums to Fs and Fe.
+__device__ __forceinline__ void tile_forces(const TileArgs& a, double Dx, double Dy, double Dz, const double bt[3],
+                                            double acc[4][3], double Fs[3], double Fe[3])
 {
     if (a.add_app) {
         const double* s = a.sh;
@@ -173,7 +180,6 @@ __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, doubl
             acc[qp][2] += sb2;
         }
     }
-    double Fs[3] = {0, 0, 0}, Fe[3] = {0, 0, 0};
 #pragma unroll
     for (int qp = 0; qp < 4; ++qp) {
         const double fx = acc[qp][1] * Dz - acc[qp][2] * Dy;
@@ -183,6 +189,10 @@ __device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, doubl
         Fs[0] = fma(ws, fx, Fs[0]); Fs[1] = fma(ws, fy, Fs[1]); Fs[2] = fma(ws, fz, Fs[2]);
         Fe[0] = fma(we, fx, Fe[0]); Fe[1] = fma(we, fy, Fe[1]); Fe[2] = fma(we, fz, Fe[2]);
     }
+}
+
+__device__ __forceinline__ void tile_store(const TileArgs& a, int64_t seg, const double Fs[3], const double Fe[3])
+{
     double* fp = a.fp + (seg - a.node_base);
     const int64_t st = a.fp_stride;
     fp[0 * st] = Fs[0];
@@ -242,16 +252,28 @@ static __device__ __noinline__ void near_flush(const double* __restrict__ pos, i
     const int64_t seg_o = __shfl_sync(0xffffffffu, (long long)seg, (int)((e.y >> 2) & 31u));
     double3 d = make_double3(0.0, 0.0, 0.0);
     if (lane < cnt) d = near_field_fp64(pos, n, nxt, src, seg_o, (int64_t)e.x, (int)(e.y & 3u), k64);
-    for (int k = 0; k < cnt; ++k) {
+    // Every lane adds its own entries in queue order, one entry of each lane at a
+    // time.  (A loop over the 32 entries would issue 96 FP64 additions for one
+    // lane each, nearly as many as the field itself takes.)
+    const unsigned own = (e.y >> 2) & 31u;
+    unsigned mine = __ballot_sync(0xffffffffu, lane < cnt);  // entries whose owner is this lane, bit by bit of its number
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+        const unsigned set = __ballot_sync(0xffffffffu, (own >> b) & 1u);
+        mine &= ((lane >> b) & 1) ? set : ~set;
+    }
+    while (__any_sync(0xffffffffu, mine != 0u)) {
+        const int k = mine ? __ffs(mine) - 1 : lane;
         const double dx = __shfl_sync(0xffffffffu, d.x, k);
         const double dy = __shfl_sync(0xffffffffu, d.y, k);
         const double dz = __shfl_sync(0xffffffffu, d.z, k);
         const unsigned tag = __shfl_sync(0xffffffffu, e.y, k);
-        if ((int)((tag >> 2) & 31u) == lane) {
+        if (mine) {
             double* acc = nacc + 3 * (int)(tag & 3u) * tpb + threadIdx.x;
             acc[0] += dx;
             acc[tpb] += dy;
             acc[2 * tpb] += dz;
+            mine &= mine - 1u;
         }
     }
 }
@@ -289,15 +311,16 @@ __device__ __forceinline__ void near_shift(uint2* q, int cnt)
 // length of DF_FAR or more, is evaluated in FP64.  A tile is one warp's: no lane waits for
 // another warp, and a small network gives as many tiles as it has warps.
 constexpr int DF_REC = 64;            // floats of a staged source record
-constexpr int DF_TILE = 16;           // sources per staged tile
-constexpr int DF_GROUP = 4;           // staged tiles per group of double-float sums
+constexpr int DF_TILE = 12;           // sources per staged tile (16 blocks of 13 KB fit one SM)
+constexpr int DF_GROUP = 5;           // staged tiles per group of double-float sums
 
 struct DFSmem {
     // per source: t, e, n (h x 3, l x 3 each), L, L^2, bt, be (h, l each), every
     // value in both lanes (26 float2), then x (9), the squared near limit
     float4 rec[DF_TILE * DF_REC / 4];
     float2 sum[16 * 32];  // double-float sums: [chain * 8 + 2 * e + part][thread], e = 3: along b'
-    double nacc[12 * 32];  // FP64 sums: [qp * 3 + e][thread]
+    double facc[6 * 32];   // FP64 far-field parts of the nodal forces: [start, end * 3 + e][thread]
+    double nacc[12 * 32];  // FP64 near-field sums: [qp * 3 + e][thread]
     double k64[3];          // {a2, c1, c2} for the near field
     uint2 queue[NEAR_Q];
 };
@@ -309,7 +332,6 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
     const int64_t n = a.n;
     const bool active = threadIdx.x < a.t_count;
     const int64_t seg = active ? a.tgt[a.t_begin + threadIdx.x] : a.tgt[a.t_begin];
-    const int64_t sb = a.nxt[seg];
     float xt[9], lim_t;
     DF1 D[3];
     DF2 bt[3];
@@ -319,15 +341,16 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
 #pragma unroll
         for (int k = 0; k < 9; ++k) xt[k] = fr[k];
         lim_t = fr[35];
-        const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            D[k] = df_split((a.pos[k * n + sb] - a.pos[k * n + seg]) * SC);
+            D[k] = DF1{fr[36 + k], fr[39 + k]};
+            bt[k] = DF2{p_all(fr[42 + k]), p_all(fr[45 + k])};
             wide = wide || !(fabsf(D[k].h) < (float)(DF_FAR * SC));
-            bt[k] = df_all(df_split(tr[8 + k]));
         }
     }
     const DFConst K = c.df;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sm.facc[k * 32 + threadIdx.x] = 0.0;
 #pragma unroll
     for (int k = 0; k < 12; ++k) sm.nacc[k * 32 + threadIdx.x] = 0.0;
 #pragma unroll
@@ -342,6 +365,7 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
     uint2* wq = sm.queue;
     int qn = 0;  // entries waiting in this warp's queue (warp-uniform)
     int open = 0;  // tiles in the open group
+    bool fp64 = a.add_app;  // (warp-uniform) the FP64 sums hold something
 
     for (int64_t j0 = a.js; j0 < a.je; j0 += DF_TILE) {
         const int cnt = (int)min((int64_t)DF_TILE, a.je - j0);
@@ -441,49 +465,71 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
                 while (qn >= 32) {
                     __syncwarp();
                     near_flush(a.pos, n, a.nxt, a.src, sm.k64, seg, wq, 32, sm.nacc, 32);
+                    fp64 = true;
                     near_shift(wq, qn);
                     qn -= 32;
                 }
             }
         }
         if (++open == DF_GROUP || j0 + DF_TILE >= a.je) {
-            // the group's sums to FP64, restoring the factor c2 and the unit of length
+            // the group's nodal force parts sum_q w (s_q x D), still in double-float, then to FP64
             open = 0;
-            const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
-            const double k2 = c.c2 * SC;
-#pragma unroll 1
+            DF2 F[6];  // lanes: the chains' first and second points
+#pragma unroll
             for (int ch = 0; ch < 2; ++ch) {
                 float2* q = sm.sum + (ch * 8) * 32 + threadIdx.x;
-                const double bx = (double)q[6 * 32].x + (double)q[7 * 32].x;
-                const double by = (double)q[6 * 32].y + (double)q[7 * 32].y;
+                DF2 s[3];
+                const DF2 b = {q[6 * 32], q[7 * 32]};
 #pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    double* acc = sm.nacc + (6 * ch + e) * 32 + threadIdx.x;
-                    const float2 h = q[2 * e * 32], l = q[(2 * e + 1) * 32];
-                    acc[0] = fma(k2, fma(bx, tr[8 + e], (double)h.x + (double)l.x), acc[0]);
-                    acc[3 * 32] = fma(k2, fma(by, tr[8 + e], (double)h.y + (double)l.y), acc[3 * 32]);
-                }
+                for (int e = 0; e < 3; ++e) s[e] = df_fma(b, bt[e], DF2{q[2 * e * 32], q[(2 * e + 1) * 32]});
 #pragma unroll
                 for (int k = 0; k < 8; ++k) q[k * 32] = p_all(0.0f);
+                const DF2 we = df_pair2(df_from(gl4_w(2 * ch) * gl4_xi(2 * ch)), df_from(gl4_w(2 * ch + 1) * gl4_xi(2 * ch + 1)));
+                const DF2 ws = df_pair2(df_from(gl4_w(2 * ch) * (1.0 - gl4_xi(2 * ch))),
+                                        df_from(gl4_w(2 * ch + 1) * (1.0 - gl4_xi(2 * ch + 1))));
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    const int i = (e + 1) % 3, j = (e + 2) % 3;
+                    const DF2 f = df_fma(s[i], df_all(D[j]), df_neg(df_mul(s[j], df_all(D[i]))));
+                    F[e] = ch ? df_fma(f, ws, F[e]) : df_mul(f, ws);
+                    F[3 + e] = ch ? df_fma(f, we, F[3 + e]) : df_mul(f, we);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const DF2 t = df_norm(df_add(df_lane_x(F[k]), df_lane_y(F[k])));
+                double* acc = sm.facc + k * 32 + threadIdx.x;
+                acc[0] = fma(c.c2, f2d_seed0(t.h.x) + f2d_seed0(t.l.x), acc[0]);
             }
         }
     }
     if (qn > 0) {
         __syncwarp();
         near_flush(a.pos, n, a.nxt, a.src, sm.k64, seg, wq, qn, sm.nacc, 32);
+        fp64 = true;
     }
     __syncwarp();
     if (!active) return;
-    const double xa = a.pos[seg], ya = a.pos[n + seg], za = a.pos[2 * n + seg];
-    const double Dx = a.pos[sb] - xa, Dy = a.pos[n + sb] - ya, Dz = a.pos[2 * n + sb] - za;
-    const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
-    const double b64[3] = {tr[8], tr[9], tr[10]};
-    double acc[4][3];
+    double Fs[3], Fe[3];
 #pragma unroll
-    for (int qp = 0; qp < 4; ++qp)
+    for (int e = 0; e < 3; ++e) {
+        Fs[e] = sm.facc[e * 32 + threadIdx.x];
+        Fe[e] = sm.facc[(3 + e) * 32 + threadIdx.x];
+    }
+    if (fp64) {
+        const int64_t sb = a.nxt[seg];
+        const double xa = a.pos[seg], ya = a.pos[n + seg], za = a.pos[2 * n + seg];
+        const double Dx = a.pos[sb] - xa, Dy = a.pos[n + sb] - ya, Dz = a.pos[2 * n + sb] - za;
+        const double* tr = a.src + (int64_t)SRC_STRIDE * seg;
+        const double b64[3] = {tr[8], tr[9], tr[10]};
+        double acc[4][3];
 #pragma unroll
-        for (int e = 0; e < 3; ++e) acc[qp][e] = sm.nacc[(3 * qp + e) * 32 + threadIdx.x];
-    tile_store(a, seg, Dx, Dy, Dz, b64, acc);
+        for (int qp = 0; qp < 4; ++qp)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) acc[qp][e] = sm.nacc[(3 * qp + e) * 32 + threadIdx.x];
+        tile_forces(a, Dx, Dy, Dz, b64, acc, Fs, Fe);
+    }
+    tile_store(a, seg, Fs, Fe);
 }
 
 // ----------------------------------------------------------------- mixed
@@ -891,7 +937,9 @@ __device__ __forceinline__ void pair_tile_mixed(const TileArgs& a, const Consts&
     for (int qp = 0; qp < 4; ++qp)
 #pragma unroll
         for (int e = 0; e < 3; ++e) acc[qp][e] = sm.nacc[(3 * qp + e) * TPB + threadIdx.x];
-    tile_store(a, seg, Dx, Dy, Dz, bt, acc);
+    double Fs[3] = {0.0, 0.0, 0.0}, Fe[3] = {0.0, 0.0, 0.0};
+    tile_forces(a, Dx, Dy, Dz, bt, acc, Fs, Fe);
+    tile_store(a, seg, Fs, Fe);
 }
 
 }  // namespace ptadd

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "ptadd_internal.cuh"
+#include "step.cuh"
 
 namespace ptadd {
 
@@ -49,7 +50,7 @@ static ptadd_status dalloc(T** p, size_t count)
 static void free_network(DevNetwork& n)
 {
     void* ptrs[] = {n.pos[0], n.pos[1], n.nxt,   n.prv,   n.loop_of, n.loop_b,  n.loop_n, n.pinned, n.tgt_burst,
-                    n.tgt_all, n.src,    n.fpart, n.vel,   n.force,   n.partial, n.acc,    n.flag,   n.staging,
+                    n.tgt_all, n.src,    n.fpart, n.vel,   n.force,   n.part,   n.grp_off, n.real_grp, n.acc,    n.flag,   n.staging,
                     n.src32,   n.srcdf, n.near_count, n.k64, n.loop_off, n.cm_scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -212,7 +213,10 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
         for (int64_t nt : {net.n_tgt_burst, n})
             net.max_chunks = std::max(net.max_chunks, choose_chunks(nt, n, FPART_MAX_CHUNKS, prec));
-    net.max_red_blocks = (int)((n + 255) / 256);
+    const int64_t node_off[2] = {0, n};
+    const StepGroups grp = step_groups(n_loops, loop_off, 1, node_off);
+    net.n_grp = grp.real_grp[1];
+    net.grp_whole = grp.whole;
 
     ptadd_status st = PTADD_OK;
 #define ALLOC(p, cnt)                              \
@@ -231,7 +235,9 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     ALLOC(net.fpart, (size_t)net.max_chunks * 6 * n);
     ALLOC(net.vel, 3 * n);
     ALLOC(net.force, 3 * n);
-    ALLOC(net.partial, (size_t)net.max_red_blocks * 13);
+    ALLOC(net.part, (size_t)net.n_grp * 16);
+    ALLOC(net.grp_off, grp.off.size());
+    ALLOC(net.real_grp, 2);
     ALLOC(net.acc, 16);
     ALLOC(net.flag, 1);
     ALLOC(net.staging, 3 * n);
@@ -240,7 +246,7 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     ALLOC(net.near_count, 1);
     ALLOC(net.k64, 4);
     ALLOC(net.loop_off, n_loops + 1);
-    ALLOC(net.cm_scratch, 5 * n);
+    ALLOC(net.cm_scratch, 10 * n);
 #undef ALLOC
     if (st != PTADD_OK) {
         free_network(net);
@@ -261,7 +267,8 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     if (!tb.empty())
         PTADD_CUDA(cudaMemcpyAsync(net.tgt_burst, tb.data(), tb.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     PTADD_CUDA(cudaMemcpyAsync(net.tgt_all, ta.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    PTADD_CUDA(cudaMemsetAsync(net.fpart, 0, (size_t)net.max_chunks * 6 * n * sizeof(double), s));
+    PTADD_CUDA(cudaMemcpyAsync(net.grp_off, grp.off.data(), grp.off.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    PTADD_CUDA(cudaMemcpyAsync(net.real_grp, grp.real_grp.data(), 2 * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     PTADD_CUDA(cudaMemsetAsync(net.acc, 0, 16 * sizeof(double), s));
     PTADD_CUDA(cudaMemsetAsync(net.flag, 0, sizeof(int), s));
     PTADD_CUDA(cudaMemsetAsync(net.near_count, 0, sizeof(unsigned long long), s));
@@ -317,20 +324,16 @@ static ptadd_status take_events(ptadd_ctx* ctx, std::pair<cudaEvent_t, cudaEvent
     return PTADD_OK;
 }
 
-// forces at the current positions for a target list (into net.force, net.vel)
-static ptadd_status eval_forces(ptadd_ctx* ctx, const int32_t* tgt, int64_t n_tgt)
+// the pair stage for a target list, timed if asked; the records are up to date
+static ptadd_status eval_pairs(ptadd_ctx* ctx, const Consts& c, const int32_t* tgt, int64_t n_tgt, int chunks)
 {
     DevNetwork& net = ctx->net;
-    const Consts c = make_consts(ctx);
+    if (n_tgt == 0) return PTADD_OK;
     double sh[6];
     for (int k = 0; k < 6; ++k) sh[k] = ctx->sig_app[k] / ctx->mat.mu;
-    const int chunks = choose_chunks(n_tgt, net.n_nodes, net.max_chunks, (int)ctx->prec);
     cudaStream_t s = ctx->stream;
-    if (n_tgt < net.n_nodes)
-        PTADD_CUDA(cudaMemsetAsync(net.fpart, 0, (size_t)chunks * 6 * net.n_nodes * sizeof(double), s));
-    PTADD_CUDA(launch_seg_prep(net, (int)ctx->prec, c, s));
     std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-    if (ctx->timing && n_tgt > 0) {
+    if (ctx->timing) {
         ptadd_status st = take_events(ctx, ev);
         if (st != PTADD_OK) return st;
         PTADD_CUDA(cudaEventRecord(ev.first, s));
@@ -340,12 +343,54 @@ static ptadd_status eval_forces(ptadd_ctx* ctx, const int32_t* tgt, int64_t n_tg
         PTADD_CUDA(cudaEventRecord(ev.second, s));
         ctx->ev_open.push_back(ev);
     }
-    PTADD_CUDA(launch_node_velocity(net, chunks, s));
-    ctx->kernel_launches += 2 + (n_tgt > 0 ? 1 : 0);
-    if (n_tgt > 0) {
-        ctx->pair_launches += 1;
-        ctx->pair_evals += n_tgt * net.n_nodes;
-    }
+    ctx->kernel_launches += 1;
+    ctx->pair_launches += 1;
+    ctx->pair_evals += n_tgt * net.n_nodes;
+    return PTADD_OK;
+}
+
+static StepArgs step_args(const ptadd_ctx* ctx, const Consts& c, int chunks, double dt_hat)
+{
+    const DevNetwork& net = ctx->net;
+    const bool mixed = ctx->prec == PTADD_MIXED;
+    StepArgs a;
+    a.n = net.n_nodes;
+    a.pos = net.pos[net.cur];
+    a.pos_next = net.pos[1 - net.cur];
+    a.nxt = net.nxt;
+    a.prv = net.prv;
+    a.loop_of = net.loop_of;
+    a.loop_b = net.loop_b;
+    a.loop_n = net.loop_n;
+    a.loop_off = net.loop_off;
+    a.pinned = net.pinned;
+    a.grp_off = net.grp_off;
+    a.chunks = chunks;
+    a.fpart = net.fpart;
+    a.vel = net.vel;
+    a.scr = net.cm_scratch;
+    a.src = net.src;
+    a.src32 = mixed ? net.src32 : nullptr;
+    a.srcdf = mixed ? nullptr : net.srcdf;
+    for (int k = 0; k < 3; ++k) a.org[k] = net.origin[k];
+    a.a2 = c.a2;
+    a.dt = dt_hat;
+    a.part = net.part;
+    a.flag = net.flag;
+    return a;
+}
+
+// forces of every node at the current positions (into net.force)
+static ptadd_status eval_forces(ptadd_ctx* ctx)
+{
+    DevNetwork& net = ctx->net;
+    const Consts c = make_consts(ctx);
+    const int chunks = choose_chunks(net.n_nodes, net.n_nodes, net.max_chunks, (int)ctx->prec);
+    PTADD_CUDA(launch_seg_prep(net, (int)ctx->prec, c, ctx->stream));
+    ptadd_status st = eval_pairs(ctx, c, net.tgt_all, net.n_nodes, chunks);
+    if (st != PTADD_OK) return st;
+    PTADD_CUDA(launch_node_force(step_args(ctx, c, chunks, 0.0), net.force, ctx->stream));
+    ctx->kernel_launches += 2;
     return PTADD_OK;
 }
 
@@ -389,23 +434,34 @@ ptadd_status ptadd_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, double Lp
     const double dt_hat = dt * ctx->mat.mu / ctx->mat.B;
     PTADD_CUDA(cudaMemsetAsync(net.acc, 0, 16 * sizeof(double), s));
     PTADD_CUDA(cudaMemsetAsync(net.flag, 0, sizeof(int), s));
+    const Consts c = make_consts(ctx);
+    const int chunks = choose_chunks(net.n_tgt_burst, net.n_nodes, net.max_chunks, (int)ctx->prec);
+    const int mob = STEP_NODE | (ctx->consistent_mass ? STEP_CONSISTENT : 0);
+    if (n_steps > 0) {
+        PTADD_CUDA(cudaMemsetAsync(net.part, 0, (size_t)net.n_grp * 16 * sizeof(double), s));
+        PTADD_CUDA(launch_seg_prep(net, (int)ctx->prec, c, s));
+        ctx->kernel_launches += 1;
+    }
     for (int64_t it = 0; it < n_steps; ++it) {
-        ptadd_status st = eval_forces(ctx, net.tgt_burst, net.n_tgt_burst);
+        ptadd_status st = eval_pairs(ctx, c, net.tgt_burst, net.n_tgt_burst, chunks);
         if (st != PTADD_OK) return st;
-        if (ctx->consistent_mass) {
-            PTADD_CUDA(launch_consistent_velocity(net, s));
-            ctx->kernel_launches += 1;
-        }
+        const StepArgs a = step_args(ctx, c, chunks, dt_hat);
+        const int move = STEP_EULER | (it + 1 < n_steps ? STEP_PREP : 0);
         if (ctx->junc) {
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob, s, &ctx->kernel_launches));
             PTADD_CUDA(launch_junction_update(ctx, s));
-            ctx->kernel_launches += 3;
-        }
-        PTADD_CUDA(launch_lp_euler(net, dt_hat, s));
-        ctx->kernel_launches += 2;
-        if (ctx->junc) {
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, move, s, &ctx->kernel_launches));
+            PTADD_CUDA(launch_step_finish(1, net.real_grp, net.part, true, net.acc, s));
             PTADD_CUDA(launch_junction_event(ctx, dt, dt_hat, s));
-            ctx->kernel_launches += 1;
+            ctx->kernel_launches += 5;
+        } else {
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob | move, s, &ctx->kernel_launches));
         }
+        net.cur = 1 - net.cur;
+    }
+    if (n_steps > 0) {
+        PTADD_CUDA(launch_step_finish(1, net.real_grp, net.part, false, net.acc, s));
+        ctx->kernel_launches += 1;
     }
     double acc[16];
     int flag = 0;
@@ -567,7 +623,7 @@ ptadd_status ptadd_get_forces(ptadd_ctx* ctx, double* F)
         return PTADD_ERR_STATE;
     }
     if (!F) return arg_error("F is NULL");
-    ptadd_status st = eval_forces(ctx, ctx->net.tgt_all, ctx->net.n_nodes);
+    ptadd_status st = eval_forces(ctx);
     if (st != PTADD_OK) return st;
     return read_soa(ctx, ctx->net.force, ctx->mat.mu * ctx->len_unit * ctx->len_unit, F);
 }
@@ -580,7 +636,7 @@ ptadd_status ptadd_get_forces_dev(ptadd_ctx* ctx, double* F_dev)
         return PTADD_ERR_STATE;
     }
     if (!F_dev) return arg_error("F_dev is NULL");
-    ptadd_status st = eval_forces(ctx, ctx->net.tgt_all, ctx->net.n_nodes);
+    ptadd_status st = eval_forces(ctx);
     if (st != PTADD_OK) return st;
     const int64_t n = ctx->net.n_nodes;
     soa_to_aos_scaled<<<(unsigned)((3 * n + 255) / 256), 256, 0, ctx->stream>>>(

@@ -49,12 +49,13 @@ constexpr int SRC_STRIDE = 16;
 // own (integer origin Ot nearby) as (x1_hi - Ot) + x1_lo with one rounding,
 // and R0 = x - x1 keeps ~1e-7 relative accuracy for every pair.
 constexpr int SRC32_STRIDE = 16;
-// Double-float record of the FP64 path (36 floats, lengths scaled by 2^DF_SCALE):
+// Double-float record of the FP64 path (48 floats, lengths scaled by 2^DF_SCALE):
 //   [0..8] x1 - origin per coordinate as an integer, a multiple of 2^-23 below
 //   1/2 and the rest   [9..11] t high parts [12..14] t low parts   [15..20] e, the
 //   same   [21..26] n = t x e   [27..28] L   [29..30] L^2   [31..32] b.t   [33..34] b.e
-//   [35] squared near limit of the segment (df_field.cuh has the frame t, e, n)
-constexpr int SRCDF_STRIDE = 36;
+//   [35] squared near limit of the segment (df_field.cuh has the frame t, e, n);
+//   for the segment as a target: [36..41] D = x2 - x1, [42..47] b (high parts, low parts)
+constexpr int SRCDF_STRIDE = 48;
 // Near field of the mixed path: point-to-segment distance below 10 a, with a
 // 1 % margin in favour of FP64 on the FP32 estimate of that distance.
 constexpr double NEAR_FACTOR = 10.1;
@@ -80,19 +81,22 @@ struct DevNetwork {
     bool origin_node0 = false;     // instead: node 0's position rounded (read on the device)
     unsigned long long* near_count = nullptr;  // FP64 point-pairs of the mixed path
     double* k64 = nullptr;         // {a2, c1, c2} for the near-field path of the mixed kernel
-    double* fpart = nullptr;       // [max_chunks*6*n] partial nodal-force parts
+    double* fpart = nullptr;       // [max_chunks*6*n] partial nodal-force parts (targets' entries only are written)
     int max_chunks = 0;
     double* vel = nullptr;         // SoA [3*n]
     double* force = nullptr;       // SoA [3*n] (last evaluated nodal force)
-    double* partial = nullptr;     // [max_blocks*13]
-    int max_red_blocks = 0;
+    int32_t* grp_off = nullptr;    // [n_grp + 1] node groups of the step kernels (step.cuh)
+    int32_t* real_grp = nullptr;   // {0, n_grp}
+    int n_grp = 0;
+    bool grp_whole = true;
+    double* part = nullptr;        // [16*n_grp] their sums
     double* acc = nullptr;         // [16]: 0..8 sum Lp dt, 9 sum rho dt, 11 line length of the last
                                    // step, 12 time jumped over while stuck (junctions), 13..15 sum
                                    // (sum_s L vbar) dt (polar velocity)
     int* flag = nullptr;           // non-finite flag
     double* staging = nullptr;     // [3*n] AoS SI positions in / out
     int64_t* loop_off = nullptr;   // [n_loops + 1] first node of each loop (consistent mobility)
-    double* cm_scratch = nullptr;  // [5*n] elimination factors of the consistent mobility
+    double* cm_scratch = nullptr;  // [10*n] rows of the consistent mobility's system
     double volume = 0;             // m^3
 };
 
@@ -119,19 +123,6 @@ cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& 
 // pair stage: writes fpart[chunk][6][seg] for the listed targets
 cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt, int chunks,
                         int precision, const Consts& c, const double sig_hat[6], cudaStream_t st);
-// node stage: F = sum of parts, v = P F / M (0 if pinned); writes net.force / net.vel
-cudaError_t launch_node_velocity(const DevNetwork& net, int chunks, cudaStream_t st);
-// consistent mobility (Eq. 2.1 with its Galerkin mass matrix): M v = P F per
-// loop, v = 0 at pinned nodes; replaces net.vel from net.force
-cudaError_t launch_consistent_velocity(const DevNetwork& net, cudaStream_t st);
-// the same on raw arrays (loops [loop_off[k], loop_off[k+1]) of n nodes, SoA
-// positions, forces and velocities; scr: 5 n doubles), for the batch
-cudaError_t launch_consistent_velocity_raw(int64_t n_loops, const int64_t* loop_off, const double* pos, int64_t n,
-                                           const double* force, const uint8_t* pinned, const double* loop_n,
-                                           double* vel, double* scr, cudaStream_t st);
-// Lp/rho sample of the step-start state, Euler update into the other buffer,
-// and the fixed-order reduction into net.acc (weighted by dt_hat)
-cudaError_t launch_lp_euler(DevNetwork& net, double dt_hat, cudaStream_t st);
 // sources per FP64 work item for a number of one-warp target tiles
 int64_t fp64_chunk_len(int64_t tiles, int64_t n_src);
 int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision);
