@@ -7,8 +7,8 @@
 //   forward   Z_l = H_{l-1} W_l^T + b_l        (A = H_{l-1} [B x din], B = W_l [dout x din])
 //   dH        dH_{l-1} = dZ_l W_l              (A = dZ_l [B x dout], B = W_l^T [din x dout])
 //   dW        dW_l = dZ_l^T H_{l-1}            (A = dZ_l^T [dout x B], B = H_{l-1}^T [din x B])
-// so the epilogues also write transposed BF16 copies of H and dZ, and Adam
-// keeps W and W^T in BF16 next to the FP32 master.  Padding: the 30 inputs
+// so training also writes transposed BF16 copies of H and dZ, and Adam
+// keeps W and W^T in BF16 next to the FP32 master (mlp_train.cu).  Padding: the 30 inputs
 // sit in 32 columns, the 6 outputs in 16 rows of the last layer; padded
 // weights stay exactly zero (their gradients are zero).
 //
@@ -30,14 +30,13 @@
 #include <numeric>
 #include <vector>
 
+#include "mlp_train.cuh"
 #include "ptadd_internal.cuh"
 #include "tc_gemm.cuh"
 
 namespace ptadd {
 
 constexpr int NIN = 30, NOUT = 6, NH = 256;
-constexpr int DIN_P[4] = {32, 256, 256, 256};
-constexpr int DOUT_P[4] = {256, 256, 256, 16};
 constexpr int DIN_U[4] = {30, 256, 256, 256};
 constexpr int DOUT_U[4] = {256, 256, 256, 6};
 constexpr double RHO_FLOOR = 1e10;
@@ -51,7 +50,7 @@ struct MlpDev {
     __nv_bfloat16* Wc = nullptr;  // layers 2, 3 staged for the fused inference kernel (bias block + 4 x 256 x 64 each)
     __nv_bfloat16 *X = nullptr, *Xt = nullptr, *Hb[3] = {}, *Ht[3] = {}, *dY = nullptr, *dYt = nullptr;
     __nv_bfloat16 *dZ[3] = {}, *dZt[3] = {};
-    float *Z[3] = {}, *Y = nullptr, *T = nullptr, *loss_part = nullptr;
+    float *Y = nullptr, *loss_part = nullptr;
     int* err = nullptr;
     int64_t step = 0;
     // closure-level maps (host)
@@ -81,7 +80,7 @@ ptadd_status m_alloc(T** p, size_t count)
 
 void free_work(MlpDev& m)
 {
-    void* ptrs[] = {m.X, m.Xt, m.dY, m.dYt, m.Y, m.T, m.loss_part};
+    void* ptrs[] = {m.X, m.Xt, m.dY, m.dYt, m.Y, m.loss_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int l = 0; l < 3; ++l) {
@@ -89,12 +88,10 @@ void free_work(MlpDev& m)
         cudaFree(m.Ht[l]);
         cudaFree(m.dZ[l]);
         cudaFree(m.dZt[l]);
-        cudaFree(m.Z[l]);
         m.Hb[l] = m.Ht[l] = m.dZ[l] = m.dZt[l] = nullptr;
-        m.Z[l] = nullptr;
     }
     m.X = m.Xt = m.dY = m.dYt = nullptr;
-    m.Y = m.T = m.loss_part = nullptr;
+    m.Y = m.loss_part = nullptr;
     m.cap = 0;
 }
 
@@ -116,7 +113,7 @@ ptadd_status alloc_params(MlpDev& m)
 {
     ptadd_status st = PTADD_OK;
     for (int l = 0; l < 4 && st == PTADD_OK; ++l) {
-        const size_t nw = (size_t)DOUT_P[l] * DIN_P[l], nb = DOUT_P[l];
+        const size_t nw = (size_t)dout_p(l) * din_p(l), nb = dout_p(l);
         float** f[] = {&m.W[l], &m.mW[l], &m.vW[l], &m.gW[l]};
         for (float** p : f)
             if (st == PTADD_OK) st = m_alloc(p, nw);
@@ -147,13 +144,11 @@ ptadd_status ensure_work(MlpDev& m, int64_t rows)
         WA(m.Ht[l], need * NH);
         WA(m.dZ[l], need * NH);
         WA(m.dZt[l], need * NH);
-        WA(m.Z[l], need * NH);
     }
     WA(m.dY, need * 16);
     WA(m.dYt, need * 16);
     WA(m.Y, need * 16);
-    WA(m.T, need * 16);
-    WA(m.loss_part, (need + 255) / 256);
+    WA(m.loss_part, need / 128);
 #undef WA
     if (st != PTADD_OK) {
         free_work(m);
@@ -176,94 +171,14 @@ __global__ void mlp_sync_bf16(const float* __restrict__ W, int dout, int din, __
     Wt[(int64_t)c * dout + o] = v;
 }
 
-// Adam on one parameter array (FP32 master), Kingma & Ba bias correction.
-__global__ void mlp_adam(int n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                         float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
-// Normalised inputs [n x 30] (FP32) -> X [rows x 32] BF16 and X^T [32 x rows]; zero padding.
-__global__ void mlp_pack_x(int64_t n, int64_t rows, const float* __restrict__ xn, const int32_t* __restrict__ idx,
-                           __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Xt)
+// Normalised inputs [n x 30] (FP32) -> X [rows x 32] BF16; zero padding.
+__global__ void mlp_pack_x(int64_t n, int64_t rows, const float* __restrict__ xn, __nv_bfloat16* __restrict__ X)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= rows * 32) return;
     const int64_t r = i / 32;
     const int c = (int)(i % 32);
-    float v = 0.0f;
-    if (r < n && c < NIN) {
-        const int64_t src = idx ? idx[r] : r;
-        v = xn[src * NIN + c];
-    }
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    X[r * 32 + c] = h;
-    Xt[(int64_t)c * rows + r] = h;
-}
-
-__global__ void mlp_pack_t(int64_t n, int64_t rows, const float* __restrict__ yn, const int32_t* __restrict__ idx,
-                           float* __restrict__ T)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= rows * 16) return;
-    const int64_t r = i / 16;
-    const int c = (int)(i % 16);
-    float v = 0.0f;
-    if (r < n && c < NOUT) {
-        const int64_t src = idx ? idx[r] : r;
-        v = yn[src * NOUT + c];
-    }
-    T[i] = v;
-}
-
-// dY = 2 (Y - T) / (n 6) on the n valid rows and 6 outputs (zero elsewhere),
-// BF16 in both layouts; per-block partial loss sums.
-__global__ void mlp_loss_dy(int64_t n, int64_t rows, const float* __restrict__ Y, const float* __restrict__ T,
-                            __nv_bfloat16* __restrict__ dY, __nv_bfloat16* __restrict__ dYt, float* __restrict__ part)
-{
-    __shared__ float red[256];
-    const int64_t r = blockIdx.x * (int64_t)256 + threadIdx.x;
-    const float scale = 1.0f / ((float)n * NOUT);
-    float loss = 0.0f;
-    if (r < rows) {
-        for (int c = 0; c < 16; ++c) {
-            float d = 0.0f;
-            if (r < n && c < NOUT) {
-                const float e = Y[r * 16 + c] - T[r * 16 + c];
-                loss += e * e * scale;
-                d = 2.0f * e * scale;
-            }
-            const __nv_bfloat16 h = __float2bfloat16_rn(d);
-            dY[r * 16 + c] = h;
-            dYt[(int64_t)c * rows + r] = h;
-        }
-    }
-    red[threadIdx.x] = loss;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// Bias gradients: row sums of the transposed dZ^T [dout x rows] (one warp per row).
-__global__ void mlp_bias_grad(int dout, int64_t rows, const __nv_bfloat16* __restrict__ dZt, float* __restrict__ gb)
-{
-    const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (row >= dout) return;
-    float s = 0.0f;
-    for (int64_t k = lane; k < rows; k += 32) s += __bfloat162float(dZt[(int64_t)row * rows + k]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) gb[row] = s;
+    X[i] = __float2bfloat16_rn(r < n && c < NIN ? xn[r * NIN + c] : 0.0f);
 }
 
 // Y [rows x 16] -> normalised outputs [n x 6]
@@ -291,20 +206,16 @@ GemmArgs gemm(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64
     return g;
 }
 
-// forward of `rows` packed rows (X already packed); train = keep Z, H^T
-cudaError_t forward(MlpDev& m, int64_t rows, bool train, cudaStream_t s, int64_t* launches)
+// forward of `rows` packed rows (X already packed)
+cudaError_t forward(MlpDev& m, int64_t rows, cudaStream_t s, int64_t* launches)
 {
     const __nv_bfloat16* in = m.X;
     int64_t ld_in = 32;
     for (int l = 0; l < 3; ++l) {
-        GemmArgs g = gemm(in, ld_in, m.Wb[l], DIN_P[l], rows, NH, DIN_P[l], EPI_BIAS_GELU, m.err);
+        GemmArgs g = gemm(in, ld_in, m.Wb[l], din_p(l), rows, NH, din_p(l), EPI_BIAS_GELU, m.err);
         g.bias = m.b[l];
-        g.out_f32 = train ? m.Z[l] : nullptr;
-        g.ld_out = NH;
         g.out_bf16 = m.Hb[l];
         g.ld_bf16 = NH;
-        g.out_bf16_t = train ? m.Ht[l] : nullptr;
-        g.ld_t = rows;
         cudaError_t e = launch_tc_gemm(g, s);
         if (e != cudaSuccess) return e;
         in = m.Hb[l];
@@ -318,70 +229,51 @@ cudaError_t forward(MlpDev& m, int64_t rows, bool train, cudaStream_t s, int64_t
     return launch_tc_gemm(g, s);
 }
 
-// loss, backward, bias gradients (rows padded to a multiple of 16; n valid)
-cudaError_t backward(MlpDev& m, int64_t n, int64_t rows, cudaStream_t s, int64_t* launches)
+// arguments of a minibatch: samples idx (or 0 .. n - 1) of the device arrays xn, yn
+TrainArgs train_args(MlpDev& m, int64_t n, int64_t rows, const float* xn, const float* yn, const int32_t* idx,
+                     float* loss_part)
 {
-    const unsigned nb = (unsigned)((rows + 255) / 256);
-    mlp_loss_dy<<<nb, 256, 0, s>>>(n, rows, m.Y, m.T, m.dY, m.dYt, m.loss_part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const __nv_bfloat16* dz = m.dY;   // [rows x dout]
-    const __nv_bfloat16* dzt = m.dYt; // [dout x rows]
-    for (int l = 3; l >= 0; --l) {
-        // dW_l = dZ_l^T H_{l-1}
-        const __nv_bfloat16* hin_t = l > 0 ? m.Ht[l - 1] : m.Xt;
-        GemmArgs g = gemm(dzt, rows, hin_t, rows, DOUT_P[l], DIN_P[l], (int)rows, EPI_STORE, m.err);
-        g.out_f32 = m.gW[l];
-        g.ld_out = DIN_P[l];
-        e = launch_tc_gemm(g, s);
-        if (e != cudaSuccess) return e;
-        mlp_bias_grad<<<(DOUT_P[l] + 7) / 8, 256, 0, s>>>(DOUT_P[l], rows, dzt, m.gb[l]);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        *launches += 2;
-        if (l == 0) break;
-        // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})
-        GemmArgs h = gemm(dz, DOUT_P[l], m.Wt[l], DOUT_P[l], rows, DIN_P[l], DOUT_P[l], EPI_DGELU, m.err);
-        h.zin = m.Z[l - 1];
-        h.ld_z = NH;
-        h.out_bf16 = m.dZ[l - 1];
-        h.ld_bf16 = NH;
-        h.out_bf16_t = m.dZt[l - 1];
-        h.ld_t = rows;
-        e = launch_tc_gemm(h, s);
-        if (e != cudaSuccess) return e;
-        *launches += 1;
-        dz = m.dZ[l - 1];
-        dzt = m.dZt[l - 1];
+    TrainArgs g;
+    g.xn = xn;
+    g.yn = yn;
+    g.idx = idx;
+    g.n = n;
+    g.rows = rows;
+    for (int l = 0; l < 4; ++l) {
+        g.Wb[l] = m.Wb[l];
+        g.Wt[l] = m.Wt[l];
+        g.W[l] = m.W[l];
+        g.b[l] = m.b[l];
+        g.mW[l] = m.mW[l];
+        g.vW[l] = m.vW[l];
+        g.mb[l] = m.mb[l];
+        g.vb[l] = m.vb[l];
+        g.gW[l] = m.gW[l];
+        g.gb[l] = m.gb[l];
     }
-    *launches += 1;
-    return cudaSuccess;
+    for (int l = 0; l < 3; ++l) {
+        g.Hb[l] = m.Hb[l];
+        g.Ht[l] = m.Ht[l];
+        g.dZ[l] = m.dZ[l];
+        g.dZt[l] = m.dZt[l];
+    }
+    g.Xt = m.Xt;
+    g.dY = m.dY;
+    g.dYt = m.dYt;
+    g.loss_part = loss_part;
+    g.err = m.err;
+    return g;
 }
 
 cudaError_t sync_bf16(MlpDev& m, cudaStream_t s)
 {
     for (int l = 0; l < 4; ++l) {
-        const int n = DOUT_P[l] * DIN_P[l];
-        mlp_sync_bf16<<<(n + 255) / 256, 256, 0, s>>>(m.W[l], DOUT_P[l], DIN_P[l], m.Wb[l], m.Wt[l]);
+        const int n = dout_p(l) * din_p(l);
+        mlp_sync_bf16<<<(n + 255) / 256, 256, 0, s>>>(m.W[l], dout_p(l), din_p(l), m.Wb[l], m.Wt[l]);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t adam_all(MlpDev& m, float lr, float b1, float b2, float eps, cudaStream_t s)
-{
-    m.step += 1;
-    const float c1 = 1.0f - powf(b1, (float)m.step), c2 = 1.0f - powf(b2, (float)m.step);
-    for (int l = 0; l < 4; ++l) {
-        const int nw = DOUT_P[l] * DIN_P[l], nbias = DOUT_P[l];
-        mlp_adam<<<(nw + 255) / 256, 256, 0, s>>>(nw, m.W[l], m.gW[l], m.mW[l], m.vW[l], lr, b1, b2, eps, c1, c2);
-        mlp_adam<<<(nbias + 255) / 256, 256, 0, s>>>(nbias, m.b[l], m.gb[l], m.mb[l], m.vb[l], lr, b1, b2, eps, c1,
-                                                     c2);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return sync_bf16(m, s);
 }
 
 // packed (unpadded, oracle order) <-> padded device layout
@@ -394,7 +286,7 @@ int64_t packed_count()
 
 ptadd_status read_loss(MlpDev& m, int64_t rows, cudaStream_t s, float* loss)
 {
-    const int nb = (int)((rows + 255) / 256);
+    const int nb = (int)((rows + 127) / 128);
     std::vector<float> part(nb);
     PTADD_CUDA(cudaMemcpyAsync(part.data(), m.loss_part, nb * sizeof(float), cudaMemcpyDeviceToHost, s));
     int err = 0;
@@ -475,9 +367,9 @@ ptadd_status ptadd_mlp_set_params(ptadd_ctx* ctx, const float* p, int64_t count)
     cudaStream_t s = ctx->own_stream;
     int64_t off = 0;
     for (int l = 0; l < 4; ++l) {
-        std::vector<float> W((size_t)DOUT_P[l] * DIN_P[l], 0.0f), b(DOUT_P[l], 0.0f);
+        std::vector<float> W((size_t)dout_p(l) * din_p(l), 0.0f), b(dout_p(l), 0.0f);
         for (int o = 0; o < DOUT_U[l]; ++o)
-            for (int c = 0; c < DIN_U[l]; ++c) W[(size_t)o * DIN_P[l] + c] = p[off++];
+            for (int c = 0; c < DIN_U[l]; ++c) W[(size_t)o * din_p(l) + c] = p[off++];
         for (int o = 0; o < DOUT_U[l]; ++o) b[o] = p[off++];
         PTADD_CUDA(cudaMemcpyAsync(m.W[l], W.data(), W.size() * 4, cudaMemcpyHostToDevice, s));
         PTADD_CUDA(cudaMemcpyAsync(m.b[l], b.data(), b.size() * 4, cudaMemcpyHostToDevice, s));
@@ -504,12 +396,12 @@ ptadd_status ptadd_mlp_get_params(ptadd_ctx* ctx, float* p, int64_t count)
     cudaStream_t s = ctx->own_stream;
     int64_t off = 0;
     for (int l = 0; l < 4; ++l) {
-        std::vector<float> W((size_t)DOUT_P[l] * DIN_P[l]), b(DOUT_P[l]);
+        std::vector<float> W((size_t)dout_p(l) * din_p(l)), b(dout_p(l));
         PTADD_CUDA(cudaMemcpyAsync(W.data(), m.W[l], W.size() * 4, cudaMemcpyDeviceToHost, s));
         PTADD_CUDA(cudaMemcpyAsync(b.data(), m.b[l], b.size() * 4, cudaMemcpyDeviceToHost, s));
         PTADD_CUDA(cudaStreamSynchronize(s));
         for (int o = 0; o < DOUT_U[l]; ++o)
-            for (int c = 0; c < DIN_U[l]; ++c) p[off++] = W[(size_t)o * DIN_P[l] + c];
+            for (int c = 0; c < DIN_U[l]; ++c) p[off++] = W[(size_t)o * din_p(l) + c];
         for (int o = 0; o < DOUT_U[l]; ++o) p[off++] = b[o];
     }
     return PTADD_OK;
@@ -553,13 +445,8 @@ ptadd_status ptadd_mlp_loss_grad(ptadd_ctx* ctx, int64_t n, const float* xn, con
     int64_t launches = 0;
     cudaError_t e = cudaMemcpyAsync(dx, xn, (size_t)n * NIN * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dy, yn, (size_t)n * NOUT * 4, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) {
-        mlp_pack_x<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(n, rows, dx, nullptr, m.X, m.Xt);
-        mlp_pack_t<<<(unsigned)((rows * 16 + 255) / 256), 256, 0, s>>>(n, rows, dy, nullptr, m.T);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = forward(m, rows, true, s, &launches);
-    if (e == cudaSuccess) e = backward(m, n, rows, s, &launches);
+    if (e == cudaSuccess) e = launch_mlp_train(train_args(m, n, rows, dx, dy, nullptr, m.loss_part), s);
+    launches += 2;
     if (e != cudaSuccess) {
         cudaFree(dx);
         cudaFree(dy);
@@ -573,16 +460,16 @@ ptadd_status ptadd_mlp_loss_grad(ptadd_ctx* ctx, int64_t n, const float* xn, con
     if (grad) {
         int64_t off = 0;
         for (int l = 0; l < 4; ++l) {
-            std::vector<float> W((size_t)DOUT_P[l] * DIN_P[l]), b(DOUT_P[l]);
+            std::vector<float> W((size_t)dout_p(l) * din_p(l)), b(dout_p(l));
             PTADD_CUDA(cudaMemcpyAsync(W.data(), m.gW[l], W.size() * 4, cudaMemcpyDeviceToHost, s));
             PTADD_CUDA(cudaMemcpyAsync(b.data(), m.gb[l], b.size() * 4, cudaMemcpyDeviceToHost, s));
             PTADD_CUDA(cudaStreamSynchronize(s));
             for (int o = 0; o < DOUT_U[l]; ++o)
-                for (int c = 0; c < DIN_U[l]; ++c) grad[off++] = W[(size_t)o * DIN_P[l] + c];
+                for (int c = 0; c < DIN_U[l]; ++c) grad[off++] = W[(size_t)o * din_p(l) + c];
             for (int o = 0; o < DOUT_U[l]; ++o) grad[off++] = b[o];
         }
     }
-    ctx->kernel_launches += launches + 2;
+    ctx->kernel_launches += launches;
     return PTADD_OK;
 }
 
@@ -602,7 +489,7 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
     int32_t* didx = nullptr;
     // per-minibatch loss partials of an epoch, kept on the device and read once
     // per epoch (reading them per minibatch would stall the stream every time)
-    const int nb = (int)((rows + 255) / 256);
+    const int nb = (int)((rows + 127) / 128);
     const int64_t nbatches = n / batch;
     if ((st = m_alloc(&dx, (size_t)n * NIN)) != PTADD_OK) return st;
     if ((st = m_alloc(&dy, (size_t)n * NOUT)) != PTADD_OK || (st = m_alloc(&didx, (size_t)n)) != PTADD_OK ||
@@ -626,16 +513,17 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
         double ep_loss = 0.0;
         int nbatch = 0;
         for (int64_t b0 = 0; b0 + batch <= n && e == cudaSuccess; b0 += batch) {  // full batches only
-            mlp_pack_x<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(batch, rows, dx, didx + b0, m.X, m.Xt);
-            mlp_pack_t<<<(unsigned)((rows * 16 + 255) / 256), 256, 0, s>>>(batch, rows, dy, didx + b0, m.T);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) e = forward(m, rows, true, s, &launches);
-            if (e == cudaSuccess) e = backward(m, batch, rows, s, &launches);
-            if (e == cudaSuccess) e = adam_all(m, lr, 0.9f, 0.999f, 1e-8f, s);
-            launches += 2 + 8 + 4;
-            if (e == cudaSuccess && loss_per_epoch)
-                e = cudaMemcpyAsync(dloss + (size_t)nbatch * nb, m.loss_part, nb * sizeof(float),
-                                    cudaMemcpyDeviceToDevice, s);
+            TrainArgs g = train_args(m, batch, rows, dx, dy, didx + b0, dloss + (size_t)nbatch * nb);
+            m.step += 1;
+            g.adam = 1;
+            g.lr = lr;
+            g.b1 = 0.9f;
+            g.b2 = 0.999f;
+            g.eps = 1e-8f;
+            g.c1 = 1.0f - powf(g.b1, (float)m.step);
+            g.c2 = 1.0f - powf(g.b2, (float)m.step);
+            e = launch_mlp_train(g, s);
+            launches += 2;
             ++nbatch;
         }
         if (e == cudaSuccess && loss_per_epoch && nbatch)
@@ -703,8 +591,8 @@ ptadd_status ptadd_mlp_forward(ptadd_ctx* ctx, int64_t n, const float* xn, float
         const int64_t rows = (k + 127) / 128 * 128;
         e = cudaMemcpyAsync(dx, xn + r0 * NIN, (size_t)k * NIN * 4, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) break;
-        mlp_pack_x<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(k, rows, dx, nullptr, m.X, m.Xt);
-        e = forward(m, rows, false, s, &launches);
+        mlp_pack_x<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(k, rows, dx, m.X);
+        e = forward(m, rows, s, &launches);
         if (e != cudaSuccess) break;
         mlp_unpack_y<<<(unsigned)((k * NOUT + 255) / 256), 256, 0, s>>>(k, m.Y, dy);
         e = cudaMemcpyAsync(yn + r0 * NOUT, dy, (size_t)k * NOUT * 4, cudaMemcpyDeviceToHost, s);

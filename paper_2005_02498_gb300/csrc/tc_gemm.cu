@@ -98,48 +98,18 @@ __global__ void __launch_bounds__(GEMM_THREADS) tc_gemm_kernel(GemmArgs g)
                     }
                     o[i] = w;
                 }
-            } else if (g.epi == EPI_STORE_T) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) g.out_f32[(int64_t)(c + i) * g.ld_out + r] = v[i];
             } else {
-                // EPI_BIAS_GELU: z = C + bias (kept in FP32 if asked), h = GELU(z);
-                // EPI_DGELU: h = C * GELU'(zin).  h -> BF16, row-major and/or transposed
+                // EPI_BIAS_GELU
                 uint32_t hw[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    float h0, h1;
-                    if (g.epi == EPI_BIAS_GELU) {
-                        const float z0 = v[2 * i] + g.bias[c + 2 * i], z1 = v[2 * i + 1] + g.bias[c + 2 * i + 1];
-                        v[2 * i] = z0;
-                        v[2 * i + 1] = z1;
-                        h0 = gelu_f(z0);
-                        h1 = gelu_f(z1);
-                    } else {
-                        const float2 zi = *reinterpret_cast<const float2*>(g.zin + r * g.ld_z + c + 2 * i);
-                        h0 = v[2 * i] * gelu_grad_f(zi.x);
-                        h1 = v[2 * i + 1] * gelu_grad_f(zi.y);
-                    }
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(h0, h1);
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(gelu_f(v[2 * i] + g.bias[c + 2 * i]),
+                                                                   gelu_f(v[2 * i + 1] + g.bias[c + 2 * i + 1]));
                     hw[i] = *reinterpret_cast<const uint32_t*>(&h);
                 }
-                if (g.epi == EPI_BIAS_GELU && g.out_f32) {
-                    float4* o = reinterpret_cast<float4*>(g.out_f32 + r * g.ld_out + c);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                }
-                if (g.out_bf16) {
-                    uint4* o = reinterpret_cast<uint4*>(g.out_bf16 + r * g.ld_bf16 + c);
-                    o[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                    o[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
-                }
-                if (g.out_bf16_t) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&hw[i]);
-                        g.out_bf16_t[(int64_t)(c + 2 * i) * g.ld_t + r] = h.x;
-                        g.out_bf16_t[(int64_t)(c + 2 * i + 1) * g.ld_t + r] = h.y;
-                    }
-                }
+                uint4* o = reinterpret_cast<uint4*>(g.out_bf16 + r * g.ld_bf16 + c);
+                o[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                o[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
             }
         }
     } else if (threadIdx.x == 0) {

@@ -125,9 +125,7 @@ __host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N)
 enum GemmEpi : int {
     EPI_STORE = 0,      // C -> out_f32 (row-major)
     EPI_BIAS = 1,       // C + bias -> out_f32
-    EPI_BIAS_GELU = 2,  // z = C + bias -> out_f32 (z), GELU(z) -> out_bf16 (+ transposed)
-    EPI_DGELU = 3,      // C * GELU'(zin) -> out_bf16 (+ transposed)
-    EPI_STORE_T = 4,    // C -> out_f32 transposed: out[c * ld_out + r]
+    EPI_BIAS_GELU = 2,  // GELU(C + bias) -> out_bf16
 };
 
 struct GemmArgs {
@@ -144,10 +142,6 @@ struct GemmArgs {
     int64_t ld_out;
     __nv_bfloat16* out_bf16;
     int64_t ld_bf16;
-    __nv_bfloat16* out_bf16_t;  // element (r, c) at [c * ld_t + r]
-    int64_t ld_t;
-    const float* zin;
-    int64_t ld_z;
     int* err;  // set to 1 if an MMA wait gave up
     int withhold_mma;  // self-test of the bounded waits: issue no MMA and no commit
 };
@@ -162,10 +156,6 @@ constexpr int GEMM_SMEM = 2 * GEMM_STAGE + 1024;     // two stages + alignment s
 constexpr long long MBAR_WAIT_LIMIT = 4000000000LL;  // ~2 s of SM clocks
 
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
 
 // Asynchronous copy of a [rows x 64] K-chunk (columns k0..k0+63 of a
 // K-contiguous matrix, rows row0..row0+rows-1) into the canonical layout at
