@@ -59,8 +59,13 @@ cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& 
 // same order (broadcast reads) and accumulates (sigma b') at its 4 Gauss points.
 constexpr int MIX_TPB = 128;
 constexpr int MIX_MAX_CHUNKS = 64;
-constexpr int MIX_TILE = 192;  // sources per staged tile: 3 blocks of 66.5 KB fit one SM's shared memory
-constexpr int MIX_MINB = 3;  // resident blocks per SM the register budget is sized for
+constexpr int MIX_TILE = 192;  // sources per tile (one plain FP32 sum), staged 64 at a time
+// Resident blocks per SM.  Bound by the FP32 pipe (183 packed instructions per
+// source and warp, two cycles each); four blocks at 128 registers (24 bytes
+// spilled outside the loop's arithmetic) keep it busier than three at 160: 32 768
+// segments 13.50 against 13.90 ms per launch, 8192 segments 0.997 against 1.017;
+// five at 96 registers 13.64 and 1.024.
+constexpr int MIX_MINB = 4;
 
 // FP64 path.  Bound by the FP32 pipe: about 1550 packed FP32 instructions per
 // source and warp, two pipe cycles each (3100 of the 3650 cycles that a source
@@ -105,28 +110,25 @@ __global__ void __launch_bounds__(MIX_TPB, MIX_MINB) pair_mixed_kernel(TileArgs 
     pair_tile_mixed<MIX_TILE, MIX_TPB>(a, c, near2, sm);
 }
 
-// SMs and resident pair blocks per SM, queried once per device and precision.
-static void pair_slots(int mixed, int& sms, int& per_sm)
+// SMs and resident blocks per SM of the FP64 kernel, queried once per device.
+static void pair_slots(int& sms, int& per_sm)
 {
-    static std::atomic<int> cached[64][2][2];  // [device][mixed] -> {sms, blocks per SM}; 0: not yet
+    static std::atomic<int> cached[64][2];  // [device] -> {sms, blocks per SM}; 0: not yet
     int dev = 0;
     sms = 152;
-    per_sm = 2;
+    per_sm = 16;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
-        cached[dev][mixed][0].load(std::memory_order_acquire) > 0) {
-        sms = cached[dev][mixed][0].load(std::memory_order_relaxed);
-        per_sm = cached[dev][mixed][1].load(std::memory_order_relaxed);
+        cached[dev][0].load(std::memory_order_acquire) > 0) {
+        sms = cached[dev][0].load(std::memory_order_relaxed);
+        per_sm = cached[dev][1].load(std::memory_order_relaxed);
         return;
     }
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (mixed)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_mixed_kernel, MIX_TPB, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_fp64_kernel, 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pair_fp64_kernel, 32, 0);
     if (per_sm < 1) per_sm = 1;
     if (dev >= 0 && dev < 64) {
-        cached[dev][mixed][1].store(per_sm, std::memory_order_relaxed);
-        cached[dev][mixed][0].store(sms, std::memory_order_release);
+        cached[dev][1].store(per_sm, std::memory_order_relaxed);
+        cached[dev][0].store(sms, std::memory_order_release);
     }
 }
 
@@ -142,7 +144,7 @@ int64_t fp64_chunk_len(int64_t tiles, int64_t n_src)
     // sources 101 / 57 / 35 in 20 / 10 / 5; 1041 x 1485 244 / 220 / 190 in 23 / 12 /
     // 6; 8192 segments 6330 / 6163 / 6155 in 128 / 64 / 32.
     int sms, per_sm;
-    pair_slots(0, sms, per_sm);
+    pair_slots(sms, per_sm);
     const int64_t slots = (int64_t)sms * per_sm;
     tiles = std::max<int64_t>(tiles, 1);
     int64_t ch = std::min((16 * slots + tiles - 1) / tiles, n_src / 64);
@@ -159,21 +161,23 @@ int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
         len = std::max(len, (n_src + max_chunks - 1) / max_chunks);
         return (int)((n_src + len - 1) / len);
     }
-    // About 16 waves of resident blocks, so that the blocks still running
+    // About 48 blocks per SM (12 waves), so that the blocks still running
     // when the others have finished (the tail) cost a few per cent; chunks of
     // at least 256 sources, so the per-block set-up and the nodal
     // output stay small next to the pair work, unless that leaves less than
-    // one wave (a small network): then chunks down to 32 sources, so that the
-    // few targets' work (and their FP64 near pairs) spreads over more SMs.
+    // three blocks per SM (a small network): then chunks down to 32 sources, so that the
+    // few targets' work (and their FP64 near pairs) spreads over more SMs.  The
+    // numbers do not follow the occupancy: a chunk's start is where the FP32 sums
+    // start, and moving it moves averaged rates by 1e-9.
     int sms, per_sm;
-    pair_slots(1, sms, per_sm);
+    pair_slots(sms, per_sm);
     const int64_t tiles_t = (n_tgt + MIX_TPB - 1) / MIX_TPB;
     int64_t cap = n_src / 256;
-    if (tiles_t * cap < (int64_t)sms * per_sm) cap = std::max<int64_t>(cap, n_src / 32);
+    if (tiles_t * cap < (int64_t)sms * 3) cap = std::max<int64_t>(cap, n_src / 32);
     if (cap > MIX_MAX_CHUNKS) cap = MIX_MAX_CHUNKS;
     if (cap > max_chunks) cap = max_chunks;
     if (cap < 1) cap = 1;
-    const int64_t want_blocks = (int64_t)sms * per_sm * 16;
+    const int64_t want_blocks = (int64_t)sms * 48;
     int64_t ch = (want_blocks + tiles_t - 1) / (tiles_t > 0 ? tiles_t : 1);
     if (ch > cap) ch = cap;
     if (ch < 1) ch = 1;

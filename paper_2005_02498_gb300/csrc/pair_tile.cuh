@@ -567,11 +567,9 @@ __device__ __forceinline__ void kahan_add2(float2& s, float2& c, float2 v)
     c = sub2(sub2(t, s), y);
     s = t;
 }
-// sources summed plainly before a compensated add: no fewer than a staged
-// tile holds, so each tile's sources form one plain group
-constexpr int SUM_GROUP = 256;
-// sources of one group handled per loop iteration (two independent chains)
-constexpr int MIX_UNROLL = 2;
+// A tile's sources are staged this many at a time, so that four blocks fit an
+// SM's shared memory (41 KB each); their plain sums run over the whole tile.
+constexpr int MIX_STAGE = 64;
 // keep a register value opaque, so the compiler holds it instead of
 // recomputing it from its (FP64) inputs inside the loop
 __device__ __forceinline__ void opaque(float& x) { asm volatile("" : "+f"(x)); }
@@ -711,7 +709,7 @@ __device__ __forceinline__ void seg_coef2(const Geo2& G, const Src2& S, const fl
 
 template <int TILE, int TPB>
 struct MixSmem {
-    float2 tile[TILE * MIX_REC];  // source records (MIX_REC float2 each)
+    float2 tile[MIX_STAGE * MIX_REC];  // source records (MIX_REC float2 each)
     double nacc[12 * TPB];             // FP64 sums: [qp * 3 + e][thread]
     float2 ksum[12 * TPB];             // Kahan sums of the work item: [p * 3 + e][thread], then compensations
     uint2 queue[TPB / 32][NEAR_Q];
@@ -784,8 +782,19 @@ __device__ __forceinline__ void pair_tile_mixed(const TileArgs& a, const Consts&
     int qn = 0;             // entries waiting in this warp's queue (warp-uniform)
     unsigned near_warp = 0;  // near point-pairs of this warp (warp-uniform)
 
-    for (int64_t j0 = a.js; j0 < a.je; j0 += TILE) {
-        const int cnt = (int)min((int64_t)TILE, a.je - j0);
+    static_assert(TILE % MIX_STAGE == 0, "a tile is a whole number of stages");
+    // plain sums of the open tile's sources (/ c2); the b' term's coefficient is
+    // summed on its own (b' is the target's)
+    float2 SG[2][3], SB[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        SB[p] = f2(0.0f);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) SG[p][e] = f2(0.0f);
+    }
+    int open = 0;  // sources staged of the open tile
+    for (int64_t j0 = a.js; j0 < a.je; j0 += MIX_STAGE) {
+        const int cnt = (int)min((int64_t)MIX_STAGE, a.je - j0);
         __syncthreads();
         for (int js = threadIdx.x; js < cnt; js += blockDim.x) {
             const float4* g = reinterpret_cast<const float4*>(a.src32 + (int64_t)SRC32_STRIDE * (j0 + js));
@@ -807,110 +816,107 @@ __device__ __forceinline__ void pair_tile_mixed(const TileArgs& a, const Consts&
             d[11] = make_float4(v[6] * v[6], v[6] * v[6], v[6] + v[6], v[6] + v[6]);
         }
         __syncthreads();
-        // plain sums of the current group of SUM_GROUP sources (/ c2); the
-        // b' term's coefficient is summed on its own (b' is the target's)
-        float2 SG[2][3], SB[2];
-        for (int g0 = 0; g0 < cnt; g0 += SUM_GROUP) {
-            const int g1 = min(cnt, g0 + SUM_GROUP);
+        for (int jj = 0; jj < cnt; ++jj) {
+            const float2* r = sm.tile + jj * MIX_REC;
+            if (!(r[6].x > 0.0f)) continue;  // zero-length source (uniform branch)
+            Src2 S;
+            S.L = r[6];
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                S.t[e] = r[7 + e];
+                S.b[e] = r[10 + e];
+                S.q[e] = r[13 + e];
+                S.nt[e] = r[16 + e];
+                S.nb[e] = r[19 + e];
+            }
+            S.LL = r[22];
+            S.L2 = r[23];
+            Pair2 P;
+            // (scalar: both lanes hold the same value)
+            P.tb = f2(__fmaf_rn(S.t[0].x, btf[0], __fmaf_rn(S.t[1].x, btf[1], __fmul_rn(S.t[2].x, btf[2]))));
+            P.qb = f2(__fmaf_rn(S.q[0].x, btf[0], __fmaf_rn(S.q[1].x, btf[1], __fmul_rn(S.q[2].x, btf[2]))));
+            P.ntb = neg2(P.tb);
+            P.nqb = neg2(P.qb);
+            // the source start in this thread's frame
+            float x1t[3];
+#pragma unroll
+            for (int e = 0; e < 3; ++e) x1t[e] = (r[e].x + nOt[e]) + r[3 + e].x;
+            // near test of both Gauss-point pairs first (point-to-segment
+            // distance), then the coefficients (near lanes give 0)
+            Geo2 G[2];
+            bool nrq[2][2];
+            bool same_all = true;
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                SB[p] = f2(0.0f);
+                float2 R0[3];
 #pragma unroll
-                for (int e = 0; e < 3; ++e) SG[p][e] = f2(0.0f);
+                for (int e = 0; e < 3; ++e) R0[e] = sub2(XT[p][e], f2(x1t[e]));
+                seg_geo2(R0, S, a2, G[p]);
+                const float2 ny = G[p].ny, u2 = G[p].u2;
+                // y < 0: nearest to x1; y > L: nearest to x2; else to the line
+                const float2 dd = sel2(ny.x > 0.0f, ny.y > 0.0f, G[p].r1s,
+                                       sel2(u2.x < 0.0f, u2.y < 0.0f, G[p].r2s, G[p].d2));
+                nrq[p][0] = active && dd.x < near2;
+                nrq[p][1] = active && dd.y < near2;
+                same_all = same_all && (ny.x >= 0.0f || u2.x <= 0.0f) && (ny.y >= 0.0f || u2.y <= 0.0f);
             }
-#pragma unroll MIX_UNROLL
-            for (int jj = g0; jj < g1; ++jj) {
-                const float2* r = sm.tile + jj * MIX_REC;
-                if (!(r[6].x > 0.0f)) continue;  // zero-length source (uniform branch)
-                Src2 S;
-                S.L = r[6];
+            const bool uni = __all_sync(0xffffffffu, same_all);
+            // both Gauss-point pairs in one straight block per branch, so
+            // that their two chains interleave
+            Coef2 C[2];
+            if (uni) {
+                seg_coef2<1>(G[0], S, bt2, P, a2, nr, nra2, kn, nrq[0][0], nrq[0][1], C[0]);
+                seg_coef2<1>(G[1], S, bt2, P, a2, nr, nra2, kn, nrq[1][0], nrq[1][1], C[1]);
+            } else {
+                seg_coef2<0>(G[0], S, bt2, P, a2, nr, nra2, kn, nrq[0][0], nrq[0][1], C[0]);
+                seg_coef2<0>(G[1], S, bt2, P, a2, nr, nra2, kn, nrq[1][0], nrq[1][1], C[1]);
+            }
 #pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    S.t[e] = r[7 + e];
-                    S.b[e] = r[10 + e];
-                    S.q[e] = r[13 + e];
-                    S.nt[e] = r[16 + e];
-                    S.nb[e] = r[19 + e];
+            for (int p = 0; p < 2; ++p) {
+                SB[p] = fma2(C[p].Q, C[p].cb, SB[p]);  // (times b' when the group closes)
+#pragma unroll
+                for (int e = 0; e < 3; ++e)
+                    SG[p][e] = fma2(C[p].Q, fma2(C[p].cRxb, C[p].X[e], fma2(C[p].cq, S.q[e],
+                                    fma2(C[p].cRp, G[p].Rp[e], mul2(C[p].ct, S.t[e])))), SG[p][e]);
+            }
+            if (__any_sync(0xffffffffu, nrq[0][0] || nrq[0][1] || nrq[1][0] || nrq[1][1])) {
+                const unsigned js = (unsigned)(j0 + jj);
+#pragma unroll
+                for (int qp = 0; qp < 4; ++qp) {
+                    const bool mine = nrq[qp >> 1][qp & 1];
+                    const unsigned bal = __ballot_sync(0xffffffffu, mine);
+                    if (mine) wq[qn + __popc(bal & lt)] = make_uint2(js, ((unsigned)lane << 2) | (unsigned)qp);
+                    qn += __popc(bal);
+                    near_warp += (unsigned)__popc(bal);
                 }
-                S.LL = r[22];
-                S.L2 = r[23];
-                Pair2 P;
-                P.tb = fma2(S.t[0], bt2[0], fma2(S.t[1], bt2[1], mul2(S.t[2], bt2[2])));
-                P.qb = fma2(S.q[0], bt2[0], fma2(S.q[1], bt2[1], mul2(S.q[2], bt2[2])));
-                P.ntb = neg2(P.tb);
-                P.nqb = neg2(P.qb);
-                // the source start in this thread's frame
-                float x1t[3];
-#pragma unroll
-                for (int e = 0; e < 3; ++e) x1t[e] = (r[e].x + nOt[e]) + r[3 + e].x;
-                // near test of both Gauss-point pairs first (point-to-segment
-                // distance), then the coefficients (near lanes give 0)
-                Geo2 G[2];
-                bool nrq[2][2];
-                bool same_all = true;
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    float2 R0[3];
-#pragma unroll
-                    for (int e = 0; e < 3; ++e) R0[e] = sub2(XT[p][e], f2(x1t[e]));
-                    seg_geo2(R0, S, a2, G[p]);
-                    const float2 ny = G[p].ny, u2 = G[p].u2;
-                    // y < 0: nearest to x1; y > L: nearest to x2; else to the line
-                    const float2 dd = sel2(ny.x > 0.0f, ny.y > 0.0f, G[p].r1s,
-                                           sel2(u2.x < 0.0f, u2.y < 0.0f, G[p].r2s, G[p].d2));
-                    nrq[p][0] = active && dd.x < near2;
-                    nrq[p][1] = active && dd.y < near2;
-                    same_all = same_all && (ny.x >= 0.0f || u2.x <= 0.0f) && (ny.y >= 0.0f || u2.y <= 0.0f);
-                }
-                const bool uni = __all_sync(0xffffffffu, same_all);
-                // both Gauss-point pairs in one straight block per branch, so
-                // that their two chains interleave
-                Coef2 C[2];
-                if (uni) {
-                    seg_coef2<1>(G[0], S, bt2, P, a2, nr, nra2, kn, nrq[0][0], nrq[0][1], C[0]);
-                    seg_coef2<1>(G[1], S, bt2, P, a2, nr, nra2, kn, nrq[1][0], nrq[1][1], C[1]);
-                } else {
-                    seg_coef2<0>(G[0], S, bt2, P, a2, nr, nra2, kn, nrq[0][0], nrq[0][1], C[0]);
-                    seg_coef2<0>(G[1], S, bt2, P, a2, nr, nra2, kn, nrq[1][0], nrq[1][1], C[1]);
-                }
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    SB[p] = fma2(C[p].Q, C[p].cb, SB[p]);  // (times b' when the group closes)
-#pragma unroll
-                    for (int e = 0; e < 3; ++e)
-                        SG[p][e] = fma2(C[p].Q, fma2(C[p].cRxb, C[p].X[e], fma2(C[p].cq, S.q[e],
-                                        fma2(C[p].cRp, G[p].Rp[e], mul2(C[p].ct, S.t[e])))), SG[p][e]);
-                }
-                if (__any_sync(0xffffffffu, nrq[0][0] || nrq[0][1] || nrq[1][0] || nrq[1][1])) {
-                    const unsigned js = (unsigned)(j0 + jj);
-#pragma unroll
-                    for (int qp = 0; qp < 4; ++qp) {
-                        const bool mine = nrq[qp >> 1][qp & 1];
-                        const unsigned bal = __ballot_sync(0xffffffffu, mine);
-                        if (mine) wq[qn + __popc(bal & lt)] = make_uint2(js, ((unsigned)lane << 2) | (unsigned)qp);
-                        qn += __popc(bal);
-                        near_warp += (unsigned)__popc(bal);
-                    }
-                    while (qn >= 32) {
-                        __syncwarp();
-                        near_flush(a.pos, n, a.nxt, a.src, a.k64, seg, wq, 32, sm.nacc, TPB);
-                        near_shift(wq, qn);
-                        qn -= 32;
-                    }
+                while (qn >= 32) {
+                    __syncwarp();
+                    near_flush(a.pos, n, a.nxt, a.src, a.k64, seg, wq, 32, sm.nacc, TPB);
+                    near_shift(wq, qn);
+                    qn -= 32;
                 }
             }
-            // close the group
+        }
+        // close the tile
+        open += MIX_STAGE;
+        if (open < TILE && j0 + MIX_STAGE < a.je) continue;
+        open = 0;
 #pragma unroll
-            for (int p = 0; p < 2; ++p)
+        for (int p = 0; p < 2; ++p)
 #pragma unroll
-                for (int e = 0; e < 3; ++e) SG[p][e] = fma2(SB[p], bt2[e], SG[p][e]);
+            for (int e = 0; e < 3; ++e) SG[p][e] = fma2(SB[p], bt2[e], SG[p][e]);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                float2 sk = sm.ksum[k * TPB + threadIdx.x], ck = sm.ksum[(6 + k) * TPB + threadIdx.x];
-                kahan_add2(sk, ck, SG[k / 3][k % 3]);
-                sm.ksum[k * TPB + threadIdx.x] = sk;
-                sm.ksum[(6 + k) * TPB + threadIdx.x] = ck;
-            }
+        for (int k = 0; k < 6; ++k) {
+            float2 sk = sm.ksum[k * TPB + threadIdx.x], ck = sm.ksum[(6 + k) * TPB + threadIdx.x];
+            kahan_add2(sk, ck, SG[k / 3][k % 3]);
+            sm.ksum[k * TPB + threadIdx.x] = sk;
+            sm.ksum[(6 + k) * TPB + threadIdx.x] = ck;
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            SB[p] = f2(0.0f);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) SG[p][e] = f2(0.0f);
         }
     }
     // compensated sums of the work item's sources to FP64, restoring the factor c2
