@@ -57,15 +57,15 @@ cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& 
 // warp), y = source chunks.  Each block runs one tile (pair_tile.cuh): it
 // stages source records through shared memory; every thread walks them in the
 // same order (broadcast reads) and accumulates (sigma b') at its 4 Gauss points.
-constexpr int MIX_TPB = 128;
+constexpr int MIX_TPB = 32;
 constexpr int MIX_MAX_CHUNKS = 64;
-constexpr int MIX_TILE = 192;  // sources per tile (one plain FP32 sum), staged 64 at a time
-// Resident blocks per SM.  Bound by the FP32 pipe (183 packed instructions per
-// source and warp, two cycles each); four blocks at 128 registers (24 bytes
-// spilled outside the loop's arithmetic) keep it busier than three at 160: 32 768
-// segments 13.50 against 13.90 ms per launch, 8192 segments 0.997 against 1.017;
-// five at 96 registers 13.64 and 1.024.
-constexpr int MIX_MINB = 4;
+constexpr int MIX_TILE = 192;  // sources per tile (one plain FP32 sum), staged 32 at a time
+// One-warp blocks, 16 per SM.  Bound by the FP32 pipe (183 packed instructions per
+// source and warp, two cycles each); 16 warps at 128 registers (16 bytes spilled
+// outside the loop's arithmetic) keep it busier than 12 at 160.  32 768 / 8192 segments:
+// 13.28 / 0.947 ms per launch, blocks of two warps 13.38 / 0.948, of four 13.41 / 0.987
+// (the tail is a warp's tile long, not a block's), three blocks of four warps 13.82 / 1.066.
+constexpr int MIX_MINB = 16;
 
 // FP64 path.  Bound by the FP32 pipe: about 1550 packed FP32 instructions per
 // source and warp, two pipe cycles each (3100 of the 3650 cycles that a source
@@ -171,7 +171,7 @@ int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
     // start, and moving it moves averaged rates by 1e-9.
     int sms, per_sm;
     pair_slots(sms, per_sm);
-    const int64_t tiles_t = (n_tgt + MIX_TPB - 1) / MIX_TPB;
+    const int64_t tiles_t = (n_tgt + 127) / 128;
     int64_t cap = n_src / 256;
     if (tiles_t * cap < (int64_t)sms * 3) cap = std::max<int64_t>(cap, n_src / 32);
     if (cap > MIX_MAX_CHUNKS) cap = MIX_MAX_CHUNKS;

@@ -567,9 +567,10 @@ __device__ __forceinline__ void kahan_add2(float2& s, float2& c, float2 v)
     c = sub2(sub2(t, s), y);
     s = t;
 }
-// A tile's sources are staged this many at a time, so that four blocks fit an
-// SM's shared memory (41 KB each); their plain sums run over the whole tile.
-constexpr int MIX_STAGE = 64;
+// A tile's sources are staged this many at a time, so that 16 warps' worth of blocks
+// fit an SM's shared memory; their plain sums run over the whole tile.
+template <int TPB>
+constexpr int mix_stage() { return TPB == 32 ? 32 : 64; }
 // keep a register value opaque, so the compiler holds it instead of
 // recomputing it from its (FP64) inputs inside the loop
 __device__ __forceinline__ void opaque(float& x) { asm volatile("" : "+f"(x)); }
@@ -709,7 +710,7 @@ __device__ __forceinline__ void seg_coef2(const Geo2& G, const Src2& S, const fl
 
 template <int TILE, int TPB>
 struct MixSmem {
-    float2 tile[MIX_STAGE * MIX_REC];  // source records (MIX_REC float2 each)
+    float2 tile[mix_stage<TPB>() * MIX_REC];  // source records (MIX_REC float2 each)
     double nacc[12 * TPB];             // FP64 sums: [qp * 3 + e][thread]
     float2 ksum[12 * TPB];             // Kahan sums of the work item: [p * 3 + e][thread], then compensations
     uint2 queue[TPB / 32][NEAR_Q];
@@ -782,6 +783,7 @@ __device__ __forceinline__ void pair_tile_mixed(const TileArgs& a, const Consts&
     int qn = 0;             // entries waiting in this warp's queue (warp-uniform)
     unsigned near_warp = 0;  // near point-pairs of this warp (warp-uniform)
 
+    constexpr int MIX_STAGE = mix_stage<TPB>();
     static_assert(TILE % MIX_STAGE == 0, "a tile is a whole number of stages");
     // plain sums of the open tile's sources (/ c2); the b' term's coefficient is
     // summed on its own (b' is the target's)
