@@ -47,7 +47,7 @@ struct MlpDev {
     int64_t cap = 0;  // row capacity of the work buffers (multiple of 128)
     float *W[4] = {}, *b[4] = {}, *mW[4] = {}, *vW[4] = {}, *mb[4] = {}, *vb[4] = {}, *gW[4] = {}, *gb[4] = {};
     __nv_bfloat16 *Wb[4] = {}, *Wt[4] = {};
-    __nv_bfloat16* Wc = nullptr;  // layers 2, 3 staged for the fused inference kernel (bias block + 4 x 256 x 64 each)
+    uint8_t* stage = nullptr;  // operands laid out for the fused inference kernel, current with the parameters and maps
     __nv_bfloat16 *X = nullptr, *Xt = nullptr, *Hb[3] = {}, *Ht[3] = {}, *dY = nullptr, *dYt = nullptr;
     __nv_bfloat16 *dZ[3] = {}, *dZt[3] = {};
     float *Y = nullptr, *loss_part = nullptr;
@@ -105,7 +105,7 @@ void free_mlp(MlpDev& m)
     }
     if (m.err) cudaFree(m.err);
     if (m.d_norm) cudaFree(m.d_norm);
-    if (m.Wc) cudaFree(m.Wc);
+    if (m.stage) cudaFree(m.stage);
     m = MlpDev{};
 }
 
@@ -124,7 +124,7 @@ ptadd_status alloc_params(MlpDev& m)
         if (st == PTADD_OK) st = m_alloc(&m.Wt[l], nw);
     }
     if (st == PTADD_OK) st = m_alloc(&m.err, 1);
-    if (st == PTADD_OK) st = m_alloc(&m.Wc, (size_t)2 * (256 * 16 + 4 * 256 * 64));
+    if (st == PTADD_OK) st = m_alloc(&m.stage, mlp_infer_stage_bytes());
     if (st == PTADD_OK) st = m_alloc(&m.d_norm, 4 * NIN + 2 * NOUT + NIN * NIN + 1);
     return st;
 }
@@ -276,6 +276,15 @@ cudaError_t sync_bf16(MlpDev& m, cudaStream_t s)
     return cudaSuccess;
 }
 
+// the inference kernel's operands from the current parameters and maps (if there are maps)
+cudaError_t stage_inference(MlpDev& m, cudaStream_t s)
+{
+    if (!m.have_norm) return cudaSuccess;
+    const __nv_bfloat16* W[4] = {m.Wb[0], m.Wb[1], m.Wb[2], m.Wb[3]};
+    const float* b[4] = {m.b[0], m.b[1], m.b[2], m.b[3]};
+    return launch_mlp_infer_stage(m.d_norm, W, b, m.stage, s);
+}
+
 // packed (unpadded, oracle order) <-> padded device layout
 int64_t packed_count()
 {
@@ -380,6 +389,7 @@ ptadd_status ptadd_mlp_set_params(ptadd_ctx* ctx, const float* p, int64_t count)
         PTADD_CUDA(cudaStreamSynchronize(s));  // W, b are host temporaries
     }
     PTADD_CUDA(sync_bf16(m, s));
+    PTADD_CUDA(stage_inference(m, s));
     PTADD_CUDA(cudaMemsetAsync(m.err, 0, sizeof(int), s));
     PTADD_CUDA(cudaStreamSynchronize(s));
     m.step = 0;
@@ -549,6 +559,8 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
             }
         }
     }
+    if (e == cudaSuccess) e = stage_inference(m, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // predictions may run on another stream
     cudaFree(dx);
     cudaFree(dy);
     cudaFree(didx);
@@ -646,6 +658,14 @@ static ptadd_status upload_maps(MlpDev& m)
     return PTADD_OK;
 }
 
+// The inference operands after the maps have changed.
+static ptadd_status stage_maps(ptadd_ctx* ctx)
+{
+    PTADD_CUDA(stage_inference(*ctx->mlp, ctx->own_stream));
+    PTADD_CUDA(cudaStreamSynchronize(ctx->own_stream));
+    return PTADD_OK;
+}
+
 static double host_feature(const double* raw, int c)
 {
     // the inference kernel's arithmetic: the input rounded to FP32, then FP32 operations
@@ -737,6 +757,7 @@ ptadd_status ptadd_surrogate_fit(ptadd_ctx* ctx, int64_t n, const double* feat, 
     m.d2_thr = sorted[(size_t)std::min<int64_t>(n - 1, (int64_t)ceil(0.99 * n) - 1)];
     m.have_norm = true;
     ptadd_status st = upload_maps(m);
+    if (st == PTADD_OK) st = stage_maps(ctx);
     if (st != PTADD_OK) return st;
     // normalised training arrays
     std::vector<float> xn((size_t)n * NIN), yn((size_t)n * NOUT);
@@ -760,10 +781,8 @@ ptadd_status ptadd_surrogate_predict_dev(ptadd_ctx* ctx, int64_t n, const double
     }
     if (n < 1 || !feat_dev || !lp6_dev) return marg("need n >= 1 and arrays");
     // one fused persistent kernel: input map, trust region, the four layers, output map
-    const __nv_bfloat16* W[4] = {m.Wb[0], m.Wb[1], m.Wb[2], m.Wb[3]};
-    const float* b[4] = {m.b[0], m.b[1], m.b[2], m.b[3]};
-    PTADD_CUDA(launch_mlp_infer(feat_dev, n, m.d_norm, W, b, m.Wc, lp6_dev, in_region_dev, m.err, ctx->stream));
-    ctx->kernel_launches += 2;
+    PTADD_CUDA(launch_mlp_infer(feat_dev, n, m.stage, lp6_dev, in_region_dev, m.err, ctx->stream));
+    ctx->kernel_launches += 1;
     return PTADD_OK;
 }
 
@@ -877,7 +896,7 @@ ptadd_status ptadd_surrogate_set_state(ptadd_ctx* ctx, const void* buf, size_t b
     st = upload_maps(m);
     if (st != PTADD_OK) return st;
     m.have_norm = true;
-    return PTADD_OK;
+    return stage_maps(ctx);
 }
 
 }  // extern "C"

@@ -1,27 +1,32 @@
 // mlp_infer.cu -- fused surrogate inference: raw closure inputs -> sym(Lp),
 // the whole 30 -> 256 -> 256 -> 256 -> 6 network in one persistent kernel.
 //
-// One CTA per SM walks 128-row tiles of the input with 18 warps in three roles:
+// A pair of CTAs (a cluster of 2, one CTA per SM) walks pairs of 128-row tiles of the input.
+// The tensor cores of the two SMs work as one (cta_group::2: M = 256, the rows of both
+// tiles; each SM holds its own rows of A and D and half of the rows of every weight), so
+// that all weights stay in shared memory: 64 KB per hidden layer and CTA.  Each CTA has
+// 18 warps in three roles:
 //   * warps 0-15 ("epilogue warps"): per tile they map and standardise the
 //     raw features (sigma / 200 MPa, log10(rho + 1e10)) into the FP16
 //     layer-1 operand (and its rounding residual, for the trust region), test
-//     the box of the trust region, prefetch the features of the tile after
-//     next with cp.async, and run the epilogues: accumulator + bias -> GELU
-//     -> FP16 activations in shared memory, 64 columns at a time (warp w:
-//     TMEM lanes 32 (w mod 4) .. +31, i.e. its rows, and 16 columns), the
-//     Mahalanobis test, and the de-standardised FP64 outputs.  The map of
-//     tile t + 1 runs right after the layer-3 epilogue of tile t, so the
-//     tensor core starts layer 1 of the next tile while the epilogue warps
-//     wait for layer 4 of this one;
-//   * warp 16, lane 0 ("MMA issuer"): issues every tcgen05 MMA, each
-//     weight K-slice as soon as its activation chunk and its weights are in
-//     shared memory, and never waits for an MMA to finish;
-//   * warp 17, lane 0 ("weight producer"): streams layers 2 and 3 (a bias
-//     block, then the weights in K-chunks) through NST shared-memory stages
-//     in bulk copies (cp.async.bulk, completion counted on an mbarrier) from
-//     a copy pre-tiled into the canonical operand layout, refilling a stage
-//     once the MMAs that read it are done (tcgen05.commit on the stage's
-//     "empty" barrier).
+//     the box of the trust region, and run the epilogues: accumulator -> GELU ->
+//     FP16 activations in shared memory, 64 columns at a time (warp w: TMEM
+//     lanes 32 (w mod 4) .. +31, i.e. its rows, and 16 columns), the Mahalanobis
+//     test, and the de-standardised FP64 outputs.  The map of tile t + 1 runs after
+//     tile t's second hidden epilogue, beside layer 3; its features were loaded into
+//     registers, coalesced, a tile ahead;
+//   * warp 16, lane 0 of the first CTA ("MMA issuer"): issues every tcgen05 MMA of the
+//     pair, each K-slice as soon as its activation chunk is in both shared
+//     memories, and never waits for an MMA to finish;
+//   * warp 17, lane 0: copies the CTA's resident operands in, once (three bulk copies
+//     from a copy laid out in global memory when the parameters or maps change).
+// What bounds it: the chain through one tile.  A layer's MMAs take 2450 cycles (17 of
+// 256 x 256 x 16), its GELUs 2000 (the special-function unit: 128 x 256 tanh at 16 per
+// clock), and only the part after the first chunk of a layer overlaps; the activations of a
+// second pair of tiles would not fit beside the weights.  10^6 rows take 392 us.  One CTA
+// per tile with weights streamed from L2 through two 32 KB stages took 468 us: a stage came
+// back to the issuer some 1700 cycles after its commit, so a layer took 4300 cycles
+// at any copy rate.  Seven 16 KB stages (528 us) and two tiles in flight per SM (477 us) did not help.
 // Trust region: the distance d2 = |L^-1 z|^2 is a 128 x 32 x 32 product,
 // W = Z L^-T, that the tensor core computes next to layer 1 (into 32 spare
 // columns of the second accumulator) in split FP16: z = z_hi + z_lo with
@@ -36,16 +41,19 @@
 // chunk c + 1 of layer l's accumulator into activations, the tensor core
 // already runs layer l + 1 on chunk c (its K-slice 64 c .. 64 c + 63).  So
 // the GELU work of a layer runs beside the next layer's MMAs instead of
-// between them.  Per tile: xbar (layer-1 operand ready, 512 arrivals),
-// hbar[4] (activation chunk ready, 512 arrivals each; a chunk's barrier
-// cannot run two phases ahead of the MMA issuer, because its next phase needs
-// the next layer's accumulator, which needs this phase), accbar[4] (layer l's
-// MMAs complete, tcgen05.commit; one barrier per layer, because layer 1 of the
-// next tile may complete before the epilogue has waited for layer 4 of this
-// one), full[NST] / empty[NST] (the weight stages).  Every wait has an
-// iteration limit; a wait that gives up raises a CTA-wide abort flag, every
-// role leaves its loop, the MMA issuer waits (bounded) for its last MMAs and
-// the producer for its last bulk copies, and the kernel frees its tensor
+// between them.  Barriers of the pair, in the first CTA, one arrival per epilogue warp of
+// both: xbar (layer-1 operand ready), hbar[4] (activation chunk ready; it cannot run two
+// phases ahead of the MMA issuer, because its next phase needs the next layer's
+// accumulator, which needs this phase), wbar (W2 and W3 are there).  In each CTA:
+// accbar[4] (layer l's MMAs complete, tcgen05.commit to both CTAs; one barrier per layer,
+// because layer 1 of the next tile may complete before the epilogue has waited for layer 4
+// of this one), lxbar (this CTA's box tests).  The arrivals at the other CTA carry the
+// default (CTA) scope: what they hand over is this CTA's own shared memory, which the
+// writing lanes have already made visible to the tensor core's proxy; a release at
+// cluster scope waits for the thread's outputs on their way to global memory (557 us).
+// Every wait has an iteration limit; a wait that gives up raises the abort flags of both
+// CTAs, every role leaves its loop, the MMA issuer waits (bounded) for its last MMAs and
+// warp 17 for its copies, and after a barrier of the cluster the kernel frees its tensor
 // memory and sets the error flag.
 //
 // Operands are FP16 (the trained weights are BF16, which FP16 holds exactly
@@ -61,7 +69,8 @@
 // b_hi)): layer 1's rides in the two padding columns of its K = 32 operand
 // (inputs 1 there, W1's columns the bias), layers 2 and 3 start with one
 // K = 16 MMA of a constant operand (1 in K columns 0 and 1) against a bias
-// block streamed ahead of the layer's weights.  So an activation pair costs
+// block whose K columns 0, 1 (layer 2) or 2, 3 (layer 3) hold the two parts; the eight equal
+// rows of the constant operand are read at a stride of zero.  So an activation pair costs
 // one conversion, four f16x2 FMA-pipe operations and one special-function
 // operation.
 #include <cuda_bf16.h>
@@ -77,61 +86,102 @@ namespace {
 
 constexpr int EW = 16;             // epilogue warps
 constexpr int IT = 32 * EW;        // epilogue threads (rows per tile: 128)
-constexpr int IT_ALL = IT + 64;    // + the MMA warp and the weight-producer warp
+constexpr int IT_ALL = IT + 64;    // + the MMA warp and the warp that copies the resident operands in
 constexpr int NF = 30, NO = 6;
-constexpr int X_BYTES = 128 * 32 * 2;   // layer-1 A operand (FP16), SBO 512
-constexpr int W1_BYTES = 256 * 32 * 2;  // SBO 512
-constexpr int W4_BYTES = 16 * 256 * 2;  // SBO 4096
+constexpr int X_BYTES = 128 * 32 * 2;   // layer-1 A operand (FP16) or its residual, SBO 512
 constexpr int H_BYTES = 128 * 256 * 2;  // hidden activations, SBO 4096
-constexpr int KCH = 64;                 // K per streamed weight chunk
-constexpr int NST = 2;                  // weight stages in shared memory
-constexpr int CPL = 256 / KCH;          // chunks per layer (W2, W3)
-constexpr int WC_BYTES = 256 * KCH * 2; // one K-chunk of W2 or W3, 8-row groups 16 KCH bytes apart
-constexpr int BB_BYTES = 256 * 16 * 2;  // a layer's bias block: 256 rows x K 16 (b_hi, b_lo, 0...), SBO 256
-constexpr int IPL = CPL + 1;            // stream items per layer: the bias block, then the K-chunks
-constexpr int LAYER_BYTES = BB_BYTES + CPL * WC_BYTES;
-constexpr int ONES_BYTES = 128 * 16 * 2;  // A operand of the bias MMA: K columns 0, 1 = 1, the rest 0
-constexpr int NV_FLOATS = 4 * NF + 2 * NO + NF * NF + 1;
-constexpr int LI_BYTES = 32 * 32 * 2;   // L_hi or L_lo: 32 rows (i) x 32 K (j), SBO 512
-constexpr int MAHA_COL = 288;           // TMEM columns of W (second accumulator, clear of layer 4's 16)
-constexpr int OFF_X = 0;
+// the B operands: this CTA's half of the rows (output columns) of each
+constexpr int W1_BYTES = 128 * 32 * 2;   // SBO 512
+constexpr int WH_BYTES = 128 * 256 * 2;  // W2 / 2 or W3 / 2, SBO 4096
+constexpr int W4_BYTES = 8 * 256 * 2;    // SBO 4096
+constexpr int LI_BYTES = 16 * 32 * 2;    // L_hi or L_lo: rows (i) x 32 K (j), SBO 512
+constexpr int BB_BYTES = 128 * 8 * 2;    // biases of layers 2 and 3: K columns 0, 1 and 2, 3 (two FP16 parts each), SBO 128
+constexpr int ONES_BYTES = 8 * 16 * 2;   // A operand of a bias MMA: 8 equal rows, 1 in the layer's two K columns, else 0
+constexpr int MAHA_COL = 288;            // TMEM columns of W (second accumulator, clear of layer 4's 16)
+// maps as the kernel keeps them (floats): xm, 1/xs, ym, ys, box lo, box hi, d2 threshold, 1/s^2, layer 4's bias
+constexpr int NV_XM = 0, NV_XR = NV_XM + NF, NV_YM = NV_XR + NF, NV_YS = NV_YM + NO, NV_LO = NV_YS + NO,
+              NV_HI = NV_LO + NF, NV_THR = NV_HI + NF, NV_S2 = NV_THR + 1, NV_B4 = NV_S2 + 1, NV_COUNT = NV_B4 + 16;
+constexpr int NV_BYTES = (NV_COUNT * 4 + 127) / 128 * 128;
+// what stays in shared memory, laid out in global memory as it is there, one block per
+// CTA of a pair: two bulk copies (what layer 1 needs, then W2 and W3)
+constexpr int R_W1 = 0;
+constexpr int R_LH = R_W1 + W1_BYTES;
+constexpr int R_LL = R_LH + LI_BYTES;
+constexpr int R_W4 = R_LL + LI_BYTES;
+constexpr int R_BB = R_W4 + W4_BYTES;
+constexpr int R_ONES = R_BB + BB_BYTES;  // layer 2's, then layer 3's
+constexpr int R_NV = R_ONES + 2 * ONES_BYTES;
+constexpr int R_WH = R_NV + NV_BYTES;    // W2, then W3
+constexpr int RES_BYTES = R_WH + 2 * WH_BYTES;
+constexpr int OFF_X = 0;                  // z_hi
 constexpr int OFF_XLO = OFF_X + X_BYTES;  // z_lo, the same layout
-constexpr int OFF_W1 = OFF_XLO + X_BYTES;
-constexpr int OFF_LH = OFF_W1 + W1_BYTES;
-constexpr int OFF_LL = OFF_LH + LI_BYTES;
-constexpr int OFF_W4 = OFF_LL + LI_BYTES;
-constexpr int OFF_H = OFF_W4 + W4_BYTES;
-constexpr int OFF_WC = OFF_H + H_BYTES;
-constexpr int OFF_ONES = OFF_WC + NST * WC_BYTES;
-constexpr int OFF_NV = OFF_ONES + ONES_BYTES;
-constexpr int OFF_B = OFF_NV + ((NV_FLOATS * 4 + 15) / 16) * 16;   // layer 4's bias (16)
-constexpr int OFF_F = OFF_B + 16 * 4;                              // raw features of a tile [128][30]
-constexpr int OFF_BOX = OFF_F + 128 * NF * 8;                      // box test per quarter row [2][4][128]
-static_assert(OFF_F % 16 == 0, "bulk copies into the staging buffer need 16-byte alignment");
-constexpr int INFER_SMEM = OFF_BOX + 2 * 4 * 128;
+constexpr int OFF_H = OFF_XLO + X_BYTES;
+constexpr int OFF_RES = OFF_H + H_BYTES;
+constexpr int OFF_BOX = OFF_RES + RES_BYTES;  // box test per row [2 tiles][128]
+constexpr int INFER_SMEM = OFF_BOX + 2 * 128;
+static_assert(R_WH % 128 == 0 && RES_BYTES % 16 == 0, "bulk copies need 16-byte alignment");
+static_assert(INFER_SMEM + 512 <= 232448, "shared memory of one CTA, the barriers included");
+// raw features of a tile: 128 rows x 15 pairs, pair e = tid + IT i in thread tid's slot i
+constexpr int FPT = (128 * NF / 2 + IT - 1) / IT;
 
 __device__ __forceinline__ uint32_t canon(int r, int k, int sbo)
 {
     return (uint32_t)((r >> 3) * sbo + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
-// Item k (0 <= k < 2 IPL) of the per-tile weight stream: the bias block of
-// layer 2, W2's K-chunks, then the same for layer 3; its offset in the staged
-// copy and its size.
-__device__ __forceinline__ uint32_t item_offset(int k)
+// ------------------------------------------------ PTX of a CTA pair
+__device__ __forceinline__ uint32_t cluster_rank()
 {
-    const int l = k / IPL, i = k % IPL;
-    return (uint32_t)(l * LAYER_BYTES + (i ? BB_BYTES + (i - 1) * WC_BYTES : 0));
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
 }
-__device__ __forceinline__ uint32_t item_bytes(int k) { return (k % IPL) ? (uint32_t)WC_BYTES : (uint32_t)BB_BYTES; }
-
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src)
+// all threads of both CTAs
+__device__ __forceinline__ void cluster_sync()
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(__cvta_generic_to_global(src))
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a shared-memory address of this CTA, in the CTA of rank r of the cluster
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t r)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(r));
+    return a;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc2(uint32_t dst_smem, uint32_t ncols)
+{
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
                  : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
+}
+// One MMA of the pair, M = 256: the operands lie at the same shared-memory addresses in
+// both CTAs, A's rows 0..127 and B's first N / 2 rows in the first CTA, the others in the
+// second; each CTA's tensor memory gets its 128 rows of D, all N columns.
+__device__ __forceinline__ void tc_mma2_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate)
+{
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// completion of the MMAs issued so far, on the barrier at this address in both CTAs
+__device__ __forceinline__ void tc_commit2(uint32_t mbar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(mbar),
+        "h"((uint16_t)3)
+        : "memory");
+}
 
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar)
 {
@@ -148,23 +198,16 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                  "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(mbar)
                  : "memory");
 }
-// Raw features of one tile (rows r0 .. r0 + valid - 1, 240 valid bytes a row,
-// contiguous) into the staging buffer, the same layout: one bulk copy with its
-// completion on mbar when the input is 16-byte aligned (issued by one thread),
-// else 8-byte asynchronous copies by every epilogue thread.
-__device__ __forceinline__ void issue_features(bool bulk, uint32_t dst, const double* feat, int64_t r0, int valid,
-                                               uint32_t mbar)
+// Two consecutive raw features, loaded ahead of use: asm volatile, so that the
+// compiler leaves the load where it is.  One 16-byte load where the array is 16-byte
+// aligned (every pair then is).
+__device__ __forceinline__ void load_pair(const double* p, bool wide, double f[2])
 {
-    if (bulk) {
-        if (threadIdx.x == 0) {
-            fence_async_smem();  // the buffer's last reads were generic
-            mbar_expect_tx(mbar, (uint32_t)valid * 240u);
-            bulk_g2s(dst, feat + r0 * 30, (uint32_t)valid * 240u, mbar);
-        }
-    } else {
-        for (int e = threadIdx.x; e < valid * 30; e += IT) cp_async8(dst + (uint32_t)e * 8, feat + r0 * 30 + e);
-        cp_async_commit();
-    }
+    asm volatile(
+        "{\n .reg .pred w;\n setp.ne.b32 w, %3, 0;\n @w ld.global.nc.v2.f64 {%0, %1}, [%2];\n"
+        " @!w ld.global.nc.f64 %0, [%2];\n @!w ld.global.nc.f64 %1, [%2 + 8];\n}\n"
+        : "=&d"(f[0]), "=&d"(f[1])
+        : "l"(p), "r"((int)wide));
 }
 
 // 2 GELU(z) of two values in f16x2 (see the header for the approximation)
@@ -180,7 +223,7 @@ __device__ __forceinline__ uint32_t gelu2x2_f16(float2 z)
 }
 
 // 16 consecutive FP32 columns of this thread's TMEM lane, without waiting:
-// the registers hold the values only after the next tmem_wait_ld().
+// the registers hold the values only after tmem_wait_ld16 on them.
 __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t r[16])
 {
     asm volatile(
@@ -191,18 +234,23 @@ __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t r[16])
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for every load issued so far; the loaded registers pass through the
+// statement, so that no use of them is scheduled before it.
+__device__ __forceinline__ void tmem_wait_ld16(uint32_t r[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
 
-// Accumulator values (16 columns from c0) [+ bias] -> 2 GELU as 8 f16x2 words.
-template <bool BIAS>
-__device__ __forceinline__ void gelu16(const uint32_t r[16], int c0, const float* __restrict__ bias, uint32_t w[8])
+// Accumulator values (16 columns; the bias is in them) -> 2 GELU as 8 f16x2 words.
+__device__ __forceinline__ void gelu16(const uint32_t r[16], uint32_t w[8])
 {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float2 z = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-        if (BIAS) z = __fadd2_rn(z, *reinterpret_cast<const float2*>(bias + c0 + 2 * i));
-        w[i] = gelu2x2_f16(z);
-    }
+    for (int i = 0; i < 8; ++i)
+        w[i] = gelu2x2_f16(make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])));
 }
 // ... into H (row, columns c0 .. c0 + 15)
 __device__ __forceinline__ void store16(const uint32_t w[8], int row, int c0, uint8_t* sH)
@@ -233,32 +281,37 @@ __device__ __forceinline__ uint4 bf16x8_to_f16x8(uint4 v, float scale)
     return make_uint4(out[0], out[1], out[2], out[3]);
 }
 
-// IEEE-754 round-to-nearest-even FP64 -> FP32 and exact FP32 -> FP64 on the
-// integer pipe, for values in the normal FP32 range (others take the
-// hardware conversion, which on this GPU runs on the 1/64-rate FP64 pipe).
+// FP64 -> FP32 (round to nearest even; results below FP32's normal range become
+// zeros, which no caller can tell from them) and FP32 -> FP64 (exact) on the integer
+// pipe: the conversion instructions run on the FP64 pipe, 2 lanes per clock on this GPU,
+// and are issued even where a select discards their result.
 __device__ __forceinline__ float d2f_rn(double x)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
-    if (e < 1023u - 126u || e > 1023u + 127u) return (float)x;  // zero, FP32-subnormal range, overflow, inf, nan
-    const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-    unsigned f = ((unsigned)(b >> 32) & 0x80000000u) | ((e - 896u) << 23) | (unsigned)(m >> 29);
-    const unsigned rest = (unsigned)m & 0x1FFFFFFFu;  // the 29 dropped bits
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu, sign = hi & 0x80000000u;
+    uint32_t f = ((e - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1FFFFFFFu;  // the 29 dropped bits
     f += (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) ? 1u : 0u;  // carries into the exponent
-    return __uint_as_float(f);
+    if (e < 897u) f = 0u;
+    if (e > 1150u) f = (e == 0x7FFu && ((hi & 0xFFFFFu) | lo)) ? 0x7FFFFFFFu : 0x7F800000u;
+    return __uint_as_float(sign | f);
 }
 __device__ __forceinline__ double f2d(float x)
 {
-    const unsigned u = __float_as_uint(x);
-    const unsigned e = (u >> 23) & 0xFFu;
-    if (e == 0u || e == 0xFFu) return (double)x;  // zero, subnormal, inf, nan
-    const unsigned long long b = ((unsigned long long)(u & 0x80000000u) << 32) |
-                                 ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29);
-    return __longlong_as_double((long long)b);
+    const uint32_t u = __float_as_uint(x), sign = u & 0x80000000u;
+    uint32_t m = u & 0x7FFFFFu, e = (u >> 23) & 0xFFu;
+    if (e == 0u && m) {  // subnormal
+        const int up = __clz((int)m) - 8;
+        m = (m << up) & 0x7FFFFFu;
+        e = (uint32_t)(897 - up);
+    } else {
+        e = e == 0u ? 0u : e == 0xFFu ? 0x7FFu : e + 896u;
+    }
+    return __hiloint2double((int)(sign | (e << 20) | (m >> 3)), (int)(m << 29));
 }
 
-// Bounded wait on an mbarrier phase that also gives up when another role has
-// raised the CTA's abort flag: false if the phase did not complete.
+// Bounded wait on an mbarrier phase that also gives up when another role of the pair
+// has raised the abort flag: false if the phase did not complete.
 __device__ __forceinline__ bool wait_or_abort(uint32_t mbar, uint32_t parity, volatile int* abort_flag)
 {
     const long long t0 = clock64();
@@ -269,237 +322,192 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t mbar, uint32_t parity, vo
     return true;
 }
 
-// epilogue-warp barrier (named barrier 1; the MMA and producer warps do not take part)
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(IT) : "memory"); }
-
-// sigma / 200 MPa, or log10(rho + 1e10), from the FP64 input rounded to FP32
-// (all FP32 arithmetic: the FP64 pipe is slow on this part)
-__device__ __forceinline__ float raw_feature(double v, bool stress)
+// Features k (even) and k + 1 from the FP64 input rounded to FP32: sigma / 200 MPa (k < 6)
+// or log10(rho + 1e10), less the mean, times the reciprocal deviation; all FP32 arithmetic
+// (the FP64 pipe is slow on this part).  Every rounding is written out, because a
+// last-bit difference here can flip the operand's FP16 rounding: the product by log10(2) is
+// rounded before the subtraction, except in columns 6 and 7 of each 8, where the two
+// are one fused operation.
+__device__ __forceinline__ float standardise(double v, int k, float mean, float rdev)
 {
+    constexpr float LOG10_2 = 0.30102999566398120f;
     const float x = d2f_rn(v);
-    return stress ? x * (float)(1.0 / 200e6) : __log10f(x + 1e10f);
+    float c;
+    if (k < 6) {
+        c = __fsub_rn(__fmul_rn(x, (float)(1.0 / 200e6)), mean);
+    } else {
+        const float l = __log2f(x + 1e10f);
+        c = (k & 7) == 6 ? fmaf(l, LOG10_2, -mean) : __fsub_rn(__fmul_rn(l, LOG10_2), mean);
+    }
+    return __fmul_rn(c, rdev);
 }
 
 struct InferArgs {
     const double* feat;  // [n x 30]
     int64_t n;
-    int feat_bulk;       // feat is 16-byte aligned: one bulk copy per tile
-    const float* nv;     // xm, xs, ym, ys, box lo, box hi, inverse Cholesky factor, d2 threshold
-    const __nv_bfloat16* W[4];
-    const __half* Wc;    // per layer 2, 3: bias block, then W / 2 (FP16) in CPL pre-tiled K-chunks of 256 x KCH
-    const float* b[4];
+    int feat_wide;       // feat is 16-byte aligned
+    const uint8_t* res;  // [2][RES_BYTES]: what stays in shared memory, per CTA of a pair
     double* lp6;         // [n x 6]
     uint8_t* in_region;  // [n] or null
     int* err;
 };
 
-__global__ void __launch_bounds__(IT_ALL, 1) mlp_infer_kernel(InferArgs g)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(IT_ALL, 1) mlp_infer_kernel(InferArgs g)
 {
     // every region below starts at a multiple of 16 bytes, all the no-swizzle
     // operand layouts need; pointers derived from the array itself keep the
     // compiler's shared-memory address space (plain shared loads and stores)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t xbar, hbar[4], accbar[4], full[NST], empty[NST], drainbar, fbar;
+    __shared__ __align__(8) uint64_t xbar, lxbar, hbar[4], accbar[4], wbar, drainbar, resbar, whbar;
     __shared__ uint32_t tmem_base;
-    __shared__ unsigned li_max;  // bits of max |L^-1| (non-negative floats order as integers)
     __shared__ volatile int abort_flag;
     uint8_t* base = smem_raw;
     uint8_t* sX = base + OFF_X;
-    uint8_t* sW1 = base + OFF_W1;
-    uint8_t* sW4 = base + OFF_W4;
-    uint8_t* sH = base + OFF_H;
     uint8_t* sXlo = base + OFF_XLO;
-    float* snv = reinterpret_cast<float*>(base + OFF_NV);
+    uint8_t* sH = base + OFF_H;
     uint8_t* sBox = base + OFF_BOX;
-    const uint32_t uX = smem_u32(sX), uW1 = smem_u32(sW1), uW4 = smem_u32(sW4), uH = smem_u32(sH);
-    const uint32_t uXlo = smem_u32(sXlo), uLH = smem_u32(base + OFF_LH), uLL = smem_u32(base + OFF_LL);
-    const uint32_t uWC = smem_u32(base + OFF_WC), uOnes = smem_u32(base + OFF_ONES);
+    const float* snv = reinterpret_cast<const float*>(base + OFF_RES + R_NV);
+    const uint32_t uX = smem_u32(sX), uXlo = smem_u32(sXlo), uH = smem_u32(sH);
+    const uint32_t uR = smem_u32(base + OFF_RES);
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int64_t n_tiles = (g.n + 127) / 128;
-    if ((int64_t)blockIdx.x >= n_tiles) return;  // whole CTA, before any allocation
-    const int64_t my_tiles = (n_tiles - 1 - blockIdx.x) / gridDim.x + 1;
-    const int64_t Q = 2 * IPL * my_tiles;  // items of the W2/W3 stream
-    const uint32_t ux = smem_u32(&xbar), uacc0 = smem_u32(&accbar[0]);
-    const uint32_t uh0 = smem_u32(&hbar[0]), ufull0 = smem_u32(&full[0]), uempty0 = smem_u32(&empty[0]);
+    const uint32_t rank = cluster_rank();
+    const int64_t n_pairs = (g.n + 255) / 256, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    // (no CTA leaves early: the grid has no more pairs than the input)
+    const int64_t my_tiles = (n_pairs - 1 - pair) / pairs + 1;
     // each mbarrier is 8 bytes: barrier k of an array at u0 + 8 k
+    const uint32_t ux = smem_u32(&xbar), ulx = smem_u32(&lxbar), uacc0 = smem_u32(accbar), uh0 = smem_u32(hbar);
+    const uint32_t ures = smem_u32(&resbar), uwh = smem_u32(&whbar), uw = smem_u32(&wbar), udrain = smem_u32(&drainbar);
+    const uint32_t uabort = smem_u32(const_cast<int*>(&abort_flag));
 
-    if (warp == 0) {
-        tmem_alloc(smem_u32(&tmem_base), 512);
-        tmem_relinquish();
-    }
+    if (warp == 0) tmem_alloc2(smem_u32(&tmem_base), 512);
     if (tid == 0) {
         abort_flag = 0;
-        mbar_init(ux, IT);
-        for (int c = 0; c < 4; ++c) mbar_init(uh0 + 8 * c, IT);
+        mbar_init(ux, 2 * EW);
+        mbar_init(ulx, EW);
+        for (int c = 0; c < 4; ++c) mbar_init(uh0 + 8 * c, 2 * EW);
         for (int l = 0; l < 4; ++l) mbar_init(uacc0 + 8 * l, 1);
-        li_max = 0u;
-        mbar_init(smem_u32(&drainbar), 1);
-        mbar_init(smem_u32(&fbar), 1);
-        for (int k = 0; k < NST; ++k) {
-            mbar_init(ufull0 + 8 * k, 1);
-            mbar_init(uempty0 + 8 * k, 1);
-        }
+        mbar_init(uw, 2);
+        mbar_init(udrain, 1);
+        mbar_init(ures, 1);
+        mbar_init(uwh, 1);
     }
-    // resident operands and maps
-    for (int e = tid; e < 256 * 4; e += IT_ALL) {  // W1: 256 rows x 32 K (4 x 8-element groups)
-        const int r = e >> 2, kc = e & 3;
-        uint4 v = bf16x8_to_f16x8(*reinterpret_cast<const uint4*>(g.W[0] + (int64_t)r * 32 + kc * 8), 1.0f);
-        if (kc == 3) {  // K columns 30, 31: the bias in two FP16 parts
-            const float bb = g.b[0][r];
-            const __half hi = __float2half_rn(bb), lo = __float2half_rn(bb - __half2float(hi));
-            const __half2 h2 = __halves2half2(hi, lo);
-            v.w = *reinterpret_cast<const uint32_t*>(&h2);
-        }
-        *reinterpret_cast<uint4*>(sW1 + (r >> 3) * 512 + kc * 128 + (r & 7) * 16) = v;
+    if (tid < 256) sBox[tid] = 1;
+    // the bias columns of the layer-1 operand (inputs 1 there, residual 0) stay as they are
+    if (tid < 128) {
+        *reinterpret_cast<uint32_t*>(sX + canon(tid, NF, 512)) = 0x3c003c00u;
+        *reinterpret_cast<uint32_t*>(sXlo + canon(tid, NF, 512)) = 0u;
     }
-    for (int e = tid; e < 16 * 32; e += IT_ALL) {  // W4 / 2: 16 rows x 256 K
-        const int r = e >> 5, kc = e & 31;
-        *reinterpret_cast<uint4*>(sW4 + (r >> 3) * 4096 + kc * 128 + (r & 7) * 16) =
-            bf16x8_to_f16x8(*reinterpret_cast<const uint4*>(g.W[3] + (int64_t)r * 256 + kc * 8), 0.5f);
-    }
-    for (int e = tid; e < NV_FLOATS; e += IT_ALL)  // (the deviations xs are kept as reciprocals)
-        snv[e] = (e >= NF && e < 2 * NF) ? 1.0f / g.nv[e] : g.nv[e];
-    const float* gLi = g.nv + 4 * NF + 2 * NO;  // L^-1, NF x NF row-major, lower triangle
-    __syncthreads();  // li_max is cleared
-    for (int e = tid; e < NF * NF; e += IT_ALL) atomicMax(&li_max, __float_as_uint(fabsf(gLi[e])));
-    __syncthreads();
-    int li_exp = 0;
-    frexpf(__uint_as_float(li_max), &li_exp);
-    const int li_k = li_max ? max(-60, min(60, 14 - li_exp)) : 0;  // s = 2^li_k
-    const float li_s = ldexpf(1.0f, li_k), inv_s2 = ldexpf(1.0f, -2 * li_k);
-    for (int e = tid; e < 32 * 32; e += IT_ALL) {  // s L^-1 = L_hi + L_lo, rows i and K columns j, zero-padded
-        const int i = e >> 5, j = e & 31;
-        const float v = (i < NF && j <= i) ? gLi[i * NF + j] * li_s : 0.0f;
-        const __half hi = __float2half_rn(v);
-        *reinterpret_cast<__half*>(base + OFF_LH + canon(i, j, 512)) = hi;
-        *reinterpret_cast<__half*>(base + OFF_LL + canon(i, j, 512)) = __float2half_rn(v - __half2float(hi));
-    }
-    float* sB = reinterpret_cast<float*>(base + OFF_B);
-    for (int e = tid; e < 16; e += IT_ALL) sB[e] = g.b[3][e];
-    for (int e = tid; e < 128 * 16; e += IT_ALL) {  // the ones operand of the bias MMAs
-        const int r = e >> 4, k = e & 15;
-        *reinterpret_cast<__half*>(base + OFF_ONES + canon(r, k, 256)) = __float2half_rn(k < 2 ? 1.0f : 0.0f);
-    }
-    const uint32_t uF = smem_u32(base + OFF_F), ufbar = smem_u32(&fbar);
-    const double* sF = reinterpret_cast<const double*>(base + OFF_F);
-    const bool fbulk = g.feat_bulk != 0;
-    fence_async_smem();  // the resident operands were written by the generic proxy
+    fence_async_smem();
     tc_fence_before();
-    __syncthreads();  // (the barrier inits are visible)
-    if (tid < IT)
-        issue_features(fbulk, uF, g.feat, (int64_t)blockIdx.x * 128,
-                       (int)min((int64_t)128, g.n - (int64_t)blockIdx.x * 128), ufbar);
+    __syncthreads();
+    cluster_sync();  // the barrier inits and both halves of the tensor memory are there
     tc_fence_after();
     const uint32_t tmem = tmem_base;
     bool ok = true;
+    auto raise_abort = [&]() {  // in both CTAs
+        for (uint32_t r = 0; r < 2; ++r)
+            asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(in_cta(uabort, r)), "r"(1) : "memory");
+    };
 
     if (warp == EW + 1) {
-        // ------------------------------------------------ weight producer
+        // ------------------------------------------------ the resident operands
         if ((tid & 31) == 0) {
-            int64_t issued = 0;
-            for (; issued < Q; ++issued) {
-                const uint32_t st = (uint32_t)(issued % NST);
-                if (issued >= NST &&  // the stage's previous chunk must have been read by its MMAs
-                    !wait_or_abort(uempty0 + 8 * st, (uint32_t)(((issued - NST) / NST) & 1), &abort_flag)) {
-                    abort_flag = 1;
-                    break;
-                }
-                const int k = (int)(issued % (2 * IPL));
-                mbar_expect_tx(ufull0 + 8 * st, item_bytes(k));
-                bulk_g2s(uWC + st * WC_BYTES, reinterpret_cast<const uint8_t*>(g.Wc) + item_offset(k), item_bytes(k),
-                         ufull0 + 8 * st);
+            const uint8_t* res = g.res + (size_t)rank * RES_BYTES;
+            mbar_expect_tx(ures, R_WH);
+            bulk_g2s(uR, res, R_WH, ures);
+            mbar_expect_tx(uwh, 2 * WH_BYTES);
+            bulk_g2s(uR + R_WH, res + R_WH, WH_BYTES, uwh);
+            bulk_g2s(uR + R_WH + WH_BYTES, res + R_WH + WH_BYTES, WH_BYTES, uwh);
+            // (no copy may still be landing when the CTA leaves: both are waited for, bounded)
+            if (!mbar_wait_bounded(ures, 0u, MBAR_WAIT_LIMIT) || !mbar_wait_bounded(uwh, 0u, MBAR_WAIT_LIMIT)) {
+                raise_abort();
+                atomicExch(g.err, 1);
             }
-            // no copy may still be landing when the CTA leaves: wait (bounded)
-            // for the last copy into each stage
-            for (int64_t j = issued > NST ? issued - NST : 0; j < issued; ++j)
-                mbar_wait_bounded(ufull0 + 8 * (uint32_t)(j % NST), (uint32_t)((j / NST) & 1), MBAR_WAIT_LIMIT);
-            if (abort_flag) atomicExch(g.err, 1);
+            mbar_arrive_cluster(in_cta(uw, 0));
         }
     } else if (warp == EW) {
-        // ------------------------------------------------ MMA issuer
-        if ((tid & 31) == 0) {
-            const uint32_t id_h = idesc_f16_f32(128, 256), id_o = idesc_f16_f32(128, 16);
-            const uint32_t id_m = idesc_f16_f32(128, 32);
+        // ------------------------------------------------ MMA issuer of the pair
+        if (rank == 0 && (tid & 31) == 0) {
+            const uint32_t id_h = idesc_f16_f32(256, 256), id_o = idesc_f16_f32(256, 16);
+            const uint32_t id_m = idesc_f16_f32(256, 32);
             const uint32_t accA = tmem, accB = tmem + 256;
-            int64_t q = 0;              // weight chunks consumed
             uint32_t xph = 0, hph = 0;  // hph bit kc: parity of hbar[kc]
             bool mma_out = false;       // MMAs issued (for the abort path)
-            for (int64_t it = 0; it < my_tiles && ok; ++it) {
-                // layer 1: X [128 x 32] W1^T -> A
-                ok = wait_or_abort(ux, xph, &abort_flag);
-                xph ^= 1u;
-                if (!ok) break;
+            auto chunk = [&](int kc) {  // activation chunk kc of the current layer is ready
+                const bool w = wait_or_abort(uh0 + 8 * kc, (hph >> kc) & 1u, &abort_flag);
+                hph ^= 1u << kc;
                 tc_fence_after();
-                for (int s = 0; s < 2; ++s)
-                    tc_mma_f16(accA, smem_desc(uX + s * 256, 128, 512), smem_desc(uW1 + s * 256, 128, 512), id_h,
-                               s ? 1u : 0u);
-                // trust region: W = z_hi L_hi + z_hi L_lo + z_lo L_hi (kind::f16 with FP16 operands)
+                return w;
+            };
+            // trust region: W = z_hi L_hi + z_hi L_lo + z_lo L_hi (kind::f16 with FP16 operands),
+            // as soon as the tile's input map is ready
+            auto trust = [&]() {
+                const bool w = wait_or_abort(ux, xph, &abort_flag);
+                xph ^= 1u;
+                if (!w) return false;
+                tc_fence_after();
                 for (int s = 0; s < 2; ++s) {
                     const uint64_t zh = smem_desc(uX + s * 256, 128, 512), zl = smem_desc(uXlo + s * 256, 128, 512);
-                    const uint64_t lh = smem_desc(uLH + s * 256, 128, 512), ll = smem_desc(uLL + s * 256, 128, 512);
-                    tc_mma_f16(tmem + MAHA_COL, zh, lh, id_m, s ? 1u : 0u);
-                    tc_mma_f16(tmem + MAHA_COL, zh, ll, id_m, 1u);
-                    tc_mma_f16(tmem + MAHA_COL, zl, lh, id_m, 1u);
+                    const uint64_t lh = smem_desc(uR + R_LH + s * 256, 128, 512);
+                    const uint64_t ll = smem_desc(uR + R_LL + s * 256, 128, 512);
+                    tc_mma2_f16(tmem + MAHA_COL, zh, lh, id_m, s ? 1u : 0u);
+                    tc_mma2_f16(tmem + MAHA_COL, zh, ll, id_m, 1u);
+                    tc_mma2_f16(tmem + MAHA_COL, zl, lh, id_m, 1u);
                 }
-                tc_commit(uacc0);
                 mma_out = true;
+                return true;
+            };
+            // layer 1: X [128 x 32] W1^T -> A
+            auto layer1 = [&]() {
+                for (int s = 0; s < 2; ++s)
+                    tc_mma2_f16(accA, smem_desc(uX + s * 256, 128, 512), smem_desc(uR + R_W1 + s * 256, 128, 512), id_h,
+                                s ? 1u : 0u);
+                tc_commit2(uacc0);
+            };
+            if ((ok = trust())) {
+                layer1();
+                ok = wait_or_abort(uw, 0u, &abort_flag);
+                tc_fence_after();
+            }
+            for (int64_t it = 0; it < my_tiles && ok; ++it) {
                 // layers 2, 3: H [128 x 256] W^T, K-slice by K-slice as soon as the
-                // epilogue has written its activation chunk and the weights have landed
+                // epilogues of both CTAs have written their activation chunk
                 for (int l = 1; l <= 2 && ok; ++l) {
-                    const uint32_t acc = (l == 1) ? accB : accA;
-                    for (int jj = 0; jj < CPL; ++jj, ++q) {
-                        const int kc = jj * KCH / 64;  // the activation chunk this K-slice lies in
-                        if ((jj * KCH) % 64 == 0) {
-                            ok = wait_or_abort(uh0 + 8 * kc, (hph >> kc) & 1u, &abort_flag);
-                            hph ^= 1u << kc;
-                            if (!ok) break;
-                        }
-                        if (jj == 0) {
-                            // the bias first: ones [128 x 16] (b_hi, b_lo, 0..)^T sets the
-                            // accumulator (only now: the previous layer's epilogue has read it)
-                            const uint32_t st = (uint32_t)(q % NST);
-                            ok = wait_or_abort(ufull0 + 8 * st, (uint32_t)((q / NST) & 1), &abort_flag);
-                            if (!ok) break;
-                            tc_fence_after();
-                            tc_mma_f16(acc, smem_desc(uOnes, 128, 256), smem_desc(uWC + st * WC_BYTES, 128, 256), id_h,
-                                       0u);
-                            tc_commit(uempty0 + 8 * st);
-                            ++q;
-                        }
-                        const uint32_t st = (uint32_t)(q % NST);
-                        ok = wait_or_abort(ufull0 + 8 * st, (uint32_t)((q / NST) & 1), &abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t ub = uWC + st * WC_BYTES;
-                        for (int s = 0; s < KCH / 16; ++s)
-                            tc_mma_f16(acc, smem_desc(uH + (jj * (KCH / 16) + s) * 256, 128, 4096),
-                                       smem_desc(ub + s * 256, 128, 16 * KCH), id_h, 1u);
-                        tc_commit(uempty0 + 8 * st);  // the stage is free once these MMAs are done
+                    const uint32_t acc = (l == 1) ? accB : accA, uW = uR + R_WH + (l - 1) * WH_BYTES;
+                    for (int kc = 0; kc < 4; ++kc) {
+                        if (!(ok = chunk(kc))) break;
+                        // the bias first: ones [128 x 16] (b_hi, b_lo, 0..)^T sets the accumulator
+                        // (only now: the previous layer's epilogue has read it)
+                        if (kc == 0)
+                            tc_mma2_f16(acc, smem_desc(uR + R_ONES + (l - 1) * ONES_BYTES, 128, 0),
+                                        smem_desc(uR + R_BB, 0, 128), id_h, 0u);
+                        for (int k = 4 * kc; k < 4 * kc + 4; ++k)
+                            tc_mma2_f16(acc, smem_desc(uH + k * 256, 128, 4096), smem_desc(uW + k * 256, 128, 4096),
+                                        id_h, 1u);
                     }
-                    if (!ok) break;
-                    tc_commit(uacc0 + 8 * l);
+                    if (ok) tc_commit2(uacc0 + 8 * l);
                 }
-                if (!ok) break;
+                const bool more = it + 1 < my_tiles;
+                // (the second accumulator is free but for layer 4's columns)
+                if (ok && more) ok = trust();
                 // layer 4: H [128 x 256] W4^T -> B (16 columns, 6 used)
                 for (int kc = 0; kc < 4 && ok; ++kc) {
-                    ok = wait_or_abort(uh0 + 8 * kc, (hph >> kc) & 1u, &abort_flag);
-                    hph ^= 1u << kc;
-                    if (!ok) break;
-                    tc_fence_after();
+                    if (!(ok = chunk(kc))) break;
                     for (int s = 4 * kc; s < 4 * kc + 4; ++s)
-                        tc_mma_f16(accB, smem_desc(uH + s * 256, 128, 4096), smem_desc(uW4 + s * 256, 128, 4096),
-                                   id_o, s ? 1u : 0u);
+                        tc_mma2_f16(accB, smem_desc(uH + s * 256, 128, 4096), smem_desc(uR + R_W4 + s * 256, 128, 4096),
+                                    id_o, s ? 1u : 0u);
                 }
                 if (!ok) break;
-                tc_commit(uacc0 + 24);
+                tc_commit2(uacc0 + 24);
+                if (more) layer1();  // (every layer-3 chunk, accumulator A, has been read)
             }
             if (!ok) {
-                abort_flag = 1;
-                // the tensor core may still be busy: wait (bounded) for a commit
+                raise_abort();
+                // the tensor cores may still be busy: wait (bounded) for a commit
                 // of everything issued before the tensor memory is freed
                 if (mma_out) {
-                    tc_commit(smem_u32(&drainbar));
-                    mbar_wait_bounded(smem_u32(&drainbar), 0u, MBAR_WAIT_LIMIT);
+                    tc_commit2(udrain);
+                    mbar_wait_bounded(udrain, 0u, MBAR_WAIT_LIMIT);
                 }
                 atomicExch(g.err, 1);
             }
@@ -507,189 +515,246 @@ __global__ void __launch_bounds__(IT_ALL, 1) mlp_infer_kernel(InferArgs g)
     } else {
         // ------------------------------------------------ epilogue warps
         const int lg = warp & 3, cs = warp >> 2;  // TMEM lane group (rows) and 16-column slice of a chunk
-        const int erow = 32 * lg + (tid & 31);
+        const int lane = tid & 31, erow = 32 * lg + lane;
         const uint32_t tmem_row = tmem + ((uint32_t)(32 * lg) << 16);
-        // input-map roles: row and quarter (8 of the 32 operand columns)
-        const int mrow = tid & 127, part = tid >> 7;
-        const float* xm = snv;
-        const float* xr = snv + NF;  // 1 / xs
-        const float* ym = snv + 2 * NF;
-        const float* ys = ym + NO;
-        const float* lo = snv + 2 * NF + 2 * NO;
-        const float* hi = lo + NF;
-        const float d2_thr = snv[4 * NF + 2 * NO + NF * NF];
-        uint32_t accph = 0;  // bit l: parity of accbar[l]
+        const uint32_t ux_lead = in_cta(ux, 0), uh_lead = in_cta(uh0, 0);
+        uint32_t accph = 0, xph = 0;  // bit l: parity of accbar[l]; of lxbar
         auto wait_acc = [&](int l) {
             const bool w = wait_or_abort(uacc0 + 8 * l, (accph >> l) & 1u, &abort_flag);
             accph ^= 1u << l;
-            if (!w) abort_flag = 1;
+            if (!w) raise_abort();
             tc_fence_after();
             return w;
         };
-        // hand a finished operand chunk to the MMA issuer
-        auto publish = [&](uint32_t mbar) {
+        // hand this warp's finished share of an operand chunk to the MMA issuer
+        auto publish = [&](uint32_t mbar_lead) {
             fence_async_smem();
             tc_fence_before();
-            mbar_arrive(mbar);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(mbar_lead);
         };
-        // the input map of tile it: raw features (prefetched into the staging
-        // buffer) -> the FP16 layer-1 operand z_hi, its residual z_lo and this
-        // quarter row's box test; then the prefetch of tile it + 1
-        int fpend = 0;  // tile whose feature copy is in flight, or -1
+        auto first_row = [&](int64_t it) { return ((pair + it * pairs) * 2 + rank) * 128; };
+        // (the second tile of the last pair may have no rows)
+        auto rows_of = [&](int64_t it) { return (int)max((int64_t)0, min((int64_t)128, g.n - first_row(it))); };
+        double f[FPT][2];  // raw features of the next tile
+        const bool wide = g.feat_wide != 0;
+        auto fetch = [&](int64_t it) {
+            // unconditional loads (of the first pair where there is nothing to load): a load in
+            // a branch is waited for where the branch ends, here a tile too early
+            const int np = it < my_tiles ? (NF / 2) * rows_of(it) : 0;
+            const double* p = g.feat + first_row(it) * NF;
+#pragma unroll
+            for (int i = 0; i < FPT; ++i)
+                load_pair(tid + IT * i < np ? p + 2 * (tid + IT * i) : g.feat, wide, f[i]);
+        };
+        // the input map of tile it (its features are in f): the FP16 layer-1 operand z_hi,
+        // its residual z_lo and the box test; then the loads for the tile after it
         auto map_tile = [&](int64_t it) {
-            const int64_t r0 = ((int64_t)blockIdx.x + it * gridDim.x) * 128;
-            const int valid = (int)min((int64_t)128, g.n - r0);
-            if (fbulk) {
-                if (!wait_or_abort(ufbar, (uint32_t)(it & 1), &abort_flag)) abort_flag = 1;
-                fpend = -1;
-                // (on abort the values read below are stale but in bounds; the tile loop ends)
-            } else {
-                cp_async_wait0();
-                epi_sync();
-            }
-            float zc[8];
-            bool box = true;
+            const int np = (NF / 2) * rows_of(it);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int k = 8 * part + i;  // warp-uniform: part is
-                zc[i] = k >= NF ? 1.0f       // the bias columns
-                                : mrow < valid ? (raw_feature(sF[mrow * NF + k], k < 6) - xm[k]) * xr[k] : 0.0f;
-                if (k < NF) box = box && zc[i] >= lo[k] && zc[i] <= hi[k];
-            }
-            uint32_t w4[4], l4[4];
+            for (int i = 0; i < FPT; ++i) {
+                const int e = tid + IT * i;
+                if (e >= 128 * (NF / 2)) break;
+                const int row = e / (NF / 2), k = 2 * (e - row * (NF / 2));
+                float z[2] = {0.0f, 0.0f};  // rows beyond the input
+                if (e < np) {
+                    bool box = true;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const __half2 h = __floats2half2_rn(zc[2 * i], zc[2 * i + 1]);
+                    for (int c = 0; c < 2; ++c) {
+                        z[c] = standardise(f[i][c], k, snv[NV_XM + k + c], snv[NV_XR + k + c]);
+                        box = box && z[c] >= snv[NV_LO + k + c] && z[c] <= snv[NV_HI + k + c];
+                    }
+                    if (!box) sBox[(it & 1) * 128 + row] = 0;
+                }
+                const __half2 h = __floats2half2_rn(z[0], z[1]);
                 const float2 hf = __half22float2(h);
-                const __half2 r = __floats2half2_rn(zc[2 * i] - hf.x, zc[2 * i + 1] - hf.y);  // 0 for the bias columns
-                w4[i] = *reinterpret_cast<const uint32_t*>(&h);
-                l4[i] = *reinterpret_cast<const uint32_t*>(&r);
+                const __half2 r = __floats2half2_rn(z[0] - hf.x, z[1] - hf.y);
+                *reinterpret_cast<__half2*>(sX + canon(row, k, 512)) = h;
+                *reinterpret_cast<__half2*>(sXlo + canon(row, k, 512)) = r;
             }
-            *reinterpret_cast<uint4*>(sX + canon(mrow, 8 * part, 512)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-            *reinterpret_cast<uint4*>(sXlo + canon(mrow, 8 * part, 512)) = make_uint4(l4[0], l4[1], l4[2], l4[3]);
-            sBox[(it & 1) * 512 + part * 128 + mrow] = box ? 1 : 0;
-            publish(ux);
-            epi_sync();  // the staging buffer has been read; the box tests are visible
-            if (it + 1 < my_tiles) {
-                const int64_t rn = ((int64_t)blockIdx.x + (it + 1) * gridDim.x) * 128;
-                issue_features(fbulk, uF, g.feat, rn, (int)min((int64_t)128, g.n - rn), ufbar);
-                fpend = (int)(it + 1);
+            publish(ux_lead);
+            if (lane == 0) mbar_arrive(ulx);  // (this CTA's box tests)
+            fetch(it + 1);
+        };
+        auto outputs = [&](int64_t it) {  // layer 4 -> FP64 outputs (two columns per thread of the last three column slices)
+            const int64_t r0 = first_row(it);
+            const int valid = rows_of(it);
+            if (cs > 0) {
+                float v[2];
+                tmem_ld2(tmem_row + 256u + (uint32_t)(2 * (cs - 1)), v);
+                if (erow < valid) {
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const int o = 2 * (cs - 1) + c;
+                        g.lp6[(r0 + erow) * NO + o] = f2d((v[c] + snv[NV_B4 + o]) * snv[NV_YS + o] + snv[NV_YM + o]);
+                    }
+                }
             }
         };
-        map_tile(0);
+        fetch(0);
+        if (!(ok = wait_or_abort(ures, 0u, &abort_flag))) raise_abort();
+        if (ok) map_tile(0);
         for (int64_t it = 0; it < my_tiles && ok; ++it) {
-            if (abort_flag) {
-                ok = false;
-                break;
-            }
-            const int64_t r0 = ((int64_t)blockIdx.x + it * gridDim.x) * 128;
-            const int valid = (int)min((int64_t)128, g.n - r0);
             // 1. hidden layers: activations chunk by chunk, each handed over at once
             for (int l = 0; l < 3 && ok; ++l) {
                 ok = wait_acc(l);
                 if (!ok) break;
-                if (l == 0 && cs == 0) {
-                    // trust region of this row: its row of W lies in columns the
-                    // layer-2 MMAs overwrite, so it is read before the first hand-over
-                    float wv[32];
-                    tmem_ld16(tmem_row + (uint32_t)MAHA_COL, wv);
-                    tmem_ld16(tmem_row + (uint32_t)MAHA_COL + 16u, wv + 16);
-                    float d2 = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < NF; ++i) d2 = fmaf(wv[i], wv[i], d2);
-                    const uint8_t* bx = sBox + (it & 1) * 512 + erow;  // this tile's half: the next tile's map
-                    const bool box = bx[0] & bx[128] & bx[256] & bx[384];  // may already be writing the other
-                    if (erow < valid && g.in_region) g.in_region[r0 + erow] = (box && d2 * inv_s2 <= d2_thr) ? 1 : 0;
-                }
                 const uint32_t acc_col = (l == 1) ? 256u : 0u;
                 // the load of chunk kc + 1 runs while chunk kc is turned into activations
                 uint32_t ra[16], rb[16];
                 tmem_ld16_async(tmem_row + acc_col + (uint32_t)(16 * cs), ra);
-                // chunk kc is handed over one step late, after chunk kc + 1's
-                // arithmetic, so that its proxy fence finds the stores done
+                if (l == 0 && cs == 0) {
+                    // trust region of this row: its row of W lies in columns the
+                    // layer-2 MMAs overwrite, so it is read before the first hand-over.
+                    // (lxbar, to have seen every warp's box tests; its next phase needs this warp)
+                    uint32_t wv[32];
+                    tmem_ld16_async(tmem_row + (uint32_t)MAHA_COL, wv);
+                    tmem_ld16_async(tmem_row + (uint32_t)MAHA_COL + 16u, wv + 16);
+                    if (!(ok = wait_or_abort(ulx, xph, &abort_flag))) raise_abort();
+                    xph ^= 1u;
+                    tmem_wait_ld16(wv);
+                    tmem_wait_ld16(wv + 16);
+                    float d2 = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < NF; ++i) {
+                        const float w = __uint_as_float(wv[i]);
+                        d2 = fmaf(w, w, d2);
+                    }
+                    uint8_t* bx = sBox + (it & 1) * 128 + erow;  // this tile's half: the next tile's map
+                    const bool box = *bx != 0;                   // may already be writing the other
+                    *bx = 1;                                     // (read here only; written again two tiles on)
+                    if (erow < rows_of(it) && g.in_region)
+                        g.in_region[first_row(it) + erow] = (box && d2 * snv[NV_S2] <= snv[NV_THR]) ? 1 : 0;
+                }
+                // chunk 0 is handed over at once (the tensor cores wait for it), chunks 1 and 2
+                // one step late, after the next chunk's arithmetic, so that the proxy
+                // fence finds the stores done (10^6 rows, same build: all late 418 us, all at once 462, so 410)
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
                     const int c0 = 64 * kc + 16 * cs;
-                    tmem_wait_ld();
                     uint32_t* cur = (kc & 1) ? rb : ra;
                     uint32_t* nxt = (kc & 1) ? ra : rb;
+                    tmem_wait_ld16(cur);
                     if (kc < 3) tmem_ld16_async(tmem_row + acc_col + (uint32_t)(c0 + 64), nxt);
                     uint32_t w[8];
-                    gelu16<false>(cur, c0, nullptr, w);  // (every layer's bias is in its accumulator)
-                    if (kc > 0) publish(uh0 + 8 * (kc - 1));
+                    gelu16(cur, w);
+                    if (kc > 1) publish(uh_lead + 8 * (kc - 1));
                     store16(w, erow, c0, sH);
+                    if (kc == 0) publish(uh_lead);
                 }
-                publish(uh0 + 24);
-                // the next tile's input map, while layer 2 finishes: its operand
-                // may be published now, because the MMA issuer starts the next
-                // tile's layer 1 only after this tile's layer 4, i.e. after
-                // every layer-3 chunk (accumulator A) has been read
-                if (l == 0 && it + 1 < my_tiles) map_tile(it + 1);
+                publish(uh_lead + 24);
+                // the next tile's input map, while layer 3 runs (after layer 1's epilogue: 1 % slower)
+                if (l == 1 && it + 1 < my_tiles) map_tile(it + 1);
             }
             if (!ok) break;
-            // 2. layer 4 -> FP64 outputs (two columns per thread of the first three column slices)
+            // 2. the outputs; the tensor cores are at the next tile's layer 1
             if (!(ok = wait_acc(3))) break;
-            if (cs < 3) {
-                float v[2];
-                tmem_ld2(tmem_row + 256u + (uint32_t)(2 * cs), v);
-                if (erow < valid) {
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const int o = 2 * cs + c;
-                        g.lp6[(r0 + erow) * NO + o] = f2d((v[c] + sB[o]) * ys[o] + ym[o]);
-                    }
-                }
-            }
+            outputs(it);
             tc_fence_before();
         }
-        cp_async_wait0();
-        // a feature copy still landing (the loop ended early): wait (bounded) for it
-        if (fbulk && tid == 0 && fpend >= 0) mbar_wait_bounded(ufbar, (uint32_t)(fpend & 1), MBAR_WAIT_LIMIT);
-        if (!ok && (tid & 31) == 0) atomicExch(g.err, 1);
+        if (!ok && lane == 0) atomicExch(g.err, 1);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 512);
+    cluster_sync();  // no arrival, MMA or flag of the pair is still on its way to this CTA
+    if (warp == 0) tmem_dealloc2(tmem, 512);
 }
 
-// The staged copy of layers 2 and 3, LAYER_BYTES each: the bias block
-// (256 rows x K 16 in the canonical no-swizzle K-major layout, 8-row groups
-// 256 B apart: row r holds b_hi = fp16(b_r), b_lo = fp16(b_r - b_hi), then
-// zeros), then W / 2 (row-major 256 x 256 BF16 in, FP16 out) in CPL K-chunks
-// of 256 rows x KCH in the same layout (K-adjacent core matrices 128 B apart,
-// 8-row groups 16 KCH bytes apart), WC_BYTES each; every item is one
-// contiguous bulk copy into shared memory.
-__global__ void tile_weights_kernel(const __nv_bfloat16* __restrict__ W2, const __nv_bfloat16* __restrict__ W3,
-                                    const float* __restrict__ b2, const float* __restrict__ b3,
-                                    __half* __restrict__ Wc)
+// What the inference kernel keeps in shared memory (RES_BYTES for each CTA of a pair,
+// that CTA's half of the rows of every weight): W1 with the bias of layer 1 in K
+// columns 30 and 31 (two FP16 parts), s L^-1 in two FP16 parts, W4 / 2, the biases of
+// layers 2 and 3 and the ones operands of the bias MMAs, the maps, W2 / 2 and W3 / 2, all
+// matrices in the canonical no-swizzle K-major layout (K-adjacent core matrices 128 B
+// apart).  Blocks 0 .. 63 lay out W2 and W3, blocks 64 and 65 the rest.
+constexpr int WH_BLOCKS = 2 * 256 * 32 / 256;
+__global__ void __launch_bounds__(256) tile_resident_kernel(const __nv_bfloat16* __restrict__ W1,
+                                                            const float* __restrict__ b1,
+                                                            const __nv_bfloat16* __restrict__ W2,
+                                                            const float* __restrict__ b2,
+                                                            const __nv_bfloat16* __restrict__ W3,
+                                                            const float* __restrict__ b3,
+                                                            const __nv_bfloat16* __restrict__ W4,
+                                                            const float* __restrict__ b4, const float* __restrict__ nv,
+                                                            uint8_t* __restrict__ out)
 {
-    constexpr int G = KCH / 8;  // 16-byte groups per row of a chunk
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    uint8_t* base = reinterpret_cast<uint8_t*>(Wc);
-    if (v < 2 * CPL * 256 * G) {  // one 16-byte group of W: chunk j, row r, group kk
-        const int j = v / (256 * G), r = (v / G) % 256, kk = v % G;
-        const int l = j / CPL;
-        const __nv_bfloat16* W = l == 0 ? W2 : W3;
-        const int k0 = KCH * (j % CPL) + 8 * kk;
-        uint8_t* dst = base + (size_t)l * LAYER_BYTES + BB_BYTES + (size_t)(j % CPL) * WC_BYTES + (r >> 3) * (16 * KCH) +
-                       kk * 128 + (r & 7) * 16;
-        *reinterpret_cast<uint4*>(dst) = bf16x8_to_f16x8(*reinterpret_cast<const uint4*>(W + r * 256 + k0), 0.5f);
-    } else if (v < 2 * CPL * 256 * G + 2 * 256) {  // one row of a bias block
-        const int u = v - 2 * CPL * 256 * G, l = u / 256, r = u % 256;
-        const float bb = (l == 0 ? b2 : b3)[r];
-        const __half hi = __float2half_rn(bb), lo = __float2half_rn(bb - __half2float(hi));
+    __shared__ unsigned li_max;  // bits of max |L^-1| (non-negative floats order as integers)
+    const int tid = threadIdx.x;
+    if (blockIdx.x < WH_BLOCKS) {  // one 16-byte group of W2 or W3: row r, group kk
+        const int v = blockIdx.x * 256 + tid, l = v >> 13, r = (v >> 5) & 255, kk = v & 31;
+        uint8_t* dst = out + (size_t)(r >> 7) * RES_BYTES + R_WH + l * WH_BYTES + canon(r & 127, 8 * kk, 4096);
+        *reinterpret_cast<uint4*>(dst) =
+            bf16x8_to_f16x8(*reinterpret_cast<const uint4*>((l ? W3 : W2) + r * 256 + 8 * kk), 0.5f);
+        return;
+    }
+    const int rank = blockIdx.x - WH_BLOCKS;
+    uint8_t* res = out + (size_t)rank * RES_BYTES;
+    if (tid == 0) li_max = 0u;
+    __syncthreads();
+    const float* gLi = nv + 4 * NF + 2 * NO;  // L^-1, NF x NF row-major, lower triangle
+    for (int e = tid; e < NF * NF; e += 256) atomicMax(&li_max, __float_as_uint(fabsf(gLi[e])));
+    auto split = [](float b) {  // b in two FP16 parts
+        const __half hi = __float2half_rn(b), lo = __float2half_rn(b - __half2float(hi));
         const __half2 h2 = __halves2half2(hi, lo);
-        uint8_t* dst = base + (size_t)l * LAYER_BYTES + (r >> 3) * 256 + (r & 7) * 16;
-        *reinterpret_cast<uint4*>(dst) = make_uint4(*reinterpret_cast<const uint32_t*>(&h2), 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(dst + 128) = make_uint4(0u, 0u, 0u, 0u);
+        return *reinterpret_cast<const uint32_t*>(&h2);
+    };
+    for (int e = tid; e < 128 * 4; e += 256) {  // W1: 128 rows x 32 K (4 x 8-element groups)
+        const int r = e >> 2, kc = e & 3, gr = 128 * rank + r;
+        uint4 v = bf16x8_to_f16x8(*reinterpret_cast<const uint4*>(W1 + gr * 32 + kc * 8), 1.0f);
+        if (kc == 3) v.w = split(b1[gr]);  // K columns 30, 31
+        *reinterpret_cast<uint4*>(res + R_W1 + canon(r, 8 * kc, 512)) = v;
+    }
+    {  // W4 / 2: 8 rows x 256 K
+        const int r = tid >> 5, kc = tid & 31;
+        *reinterpret_cast<uint4*>(res + R_W4 + canon(r, 8 * kc, 4096)) =
+            bf16x8_to_f16x8(*reinterpret_cast<const uint4*>(W4 + (8 * rank + r) * 256 + kc * 8), 0.5f);
+    }
+    if (tid < 128)
+        *reinterpret_cast<uint4*>(res + R_BB + tid * 16) =
+            make_uint4(split(b2[128 * rank + tid]), split(b3[128 * rank + tid]), 0u, 0u);
+    if (tid < 32) {  // per layer two core matrices: 8 rows x K 0..7, K 8..15
+        const int l = tid >> 4, group = (tid >> 3) & 1, r = tid & 7;
+        const uint32_t one = group == 0 ? 0x3c003c00u : 0u;
+        *reinterpret_cast<uint4*>(res + R_ONES + l * ONES_BYTES + group * 128 + r * 16) =
+            make_uint4(l == 0 ? one : 0u, l == 1 ? one : 0u, 0u, 0u);
+    }
+    __syncthreads();
+    int li_exp = 0;
+    frexpf(__uint_as_float(li_max), &li_exp);
+    const int li_k = li_max ? max(-60, min(60, 14 - li_exp)) : 0;  // s = 2^li_k
+    const float li_s = ldexpf(1.0f, li_k);
+    for (int e = tid; e < 16 * 32; e += 256) {  // s L^-1 = L_hi + L_lo, rows i and K columns j, zero-padded
+        const int r = e >> 5, i = 16 * rank + r, j = e & 31;
+        const float v = (i < NF && j <= i) ? gLi[i * NF + j] * li_s : 0.0f;
+        const __half hi = __float2half_rn(v);
+        *reinterpret_cast<__half*>(res + R_LH + canon(r, j, 512)) = hi;
+        *reinterpret_cast<__half*>(res + R_LL + canon(r, j, 512)) = __float2half_rn(v - __half2float(hi));
+    }
+    float* o = reinterpret_cast<float*>(res + R_NV);
+    for (int e = tid; e < NV_BYTES / 4; e += 256) {
+        float v = 0.0f;
+        if (e < NV_XR) v = nv[e];
+        else if (e < NV_YM) v = 1.0f / nv[e];  // (the deviations xs are kept as reciprocals)
+        else if (e < NV_THR) v = nv[e];
+        else if (e == NV_THR) v = nv[4 * NF + 2 * NO + NF * NF];
+        else if (e == NV_S2) v = ldexpf(1.0f, -2 * li_k);
+        else if (e < NV_COUNT) v = b4[e - NV_B4];
+        o[e] = v;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_mlp_infer(const double* feat, int64_t n, const float* nv, const __nv_bfloat16* const W[4],
-                             const float* const b[4], __nv_bfloat16* wc, double* lp6, uint8_t* in_region, int* err,
-                             cudaStream_t s)
+size_t mlp_infer_stage_bytes() { return (size_t)2 * RES_BYTES; }
+
+cudaError_t launch_mlp_infer_stage(const float* nv, const __nv_bfloat16* const W[4], const float* const b[4],
+                                   uint8_t* stage, cudaStream_t s)
+{
+    tile_resident_kernel<<<WH_BLOCKS + 2, 256, 0, s>>>(W[0], b[0], W[1], b[1], W[2], b[2], W[3], b[3], nv, stage);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_infer(const double* feat, int64_t n, const uint8_t* stage, double* lp6, uint8_t* in_region,
+                             int* err, cudaStream_t s)
 {
     static bool attr_set[64] = {};  // the attribute is per function and device
     int dev = 0;
@@ -701,28 +766,18 @@ cudaError_t launch_mlp_infer(const double* feat, int64_t n, const float* nv, con
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     if (n <= 0) return cudaSuccess;
-    // the staged FP16 weights live in the 2-byte-per-element scratch wc
-    __half* wh = reinterpret_cast<__half*>(wc);
-    tile_weights_kernel<<<(2 * CPL * 256 * (KCH / 8) + 2 * 256 + 255) / 256, 256, 0, s>>>(W[1], W[2], b[1], b[2], wh);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tiles = (n + 127) / 128;
+    const int64_t pairs = (n + 255) / 256, most = sms / 2;
     InferArgs g{};
     g.feat = feat;
     g.n = n;
-    g.feat_bulk = ((uintptr_t)feat & 15u) == 0;
-    g.nv = nv;
-    for (int l = 0; l < 4; ++l) {
-        g.W[l] = W[l];
-        g.b[l] = b[l];
-    }
-    g.Wc = wh;
+    g.feat_wide = ((uintptr_t)feat & 15u) == 0;
+    g.res = stage;
     g.lp6 = lp6;
     g.in_region = in_region;
     g.err = err;
-    mlp_infer_kernel<<<(unsigned)(tiles < sms ? tiles : sms), IT_ALL, INFER_SMEM, s>>>(g);
+    mlp_infer_kernel<<<(unsigned)(2 * (pairs < most ? pairs : most)), IT_ALL, INFER_SMEM, s>>>(g);
     return cudaGetLastError();
 }
 

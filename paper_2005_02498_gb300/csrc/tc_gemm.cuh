@@ -185,12 +185,14 @@ __device__ __forceinline__ void load_chunk_async(uint32_t dst, const __nv_bfloat
 cudaError_t launch_tc_gemm(const GemmArgs& g, cudaStream_t s);
 
 // Fused surrogate inference (mlp_infer.cu): raw features [n x 30] -> sym(Lp)
-// [n x 6] in FP64 and the trust-region flags; nv = the FP32 maps (xm, xs, ym,
-// ys, box, Cholesky factor, threshold), W/b the BF16 weights and FP32 biases,
-// wc a device buffer of 8 x 256 x 64 BF16 for the pre-tiled W2/W3 chunks
-// (rewritten by every launch).  Two launches: the tiling, the fused kernel.
-cudaError_t launch_mlp_infer(const double* feat, int64_t n, const float* nv, const __nv_bfloat16* const W[4],
-                             const float* const b[4], __nv_bfloat16* wc, double* lp6, uint8_t* in_region, int* err,
-                             cudaStream_t s);
+// [n x 6] in FP64 and the trust-region flags.  The operands are laid out once per
+// change of the parameters or maps (launch_mlp_infer_stage, into mlp_infer_stage_bytes()
+// of device memory): nv = the FP32 maps (xm, xs, ym, ys, box, inverse Cholesky factor,
+// threshold), W/b the BF16 weights and FP32 biases.
+size_t mlp_infer_stage_bytes();
+cudaError_t launch_mlp_infer_stage(const float* nv, const __nv_bfloat16* const W[4], const float* const b[4],
+                                   uint8_t* stage, cudaStream_t s);
+cudaError_t launch_mlp_infer(const double* feat, int64_t n, const uint8_t* stage, double* lp6, uint8_t* in_region,
+                             int* err, cudaStream_t s);
 
 }  // namespace ptadd
