@@ -48,8 +48,8 @@ struct MlpDev {
     float *W[4] = {}, *b[4] = {}, *mW[4] = {}, *vW[4] = {}, *mb[4] = {}, *vb[4] = {}, *gW[4] = {}, *gb[4] = {};
     __nv_bfloat16 *Wb[4] = {}, *Wt[4] = {};
     uint8_t* stage = nullptr;  // operands laid out for the fused inference kernel, current with the parameters and maps
-    __nv_bfloat16 *X = nullptr, *Xt = nullptr, *Hb[3] = {}, *Ht[3] = {}, *dY = nullptr, *dYt = nullptr;
-    __nv_bfloat16 *dZ[3] = {}, *dZt[3] = {};
+    __nv_bfloat16 *X = nullptr, *Xt = nullptr, *Hb[3] = {}, *Ht[3] = {}, *dYt = nullptr;
+    __nv_bfloat16* dZt[3] = {};
     float *Y = nullptr, *loss_part = nullptr;
     int* err = nullptr;
     int64_t step = 0;
@@ -80,17 +80,16 @@ ptadd_status m_alloc(T** p, size_t count)
 
 void free_work(MlpDev& m)
 {
-    void* ptrs[] = {m.X, m.Xt, m.dY, m.dYt, m.Y, m.loss_part};
+    void* ptrs[] = {m.X, m.Xt, m.dYt, m.Y, m.loss_part};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int l = 0; l < 3; ++l) {
         cudaFree(m.Hb[l]);
         cudaFree(m.Ht[l]);
-        cudaFree(m.dZ[l]);
         cudaFree(m.dZt[l]);
-        m.Hb[l] = m.Ht[l] = m.dZ[l] = m.dZt[l] = nullptr;
+        m.Hb[l] = m.Ht[l] = m.dZt[l] = nullptr;
     }
-    m.X = m.Xt = m.dY = m.dYt = nullptr;
+    m.X = m.Xt = m.dYt = nullptr;
     m.Y = m.loss_part = nullptr;
     m.cap = 0;
 }
@@ -142,10 +141,8 @@ ptadd_status ensure_work(MlpDev& m, int64_t rows)
     for (int l = 0; l < 3; ++l) {
         WA(m.Hb[l], need * NH);
         WA(m.Ht[l], need * NH);
-        WA(m.dZ[l], need * NH);
         WA(m.dZt[l], need * NH);
     }
-    WA(m.dY, need * 16);
     WA(m.dYt, need * 16);
     WA(m.Y, need * 16);
     WA(m.loss_part, need / 128);
@@ -252,13 +249,10 @@ TrainArgs train_args(MlpDev& m, int64_t n, int64_t rows, const float* xn, const 
         g.gb[l] = m.gb[l];
     }
     for (int l = 0; l < 3; ++l) {
-        g.Hb[l] = m.Hb[l];
         g.Ht[l] = m.Ht[l];
-        g.dZ[l] = m.dZ[l];
         g.dZt[l] = m.dZt[l];
     }
     g.Xt = m.Xt;
-    g.dY = m.dY;
     g.dYt = m.dYt;
     g.loss_part = loss_part;
     g.err = m.err;

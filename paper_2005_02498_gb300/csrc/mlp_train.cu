@@ -6,20 +6,22 @@
 // and the update.  As separate launches (7 GEMMs, 4 weight-gradient GEMMs, 19
 // small kernels) a step took 255 us.
 //
-//   mlp_fb_kernel: the whole chain.  A cluster of four CTAs owns 128 rows; each CTA
-//   owns 64 of the 256 columns of every layer and keeps GELU'(Z) of its tile in
-//   registers from the forward to the backward pass.  Between layers the
-//   activations go through L2 (row-major for the next layer, transposed for the
-//   weight gradients) and a cluster barrier; the next layer's weights are
-//   loaded while the epilogue runs.
+//   mlp_fb_kernel: the whole chain.  A cluster of eight CTAs owns 128 rows; each CTA
+//   owns 32 of the 256 columns of every layer and keeps GELU'(Z) of its tile in
+//   registers from the forward to the backward pass.  A layer's columns are written into
+//   the operand buffers of all eight CTAs' shared memory, and a barrier of the cluster
+//   is the hand-over; what only the weight gradients need goes to global memory
+//   (transposed) while the others arrive, the next layer's weights are loaded while the
+//   epilogue runs.
 //   mlp_dw_kernel: every weight gradient dW = dZ^T H at once, 42 CTAs of 128 x 32
 //   outputs over all rows, with Adam and the BF16 copies in the epilogue; the bias
 //   gradients (row sums of dZ^T) in 98 more.
-// What bounds it: latency.  At 512 rows a minibatch is 16 CTAs in the first launch (48 us
-// cold: seven dependent products, a cluster barrier and an L2 round trip after each) and
-// 140 in the second (21 us); weights and activations stay in L2.  Two epochs of 8192
-// rows in minibatches of 512 take 2.65 ms (70 us a minibatch, and the host's copies of parameters
-// and data) where one launch per product, transposition, reduction and update took 8.18 ms.
+// What bounds it: latency.  At 512 rows a minibatch is 32 CTAs in the first launch (27 us:
+// seven dependent products, each with a hand-over of some 5000 cycles) and 140 in the
+// second (18 us).  Two epochs of 8192 rows in minibatches of 512 take 2.22 ms (57 us a
+// minibatch with the host's shuffle, and copies of parameters and data) where one launch per
+// product, transposition, reduction and update took 8.18 ms, and four CTAs of 64 columns
+// that exchanged their activations through L2 2.65 ms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -31,23 +33,24 @@ namespace ptadd {
 namespace {
 
 constexpr int NIN = 30, NOUT = 6, NH = 256;
-constexpr int FB_T = 512;             // threads: 4 TMEM lane groups x 4 slices of 16 columns
-constexpr int FB_N = 64;              // columns of a layer per CTA
+constexpr int FB_CL = 8;              // CTAs of a cluster
+constexpr int FB_N = NH / FB_CL;      // columns of a layer per CTA
+constexpr int FB_C = 8;               // columns per thread
+constexpr int FB_T = 128 * FB_N / FB_C;  // threads: 4 TMEM lane groups x FB_N / FB_C slices
 constexpr int A_CHUNK = 128 * 64 * 2; // one K-chunk of 64 of the A operand
 constexpr int FB_A = 4 * A_CHUNK;     // A: 128 rows x K 256
 constexpr int FB_B = 4 * FB_N * 64 * 2;
-constexpr int FB_SMEM = FB_A + FB_B;
+constexpr int FB_SMEM = 2 * FB_A + FB_B;
 constexpr int DW_T = 256, DW_N = 32, DW_KC = 8;  // threads, columns per CTA, K-chunks of 64 in shared memory
 constexpr int DW_B_CHUNK = DW_N * 64 * 2;
 constexpr int DW_SMEM = DW_KC * (A_CHUNK + DW_B_CHUNK);
 
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// generic-proxy writes to any CTA's shared memory before the tensor core's reads
+__device__ __forceinline__ void fence_async_cluster() { asm volatile("fence.proxy.async.shared::cluster;" ::: "memory"); }
 
 // K columns k0 .. k0 + 64 nchunk - 1 of rows row0 .. row0 + R - 1 of a K-contiguous matrix
 // into nchunk consecutive chunks in the canonical layout (tc_gemm.cuh); zeros beyond row_lim and K.
@@ -85,27 +88,42 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// 16 values of row r, columns c0 .. c0 + 15: BF16, row-major (ld columns) and transposed
-__device__ __forceinline__ void store16(const float h[16], __nv_bfloat16* rm, int64_t ld, __nv_bfloat16* tr, int64_t rows,
-                                        int64_t r, int c0)
+// FB_C values of a tile's row lr, columns c .. c + FB_C - 1, in BF16: into the A operand at
+// shared-memory address a of the CTAs 0 .. peers - 1 of the cluster
+__device__ __forceinline__ void share8(const float h[FB_C], uint32_t a, int lr, int c, int peers)
 {
-    uint32_t w[8];
+    const uint32_t at = a + (uint32_t)((c >> 6) * A_CHUNK + (lr >> 3) * 1024 + ((c >> 3) & 7) * 128 + (lr & 7) * 16);
+    const uint32_t w0 = pack2(h[0], h[1]), w1 = pack2(h[2], h[3]), w2 = pack2(h[4], h[5]), w3 = pack2(h[6], h[7]);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = pack2(h[2 * i], h[2 * i + 1]);
-    if (rm) {
-        uint4* o = reinterpret_cast<uint4*>(rm + r * ld + c0);
-        o[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    for (int p = 0; p < FB_CL; ++p) {
+        if (p >= peers) break;
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(at), "r"(p));
+        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w0), "r"(w1), "r"(w2), "r"(w3)
+                     : "memory");
     }
+    fence_async_cluster();
+}
+// ... and transposed [. x rows] for the weight gradients
+__device__ __forceinline__ void store_t8(const float h[FB_C], __nv_bfloat16* tr, int64_t rows, int64_t r, int c)
+{
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
-        tr[(int64_t)(c0 + 2 * i) * rows + r] = v.x;
-        tr[(int64_t)(c0 + 2 * i + 1) * rows + r] = v.y;
-    }
+    for (int i = 0; i < FB_C; ++i) tr[(int64_t)(c + i) * rows + r] = __float2bfloat16_rn(h[i]);
+}
+// 8 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8])
+{
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kernel(TrainArgs g)
+__global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_kernel(TrainArgs g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t mbar;
@@ -114,9 +132,9 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kern
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t row0 = (int64_t)blockIdx.x * 128;
     const int y = blockIdx.y, n0 = y * FB_N;
-    const uint32_t uA = smem_u32(smem), uB = uA + FB_A, mb = smem_u32(&mbar);
+    const uint32_t uA = smem_u32(smem), uB = uA + 2 * FB_A, mb = smem_u32(&mbar);
     const int lr = 32 * (warp & 3) + lane;  // this thread's row of the tile
-    const int c0 = 16 * (warp >> 2);        // and first column of its slice
+    const int c0 = FB_C * (warp >> 2);      // and first column of its slice
     const int64_t r = row0 + lr;
     const bool live = r < g.rows;
     if (warp == 0) {
@@ -124,11 +142,12 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kern
         tmem_relinquish();
     }
     if (tid == 0) mbar_init(mb, 1);
+    cluster_arrive();  // (waited for before the first write into another CTA: it has started by then)
     // layer 1: its weights, and the inputs straight from the samples
     load_operand<FB_N, FB_T>(uB, g.Wb[0], din_p(0), n0, NH, 0, din_p(0), 1);
     cp_commit();
-    {
-        const int xr = tid >> 2, part = tid & 3;
+    for (int e = tid; e < 128 * 4; e += FB_T) {
+        const int xr = e >> 2, part = e & 3;
         const int64_t gr = row0 + xr;
         float v[8];
 #pragma unroll
@@ -159,14 +178,14 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kern
     bool ok = true;
     // the operands have been issued: wait for them, multiply, wait for the product.  A wait
     // that gives up leaves the rest of the tile's products out; every barrier is still met.
-    auto multiply = [&](int steps, int N) {
+    auto multiply = [&](uint32_t ua, int steps, int N) {
         cp_wait_all();
-        fence_async_smem();
+        fence_async_cluster();  // this thread's copies, and what its barrier wait has made visible
         tc_fence_before();
         __syncthreads();
         if (tid == 0 && ok) {
             tc_fence_after();
-            issue_mma<FB_N>(tmem, uA, uB, steps, idesc_bf16_f32(128, N), false);
+            issue_mma<FB_N>(tmem, ua, uB, steps, idesc_bf16_f32(128, N), false);
             tc_commit(mb);
         }
         bool w = true;
@@ -175,57 +194,65 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kern
         ok = __syncthreads_and(ok && w);
         tc_fence_after();
     };
-    float dg[3][16];  // GELU'(Z) of this thread's values
+    // The A operand alternates between two buffers (layer l reads buffer l mod 2): a CTA writes
+    // its columns of the next operand while a slower one still multiplies from this one, and
+    // a buffer's last readers have passed a barrier of the cluster before it is written again.
+    float dg[3][FB_C];  // GELU'(Z) of this thread's values
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-        multiply(l == 0 ? 2 : 16, FB_N);
+        multiply(uA + (l & 1) * FB_A, l == 0 ? 2 : 16, FB_N);
         // the next layer's weights, while the epilogue runs
         if (l < 2)
             load_operand<FB_N, FB_T>(uB, g.Wb[l + 1], NH, n0, NH, 0, NH, 4);
         else if (y == 0)
             load_operand<FB_N, FB_T>(uB, g.Wb[3], NH, 0, dout_p(3), 0, NH, 4);
         cp_commit();
-        float z[16], h[16];
-        tmem_ld16(trow, z);
+        float z[FB_C], h[FB_C], e[FB_C];
+        tmem_ld8(trow, z);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < FB_C; ++i) {
             z[i] += g.b[l][n0 + c0 + i];
-            const float e = 1.0f + erff(z[i] * 0.70710678118654752f);
-            h[i] = 0.5f * z[i] * e;
-            dg[l][i] = 0.5f * e + z[i] * expf(-0.5f * z[i] * z[i]) * 0.39894228040143268f;
+            e[i] = 1.0f + erff(z[i] * 0.70710678118654752f);
+            h[i] = 0.5f * z[i] * e[i];
         }
-        if (live) store16(h, g.Hb[l], NH, g.Ht[l], g.rows, r, n0 + c0);
+        if (l == 0) cluster_wait();
+        share8(h, uA + ((l + 1) & 1) * FB_A, lr, n0 + c0, l < 2 ? FB_CL : 1);  // (layer 4 is the first CTA's)
         tc_fence_before();
-        cluster_sync();
-        if (l < 2 || y == 0) {
-            load_operand<128, FB_T>(uA, g.Hb[l], NH, row0, g.rows, 0, NH, 4);
-            cp_commit();
-        }
+        cluster_arrive();
+        // what only the backward pass and the weight gradients read, while the others arrive
+        if (live) store_t8(h, g.Ht[l], g.rows, r, n0 + c0);
+#pragma unroll
+        for (int i = 0; i < FB_C; ++i)
+            dg[l][i] = 0.5f * e[i] + z[i] * expf(-0.5f * z[i] * z[i]) * 0.39894228040143268f;
+        cluster_wait();
     }
     // layer 4 (one CTA of the cluster), the loss and its gradient
     if (y == 0) {
-        multiply(16, dout_p(3));
+        multiply(uA + FB_A, 16, dout_p(3));
         load_operand<FB_N, FB_T>(uB, g.Wt[3], dout_p(3), n0, NH, 0, dout_p(3), 1);
         cp_commit();
-        if (c0 == 0) {
-            float v[16], d[16], loss = 0.0f;
-            tmem_ld16(trow, v);
+        if (c0 < dout_p(3)) {
+            float v[FB_C], d[FB_C], loss = 0.0f;
+            tmem_ld8(trow, v);
             const float scale = 1.0f / ((float)g.n * NOUT);
             const bool in = r < g.n;
             const float* t = g.yn + (in ? (g.idx ? (int64_t)g.idx[r] : r) : 0) * NOUT;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < FB_C; ++i) {
                 d[i] = 0.0f;
-                if (in && i < NOUT) {
-                    const float e = v[i] + g.b[3][i] - t[i];
+                if (in && c0 + i < NOUT) {
+                    const float e = v[i] + g.b[3][c0 + i] - t[c0 + i];
                     loss += e * e * scale;
                     d[i] = 2.0f * e * scale;
                 }
             }
-            if (live) store16(d, g.dY, dout_p(3), g.dYt, g.rows, r, 0);
+            share8(d, uA, lr, c0, FB_CL);
+            if (live) store_t8(d, g.dYt, g.rows, r, c0);
+            if (c0 == 0) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-            if (lane == 0) red[warp] = loss;
+                for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+                if (lane == 0) red[warp] = loss;
+            }
         }
         __syncthreads();
         if (tid == 0) g.loss_part[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
@@ -234,28 +261,27 @@ __global__ void __cluster_dims__(1, 4, 1) __launch_bounds__(FB_T, 1) mlp_fb_kern
         cp_commit();
     }
     tc_fence_before();
-    cluster_sync();
-    load_operand<128, FB_T>(uA, g.dY, dout_p(3), row0, g.rows, 0, dout_p(3), 1);
-    cp_commit();
+    cluster_arrive();
+    cluster_wait();
     // backward: dZ_l = (dZ_{l+1} W_{l+1}) GELU'(Z_l)
 #pragma unroll
     for (int l = 2; l >= 0; --l) {
-        multiply(l == 2 ? 1 : 16, FB_N);
+        multiply(uA + (l & 1) * FB_A, l == 2 ? 1 : 16, FB_N);
         if (l > 0) {
             load_operand<FB_N, FB_T>(uB, g.Wt[l], NH, n0, NH, 0, NH, 4);
             cp_commit();
         }
-        float v[16];
-        tmem_ld16(trow, v);
+        float v[FB_C];
+        tmem_ld8(trow, v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] *= dg[l][i];
-        if (live) store16(v, l > 0 ? g.dZ[l] : nullptr, NH, g.dZt[l], g.rows, r, n0 + c0);
+        for (int i = 0; i < FB_C; ++i) v[i] *= dg[l][i];
         if (l > 0) {
+            share8(v, uA + ((l - 1) & 1) * FB_A, lr, n0 + c0, FB_CL);
             tc_fence_before();
-            cluster_sync();
-            load_operand<128, FB_T>(uA, g.dZ[l], NH, row0, g.rows, 0, NH, 4);
-            cp_commit();
+            cluster_arrive();
         }
+        if (live) store_t8(v, g.dZt[l], g.rows, r, n0 + c0);
+        if (l > 0) cluster_wait();
     }
     if (!ok && tid == 0) {
         atomicExch(g.err, 1);
@@ -415,7 +441,7 @@ cudaError_t launch_mlp_train(const TrainArgs& g, cudaStream_t s)
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     if (g.rows <= 0) return cudaSuccess;
-    mlp_fb_kernel<<<dim3((unsigned)((g.rows + 127) / 128), 4), FB_T, FB_SMEM, s>>>(g);
+    mlp_fb_kernel<<<dim3((unsigned)((g.rows + 127) / 128), FB_CL), FB_T, FB_SMEM, s>>>(g);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     mlp_dw_kernel<<<DW_TILES + BIAS_ROWS / (DW_T / 32), DW_T, DW_SMEM, s>>>(g);

@@ -21,8 +21,8 @@ struct TrainArgs {
     __nv_bfloat16 *Wb[4] = {}, *Wt[4] = {};
     float *W[4] = {}, *b[4] = {}, *mW[4] = {}, *vW[4] = {}, *mb[4] = {}, *vb[4] = {};
     float *gW[4] = {}, *gb[4] = {};  // gradients out (adam = 0)
-    // work: activations and their gradients, row-major [rows x .] and transposed [. x rows]
-    __nv_bfloat16 *Xt = nullptr, *Hb[3] = {}, *Ht[3] = {}, *dY = nullptr, *dYt = nullptr, *dZ[3] = {}, *dZt[3] = {};
+    // work: activations and their gradients, transposed [. x rows]
+    __nv_bfloat16 *Xt = nullptr, *Ht[3] = {}, *dYt = nullptr, *dZt[3] = {};
     float* loss_part = nullptr;  // [ceil(rows / 128)]
     int adam = 0;                // 1: update the parameters, 0: write the gradients
     float lr = 0, b1 = 0, b2 = 0, eps = 0, c1 = 0, c2 = 0;
