@@ -137,13 +137,13 @@ ptadd_status ensure_work(MlpDev& m, int64_t rows)
 #define WA(p, n) \
     if (st == PTADD_OK) st = m_alloc(&(p), (size_t)(n));
     WA(m.X, need * 32);
-    WA(m.Xt, need * 32);
+    WA(m.Xt, need * 128);  // (tiles of 128 columns)
     for (int l = 0; l < 3; ++l) {
         WA(m.Hb[l], need * NH);
         WA(m.Ht[l], need * NH);
         WA(m.dZt[l], need * NH);
     }
-    WA(m.dYt, need * 16);
+    WA(m.dYt, need * 128);
     WA(m.Y, need * 16);
     WA(m.loss_part, need / 128);
 #undef WA

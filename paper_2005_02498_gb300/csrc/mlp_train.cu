@@ -8,20 +8,24 @@
 //
 //   mlp_fb_kernel: the whole chain.  A cluster of eight CTAs owns 128 rows; each CTA
 //   owns 32 of the 256 columns of every layer and keeps GELU'(Z) of its tile in
-//   registers from the forward to the backward pass.  A layer's columns are written into
-//   the operand buffers of all eight CTAs' shared memory, and a barrier of the cluster
-//   is the hand-over; what only the weight gradients need goes to global memory
-//   (transposed) while the others arrive, the next layer's weights are loaded while the
-//   epilogue runs.
+//   registers from the forward to the backward pass.  A layer's columns are one
+//   contiguous piece of the next layer's operand: written in the CTA's own shared
+//   memory and sent to the other seven by bulk copies that complete on the receiver's
+//   mbarrier.  What only the weight gradients need goes to global memory while the
+//   pieces are on their way, transposed and already in the operand layout; the next layer's
+//   weights are loaded while the epilogue runs.
 //   mlp_dw_kernel: every weight gradient dW = dZ^T H at once, 42 CTAs of 128 x 32
-//   outputs over all rows, with Adam and the BF16 copies in the epilogue; the bias
-//   gradients (row sums of dZ^T) in 98 more.
-// What bounds it: latency.  At 512 rows a minibatch is 32 CTAs in the first launch (27 us:
-// seven dependent products, each with a hand-over of some 5000 cycles) and 140 in the
-// second (18 us).  Two epochs of 8192 rows in minibatches of 512 take 2.22 ms (57 us a
-// minibatch with the host's shuffle, and copies of parameters and data) where one launch per
-// product, transposition, reduction and update took 8.18 ms, and four CTAs of 64 columns
-// that exchanged their activations through L2 2.65 ms.
+//   outputs over all rows, operands by bulk copies, with Adam (parameters and moments
+//   loaded while the operands arrive) and the BF16 copies in the epilogue; the bias
+//   gradients (row sums of dZ^T) in 49 more.
+// What bounds it: latency, of seven dependent products (some 5000 cycles each: 16 MMAs 2200,
+// GELU 1500, the hand-over) and of the update.  Two epochs of 8192 rows in minibatches of 512
+// take 1.74 ms (42 us a minibatch with the host's shuffle, and copies of parameters and data).
+// Before: one launch per product, transposition, reduction and update 8.18 ms; clusters of
+// four that exchanged activations through L2 2.65 ms; pieces stored into all eight CTAs by
+// st.shared::cluster and a cluster barrier (4400 cycles a hand-over), and weight gradients
+// that gathered their operands with 16-byte copies and read the moments in the epilogue
+// (35000 cycles) 2.22 ms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -38,19 +42,44 @@ constexpr int FB_N = NH / FB_CL;      // columns of a layer per CTA
 constexpr int FB_C = 8;               // columns per thread
 constexpr int FB_T = 128 * FB_N / FB_C;  // threads: 4 TMEM lane groups x FB_N / FB_C slices
 constexpr int A_CHUNK = 128 * 64 * 2; // one K-chunk of 64 of the A operand
-constexpr int FB_A = 4 * A_CHUNK;     // A: 128 rows x K 256
+constexpr int PIECE = 128 * FB_N * 2; // a CTA's columns of an A operand: 128 rows x K 32, 8-row groups 512 B apart
+constexpr int FB_A = FB_CL * PIECE;   // A: 128 rows x K 256
 constexpr int FB_B = 4 * FB_N * 64 * 2;
 constexpr int FB_SMEM = 2 * FB_A + FB_B;
-constexpr int DW_T = 256, DW_N = 32, DW_KC = 8;  // threads, columns per CTA, K-chunks of 64 in shared memory
+constexpr int DW_T = 512, DW_N = 32, DW_KC = 8;  // threads, columns per CTA, K-chunks of 64 in shared memory
+constexpr int DW_C = DW_N / (DW_T / 128);        // columns per thread
 constexpr int DW_B_CHUNK = DW_N * 64 * 2;
 constexpr int DW_SMEM = DW_KC * (A_CHUNK + DW_B_CHUNK);
+static_assert(FB_C == 8 && DW_C == 8, "a thread's columns are one core-matrix row");
 
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// generic-proxy writes to any CTA's shared memory before the tensor core's reads
-__device__ __forceinline__ void fence_async_cluster() { asm volatile("fence.proxy.async.shared::cluster;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+// Bulk copies (16-byte aligned, a multiple of 16 bytes) into shared memory, completion on
+// an mbarrier next to the destination: from global memory, and into another CTA of the cluster.
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_s2c(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t mbar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "r"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
 
 // K columns k0 .. k0 + 64 nchunk - 1 of rows row0 .. row0 + R - 1 of a K-contiguous matrix
 // into nchunk consecutive chunks in the canonical layout (tc_gemm.cuh); zeros beyond row_lim and K.
@@ -71,15 +100,15 @@ __device__ __forceinline__ void load_operand(uint32_t dst, const __nv_bfloat16* 
     }
 }
 
-// D (+)= A B^T over `steps` K-steps of 16 from the chunks at a0 and b0 (R_B rows of B).
+// D (+)= A B^T over `steps` K-steps of 16: A in blocks of a_k steps and a_bytes bytes with 8-row
+// groups a_sbo bytes apart, B in chunks of 4 steps and R_B rows.
 template <int R_B>
-__device__ __forceinline__ void issue_mma(uint32_t tmem, uint32_t a0, uint32_t b0, int steps, uint32_t idesc, bool add)
+__device__ __forceinline__ void issue_mma(uint32_t tmem, uint32_t a0, int a_k, uint32_t a_bytes, uint32_t a_sbo, uint32_t b0,
+                                          int steps, uint32_t idesc, bool add)
 {
-    for (int s = 0; s < steps; ++s) {
-        const uint32_t c = s >> 2, o = (s & 3) * 256;
-        tc_mma_f16(tmem, smem_desc(a0 + c * A_CHUNK + o, 128, 1024), smem_desc(b0 + c * (R_B * 128) + o, 128, 1024),
-                   idesc, (add || s > 0) ? 1u : 0u);
-    }
+    for (int s = 0; s < steps; ++s)
+        tc_mma_f16(tmem, smem_desc(a0 + s / a_k * a_bytes + s % a_k * 256, 128, a_sbo),
+                   smem_desc(b0 + (s >> 2) * (R_B * 128) + (s & 3) * 256, 128, 1024), idesc, (add || s > 0) ? 1u : 0u);
 }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b)
@@ -88,27 +117,24 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// FB_C values of a tile's row lr, columns c .. c + FB_C - 1, in BF16: into the A operand at
-// shared-memory address a of the CTAs 0 .. peers - 1 of the cluster
-__device__ __forceinline__ void share8(const float h[FB_C], uint32_t a, int lr, int c, int peers)
+// FB_C = 8 values of a row, consecutive columns, as one 16-byte core-matrix row
+__device__ __forceinline__ void put8(const float h[FB_C], uint8_t* dst)
 {
-    const uint32_t at = a + (uint32_t)((c >> 6) * A_CHUNK + (lr >> 3) * 1024 + ((c >> 3) & 7) * 128 + (lr & 7) * 16);
-    const uint32_t w0 = pack2(h[0], h[1]), w1 = pack2(h[2], h[3]), w2 = pack2(h[4], h[5]), w3 = pack2(h[6], h[7]);
-#pragma unroll
-    for (int p = 0; p < FB_CL; ++p) {
-        if (p >= peers) break;
-        uint32_t dst;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(at), "r"(p));
-        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w0), "r"(w1), "r"(w2), "r"(w3)
-                     : "memory");
-    }
-    fence_async_cluster();
+    *reinterpret_cast<uint4*>(dst) = make_uint4(pack2(h[0], h[1]), pack2(h[2], h[3]), pack2(h[4], h[5]), pack2(h[6], h[7]));
 }
-// ... and transposed [. x rows] for the weight gradients
-__device__ __forceinline__ void store_t8(const float h[FB_C], __nv_bfloat16* tr, int64_t rows, int64_t r, int c)
+// The transposed activations and gradients as the weight-gradient kernel's operands: tiles of
+// 128 columns c (rows of dZ^T, H^T) x 64 rows r of the minibatch (K), each in the canonical
+// layout (16 KB, contiguous); nk tiles along K.  Element index of (c, r).
+__device__ __forceinline__ int64_t t_index(int c, int64_t r, int64_t nk)
 {
+    return ((int64_t)(c >> 7) * nk + (r >> 6)) * (A_CHUNK / 2) + ((c & 127) >> 3) * 512 + ((r & 63) >> 3) * 64 +
+           (c & 7) * 8 + (r & 7);
+}
+__device__ __forceinline__ void store_t8(const float h[FB_C], __nv_bfloat16* tr, int64_t nk, int64_t r, int c)
+{
+    __nv_bfloat16* p = tr + t_index(c, r, nk);  // c is a multiple of 8
 #pragma unroll
-    for (int i = 0; i < FB_C; ++i) tr[(int64_t)(c + i) * rows + r] = __float2bfloat16_rn(h[i]);
+    for (int i = 0; i < FB_C; ++i) p[8 * i] = __float2bfloat16_rn(h[i]);
 }
 // 8 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8])
@@ -126,23 +152,28 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8])
 __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_kernel(TrainArgs g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t mbar;
+    __shared__ __align__(8) uint64_t mbar, xbar[2];
     __shared__ uint32_t tmem_base;
     __shared__ float red[4];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t row0 = (int64_t)blockIdx.x * 128;
     const int y = blockIdx.y, n0 = y * FB_N;
-    const uint32_t uA = smem_u32(smem), uB = uA + 2 * FB_A, mb = smem_u32(&mbar);
+    const uint32_t uA = smem_u32(smem), uB = uA + 2 * FB_A, mb = smem_u32(&mbar), ux = smem_u32(xbar);
     const int lr = 32 * (warp & 3) + lane;  // this thread's row of the tile
     const int c0 = FB_C * (warp >> 2);      // and first column of its slice
     const int64_t r = row0 + lr;
     const bool live = r < g.rows;
+    const int64_t nk = (g.rows + 63) / 64;
     if (warp == 0) {
         tmem_alloc(smem_u32(&tmem_base), FB_N);
         tmem_relinquish();
     }
-    if (tid == 0) mbar_init(mb, 1);
-    cluster_arrive();  // (waited for before the first write into another CTA: it has started by then)
+    if (tid == 0) {
+        mbar_init(mb, 1);
+        mbar_init(ux, 1);
+        mbar_init(ux + 8, 1);
+    }
+    cluster_arrive();  // (waited for before the first copy into another CTA: its barriers are there by then)
     // layer 1: its weights, and the inputs straight from the samples
     load_operand<FB_N, FB_T>(uB, g.Wb[0], din_p(0), n0, NH, 0, din_p(0), 1);
     cp_commit();
@@ -161,46 +192,64 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
         uint32_t w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) w[i] = pack2(v[2 * i], v[2 * i + 1]);
-        *reinterpret_cast<uint4*>(smem + (xr >> 3) * 1024 + part * 128 + (xr & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        if (y == 1 && gr < g.rows)
+        *reinterpret_cast<uint4*>(smem + (xr >> 3) * 512 + part * 128 + (xr & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (y == 1 && gr < g.rows) {
+            __nv_bfloat16* t = g.Xt + t_index(8 * part, gr, nk);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
-                g.Xt[(int64_t)(8 * part + 2 * i) * g.rows + gr] = h.x;
-                g.Xt[(int64_t)(8 * part + 2 * i + 1) * g.rows + gr] = h.y;
+                t[16 * i] = h.x;
+                t[16 * i + 8] = h.y;
             }
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base, trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
-    uint32_t phase = 0;
+    uint32_t phase = 0, xph = 0;  // xph bit b: parity of xbar[b]
     bool ok = true;
-    // the operands have been issued: wait for them, multiply, wait for the product.  A wait
-    // that gives up leaves the rest of the tile's products out; every barrier is still met.
-    auto multiply = [&](uint32_t ua, int steps, int N) {
+    // The A operand alternates between two buffers.  A CTA writes its piece of the next one in
+    // its own shared memory and copies it into the other CTAs'; `other` bytes arrive from them.
+    // No other hand-shake is needed: a piece for a buffer is sent only after a product whose
+    // operand held every CTA's previous piece, sent after that CTA's last product from
+    // this buffer; and a piece's source is written again only after products of all its readers.
+    auto send = [&](uint32_t at, uint32_t bytes, int b, int peers) {  // to the CTAs 0 .. peers - 1
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        const int p = tid - 32;  // (not the thread that issues the MMAs)
+        if (p >= 0 && p < peers && p != y) bulk_s2c(in_cta(at, p), at, bytes, in_cta(ux + 8 * b, p));
+    };
+    // The operands have been issued: wait for them (the `other` bytes of A in buffer b from other CTAs too),
+    // multiply, wait for the product.  A wait that gives up leaves the rest of the tile's
+    // products out; every barrier is still met.
+    auto multiply = [&](int b, uint32_t other, int steps, uint32_t a_sbo, int N) {
+        if (tid == 0 && other) mbar_expect_tx(ux + 8 * b, other);
         cp_wait_all();
-        fence_async_cluster();  // this thread's copies, and what its barrier wait has made visible
+        fence_async_smem();
         tc_fence_before();
         __syncthreads();
         if (tid == 0 && ok) {
-            tc_fence_after();
-            issue_mma<FB_N>(tmem, ua, uB, steps, idesc_bf16_f32(128, N), false);
-            tc_commit(mb);
+            if (!other || mbar_wait_bounded(ux + 8 * b, (xph >> b) & 1u, MBAR_WAIT_LIMIT)) {
+                tc_fence_after();
+                issue_mma<FB_N>(tmem, uA + b * FB_A, 2, PIECE, a_sbo, uB, steps, idesc_bf16_f32(128, N), false);
+                tc_commit(mb);
+            }
         }
+        if (other) xph ^= 1u << b;
         bool w = true;
         if (ok) w = mbar_wait_bounded(mb, phase, MBAR_WAIT_LIMIT);
         phase ^= 1u;
         ok = __syncthreads_and(ok && w);
         tc_fence_after();
     };
-    // The A operand alternates between two buffers (layer l reads buffer l mod 2): a CTA writes
-    // its columns of the next operand while a slower one still multiplies from this one, and
-    // a buffer's last readers have passed a barrier of the cluster before it is written again.
+    constexpr uint32_t OTHERS = (FB_CL - 1) * PIECE, DY_BYTES = 128 * 16 * 2;
+    uint8_t* piece = smem + y * PIECE + (lr >> 3) * 512 + (c0 >> 3) * 128 + (lr & 7) * 16;  // this thread's 16 bytes
     float dg[3][FB_C];  // GELU'(Z) of this thread's values
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-        multiply(uA + (l & 1) * FB_A, l == 0 ? 2 : 16, FB_N);
+        multiply(l & 1, l == 0 ? 0u : OTHERS, l == 0 ? 2 : 16, 512, FB_N);
         // the next layer's weights, while the epilogue runs
         if (l < 2)
             load_operand<FB_N, FB_T>(uB, g.Wb[l + 1], NH, n0, NH, 0, NH, 4);
@@ -215,20 +264,19 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
             e[i] = 1.0f + erff(z[i] * 0.70710678118654752f);
             h[i] = 0.5f * z[i] * e[i];
         }
+        const int nb = (l + 1) & 1;
+        put8(h, piece + nb * FB_A);
         if (l == 0) cluster_wait();
-        share8(h, uA + ((l + 1) & 1) * FB_A, lr, n0 + c0, l < 2 ? FB_CL : 1);  // (layer 4 is the first CTA's)
-        tc_fence_before();
-        cluster_arrive();
-        // what only the backward pass and the weight gradients read, while the others arrive
-        if (live) store_t8(h, g.Ht[l], g.rows, r, n0 + c0);
+        send(uA + nb * FB_A + y * PIECE, PIECE, nb, l < 2 ? FB_CL : 1);  // (layer 4 is the first CTA's)
+        // what only the backward pass and the weight gradients read, while the pieces are on their way
+        if (live) store_t8(h, g.Ht[l], nk, r, n0 + c0);
 #pragma unroll
         for (int i = 0; i < FB_C; ++i)
             dg[l][i] = 0.5f * e[i] + z[i] * expf(-0.5f * z[i] * z[i]) * 0.39894228040143268f;
-        cluster_wait();
     }
     // layer 4 (one CTA of the cluster), the loss and its gradient
     if (y == 0) {
-        multiply(uA + FB_A, 16, dout_p(3));
+        multiply(1, OTHERS, 16, 512, dout_p(3));
         load_operand<FB_N, FB_T>(uB, g.Wt[3], dout_p(3), n0, NH, 0, dout_p(3), 1);
         cp_commit();
         if (c0 < dout_p(3)) {
@@ -246,27 +294,24 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
                     d[i] = 2.0f * e * scale;
                 }
             }
-            share8(d, uA, lr, c0, FB_CL);
-            if (live) store_t8(d, g.dYt, g.rows, r, c0);
+            put8(d, smem + (lr >> 3) * 256 + (c0 >> 3) * 128 + (lr & 7) * 16);  // K 16: 8-row groups 256 B apart
+            if (live) store_t8(d, g.dYt, nk, r, c0);
             if (c0 == 0) {
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
                 if (lane == 0) red[warp] = loss;
             }
         }
-        __syncthreads();
+        send(uA, DY_BYTES, 0, FB_CL);
         if (tid == 0) g.loss_part[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
     } else {
         load_operand<FB_N, FB_T>(uB, g.Wt[3], dout_p(3), n0, NH, 0, dout_p(3), 1);
         cp_commit();
     }
-    tc_fence_before();
-    cluster_arrive();
-    cluster_wait();
     // backward: dZ_l = (dZ_{l+1} W_{l+1}) GELU'(Z_l)
 #pragma unroll
     for (int l = 2; l >= 0; --l) {
-        multiply(uA + (l & 1) * FB_A, l == 2 ? 1 : 16, FB_N);
+        multiply(l & 1, l < 2 ? OTHERS : y == 0 ? 0u : DY_BYTES, l == 2 ? 1 : 16, l == 2 ? 256 : 512, FB_N);
         if (l > 0) {
             load_operand<FB_N, FB_T>(uB, g.Wt[l], NH, n0, NH, 0, NH, 4);
             cp_commit();
@@ -276,12 +321,11 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
 #pragma unroll
         for (int i = 0; i < FB_C; ++i) v[i] *= dg[l][i];
         if (l > 0) {
-            share8(v, uA + ((l - 1) & 1) * FB_A, lr, n0 + c0, FB_CL);
-            tc_fence_before();
-            cluster_arrive();
+            const int nb = (l - 1) & 1;
+            put8(v, piece + nb * FB_A);
+            send(uA + nb * FB_A + y * PIECE, PIECE, nb, FB_CL);
         }
-        if (live) store_t8(v, g.dZt[l], g.rows, r, n0 + c0);
-        if (l > 0) cluster_wait();
+        if (live) store_t8(v, g.dZt[l], nk, r, n0 + c0);
     }
     if (!ok && tid == 0) {
         atomicExch(g.err, 1);
@@ -291,6 +335,8 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
     }
     tc_fence_before();
     __syncthreads();
+    cluster_arrive();  // no copy of the cluster is still reading this CTA's shared memory
+    cluster_wait();
     if (warp == 0) tmem_dealloc(tmem, FB_N);
 }
 
@@ -308,10 +354,11 @@ constexpr int BIAS_ROWS = 256 + 256 + 256 + 16;
 __device__ __forceinline__ void bias_rows(const TrainArgs& g, int row)
 {
     const int l = row < 768 ? row >> 8 : 3, o = row - 256 * l, lane = threadIdx.x & 31;
-    const __nv_bfloat16* p = (l == 3 ? g.dYt : g.dZt[l]) + (int64_t)o * g.rows;
+    const __nv_bfloat16* p = l == 3 ? g.dYt : g.dZt[l];
+    const int64_t nk = (g.rows + 63) / 64;
     float s = 0.0f;
 #pragma unroll 8
-    for (int64_t k = lane; k < g.rows; k += 32) s += __bfloat162float(p[k]);
+    for (int64_t k = lane; k < g.rows; k += 32) s += __bfloat162float(p[t_index(o, k, nk)]);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
     if (lane != 0) return;
@@ -326,11 +373,11 @@ __device__ __forceinline__ void bias_rows(const TrainArgs& g, int row)
 }
 
 // CTA: one 128 x 32 tile of one layer's weight gradient (tile order: layer 1's 2, 16
-// each of layers 2 and 3, layer 4's 8); the CTAs after them eight bias rows each.
+// each of layers 2 and 3, layer 4's 8); the CTAs after them sixteen bias rows each.
 __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t mbar;
+    __shared__ __align__(8) uint64_t mbar, full;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int t = blockIdx.x, l = 0;
@@ -347,12 +394,50 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
     const int m0 = 128 * (t / nt), n0 = DW_N * (t % nt);
     const __nv_bfloat16* A = l == 3 ? g.dYt : g.dZt[l];
     const __nv_bfloat16* B = l == 0 ? g.Xt : g.Ht[l - 1];
-    const uint32_t uA = smem_u32(smem), uB = uA + DW_KC * A_CHUNK, mb = smem_u32(&mbar);
+    const uint32_t uA = smem_u32(smem), uB = uA + DW_KC * A_CHUNK, mb = smem_u32(&mbar), uf = smem_u32(&full);
+    const int64_t nk = (g.rows + 63) / 64;
     if (warp == 0) {
         tmem_alloc(smem_u32(&tmem_base), DW_N);
         tmem_relinquish();
     }
-    if (tid == 0) mbar_init(mb, 1);
+    // up to DW_KC K-chunks: A's are contiguous (16 rows of layer 4's), B's are 32 of a tile's 128 rows
+    auto fetch = [&](int64_t k0, int nc) {
+        const uint32_t ab = l == 3 ? 2048u : (uint32_t)A_CHUNK;
+        const __nv_bfloat16* a = A + t_index(m0, k0, nk);
+        const __nv_bfloat16* b = B + t_index(n0, k0, nk);
+        mbar_expect_tx(uf, nc * (ab + DW_B_CHUNK));
+        if (l < 3) bulk_g2s(uA, a, nc * A_CHUNK, uf);
+        for (int c = 0; c < nc; ++c) {
+            if (l == 3) bulk_g2s(uA + c * A_CHUNK, a + c * (A_CHUNK / 2), ab, uf);
+            bulk_g2s(uB + c * DW_B_CHUNK, b + c * (A_CHUNK / 2), DW_B_CHUNK, uf);
+        }
+    };
+    const auto chunks = [&](int64_t k0) { return (int)min((int64_t)DW_KC, nk - k0 / 64); };
+    if (tid == 0) {
+        mbar_init(mb, 1);
+        mbar_init(uf, 1);
+        fetch(0, chunks(0));
+    }
+    // this thread's outputs; parameters and moments are loaded while the operands arrive
+    const int o = m0 + 32 * (warp & 3) + lane, c = n0 + DW_C * (warp >> 2);
+    const int64_t at = (int64_t)o * din_p(l) + c;
+    const bool mine = o < dout_p(l), update = mine && g.adam;
+    float p[DW_C], m[DW_C], v[DW_C];
+    auto load8 = [&](const float* src, float (&x)[DW_C]) {
+#pragma unroll
+        for (int i = 0; i < DW_C; i += 4) {
+            const float4 q = update ? *reinterpret_cast<const float4*>(src + at + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            x[i] = q.x, x[i + 1] = q.y, x[i + 2] = q.z, x[i + 3] = q.w;
+        }
+    };
+    auto store8 = [&](float* dst, const float (&x)[DW_C]) {
+#pragma unroll
+        for (int i = 0; i < DW_C; i += 4)
+            *reinterpret_cast<float4*>(dst + at + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+    };
+    load8(g.W[l], p);
+    load8(g.mW[l], m);
+    load8(g.vW[l], v);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -360,17 +445,14 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
     uint32_t phase = 0;
     bool ok = true;
     for (int64_t k0 = 0; k0 < g.rows && ok; k0 += 64 * DW_KC) {
-        const int kn = (int)min((int64_t)64 * DW_KC, g.rows - k0), nc = (kn + 63) / 64;
-        load_operand<128, DW_T>(uA, A, g.rows, m0, dout_p(l), k0, g.rows, nc);
-        load_operand<DW_N, DW_T>(uB, B, g.rows, n0, din_p(l), k0, g.rows, nc);
-        cp_commit();
-        cp_wait_all();
-        fence_async_smem();
-        __syncthreads();
         if (tid == 0) {
-            tc_fence_after();
-            issue_mma<DW_N>(tmem, uA, uB, kn / 16, idesc_bf16_f32(128, DW_N), k0 > 0);
-            tc_commit(mb);
+            if (k0 > 0) fetch(k0, chunks(k0));
+            if (mbar_wait_bounded(uf, phase, MBAR_WAIT_LIMIT)) {
+                tc_fence_after();
+                issue_mma<DW_N>(tmem, uA, 4, A_CHUNK, 1024, uB, (int)min((int64_t)64 * DW_KC, g.rows - k0) / 16,
+                                idesc_bf16_f32(128, DW_N), k0 > 0);
+                tc_commit(mb);
+            }
         }
         ok = mbar_wait_bounded(mb, phase, MBAR_WAIT_LIMIT);
         phase ^= 1u;
@@ -378,43 +460,18 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
     }
     tc_fence_after();
     if (ok) {
-        const int o = m0 + 32 * (warp & 3) + lane, c = n0 + 16 * (warp >> 2);
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(16 * (warp >> 2)), v);
-        if (o < dout_p(l)) {
-            const int64_t at = (int64_t)o * din_p(l) + c;
-            if (!g.adam) {
-                float4* out = reinterpret_cast<float4*>(g.gW[l] + at);
+        float d[DW_C];
+        tmem_ld8(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(DW_C * (warp >> 2)), d);
+        if (mine && !g.adam) store8(g.gW[l], d);
+        if (update) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) out[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-            } else {
-                float4* pw = reinterpret_cast<float4*>(g.W[l] + at);
-                float4* pm = reinterpret_cast<float4*>(g.mW[l] + at);
-                float4* pv = reinterpret_cast<float4*>(g.vW[l] + at);
-                uint32_t w[8];
+            for (int i = 0; i < DW_C; ++i) p[i] = adam_step(p[i], d[i], m[i], v[i], g);
+            store8(g.W[l], p);
+            store8(g.mW[l], m);
+            store8(g.vW[l], v);
+            put8(p, reinterpret_cast<uint8_t*>(g.Wb[l] + at));
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float4 p = pw[i], m = pm[i], s = pv[i];
-                    p.x = adam_step(p.x, v[4 * i], m.x, s.x, g);
-                    p.y = adam_step(p.y, v[4 * i + 1], m.y, s.y, g);
-                    p.z = adam_step(p.z, v[4 * i + 2], m.z, s.z, g);
-                    p.w = adam_step(p.w, v[4 * i + 3], m.w, s.w, g);
-                    pw[i] = p;
-                    pm[i] = m;
-                    pv[i] = s;
-                    w[2 * i] = pack2(p.x, p.y);
-                    w[2 * i + 1] = pack2(p.z, p.w);
-                }
-                uint4* wb = reinterpret_cast<uint4*>(g.Wb[l] + at);
-                wb[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                wb[1] = make_uint4(w[4], w[5], w[6], w[7]);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
-                    g.Wt[l][(int64_t)(c + 2 * i) * dout_p(l) + o] = h.x;
-                    g.Wt[l][(int64_t)(c + 2 * i + 1) * dout_p(l) + o] = h.y;
-                }
-            }
+            for (int i = 0; i < DW_C; ++i) g.Wt[l][(int64_t)(c + i) * dout_p(l) + o] = __float2bfloat16_rn(p[i]);
         }
     } else if (tid == 0) {
         atomicExch(g.err, 1);

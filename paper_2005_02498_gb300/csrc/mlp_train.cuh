@@ -21,7 +21,8 @@ struct TrainArgs {
     __nv_bfloat16 *Wb[4] = {}, *Wt[4] = {};
     float *W[4] = {}, *b[4] = {}, *mW[4] = {}, *vW[4] = {}, *mb[4] = {}, *vb[4] = {};
     float *gW[4] = {}, *gb[4] = {};  // gradients out (adam = 0)
-    // work: activations and their gradients, transposed [. x rows]
+    // work: activations and their gradients, transposed: [. x rows] in tiles of 128 x 64 (mlp_train.cu),
+    // both padded to full tiles
     __nv_bfloat16 *Xt = nullptr, *Ht[3] = {}, *dYt = nullptr, *dZt[3] = {};
     float* loss_part = nullptr;  // [ceil(rows / 128)]
     int adam = 0;                // 1: update the parameters, 0: write the gradients
