@@ -45,6 +45,7 @@ constexpr double SIG_SCALE = 200e6;
 struct MlpDev {
     bool ready = false;
     int64_t cap = 0;  // row capacity of the work buffers (multiple of 128)
+    float* slab = nullptr;  // parameters, first moments, second moments, gradients: SLAB floats each (W0, b0, W1, b1, ...)
     float *W[4] = {}, *b[4] = {}, *mW[4] = {}, *vW[4] = {}, *mb[4] = {}, *vb[4] = {}, *gW[4] = {}, *gb[4] = {};
     __nv_bfloat16 *Wb[4] = {}, *Wt[4] = {};
     uint8_t* stage = nullptr;  // operands laid out for the fused inference kernel, current with the parameters and maps
@@ -59,6 +60,8 @@ struct MlpDev {
     double box_lo[NIN], box_hi[NIN];
     double chol[NIN * NIN];  // lower Cholesky factor of the training covariance (standardised x)
     double d2_thr = 0.0;
+    uint8_t* io = nullptr;  // device copies of the arrays of a host call (host_block)
+    size_t io_cap = 0;
     float* d_norm = nullptr;  // device copy (FP32): xm, xs, ym, ys, box_lo, box_hi, chol^-1, d2_thr
 };
 
@@ -98,27 +101,37 @@ void free_mlp(MlpDev& m)
 {
     free_work(m);
     for (int l = 0; l < 4; ++l) {
-        void* ptrs[] = {m.W[l], m.b[l], m.mW[l], m.vW[l], m.mb[l], m.vb[l], m.gW[l], m.gb[l], m.Wb[l], m.Wt[l]};
+        void* ptrs[] = {m.Wb[l], m.Wt[l]};
         for (void* p : ptrs)
             if (p) cudaFree(p);
     }
+    if (m.slab) cudaFree(m.slab);
+    if (m.io) cudaFree(m.io);
     if (m.err) cudaFree(m.err);
     if (m.d_norm) cudaFree(m.d_norm);
     if (m.stage) cudaFree(m.stage);
     m = MlpDev{};
 }
 
+// padded floats of all parameters
+constexpr size_t layer_floats(int l) { return (size_t)dout_p(l) * din_p(l) + dout_p(l); }
+constexpr size_t SLAB = layer_floats(0) + layer_floats(1) + layer_floats(2) + layer_floats(3);
+constexpr size_t layer_offset(int l) { return l == 0 ? 0 : layer_offset(l - 1) + layer_floats(l - 1); }
+static_assert(layer_floats(0) % 4 == 0 && layer_floats(1) % 4 == 0 && layer_floats(3) % 4 == 0, "16-byte aligned arrays");
+
 ptadd_status alloc_params(MlpDev& m)
 {
-    ptadd_status st = PTADD_OK;
+    ptadd_status st = m_alloc(&m.slab, 4 * SLAB);
     for (int l = 0; l < 4 && st == PTADD_OK; ++l) {
-        const size_t nw = (size_t)dout_p(l) * din_p(l), nb = dout_p(l);
-        float** f[] = {&m.W[l], &m.mW[l], &m.vW[l], &m.gW[l]};
-        for (float** p : f)
-            if (st == PTADD_OK) st = m_alloc(p, nw);
-        float** g[] = {&m.b[l], &m.mb[l], &m.vb[l], &m.gb[l]};
-        for (float** p : g)
-            if (st == PTADD_OK) st = m_alloc(p, nb);
+        const size_t nw = (size_t)dout_p(l) * din_p(l), at = layer_offset(l);
+        m.W[l] = m.slab + at;
+        m.mW[l] = m.W[l] + SLAB;
+        m.vW[l] = m.W[l] + 2 * SLAB;
+        m.gW[l] = m.W[l] + 3 * SLAB;
+        m.b[l] = m.W[l] + nw;
+        m.mb[l] = m.b[l] + SLAB;
+        m.vb[l] = m.b[l] + 2 * SLAB;
+        m.gb[l] = m.b[l] + 3 * SLAB;
         if (st == PTADD_OK) st = m_alloc(&m.Wb[l], nw);
         if (st == PTADD_OK) st = m_alloc(&m.Wt[l], nw);
     }
@@ -127,6 +140,40 @@ ptadd_status alloc_params(MlpDev& m)
     if (st == PTADD_OK) st = m_alloc(&m.d_norm, 4 * NIN + 2 * NOUT + NIN * NIN + 1);
     return st;
 }
+
+// Device memory for the arrays of one host call: the context's block, grown to the need and
+// kept up to IO_KEEP (an allocation and its release cost 10 to 40 us and wait for the device), beyond that
+// memory of the call's own.  Every call has waited for its work when it returns, so the
+// block is free at the next one, on whatever stream.
+constexpr size_t IO_KEEP = (size_t)64 << 20;
+struct HostBlock {
+    uint8_t* p = nullptr;
+    bool own = false;
+    ~HostBlock()
+    {
+        if (own) cudaFree(p);
+    }
+};
+ptadd_status host_block(MlpDev& m, size_t bytes, HostBlock& b)
+{
+    if (bytes > IO_KEEP) {
+        const ptadd_status st = m_alloc(&b.p, bytes);
+        b.own = st == PTADD_OK;
+        return st;
+    }
+    if (bytes > m.io_cap) {
+        if (m.io) cudaFree(m.io);
+        m.io = nullptr;
+        m.io_cap = 0;
+        const ptadd_status st = m_alloc(&m.io, bytes);
+        if (st != PTADD_OK) return st;
+        m.io_cap = bytes;
+    }
+    b.p = m.io;
+    return PTADD_OK;
+}
+// offset of the next array after `at`
+size_t next_array(size_t at, size_t bytes) { return (at + bytes + 255) / 256 * 256; }
 
 ptadd_status ensure_work(MlpDev& m, int64_t rows)
 {
@@ -287,6 +334,35 @@ int64_t packed_count()
     return c;
 }
 
+// p (packed) -> the padded layout of one kind of the slab, zeros in the padding
+std::vector<float> pad(const float* p)
+{
+    std::vector<float> q(SLAB, 0.0f);
+    for (int l = 0; l < 4; ++l) {
+        float *W = q.data() + layer_offset(l), *b = W + (size_t)dout_p(l) * din_p(l);
+        for (int o = 0; o < DOUT_U[l]; ++o, p += DIN_U[l]) memcpy(W + (size_t)o * din_p(l), p, DIN_U[l] * sizeof(float));
+        memcpy(b, p, DOUT_U[l] * sizeof(float));
+        p += DOUT_U[l];
+    }
+    return q;
+}
+// kind 0 (parameters) or 3 (gradients) of the slab -> p (packed), waiting for the stream
+cudaError_t unpad(const MlpDev& m, int kind, float* p, cudaStream_t s)
+{
+    std::vector<float> q(SLAB);
+    cudaError_t e = cudaMemcpyAsync(q.data(), m.slab + kind * SLAB, SLAB * sizeof(float), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return e;
+    for (int l = 0; l < 4; ++l) {
+        const float *W = q.data() + layer_offset(l), *b = W + (size_t)dout_p(l) * din_p(l);
+        for (int o = 0; o < DOUT_U[l]; ++o, p += DIN_U[l]) memcpy(p, W + (size_t)o * din_p(l), DIN_U[l] * sizeof(float));
+        memcpy(p, b, DOUT_U[l] * sizeof(float));
+        p += DOUT_U[l];
+    }
+    return cudaSuccess;
+}
+
 ptadd_status read_loss(MlpDev& m, int64_t rows, cudaStream_t s, float* loss)
 {
     const int nb = (int)((rows + 127) / 128);
@@ -368,20 +444,9 @@ ptadd_status ptadd_mlp_set_params(ptadd_ctx* ctx, const float* p, int64_t count)
     }
     MlpDev& m = *ctx->mlp;
     cudaStream_t s = ctx->own_stream;
-    int64_t off = 0;
-    for (int l = 0; l < 4; ++l) {
-        std::vector<float> W((size_t)dout_p(l) * din_p(l), 0.0f), b(dout_p(l), 0.0f);
-        for (int o = 0; o < DOUT_U[l]; ++o)
-            for (int c = 0; c < DIN_U[l]; ++c) W[(size_t)o * din_p(l) + c] = p[off++];
-        for (int o = 0; o < DOUT_U[l]; ++o) b[o] = p[off++];
-        PTADD_CUDA(cudaMemcpyAsync(m.W[l], W.data(), W.size() * 4, cudaMemcpyHostToDevice, s));
-        PTADD_CUDA(cudaMemcpyAsync(m.b[l], b.data(), b.size() * 4, cudaMemcpyHostToDevice, s));
-        PTADD_CUDA(cudaMemsetAsync(m.mW[l], 0, W.size() * 4, s));
-        PTADD_CUDA(cudaMemsetAsync(m.vW[l], 0, W.size() * 4, s));
-        PTADD_CUDA(cudaMemsetAsync(m.mb[l], 0, b.size() * 4, s));
-        PTADD_CUDA(cudaMemsetAsync(m.vb[l], 0, b.size() * 4, s));
-        PTADD_CUDA(cudaStreamSynchronize(s));  // W, b are host temporaries
-    }
+    const std::vector<float> q = pad(p);
+    PTADD_CUDA(cudaMemcpyAsync(m.slab, q.data(), SLAB * sizeof(float), cudaMemcpyHostToDevice, s));
+    PTADD_CUDA(cudaMemsetAsync(m.slab + SLAB, 0, 2 * SLAB * sizeof(float), s));  // Adam's moments
     PTADD_CUDA(sync_bf16(m, s));
     PTADD_CUDA(stage_inference(m, s));
     PTADD_CUDA(cudaMemsetAsync(m.err, 0, sizeof(int), s));
@@ -398,16 +463,7 @@ ptadd_status ptadd_mlp_get_params(ptadd_ctx* ctx, float* p, int64_t count)
     if (!p || count != packed_count()) return marg("parameter array must hold ptadd_mlp_param_count() floats");
     MlpDev& m = *ctx->mlp;
     cudaStream_t s = ctx->own_stream;
-    int64_t off = 0;
-    for (int l = 0; l < 4; ++l) {
-        std::vector<float> W((size_t)dout_p(l) * din_p(l)), b(dout_p(l));
-        PTADD_CUDA(cudaMemcpyAsync(W.data(), m.W[l], W.size() * 4, cudaMemcpyDeviceToHost, s));
-        PTADD_CUDA(cudaMemcpyAsync(b.data(), m.b[l], b.size() * 4, cudaMemcpyDeviceToHost, s));
-        PTADD_CUDA(cudaStreamSynchronize(s));
-        for (int o = 0; o < DOUT_U[l]; ++o)
-            for (int c = 0; c < DIN_U[l]; ++c) p[off++] = W[(size_t)o * din_p(l) + c];
-        for (int o = 0; o < DOUT_U[l]; ++o) p[off++] = b[o];
-    }
+    PTADD_CUDA(unpad(m, 0, p, s));
     return PTADD_OK;
 }
 
@@ -461,18 +517,7 @@ ptadd_status ptadd_mlp_loss_grad(ptadd_ctx* ctx, int64_t n, const float* xn, con
     cudaFree(dx);
     cudaFree(dy);
     if (st != PTADD_OK) return st;
-    if (grad) {
-        int64_t off = 0;
-        for (int l = 0; l < 4; ++l) {
-            std::vector<float> W((size_t)dout_p(l) * din_p(l)), b(dout_p(l));
-            PTADD_CUDA(cudaMemcpyAsync(W.data(), m.gW[l], W.size() * 4, cudaMemcpyDeviceToHost, s));
-            PTADD_CUDA(cudaMemcpyAsync(b.data(), m.gb[l], b.size() * 4, cudaMemcpyDeviceToHost, s));
-            PTADD_CUDA(cudaStreamSynchronize(s));
-            for (int o = 0; o < DOUT_U[l]; ++o)
-                for (int c = 0; c < DIN_U[l]; ++c) grad[off++] = W[(size_t)o * din_p(l) + c];
-            for (int o = 0; o < DOUT_U[l]; ++o) grad[off++] = b[o];
-        }
-    }
+    if (grad) PTADD_CUDA(unpad(m, 3, grad, s));
     ctx->kernel_launches += launches;
     return PTADD_OK;
 }
@@ -489,30 +534,32 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
     const int64_t rows = batch;
     st = ensure_work(m, rows);
     if (st != PTADD_OK) return st;
-    float *dx = nullptr, *dy = nullptr, *dloss = nullptr;
-    int32_t* didx = nullptr;
     // per-minibatch loss partials of an epoch, kept on the device and read once
     // per epoch (reading them per minibatch would stall the stream every time)
     const int nb = (int)((rows + 127) / 128);
     const int64_t nbatches = n / batch;
-    if ((st = m_alloc(&dx, (size_t)n * NIN)) != PTADD_OK) return st;
-    if ((st = m_alloc(&dy, (size_t)n * NOUT)) != PTADD_OK || (st = m_alloc(&didx, (size_t)n)) != PTADD_OK ||
-        (st = m_alloc(&dloss, (size_t)std::max<int64_t>(1, nbatches) * nb)) != PTADD_OK) {
-        cudaFree(dx);
-        cudaFree(dy);
-        cudaFree(didx);
-        return st;
-    }
+    HostBlock block;
+    const size_t at_y = next_array(0, (size_t)n * NIN * 4), at_idx = next_array(at_y, (size_t)n * NOUT * 4);
+    const size_t at_loss = next_array(at_idx, (size_t)n * 4);
+    if ((st = host_block(m, next_array(at_loss, (size_t)nbatches * nb * 4), block)) != PTADD_OK) return st;
+    float *dx = (float*)block.p, *dy = (float*)(block.p + at_y), *dloss = (float*)(block.p + at_loss);
+    int32_t* didx = (int32_t*)(block.p + at_idx);
     std::vector<float> hloss((size_t)std::max<int64_t>(1, nbatches) * nb);
     std::vector<int32_t> perm(n);
     std::iota(perm.begin(), perm.end(), 0);
+    // Fisher-Yates shuffle of the sample order, copied once per epoch.  The next epoch's is made
+    // while the device works on this one's minibatches (110 us at 8192 samples), in a second array: the
+    // copy of the first may still be under way.
     uint64_t rs = seed;
+    auto shuffle = [&](std::vector<int32_t>& q) {
+        for (int64_t i = n - 1; i > 0; --i) std::swap(q[i], q[splitmix64(rs) % (uint64_t)(i + 1)]);
+    };
+    std::vector<int32_t> next;
+    if (epochs > 0) shuffle(perm);
     int64_t launches = 0;
     cudaError_t e = cudaMemcpyAsync(dx, xn, (size_t)n * NIN * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dy, yn, (size_t)n * NOUT * 4, cudaMemcpyHostToDevice, s);
     for (int ep = 0; ep < epochs && e == cudaSuccess && st == PTADD_OK; ++ep) {
-        // Fisher-Yates shuffle of the sample order (host), copied once per epoch
-        for (int64_t i = n - 1; i > 0; --i) std::swap(perm[i], perm[splitmix64(rs) % (uint64_t)(i + 1)]);
         e = cudaMemcpyAsync(didx, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
         double ep_loss = 0.0;
         int nbatch = 0;
@@ -530,11 +577,16 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
             launches += 2;
             ++nbatch;
         }
+        if (e == cudaSuccess && ep + 1 < epochs) {
+            next = perm;
+            shuffle(next);
+        }
         if (e == cudaSuccess && loss_per_epoch && nbatch)
             e = cudaMemcpyAsync(hloss.data(), dloss, (size_t)nbatch * nb * sizeof(float), cudaMemcpyDeviceToHost, s);
         // a synchronisation per epoch keeps the host copy of perm safe to rewrite
         cudaError_t e2 = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = e2;
+        perm.swap(next);
         if (e == cudaSuccess && loss_per_epoch) {
             // each minibatch's loss as its partials summed in order, then the epoch mean
             for (int b = 0; b < nbatch; ++b) {
@@ -554,11 +606,8 @@ ptadd_status ptadd_mlp_train(ptadd_ctx* ctx, int64_t n, const float* xn, const f
         }
     }
     if (e == cudaSuccess) e = stage_inference(m, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // predictions may run on another stream
-    cudaFree(dx);
-    cudaFree(dy);
-    cudaFree(didx);
-    cudaFree(dloss);
+    const cudaError_t e2 = cudaStreamSynchronize(s);  // predictions may run on another stream; the block is free
+    if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) {
         set_error("surrogate training: %s", cudaGetErrorString(e));
         return PTADD_ERR_CUDA;
@@ -785,30 +834,31 @@ ptadd_status ptadd_surrogate_predict(ptadd_ctx* ctx, int64_t n, const double* fe
     ptadd_status st = need_mlp(ctx);
     if (st != PTADD_OK) return st;
     if (n < 1 || !feat || !lp6) return marg("need n >= 1 and arrays");
-    double *df = nullptr, *dl = nullptr;
-    uint8_t* dr = nullptr;
-    if ((st = m_alloc(&df, (size_t)n * NIN)) != PTADD_OK) return st;
-    if ((st = m_alloc(&dl, (size_t)n * NOUT)) != PTADD_OK || (st = m_alloc(&dr, (size_t)n)) != PTADD_OK) {
-        cudaFree(df);
-        cudaFree(dl);
-        return st;
-    }
+    // features, then outputs; flags with the error word behind them come back in one copy
+    HostBlock block;
+    const size_t at_l = next_array(0, (size_t)n * NIN * 8), at_r = next_array(at_l, (size_t)n * NOUT * 8);
+    const size_t flags = ((size_t)n + 3) / 4 * 4, tail = flags + sizeof(int);
+    if ((st = host_block(*ctx->mlp, next_array(at_r, tail), block)) != PTADD_OK) return st;
+    double *df = (double*)block.p, *dl = (double*)(block.p + at_l);
+    uint8_t* dr = block.p + at_r;
+    std::vector<uint8_t> back(tail);
     cudaStream_t s = ctx->stream;
     cudaError_t e = cudaMemcpyAsync(df, feat, (size_t)n * NIN * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) st = ptadd_surrogate_predict_dev(ctx, n, df, dl, dr);
+    if (e == cudaSuccess && st == PTADD_OK)
+        e = cudaMemcpyAsync(dr + flags, ctx->mlp->err, sizeof(int), cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess && st == PTADD_OK) e = cudaMemcpyAsync(lp6, dl, (size_t)n * NOUT * 8, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && st == PTADD_OK && in_region) e = cudaMemcpyAsync(in_region, dr, (size_t)n, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(df);
-    cudaFree(dl);
-    cudaFree(dr);
+    if (e == cudaSuccess && st == PTADD_OK) e = cudaMemcpyAsync(back.data(), dr, tail, cudaMemcpyDeviceToHost, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = e2;
     if (st != PTADD_OK) return st;
     if (e != cudaSuccess) {
         set_error("surrogate predict: %s", cudaGetErrorString(e));
         return PTADD_ERR_CUDA;
     }
+    if (in_region) memcpy(in_region, back.data(), (size_t)n);
     int err = 0;
-    PTADD_CUDA(cudaMemcpy(&err, ctx->mlp->err, sizeof(int), cudaMemcpyDeviceToHost));
+    memcpy(&err, back.data() + flags, sizeof(int));
     if (err) {
         set_error("a tensor-core wait gave up");
         return PTADD_ERR_TIMEOUT;

@@ -20,7 +20,7 @@
 //   gradients (row sums of dZ^T) in 49 more.
 // What bounds it: latency, of seven dependent products (some 5000 cycles each: 16 MMAs 2200,
 // GELU 1500, the hand-over) and of the update.  Two epochs of 8192 rows in minibatches of 512
-// take 1.74 ms (42 us a minibatch with the host's shuffle, and copies of parameters and data).
+// take 1.54 ms (39 us a minibatch, and the host's first shuffle and copies).
 // Before: one launch per product, transposition, reduction and update 8.18 ms; clusters of
 // four that exchanged activations through L2 2.65 ms; pieces stored into all eight CTAs by
 // st.shared::cluster and a cluster barrier (4400 cycles a hand-over), and weight gradients
