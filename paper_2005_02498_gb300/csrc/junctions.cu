@@ -2,30 +2,32 @@
 // thermally activated breaking (Sec. 2.2), inside the burst of
 // ptadd_advance.
 //
-// Per step, between the velocity stage and the Euler stage, three kernels:
-//   junction_release_kernel (one thread per node): a held node whose break
-//     time has come lets go (and remembers the sessile loop it left); every
-//     free node that holds nothing goes on the list of nodes looking for a
-//     junction, with its best candidate reset;
-//   junction_search_kernel (one warp per (looking node, 32 sessile
-//     segments), spread over every SM): each lane tests one sessile segment
-//     of another loop (not the one the node last left) against the capture
+// Per step, between the velocity stage and the Euler stage, two kernels:
+//   junction_search_kernel (one warp per (free node, 32 sessile segments),
+//     spread over every SM): a node that holds nothing, or whose break time has
+//     come, looks for a junction: each lane tests one sessile segment of
+//     another loop (not the one the node last left) against the capture
 //     radius; the warp's lowest passing position in the sessile list goes
 //     into the node's candidate with an atomic minimum, so the lowest-index
 //     segment wins whatever the order of the warps;
-//   junction_hold_kernel (one thread per node): forms the junction found
-//     (breaking after f a), holds the velocity of a held node at 0, and
-//     reduces the largest squared speed of the free nodes, the number of
-//     held junctions and the earliest break time with 64-bit atomics on the
-//     bit patterns of non-negative doubles, whose integer order is their
-//     numeric order, so the result does not depend on the order of the
-//     atomics.
+//   junction_hold_kernel (one thread per node): a held node whose break time
+//     has come lets go (and remembers the sessile loop it left); the junction
+//     found is formed (breaking after f a) and the candidate reset; the velocity
+//     of a held node is held at 0, and the largest squared speed of the free
+//     nodes, the number of held junctions and the earliest break time are
+//     reduced with 64-bit atomics on the bit patterns of non-negative doubles,
+//     whose integer order is their numeric order, so the result does not depend
+//     on the order of the atomics.
 // after the Euler stage:
-//   junction_event_kernel (one thread): t <- t + dt, or, if some junction is
-//     held and no free node moved more than the stuck displacement, t <- the
-//     earliest break time; the frozen interval adds (the step's line length)
-//     x (the interval) to the rho sum, nothing to the Lp sum, and the
-//     interval to the time sum.
+//   junction_event_kernel (one block): the step's line length from the groups'
+//     parts, then t <- t + dt, or, if some junction is held and no free node
+//     moved more than the stuck displacement, t <- the earliest break time; the
+//     frozen interval adds (the step's line length) x (the interval) to the rho
+//     sum, nothing to the Lp sum, and the interval to the time sum.
+// A step of a small network is a chain of launches (about 4 us each), so the release
+// has no launch of its own (the search decides it again for its node) and the
+// length is summed where it is used: 8 launches a step became 6.  1280 nodes, 64 of them
+// free: 103 -> 97 us a step, pair stage and all.
 // Distances and times are formed with explicit round-to-nearest operations,
 // no contraction, so a decision depends only on the positions and the clock.
 //
@@ -67,15 +69,26 @@ struct DevJunctions {
     double* clock = nullptr;     // [0] DD time, [1] time jumped (s)
     unsigned long long* red = nullptr;  // [0] max v^2 bits, [1] min break bits, [2] held,
                                         // [3] formed, [4] broken, [5] jumps
-    int64_t n_free = 0;          // unpinned nodes (the most that can look in one step)
-    int32_t* look = nullptr;     // nodes looking for a junction this step (any order)
-    unsigned* look_n = nullptr;  // their number (reset by the event kernel)
-    int32_t* found = nullptr;    // per node: lowest passing position in sess, or INT32_MAX
+    int64_t n_free = 0;           // unpinned nodes
+    int32_t* free_nodes = nullptr;  // their list
+    int32_t* found = nullptr;     // per node: lowest passing position in sess, or INT32_MAX (so between steps)
 };
 
 namespace {
 
 constexpr int JT = 256;
+// One warp: the step's line length from slot 13 of the groups' parts, in the order of
+// step_finish_kernel: 16 partial sums, then those in order.
+__device__ __forceinline__ double step_length(int n_groups, const double* __restrict__ part)
+{
+    const int y = threadIdx.x & 15;
+    double s = 0.0;
+    for (int g = y; g < n_groups; g += 16) s += part[16 * (int64_t)g + 13];
+    double t = __shfl_sync(0xffffffffu, s, 0);
+    for (int k = 1; k < 16; ++k) t += __shfl_sync(0xffffffffu, s, k);
+    return t;
+}
+
 constexpr unsigned long long INF_BITS = 0x7FF0000000000000ull;
 
 __device__ __forceinline__ uint64_t splitmix64_mix(uint64_t z)
@@ -110,45 +123,27 @@ __device__ __forceinline__ double seg_dist2(double x, double y, double z, const 
     return __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
 }
 
-__global__ void __launch_bounds__(JT) junction_release_kernel(
-    int64_t n, const int32_t* __restrict__ loop_of, const uint8_t* __restrict__ pinned, int32_t* __restrict__ jseg,
-    int32_t* __restrict__ jlast, const double* __restrict__ jbrk, const double* __restrict__ clock,
-    int32_t* __restrict__ look, unsigned* __restrict__ look_n, int32_t* __restrict__ found,
-    unsigned long long* __restrict__ red)
-{
-    const int64_t p = blockIdx.x * (int64_t)JT + threadIdx.x;
-    if (p >= n || pinned[p]) return;
-    int32_t js = jseg[p];
-    if (js >= 0 && jbrk[p] <= clock[0]) {
-        jlast[p] = loop_of[js];
-        jseg[p] = -1;
-        js = -1;
-        atomicAdd(&red[4], 1ull);
-    }
-    if (js < 0) {
-        found[p] = INT32_MAX;
-        look[atomicAdd(look_n, 1u)] = (int32_t)p;
-    }
-}
-
-// Block: JSW warps; warp w of block (x, y) tests look[x JSW + w] against the
+// Block: JSW warps; warp w of block (x, y) tests free node x JSW + w against the
 // sessile positions 32 y .. 32 y + 31, one per lane.
 constexpr int JSW = 8;
 
 __global__ void __launch_bounds__(32 * JSW) junction_search_kernel(
     int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt, const int32_t* __restrict__ loop_of,
-    const int32_t* __restrict__ sess, int64_t n_sess, const int32_t* __restrict__ jlast,
-    const int32_t* __restrict__ look, const unsigned* __restrict__ look_n, int32_t* __restrict__ found, double rc2)
+    const int32_t* __restrict__ sess, int64_t n_sess, const int32_t* __restrict__ jseg,
+    const int32_t* __restrict__ jlast, const double* __restrict__ jbrk, const double* __restrict__ clock,
+    const int32_t* __restrict__ free_nodes, int64_t n_free, int32_t* __restrict__ found, double rc2)
 {
-    const int li = blockIdx.x * JSW + (threadIdx.x >> 5);
-    if (li >= (int)*look_n) return;  // warp-uniform
+    const int64_t li = (int64_t)blockIdx.x * JSW + (threadIdx.x >> 5);
+    if (li >= n_free) return;  // warp-uniform, as the next one
     const int64_t k = (int64_t)blockIdx.y * 32 + (threadIdx.x & 31);
-    const int32_t p = look[li];
+    const int32_t p = free_nodes[li], js = jseg[p];
+    if (js >= 0 && !(jbrk[p] <= clock[0])) return;  // held
+    const int32_t left = js >= 0 ? loop_of[js] : jlast[p];
     bool hit = false;
     if (k < n_sess) {
         const int32_t sg = sess[k];
         const int32_t sl = loop_of[sg];
-        if (sl != loop_of[p] && sl != jlast[p]) {
+        if (sl != loop_of[p] && sl != left) {
             const int32_t e = nxt[sg];
             const double sp[6] = {pos[sg], pos[n + sg], pos[2 * n + sg], pos[e], pos[n + e], pos[2 * n + e]};
             hit = seg_dist2(pos[p], pos[n + p], pos[2 * n + p], sp) < rc2;
@@ -160,16 +155,25 @@ __global__ void __launch_bounds__(32 * JSW) junction_search_kernel(
 }
 
 __global__ void __launch_bounds__(JT) junction_hold_kernel(
-    int64_t n, const uint8_t* __restrict__ pinned, double* __restrict__ vel, const int32_t* __restrict__ sess,
-    int32_t* __restrict__ jseg, int32_t* __restrict__ jcount, double* __restrict__ jbrk,
-    const int32_t* __restrict__ found, const double* __restrict__ clock, double a, uint64_t seed,
+    int64_t n, const int32_t* __restrict__ loop_of, const uint8_t* __restrict__ pinned, double* __restrict__ vel,
+    const int32_t* __restrict__ sess, int32_t* __restrict__ jseg, int32_t* __restrict__ jlast,
+    int32_t* __restrict__ jcount, double* __restrict__ jbrk, int32_t* __restrict__ found,
+    const double* __restrict__ clock, double a, uint64_t seed,
     unsigned long long* __restrict__ red)
 {
     const int64_t p = blockIdx.x * (int64_t)JT + threadIdx.x;
     if (p >= n || pinned[p]) return;
     int32_t js = jseg[p];
-    if (js < 0 && found[p] != INT32_MAX) {
-        js = sess[found[p]];
+    if (js >= 0 && jbrk[p] <= clock[0]) {
+        jlast[p] = loop_of[js];
+        jseg[p] = -1;
+        js = -1;
+        atomicAdd(&red[4], 1ull);
+    }
+    const int32_t at = found[p];
+    if (js < 0 && at != INT32_MAX) {
+        found[p] = INT32_MAX;
+        js = sess[at];
         const int32_t k = jcount[p];
         jbrk[p] = __dadd_rn(clock[0], __dmul_rn(a, break_fraction(seed, p, k)));
         jcount[p] = k + 1;
@@ -188,12 +192,15 @@ __global__ void __launch_bounds__(JT) junction_hold_kernel(
     }
 }
 
-__global__ void junction_event_kernel(double* __restrict__ clock, unsigned long long* __restrict__ red,
-                                      double* __restrict__ acc, unsigned* __restrict__ look_n, double dt_s,
-                                      double dt_hat, double stuck_hat, double time_scale)
+__global__ void __launch_bounds__(32) junction_event_kernel(int n_groups, const double* __restrict__ part,
+                                                            double* __restrict__ clock,
+                                                            unsigned long long* __restrict__ red,
+                                                            double* __restrict__ acc, double dt_s, double dt_hat,
+                                                            double stuck_hat, double time_scale)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    *look_n = 0u;
+    const double len = step_length(n_groups, part);
+    if (threadIdx.x != 0) return;
+    acc[11] = len;
     const double t1 = __dadd_rn(clock[0], dt_s);
     const double vmax = sqrt(__longlong_as_double((long long)red[0]));
     const double tmin = __longlong_as_double((long long)red[1]);
@@ -202,7 +209,7 @@ __global__ void junction_event_kernel(double* __restrict__ clock, unsigned long 
         const double jump = __dsub_rn(tmin, t1);
         clock[1] = __dadd_rn(clock[1], jump);
         const double jh = jump * time_scale;
-        acc[9] = fma(acc[11], jh, acc[9]);
+        acc[9] = fma(len, jh, acc[9]);
         acc[12] += jh;
         red[5] += 1;
         tn = tmin;
@@ -374,7 +381,7 @@ void junctions_free(ptadd_ctx* ctx)
 {
     DevJunctions* j = ctx->junc;
     if (!j) return;
-    void* ptrs[] = {j->sess, j->seg, j->last, j->count, j->brk, j->clock, j->red, j->look, j->look_n, j->found};
+    void* ptrs[] = {j->sess, j->seg, j->last, j->count, j->brk, j->clock, j->red, j->free_nodes, j->found};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete j;
@@ -387,26 +394,24 @@ cudaError_t launch_junction_update(ptadd_ctx* ctx, cudaStream_t st)
     const DevNetwork& net = ctx->net;
     const int64_t n = net.n_nodes;
     const unsigned nb = (unsigned)((n + JT - 1) / JT);
-    junction_release_kernel<<<nb, JT, 0, st>>>(n, net.loop_of, net.pinned, j->seg, j->last, j->brk, j->clock,
-                                               j->look, j->look_n, j->found, j->red);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (j->n_free > 0 && j->n_sess > 0) {
         const dim3 grid((unsigned)((j->n_free + JSW - 1) / JSW), (unsigned)((j->n_sess + 31) / 32));
         junction_search_kernel<<<grid, 32 * JSW, 0, st>>>(n, net.pos[net.cur], net.nxt, net.loop_of, j->sess,
-                                                          j->n_sess, j->last, j->look, j->look_n, j->found, j->rc2);
+                                                          j->n_sess, j->seg, j->last, j->brk, j->clock, j->free_nodes,
+                                                          j->n_free, j->found, j->rc2);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    junction_hold_kernel<<<nb, JT, 0, st>>>(n, net.pinned, net.vel, j->sess, j->seg, j->count, j->brk, j->found,
-                                            j->clock, j->a, j->seed, j->red);
+    junction_hold_kernel<<<nb, JT, 0, st>>>(n, net.loop_of, net.pinned, net.vel, j->sess, j->seg, j->last, j->count,
+                                            j->brk, j->found, j->clock, j->a, j->seed, j->red);
     return cudaGetLastError();
 }
 
 cudaError_t launch_junction_event(ptadd_ctx* ctx, double dt_s, double dt_hat, cudaStream_t st)
 {
     DevJunctions* j = ctx->junc;
-    junction_event_kernel<<<1, 32, 0, st>>>(j->clock, j->red, ctx->net.acc, j->look_n, dt_s, dt_hat, j->stuck_hat,
+    junction_event_kernel<<<1, 32, 0, st>>>(ctx->net.n_grp, ctx->net.part, j->clock, j->red, ctx->net.acc, dt_s, dt_hat, j->stuck_hat,
                                              ctx->mat.mu / ctx->mat.B);
     return cudaGetLastError();
 }
@@ -661,11 +666,10 @@ extern "C" ptadd_status ptadd_set_junctions(ptadd_ctx* ctx, const ptadd_junction
     std::vector<int32_t> nxt(n);
     PTADD_CUDA(cudaMemcpy(pin.data(), net.pinned, n, cudaMemcpyDeviceToHost));
     PTADD_CUDA(cudaMemcpy(nxt.data(), net.nxt, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
-    std::vector<int32_t> sess;
-    int64_t n_free = 0;
+    std::vector<int32_t> sess, free_nodes;
     for (int64_t i = 0; i < n; ++i) {
         if (pin[i] && pin[nxt[i]]) sess.push_back((int32_t)i);
-        n_free += pin[i] ? 0 : 1;
+        if (!pin[i]) free_nodes.push_back((int32_t)i);
     }
 
     DevJunctions* j = new DevJunctions;
@@ -676,7 +680,7 @@ extern "C" ptadd_status ptadd_set_junctions(ptadd_ctx* ctx, const ptadd_junction
     j->stuck_hat = p->stuck_disp / l;
     j->seed = p->seed;
     j->n_sess = (int64_t)sess.size();
-    j->n_free = n_free;
+    j->n_free = (int64_t)free_nodes.size();
     cudaError_t e = cudaSuccess;
     auto al = [&](void** q, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(q, bytes > 0 ? bytes : 1);
@@ -688,8 +692,7 @@ extern "C" ptadd_status ptadd_set_junctions(ptadd_ctx* ctx, const ptadd_junction
     al((void**)&j->brk, n * sizeof(double));
     al((void**)&j->clock, 2 * sizeof(double));
     al((void**)&j->red, 6 * sizeof(unsigned long long));
-    al((void**)&j->look, (size_t)n * sizeof(int32_t));
-    al((void**)&j->look_n, sizeof(unsigned));
+    al((void**)&j->free_nodes, free_nodes.size() * sizeof(int32_t));
     al((void**)&j->found, (size_t)n * sizeof(int32_t));
     if (e != cudaSuccess) {
         set_error("ptadd_set_junctions: cudaMalloc failed: %s", cudaGetErrorString(e));
@@ -708,7 +711,10 @@ extern "C" ptadd_status ptadd_set_junctions(ptadd_ctx* ctx, const ptadd_junction
     chk(cudaMemset(j->brk, 0, n * sizeof(double)));
     chk(cudaMemcpy(j->clock, clock0, sizeof(clock0), cudaMemcpyHostToDevice));
     chk(cudaMemcpy(j->red, red0, sizeof(red0), cudaMemcpyHostToDevice));
-    chk(cudaMemset(j->look_n, 0, sizeof(unsigned)));
+    if (!free_nodes.empty())
+        chk(cudaMemcpy(j->free_nodes, free_nodes.data(), free_nodes.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    const std::vector<int32_t> none((size_t)n, INT32_MAX);
+    chk(cudaMemcpy(j->found, none.data(), none.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     if (e != cudaSuccess) {  // leave junctions off rather than half set
         set_error("ptadd_set_junctions: initialising the junction state failed: %s", cudaGetErrorString(e));
         junctions_free(ctx);

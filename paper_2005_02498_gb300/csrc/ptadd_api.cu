@@ -451,9 +451,8 @@ ptadd_status ptadd_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, double Lp
             PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob, s, &ctx->kernel_launches));
             PTADD_CUDA(launch_junction_update(ctx, s));
             PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, move, s, &ctx->kernel_launches));
-            PTADD_CUDA(launch_step_finish(1, net.real_grp, net.part, true, net.acc, s));
             PTADD_CUDA(launch_junction_event(ctx, dt, dt_hat, s));
-            ctx->kernel_launches += 5;
+            ctx->kernel_launches += 3;
         } else {
             PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob | move, s, &ctx->kernel_launches));
         }
