@@ -13,6 +13,7 @@
 #include <atomic>
 #include <math.h>
 
+#include "chain.cuh"
 #include "pair_tile.cuh"
 #include "ptadd_internal.cuh"
 #include "seg_field.cuh"
@@ -86,6 +87,8 @@ __global__ void __launch_bounds__(32, DF_MINB) pair_fp64_kernel(TileArgs base, i
                                                                 Consts c)
 {
     __shared__ DFSmem sm;
+    chain_wait();
+    chain_next();
     TileArgs a = base;
     a.t_begin = (int64_t)blockIdx.x * 32;
     a.t_count = min((int64_t)32, n_tgt - a.t_begin);
@@ -100,6 +103,8 @@ __global__ void __launch_bounds__(MIX_TPB, MIX_MINB) pair_mixed_kernel(TileArgs 
                                                              Consts c, float near2)
 {
     __shared__ MixSmem<MIX_TILE, MIX_TPB> sm;
+    chain_wait();
+    chain_next();
     TileArgs a = base;
     a.t_begin = (int64_t)blockIdx.x * MIX_TPB;
     a.t_count = min((int64_t)MIX_TPB, n_tgt - a.t_begin);
@@ -185,7 +190,7 @@ int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
 }
 
 cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt, int chunks, int precision,
-                        const Consts& c, const double sh[6], cudaStream_t st)
+                        const Consts& c, const double sh[6], cudaStream_t st, bool chained)
 {
     const int64_t n = net.n_nodes;
     if (n_tgt == 0 || n == 0) return cudaSuccess;
@@ -208,10 +213,12 @@ cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt
     if (precision == (int)PTADD_MIXED) {
         dim3 grid((unsigned)((n_tgt + MIX_TPB - 1) / MIX_TPB), (unsigned)chunks);
         const float near2 = (float)((NEAR_FACTOR * NEAR_FACTOR + 1.0) * c.a2);
+        if (chained) return launch_chained(pair_mixed_kernel, grid, MIX_TPB, 0, st, a, n_tgt, chunk_len, c, near2);
         pair_mixed_kernel<<<grid, MIX_TPB, 0, st>>>(a, n_tgt, chunk_len, c, near2);
         return cudaGetLastError();
     }
     const dim3 grid((unsigned)((n_tgt + 31) / 32), (unsigned)chunks);
+    if (chained) return launch_chained(pair_fp64_kernel, grid, 32, 0, st, a, n_tgt, chunk_len, c);
     pair_fp64_kernel<<<grid, 32, 0, st>>>(a, n_tgt, chunk_len, c);
     return cudaGetLastError();
 }

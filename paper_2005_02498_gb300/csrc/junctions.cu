@@ -27,7 +27,7 @@
 // A step of a small network is a chain of launches (about 4 us each), so the release
 // has no launch of its own (the search decides it again for its node) and the
 // length is summed where it is used: 8 launches a step became 6.  1280 nodes, 64 of them
-// free: 103 -> 97 us a step, pair stage and all.
+// free: 103 -> 97 us a step, pair stage and all (84 as a chain, chain.cuh).
 // Distances and times are formed with explicit round-to-nearest operations,
 // no contraction, so a decision depends only on the positions and the clock.
 //
@@ -51,6 +51,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "chain.cuh"
 #include "ptadd_internal.cuh"
 
 namespace ptadd {
@@ -128,11 +129,13 @@ __device__ __forceinline__ double seg_dist2(double x, double y, double z, const 
 constexpr int JSW = 8;
 
 __global__ void __launch_bounds__(32 * JSW) junction_search_kernel(
-    int64_t n, const double* __restrict__ pos, const int32_t* __restrict__ nxt, const int32_t* __restrict__ loop_of,
-    const int32_t* __restrict__ sess, int64_t n_sess, const int32_t* __restrict__ jseg,
-    const int32_t* __restrict__ jlast, const double* __restrict__ jbrk, const double* __restrict__ clock,
-    const int32_t* __restrict__ free_nodes, int64_t n_free, int32_t* __restrict__ found, double rc2)
+    int64_t n, const double* pos, const int32_t* __restrict__ nxt, const int32_t* __restrict__ loop_of,
+    const int32_t* __restrict__ sess, int64_t n_sess, const int32_t* jseg,
+    const int32_t* jlast, const double* jbrk, const double* clock,
+    const int32_t* __restrict__ free_nodes, int64_t n_free, int32_t* found, double rc2)
 {
+    chain_wait();
+    chain_next();
     const int64_t li = (int64_t)blockIdx.x * JSW + (threadIdx.x >> 5);
     if (li >= n_free) return;  // warp-uniform, as the next one
     const int64_t k = (int64_t)blockIdx.y * 32 + (threadIdx.x & 31);
@@ -155,12 +158,14 @@ __global__ void __launch_bounds__(32 * JSW) junction_search_kernel(
 }
 
 __global__ void __launch_bounds__(JT) junction_hold_kernel(
-    int64_t n, const int32_t* __restrict__ loop_of, const uint8_t* __restrict__ pinned, double* __restrict__ vel,
-    const int32_t* __restrict__ sess, int32_t* __restrict__ jseg, int32_t* __restrict__ jlast,
-    int32_t* __restrict__ jcount, double* __restrict__ jbrk, int32_t* __restrict__ found,
-    const double* __restrict__ clock, double a, uint64_t seed,
-    unsigned long long* __restrict__ red)
+    int64_t n, const int32_t* __restrict__ loop_of, const uint8_t* __restrict__ pinned, double* vel,
+    const int32_t* __restrict__ sess, int32_t* jseg, int32_t* jlast,
+    int32_t* jcount, double* jbrk, int32_t* found,
+    const double* clock, double a, uint64_t seed,
+    unsigned long long* red)
 {
+    chain_wait();
+    chain_next();
     const int64_t p = blockIdx.x * (int64_t)JT + threadIdx.x;
     if (p >= n || pinned[p]) return;
     int32_t js = jseg[p];
@@ -192,12 +197,14 @@ __global__ void __launch_bounds__(JT) junction_hold_kernel(
     }
 }
 
-__global__ void __launch_bounds__(32) junction_event_kernel(int n_groups, const double* __restrict__ part,
-                                                            double* __restrict__ clock,
-                                                            unsigned long long* __restrict__ red,
-                                                            double* __restrict__ acc, double dt_s, double dt_hat,
+__global__ void __launch_bounds__(32) junction_event_kernel(int n_groups, const double* part,
+                                                            double* clock,
+                                                            unsigned long long* red,
+                                                            double* acc, double dt_s, double dt_hat,
                                                             double stuck_hat, double time_scale)
 {
+    chain_wait();
+    chain_next();
     const double len = step_length(n_groups, part);
     if (threadIdx.x != 0) return;
     acc[11] = len;
@@ -397,23 +404,20 @@ cudaError_t launch_junction_update(ptadd_ctx* ctx, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     if (j->n_free > 0 && j->n_sess > 0) {
         const dim3 grid((unsigned)((j->n_free + JSW - 1) / JSW), (unsigned)((j->n_sess + 31) / 32));
-        junction_search_kernel<<<grid, 32 * JSW, 0, st>>>(n, net.pos[net.cur], net.nxt, net.loop_of, j->sess,
-                                                          j->n_sess, j->seg, j->last, j->brk, j->clock, j->free_nodes,
-                                                          j->n_free, j->found, j->rc2);
-        e = cudaGetLastError();
+        e = launch_chained(junction_search_kernel, grid, 32 * JSW, 0, st, n, net.pos[net.cur], net.nxt, net.loop_of,
+                           j->sess, j->n_sess, j->seg, j->last, j->brk, j->clock, j->free_nodes, j->n_free, j->found,
+                           j->rc2);
         if (e != cudaSuccess) return e;
     }
-    junction_hold_kernel<<<nb, JT, 0, st>>>(n, net.loop_of, net.pinned, net.vel, j->sess, j->seg, j->last, j->count,
-                                            j->brk, j->found, j->clock, j->a, j->seed, j->red);
-    return cudaGetLastError();
+    return launch_chained(junction_hold_kernel, nb, JT, 0, st, n, net.loop_of, net.pinned, net.vel, j->sess, j->seg,
+                          j->last, j->count, j->brk, j->found, j->clock, j->a, j->seed, j->red);
 }
 
 cudaError_t launch_junction_event(ptadd_ctx* ctx, double dt_s, double dt_hat, cudaStream_t st)
 {
     DevJunctions* j = ctx->junc;
-    junction_event_kernel<<<1, 32, 0, st>>>(ctx->net.n_grp, ctx->net.part, j->clock, j->red, ctx->net.acc, dt_s, dt_hat, j->stuck_hat,
-                                             ctx->mat.mu / ctx->mat.B);
-    return cudaGetLastError();
+    return launch_chained(junction_event_kernel, 1, 32, 0, st, ctx->net.n_grp, ctx->net.part, j->clock, j->red,
+                          ctx->net.acc, dt_s, dt_hat, j->stuck_hat, ctx->mat.mu / ctx->mat.B);
 }
 
 // blob part: seg, last, count (int32 x n each), brk (n doubles), clock[2], red[3..5]

@@ -20,7 +20,7 @@
 //   gradients (row sums of dZ^T) in 49 more.
 // What bounds it: latency, of seven dependent products (some 5000 cycles each: 16 MMAs 2200,
 // GELU 1500, the hand-over) and of the update.  Two epochs of 8192 rows in minibatches of 512
-// take 1.54 ms (39 us a minibatch, and the host's first shuffle and copies).
+// take 1.37 ms (34 us a minibatch, and the host's first shuffle and copies).
 // Before: one launch per product, transposition, reduction and update 8.18 ms; clusters of
 // four that exchanged activations through L2 2.65 ms; pieces stored into all eight CTAs by
 // st.shared::cluster and a cluster barrier (4400 cycles a hand-over), and weight gradients
@@ -29,6 +29,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "mlp_train.cuh"
 #include "tc_gemm.cuh"
 
@@ -174,6 +175,8 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
         mbar_init(ux + 8, 1);
     }
     cluster_arrive();  // (waited for before the first copy into another CTA: its barriers are there by then)
+    chain_wait();
+    chain_next();
     // layer 1: its weights, and the inputs straight from the samples
     load_operand<FB_N, FB_T>(uB, g.Wb[0], din_p(0), n0, NH, 0, din_p(0), 1);
     cp_commit();
@@ -382,6 +385,7 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int t = blockIdx.x, l = 0;
     if (t >= DW_TILES) {
+        chain_wait();
         bias_rows(g, (t - DW_TILES) * (DW_T / 32) + warp);
         return;
     }
@@ -412,6 +416,8 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
             bulk_g2s(uB + c * DW_B_CHUNK, b + c * (A_CHUNK / 2), DW_B_CHUNK, uf);
         }
     };
+    chain_wait();
+    chain_next();
     const auto chunks = [&](int64_t k0) { return (int)min((int64_t)DW_KC, nk - k0 / 64); };
     if (tid == 0) {
         mbar_init(mb, 1);
@@ -498,11 +504,9 @@ cudaError_t launch_mlp_train(const TrainArgs& g, cudaStream_t s)
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     if (g.rows <= 0) return cudaSuccess;
-    mlp_fb_kernel<<<dim3((unsigned)((g.rows + 127) / 128), FB_CL), FB_T, FB_SMEM, s>>>(g);
-    e = cudaGetLastError();
+    e = launch_chained(mlp_fb_kernel, dim3((unsigned)((g.rows + 127) / 128), FB_CL), FB_T, FB_SMEM, s, g);
     if (e != cudaSuccess) return e;
-    mlp_dw_kernel<<<DW_TILES + BIAS_ROWS / (DW_T / 32), DW_T, DW_SMEM, s>>>(g);
-    return cudaGetLastError();
+    return launch_chained(mlp_dw_kernel, DW_TILES + BIAS_ROWS / (DW_T / 32), DW_T, DW_SMEM, s, g);
 }
 
 }  // namespace ptadd

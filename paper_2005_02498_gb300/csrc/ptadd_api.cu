@@ -325,7 +325,8 @@ static ptadd_status take_events(ptadd_ctx* ctx, std::pair<cudaEvent_t, cudaEvent
 }
 
 // the pair stage for a target list, timed if asked; the records are up to date
-static ptadd_status eval_pairs(ptadd_ctx* ctx, const Consts& c, const int32_t* tgt, int64_t n_tgt, int chunks)
+static ptadd_status eval_pairs(ptadd_ctx* ctx, const Consts& c, const int32_t* tgt, int64_t n_tgt, int chunks,
+                               bool chained = false)
 {
     DevNetwork& net = ctx->net;
     if (n_tgt == 0) return PTADD_OK;
@@ -338,7 +339,7 @@ static ptadd_status eval_pairs(ptadd_ctx* ctx, const Consts& c, const int32_t* t
         if (st != PTADD_OK) return st;
         PTADD_CUDA(cudaEventRecord(ev.first, s));
     }
-    PTADD_CUDA(launch_pair(net, tgt, n_tgt, chunks, (int)ctx->prec, c, sh, s));
+    PTADD_CUDA(launch_pair(net, tgt, n_tgt, chunks, (int)ctx->prec, c, sh, s, chained));
     if (ev.first) {
         PTADD_CUDA(cudaEventRecord(ev.second, s));
         ctx->ev_open.push_back(ev);
@@ -443,18 +444,19 @@ ptadd_status ptadd_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, double Lp
         ctx->kernel_launches += 1;
     }
     for (int64_t it = 0; it < n_steps; ++it) {
-        ptadd_status st = eval_pairs(ctx, c, net.tgt_burst, net.n_tgt_burst, chunks);
+        ptadd_status st = eval_pairs(ctx, c, net.tgt_burst, net.n_tgt_burst, chunks, true);
         if (st != PTADD_OK) return st;
         const StepArgs a = step_args(ctx, c, chunks, dt_hat);
         const int move = STEP_EULER | (it + 1 < n_steps ? STEP_PREP : 0);
         if (ctx->junc) {
-            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob, s, &ctx->kernel_launches));
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob, s, &ctx->kernel_launches, true));
             PTADD_CUDA(launch_junction_update(ctx, s));
-            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, move, s, &ctx->kernel_launches));
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, move, s, &ctx->kernel_launches, true));
             PTADD_CUDA(launch_junction_event(ctx, dt, dt_hat, s));
             ctx->kernel_launches += 3;
         } else {
-            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob | move, s, &ctx->kernel_launches));
+            PTADD_CUDA(launch_step(a, net.n_grp, net.grp_whole, chunks, mob | move, s, &ctx->kernel_launches,
+                                   true));
         }
         net.cur = 1 - net.cur;
     }

@@ -122,7 +122,7 @@ inline Consts make_consts(double a_internal, double nu)
 cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& c, cudaStream_t st);
 // pair stage: writes fpart[chunk][6][seg] for the listed targets
 cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt, int chunks,
-                        int precision, const Consts& c, const double sig_hat[6], cudaStream_t st);
+                        int precision, const Consts& c, const double sig_hat[6], cudaStream_t st, bool chained = false);
 // sources per FP64 work item for a number of one-warp target tiles
 int64_t fp64_chunk_len(int64_t tiles, int64_t n_src);
 int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision);

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "pair_tile.cuh"
 #include "step.cuh"
 
@@ -148,6 +149,11 @@ __global__ void __launch_bounds__(32 * ROWS) step_kernel(StepArgs a, int what)
 {
     __shared__ double red[ROWS][3][33];
     const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
+    chain_wait();
+    // In the middle of a step the next kernel's few blocks may be set up beside these.  At its end the
+    // next kernel is the pair stage, sized to fill the SMs once: set up around these blocks it
+    // would be spread unevenly (512 segments: 78 against 75 us a step), so it comes as they end.
+    if (!(what & STEP_EULER)) chain_next();
     const int64_t lo = a.grp_off[blockIdx.x], hi = a.grp_off[blockIdx.x + 1], n = a.n;
     if (a.counter && blockIdx.x == 0 && tid == 0) *a.counter = 0u;
     if (what & STEP_NODE) {
@@ -317,16 +323,20 @@ StepGroups step_groups(int64_t n_loops, const int64_t* loop_off, int32_t R, cons
 }
 
 cudaError_t launch_step(const StepArgs& a, int n_groups, bool whole, int max_chunks, int what, cudaStream_t st,
-                        int64_t* launches)
+                        int64_t* launches, bool chained)
 {
     if (a.n == 0) return cudaSuccess;
     auto go = [&](int w) {
         // 16 rows where few blocks sum many chunks (a small network); 4 leave room for more blocks
-        if (max_chunks > 16 && n_groups <= 304)
+        *launches += 1;
+        const bool tall = max_chunks > 16 && n_groups <= 304;
+        if (chained)
+            return tall ? launch_chained(step_kernel<16>, n_groups, 512, 0, st, a, w)
+                        : launch_chained(step_kernel<4>, n_groups, 128, 0, st, a, w);
+        if (tall)
             step_kernel<16><<<n_groups, 512, 0, st>>>(a, w);
         else
             step_kernel<4><<<n_groups, 128, 0, st>>>(a, w);
-        *launches += 1;
         return cudaGetLastError();
     };
     if (whole) return go(what);

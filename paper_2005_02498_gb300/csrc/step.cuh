@@ -64,9 +64,10 @@ struct StepGroups {
 StepGroups step_groups(int64_t n_loops, const int64_t* loop_off, int32_t R, const int64_t* node_off);
 
 // The phases of one step that follow the pair stage; junctions (which act on
-// the velocities) split it with `what`.  Adds the number of launches.
+// the velocities) split it with `what`.  Adds the number of launches.  chained: in a chain of
+// kernels that all wait for the one before (chain.cuh).
 cudaError_t launch_step(const StepArgs& a, int n_groups, bool whole, int max_chunks, int what, cudaStream_t st,
-                        int64_t* launches);
+                        int64_t* launches, bool chained = false);
 // Nodal forces of every node (F, SoA [3 n]) from the pair stage's parts; 0 at pinned nodes of a batch,
 // whose segments may not have been evaluated.
 cudaError_t launch_node_force(const StepArgs& a, double* force, cudaStream_t st);
