@@ -526,6 +526,8 @@ def run_ours(args):
     if fp64_cmp:
         peak64 = sms * 2 * 2 * max_mhz * 1e6
         fp64_cmp["pair_kernel_frac_of_fp64_peak"] = fp64_cmp["pair_kernel_tflops"] * 1e12 / peak64
+        fp64_cmp["arithmetic"] = ("far pairs in double-float on the FP32 pipe, close pairs in FP64: the fraction of "
+                                  "the FP64 peak can exceed 1")
         x64 = recorded_capture("fp64").get("executed_fp64_flops_per_pair")
         if x64 is not None:
             t64 = fp64_cmp["pair_kernel_tflops"] * x64 / FLOPS_PER_PAIR
