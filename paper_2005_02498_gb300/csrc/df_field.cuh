@@ -23,9 +23,14 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
+#include <string.h>
 
 namespace ptadd {
 
+// Everything here also compiles for the host, where the arithmetic is checked against
+// 80-bit numbers pair by pair; DF_HOST_SEED stands in for the error of the hardware's
+// reciprocal approximations there.
 #define DF_FN __host__ __device__ __forceinline__
 #ifndef DF_HOST_SEED
 #define DF_HOST_SEED(y) (y)
@@ -83,6 +88,19 @@ DF_FN float2 p_rcp_seed(float2 x)
 #endif
 }
 
+// Gauss-Legendre rule on [0,1]: the textbook 4-point abscissae z and
+// weights W on [-1,1] mapped by xi = (1 + z)/2, w = W/2.
+DF_FN constexpr double gl4_xi(int qp)
+{
+    constexpr double z0 = 0.8611363115940526, z1 = 0.3399810435848563;
+    return qp == 0 ? 0.5 * (1.0 - z0) : qp == 1 ? 0.5 * (1.0 - z1) : qp == 2 ? 0.5 * (1.0 + z1) : 0.5 * (1.0 + z0);
+}
+DF_FN constexpr double gl4_w(int qp)
+{
+    constexpr double W0 = 0.3478548451374538, W1 = 0.6521451548625461;
+    return (qp == 0 || qp == 3) ? 0.5 * W0 : 0.5 * W1;
+}
+
 // ---------------------------------------------------------- double-float
 struct DF2 {
     float2 h, l;
@@ -91,7 +109,53 @@ struct DF1 {  // one value
     float h, l;
 };
 
-// the two FP32 parts of an FP64 value
+// An FP64 value to the nearest FP32 one (0 below FP32's normal range, which the
+// callers can leave out; infinite above it; NaN stays NaN) on the integer pipe: the hardware
+// conversions and every FP64 operation run on the 1/64-rate FP64 pipe.
+DF_FN float df_round(double x)
+{
+#ifdef __CUDA_ARCH__
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+#else
+    uint64_t u;
+    memcpy(&u, &x, sizeof(u));
+    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+#endif
+    const uint32_t e = (hi >> 20) & 0x7FFu, v = (hi << 3) | (lo >> 29);
+    // exponents 897 .. 1150: the field moved by 896, plus the first dropped bit, carrying upwards
+    uint32_t f = v - (896u << 23) + ((lo >> 28) & 1u);
+    if (e < 897u) f = 0u;
+    if (e > 1150u) f = e == 0x7FFu && (v & 0x7FFFFFu) ? 0x7FFFFFFFu : 0x7F800000u;
+    f |= hi & 0x80000000u;
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(f);
+#else
+    float r;
+    memcpy(&r, &f, sizeof(r));
+    return r;
+#endif
+}
+// FP32 to FP64, exact for 0, the normal range and infinities (2^128 stands for these)
+DF_FN double df_widen(float x)
+{
+#ifdef __CUDA_ARCH__
+    const uint32_t u = __float_as_uint(x);
+    const uint32_t hi = (u & 0x80000000u) | ((((u >> 23) & 0xFFu) + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
+    return x != 0.0f ? __hiloint2double((int)hi, (int)(u << 29)) : 0.0;
+#else
+    return (double)x;
+#endif
+}
+// The two FP32 parts of an FP64 value, each to nearest: h + l is within 2^-48 |x| of x, on
+// either side alike.  (Truncated parts, one integer operation fewer each, were within 2^-46 and
+// always short, and their error in the frames of the sources added up along a loop:
+// far-field part of Lp of two loops of 21 segments 3.5e-15 against 1.2e-14.)
+DF_FN DF1 df_split(double x)
+{
+    const float h = df_round(x);
+    return DF1{h, df_round(x - df_widen(h))};
+}
+// the same for a constant
 DF_FN constexpr DF1 df_from(double x) { return DF1{(float)x, (float)(x - (double)(float)x)}; }
 DF_FN DF2 df_all(DF1 a) { return DF2{p_all(a.h), p_all(a.l)}; }
 DF_FN DF2 df_pair2(DF1 a, DF1 b) { return DF2{make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
@@ -293,6 +357,25 @@ DF_FN void df_field(const DFGeo& G, const DFPair& P, DF2 L, DF2 LL, DF2 bt, DF2 
     Sn = df_fma(df_neg(cq), be, df_fma(df_neg(Gx), G.al, df_mul(cR, G.be)));
     St = df_fma(df_neg(ga), in3, df_fma(df_neg(C1), nqb, df_mul(rA0, Mt)));
     cb = df_mul(df_neg(ga), B0);
+}
+
+// The nodal force parts sum_q w_q (s_q x D) of a group of sources, from the group's sums s and
+// b (the coefficient along b') at the Gauss points of chain ch (its two points are the
+// lanes): F = start node's 3, end node's 3; chain 0 sets them, chain 1 adds.
+DF_FN void df_group_forces(int ch, DF2 s[3], DF2 b, const DF2 bt[3], const DF1 D[3], DF2 F[6])
+{
+    const double x0 = gl4_xi(2 * ch), x1 = gl4_xi(2 * ch + 1), w0 = gl4_w(2 * ch), w1 = gl4_w(2 * ch + 1);
+    const DF2 we = df_pair2(df_from(w0 * x0), df_from(w1 * x1));
+    const DF2 ws = df_pair2(df_from(w0 * (1.0 - x0)), df_from(w1 * (1.0 - x1)));
+#pragma unroll
+    for (int e = 0; e < 3; ++e) s[e] = df_fma(b, bt[e], s[e]);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int i = (e + 1) % 3, j = (e + 2) % 3;
+        const DF2 f = df_fma(s[i], df_all(D[j]), df_neg(df_mul(s[j], df_all(D[i]))));
+        F[e] = ch ? df_fma(f, ws, F[e]) : df_mul(f, ws);
+        F[3 + e] = ch ? df_fma(f, we, F[3 + e]) : df_mul(f, we);
+    }
 }
 
 }  // namespace ptadd

@@ -43,16 +43,6 @@ struct TileArgs {
 // ---------------------------------------------------------------- records
 constexpr double DF_NEAR = 32.0;      // in core widths a
 constexpr double DF_FAR = 2097152.0;  // 2^21 units
-// The two FP32 parts of an FP64 value in FP32's normal range (or 0), the first
-// by truncation: the mantissa fields are moved on the integer pipe, because the
-// hardware conversions and every FP64 operation run on the 1/64-rate FP64 pipe
-// (one FP64 subtraction is left; h + l differs from x by less than 2^-46 |x|).
-__device__ __forceinline__ DF1 df_split(double x)
-{
-    const float h = d2f_seed0(x);
-    return DF1{h, d2f_seed0(x - f2d_seed0(h))};
-}
-
 // The three FP32 parts of x - o (o an integer), scaled; NaN outside their range.
 __device__ __forceinline__ void df_parts(double x, double o, float* f)
 {
@@ -295,12 +285,12 @@ __device__ __forceinline__ void near_shift(uint2* q, int cnt)
 // FP64 results.  A (Gauss point, source) pair nearer than DF_NEAR a, or than
 // 1/16 of either segment's length, is evaluated in FP64 (near_flush); every
 // other pair in double-float arithmetic on the FP32 pipe (df_field.cuh).  The
-// rounding error of the nodal forces comes from the close pairs, whose field
-// is the largest and whose geometry cancels: against an 80-bit reference the
-// relative error of the forces (1e-12 to 3e-12 over the loop networks of 42 to
-// 1500 nodes) is the same to 0.1 % with every pair in FP64 and with the pairs
-// beyond 20 a, 32 a, 64 a or 256 a in double-float; a pair beyond 32 a errs by
-// 2e-14 of itself in the median.
+// rounding error of the nodal forces comes from the close pairs, whose field is the
+// largest and whose geometry cancels.  Against an 80-bit reference, 25 loop networks of 42
+// to 2125 segments: the forces are 1.7e-12 to 1.3e-11 off (2-norm), within 1e-4 of
+// that error what they are with every pair in FP64; Lp of the free networks 6e-14 to 1.2e-11,
+// within 0.6 % of that error.  The far pairs' share of the forces' error is 5e-15 to
+// 1.4e-14; a far pair is 2e-14 of itself off in the median, 2e-13 in 99 of 100.
 //
 // The sums over DF_GROUP tiles' sources are kept in double-float per Gauss
 // point (in shared memory: they are touched once per source, and the two
@@ -481,25 +471,16 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
                 DF2 s[3];
                 const DF2 b = {q[6 * 32], q[7 * 32]};
 #pragma unroll
-                for (int e = 0; e < 3; ++e) s[e] = df_fma(b, bt[e], DF2{q[2 * e * 32], q[(2 * e + 1) * 32]});
+                for (int e = 0; e < 3; ++e) s[e] = DF2{q[2 * e * 32], q[(2 * e + 1) * 32]};
 #pragma unroll
                 for (int k = 0; k < 8; ++k) q[k * 32] = p_all(0.0f);
-                const DF2 we = df_pair2(df_from(gl4_w(2 * ch) * gl4_xi(2 * ch)), df_from(gl4_w(2 * ch + 1) * gl4_xi(2 * ch + 1)));
-                const DF2 ws = df_pair2(df_from(gl4_w(2 * ch) * (1.0 - gl4_xi(2 * ch))),
-                                        df_from(gl4_w(2 * ch + 1) * (1.0 - gl4_xi(2 * ch + 1))));
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    const int i = (e + 1) % 3, j = (e + 2) % 3;
-                    const DF2 f = df_fma(s[i], df_all(D[j]), df_neg(df_mul(s[j], df_all(D[i]))));
-                    F[e] = ch ? df_fma(f, ws, F[e]) : df_mul(f, ws);
-                    F[3 + e] = ch ? df_fma(f, we, F[3 + e]) : df_mul(f, we);
-                }
+                df_group_forces(ch, s, b, bt, D, F);
             }
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const DF2 t = df_norm(df_add(df_lane_x(F[k]), df_lane_y(F[k])));
                 double* acc = sm.facc + k * 32 + threadIdx.x;
-                acc[0] = fma(c.c2, f2d_seed0(t.h.x) + f2d_seed0(t.l.x), acc[0]);
+                acc[0] = fma(c.c2, df_widen(t.h.x) + df_widen(t.l.x), acc[0]);
             }
         }
     }

@@ -70,13 +70,6 @@ __device__ __forceinline__ double f2d_seed(float y)
     const unsigned hi = (u & 0x80000000u) | ((((u >> 23) & 0xFFu) + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
     return __hiloint2double((int)hi, (int)(u << 29));
 }
-// The same for any finite value: 0 below FP32's normal range (an underflow
-// the callers can leave out), saturated above it.
-__device__ __forceinline__ float d2f_seed0(double x)
-{
-    return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) > 896u ? d2f_seed(x) : 0.0f;
-}
-__device__ __forceinline__ double f2d_seed0(float y) { return y != 0.0f ? f2d_seed(y) : 0.0; }
 __device__ __forceinline__ double rcp_nr(double x)
 {
     const double y = f2d_seed(rcp_approx(d2f_seed(x)));
@@ -198,19 +191,6 @@ __device__ __forceinline__ void seg_sigma_b(double R0x, double R0y, double R0z, 
     s[0] = fma(sb, bt[0], s[0]);
     s[1] = fma(sb, bt[1], s[1]);
     s[2] = fma(sb, bt[2], s[2]);
-}
-
-// Gauss-Legendre rule on [0,1]: the textbook 4-point abscissae z and
-// weights W on [-1,1] mapped by xi = (1 + z)/2, w = W/2.
-__host__ __device__ __forceinline__ constexpr double gl4_xi(int qp)
-{
-    constexpr double z0 = 0.8611363115940526, z1 = 0.3399810435848563;
-    return qp == 0 ? 0.5 * (1.0 - z0) : qp == 1 ? 0.5 * (1.0 - z1) : qp == 2 ? 0.5 * (1.0 + z1) : 0.5 * (1.0 + z0);
-}
-__host__ __device__ __forceinline__ constexpr double gl4_w(int qp)
-{
-    constexpr double W0 = 0.3478548451374538, W1 = 0.6521451548625461;
-    return (qp == 0 || qp == 3) ? 0.5 * W0 : 0.5 * W1;
 }
 
 }  // namespace ptadd
