@@ -34,6 +34,7 @@
 #include <string>
 #include <vector>
 
+#include "chunk_rule.cuh"
 #include "pair_tile.cuh"
 #include "ptadd_internal.cuh"
 #include "step.cuh"
@@ -69,7 +70,7 @@ struct DevBatch {
     float* srcdf = nullptr;
     double *fpart = nullptr, *vel = nullptr, *force = nullptr, *part = nullptr, *acc = nullptr;
     std::vector<double> last_LV;  // [3R] (1/|B|) sum L vbar of the last burst, time-averaged, SI
-    int64_t fpart_cap = 0;  // doubles
+    int64_t fpart_cap = 0;  // doubles, for the work lists so far
     // per realisation (device)
     int64_t* d_node_off = nullptr;
     int64_t* d_fp_base = nullptr;
@@ -256,20 +257,22 @@ ptadd_status bd_alloc(T** p, size_t count)
     return PTADD_OK;
 }
 
-// Targets per tile and sources per chunk of the work list.  FP64 tiles are one
-// warp's and, where the configured chunks would not fill the GPU, cut finer by
-// the rule of the single network (for the mean realisation), unless the
-// configuration was set by hand.
-void item_shape(const DevBatch& B, const BatchConfig& cfg, int prec, int64_t& tpb, int64_t& chunk_len)
+// Targets per tile and sources per chunk of every realisation.  FP64 tiles are one
+// warp's and their chunks at most the configured ones, cut finer by the rule of chunk_rule.cuh,
+// unless the configuration was set by hand.
+void item_shape(const DevBatch& B, const BatchConfig& cfg, int prec, int64_t& tpb, std::vector<int64_t>& len)
 {
     tpb = cfg.tpb;
-    chunk_len = cfg.chunk_len;
-    if (prec != (int)PTADD_MIXED && !cfg.by_hand) {
-        tpb = 32;
-        int64_t tiles = 0;
-        for (int r = 0; r < B.R; ++r) tiles += (B.tgt_off[r + 1] - B.tgt_off[r] + 31) / 32;
-        chunk_len = std::min(chunk_len, fp64_chunk_len(tiles, B.n / B.R));
+    len.assign(B.R, cfg.chunk_len);
+    if (prec == (int)PTADD_MIXED || cfg.by_hand) return;
+    tpb = 32;
+    int64_t tiles = 0;
+    std::vector<int64_t> n(B.R);
+    for (int r = 0; r < B.R; ++r) {
+        tiles += (B.tgt_off[r + 1] - B.tgt_off[r] + 31) / 32;
+        n[r] = B.node_off[r + 1] - B.node_off[r];
     }
+    len = batch_chunk_lens(fp64_slots(), tiles, n, cfg.chunk_len);
 }
 
 // Work list and fpart layout for a configuration and precision; returns the
@@ -277,15 +280,16 @@ void item_shape(const DevBatch& B, const BatchConfig& cfg, int prec, int64_t& tp
 int64_t build_items(const DevBatch& B, const BatchConfig& cfg, int prec, std::vector<WorkItem>& items,
                     std::vector<int64_t>& fp_base, std::vector<int32_t>& chunks)
 {
-    int64_t tpb, chunk_len;
-    item_shape(B, cfg, prec, tpb, chunk_len);
+    int64_t tpb;
+    std::vector<int64_t> len;
+    item_shape(B, cfg, prec, tpb, len);
     items.clear();
     fp_base.assign(B.R, 0);
     chunks.assign(B.R, 0);
     int64_t off = 0;
     for (int r = 0; r < B.R; ++r) {
         const int64_t s0 = B.node_off[r], nr = B.node_off[r + 1] - s0;
-        const int32_t nch = (int32_t)((nr + chunk_len - 1) / chunk_len);
+        const int32_t nch = (int32_t)((nr + len[r] - 1) / len[r]);
         chunks[r] = nch;
         fp_base[r] = off;
         off += (int64_t)nch * 6 * nr;
@@ -297,8 +301,8 @@ int64_t build_items(const DevBatch& B, const BatchConfig& cfg, int prec, std::ve
                 w.chunk = ch;
                 w.t_begin = (int32_t)tb;
                 w.t_count = (int32_t)std::min<int64_t>(tpb, t1 - tb);
-                w.js = (int32_t)(s0 + (int64_t)ch * chunk_len);
-                w.je = (int32_t)std::min<int64_t>(s0 + nr, w.js + chunk_len);
+                w.js = (int32_t)(s0 + (int64_t)ch * len[r]);
+                w.je = (int32_t)std::min<int64_t>(s0 + nr, w.js + len[r]);
                 items.push_back(w);
             }
     }
@@ -315,9 +319,19 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStr
     std::vector<int64_t> fp_base;
     std::vector<int32_t> chunks;
     const int64_t need = build_items(B, cfg, prec, items, fp_base, chunks);
+    // (every call of the batch has waited for its work, so its buffers are free)
+    if (B.graph) {
+        cudaGraphExecDestroy(B.graph);
+        B.graph = nullptr;
+    }
+    B.items_prec = -1;  // until the new list is complete
     if (need > B.fpart_cap) {
-        set_error("internal: partial-force buffer too small for the configuration");
-        return PTADD_ERR_STATE;
+        if (B.fpart) cudaFree(B.fpart);
+        B.fpart = nullptr;
+        B.fpart_cap = 0;
+        const ptadd_status sp = bd_alloc(&B.fpart, need);
+        if (sp != PTADD_OK) return sp;
+        B.fpart_cap = need;
     }
     if (B.d_items) cudaFree(B.d_items);
     B.d_items = nullptr;
@@ -331,10 +345,6 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStr
     B.cfg = cfg;
     B.items_prec = prec;
     B.max_chunks = *std::max_element(chunks.begin(), chunks.end());
-    if (B.graph) {
-        cudaGraphExecDestroy(B.graph);
-        B.graph = nullptr;
-    }
     return PTADD_OK;
 }
 
@@ -672,17 +682,6 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     B.tgt_off[R] = (int64_t)tgt.size();
     B.n_tgt = (int64_t)tgt.size();
 
-    // partial-force capacity: the smallest chunk length any configuration uses
-    {
-        std::vector<WorkItem> items;
-        std::vector<int64_t> fb;
-        std::vector<int32_t> ch;
-        BatchConfig smallest;
-        smallest.chunk_len = 1024;
-        for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
-            B.fpart_cap = std::max(B.fpart_cap, build_items(B, smallest, prec, items, fb, ch));
-    }
-
     ptadd_status st = PTADD_OK;
 #define BALLOC(p, cnt) \
     if (st == PTADD_OK) st = bd_alloc(&(p), (size_t)(cnt));
@@ -699,7 +698,6 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     BALLOC(B.src, SRC_STRIDE * n);
     BALLOC(B.src32, SRC32_STRIDE * n);
     BALLOC(B.srcdf, SRCDF_STRIDE * n);
-    BALLOC(B.fpart, B.fpart_cap);
     BALLOC(B.vel, 3 * n);
     BALLOC(B.force, 3 * n);
     BALLOC(B.part, 16 * (int64_t)B.n_grp);
@@ -755,7 +753,9 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     PTADD_CUDA(cudaStreamSynchronize(s));
     BatchConfig cfg;
     B.tuned = tune_lookup(tune_path(nullptr), tune_key(ctx, B, (int)ctx->prec), cfg) ? 1 : 0;
-    return apply_config(B, cfg, (int)ctx->prec, s);
+    st = apply_config(B, cfg, (int)ctx->prec, s);
+    if (st != PTADD_OK) batch_free(ctx);
+    return st;
 }
 
 ptadd_status ptadd_batch_set_stress(ptadd_ctx* ctx, const double* sig6)

@@ -14,6 +14,7 @@
 #include <math.h>
 
 #include "chain.cuh"
+#include "chunk_rule.cuh"
 #include "pair_tile.cuh"
 #include "ptadd_internal.cuh"
 #include "seg_field.cuh"
@@ -137,32 +138,17 @@ static void pair_slots(int& sms, int& per_sm)
     }
 }
 
-int64_t fp64_chunk_len(int64_t tiles, int64_t n_src)
+int64_t fp64_slots()
 {
-    // Resident one-warp tiles: 16 per SM.  Up to 16 waves of them in chunks of
-    // at least 64 sources (about one group of sums), so that the tail costs a few
-    // per cent.  Where that leaves fewer than four waves the chunks shrink to 4
-    // sources, and below that while a wave is not full: a lone warp spends 3.3 us
-    // on a source, and the FP64 near pairs of a loop (5 us per 32) sit in few
-    // chunks.  Measured, us per launch: 42 segments 29 / 22 in chunks of 3 / 1; 512
-    // segments 93 / 68 / 56 / 65 in chunks of 16 / 8 / 4 / 2; 64 targets x 1280
-    // sources 101 / 57 / 35 in 20 / 10 / 5; 1041 x 1485 244 / 220 / 190 in 23 / 12 /
-    // 6; 8192 segments 6330 / 6163 / 6155 in 128 / 64 / 32.
     int sms, per_sm;
     pair_slots(sms, per_sm);
-    const int64_t slots = (int64_t)sms * per_sm;
-    tiles = std::max<int64_t>(tiles, 1);
-    int64_t ch = std::min((16 * slots + tiles - 1) / tiles, n_src / 64);
-    if (tiles * ch < 4 * slots) ch = std::min((4 * slots + tiles - 1) / tiles, n_src / 4);
-    if (tiles * ch < slots) ch = std::min(slots / tiles, n_src);
-    ch = std::max<int64_t>(ch, 1);
-    return (n_src + ch - 1) / ch;
+    return (int64_t)sms * per_sm;
 }
 
 int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision)
 {
     if (precision != (int)PTADD_MIXED) {
-        int64_t len = fp64_chunk_len((n_tgt + 31) / 32, n_src);
+        int64_t len = chunk_len_rule(fp64_slots(), (n_tgt + 31) / 32, n_src);
         len = std::max(len, (n_src + max_chunks - 1) / max_chunks);
         return (int)((n_src + len - 1) / len);
     }

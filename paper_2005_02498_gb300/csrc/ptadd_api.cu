@@ -10,12 +10,11 @@
 #include <new>
 #include <vector>
 
+#include "chunk_rule.cuh"
 #include "ptadd_internal.cuh"
 #include "step.cuh"
 
 namespace ptadd {
-
-constexpr int FPART_MAX_CHUNKS = 512;
 
 static thread_local char g_err[1024] = "no error";
 
@@ -212,7 +211,7 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     net.max_chunks = 1;
     for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
         for (int64_t nt : {net.n_tgt_burst, n})
-            net.max_chunks = std::max(net.max_chunks, choose_chunks(nt, n, FPART_MAX_CHUNKS, prec));
+            net.max_chunks = std::max(net.max_chunks, choose_chunks(nt, n, network_max_chunks(n), prec));
     const int64_t node_off[2] = {0, n};
     const StepGroups grp = step_groups(n_loops, loop_off, 1, node_off);
     net.n_grp = grp.real_grp[1];
