@@ -221,8 +221,11 @@ typedef struct {
     int64_t n_nodes, n_loops, n_targets;
     int64_t pairs_per_step; /* sum over realisations of n_targets_r * n_nodes_r */
     int64_t work_items;     /* tiles of the persistent pair kernel per step    */
-    int32_t tile_targets;   /* autotuned: targets per tile (threads per block)  */
-    int32_t chunk_sources;  /* autotuned: sources per work item                 */
+    int32_t tile_targets;   /* targets per tile (threads per block): mixed and  *
+                             * set by hand as configured, else 32 (FP64)        */
+    int32_t chunk_sources;  /* sources per work item: mixed and set by hand as  *
+                             * configured, else the largest that FP64's rule    *
+                             * gives a realisation                              */
     int32_t tuned;          /* 1 if the configuration came from the tuner/cache */
 } ptadd_batch_info;
 
@@ -259,7 +262,10 @@ ptadd_status ptadd_batch_get_info(ptadd_ctx* ctx, ptadd_batch_info* info);
  * append it to a JSON-lines cache (cache_path, else $PTADD_TUNE_CACHE, else
  * $HOME/.cache/ptadd_tune.jsonl) keyed by GPU, library version, a hash of
  * the sources the library was built from, precision and the batch's size
- * class.  A cached entry is reused unless force != 0.
+ * class.  A cached entry is reused unless force != 0.  FP64 cuts its own
+ * tiles and chunks, of at most the candidate's length: candidates that come
+ * to the same work list are timed once, and the default (64 x 2048) is kept
+ * where all do.
  * ptadd_batch_set applies a cached entry when one exists. */
 ptadd_status ptadd_batch_autotune(ptadd_ctx* ctx, const char* cache_path, int force);
 /* Set the pair-stage configuration by hand: tile_targets (threads per

@@ -94,6 +94,7 @@ struct DevBatch {
     std::vector<double> volume, origin, sh;
     BatchConfig cfg;
     int items_prec = -1;  // precision the work list was built for
+    int tile = 0, chunk = 0;  // its targets per tile, and its longest chunk (mixed, by hand: the configured length)
     int tuned = 0;
     // graph of two steps
     cudaGraphExec_t graph = nullptr;
@@ -343,6 +344,11 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStr
     PTADD_CUDA(cudaStreamSynchronize(s));
     B.n_items = (int)items.size();
     B.cfg = cfg;
+    int64_t tpb;
+    std::vector<int64_t> len;
+    item_shape(B, cfg, prec, tpb, len);
+    B.tile = (int)tpb;
+    B.chunk = (int)*std::max_element(len.begin(), len.end());
     B.items_prec = prec;
     B.max_chunks = *std::max_element(chunks.begin(), chunks.end());
     return PTADD_OK;
@@ -1058,8 +1064,8 @@ ptadd_status ptadd_batch_get_info(ptadd_ctx* ctx, ptadd_batch_info* info)
     info->n_targets = B.n_tgt;
     info->pairs_per_step = B.pairs;
     info->work_items = B.n_items;
-    info->tile_targets = B.cfg.tpb;
-    info->chunk_sources = B.cfg.chunk_len;
+    info->tile_targets = B.tile;
+    info->chunk_sources = B.chunk;
     info->tuned = B.tuned;
     return PTADD_OK;
 }
@@ -1086,16 +1092,23 @@ ptadd_status ptadd_batch_autotune(ptadd_ctx* ctx, const char* cache_path, int fo
     cudaEvent_t e0, e1;
     PTADD_CUDA(cudaEventCreate(&e0));
     PTADD_CUDA(cudaEventCreate(&e1));
+    // the default first: of candidates that come out equal (FP64 chunks are mostly set by the rule of
+    // chunk_rule.cuh) one is timed, and the default is kept if all do
     const int tpbs[2] = {64, 128};
-    const int chunks[3] = {1024, 2048, 4096};
+    const int chunks[3] = {2048, 1024, 4096};
     BatchConfig best;
     double best_ms = INFINITY;
     ptadd_status st = PTADD_OK;
+    std::vector<std::pair<int64_t, std::vector<int64_t>>> seen;
     for (int ti = 0; ti < 2 && st == PTADD_OK; ++ti)
         for (int ci = 0; ci < 3 && st == PTADD_OK; ++ci) {
             BatchConfig cfg;
             cfg.tpb = tpbs[ti];
             cfg.chunk_len = chunks[ci];
+            std::pair<int64_t, std::vector<int64_t>> shape;
+            item_shape(B, cfg, prec, shape.first, shape.second);
+            if (std::find(seen.begin(), seen.end(), shape) != seen.end()) continue;
+            seen.push_back(shape);
             st = apply_config(B, cfg, prec, s);
             if (st != PTADD_OK) break;
             float best_rep = INFINITY;
