@@ -115,7 +115,10 @@ void ptadd_destroy(ptadd_ctx* ctx);
 /* Message of the last failed call on this host thread (never NULL). */
 const char* ptadd_last_error(void);
 
-/* Switch precision of later bursts. */
+/* Switch precision of later bursts.  With a network loaded, the buffers that
+ * only the new precision uses are made here if it has not been used yet;
+ * PTADD_ERR_NOMEM leaves the precision as it was.  A batch makes its own at the
+ * next batch call. */
 ptadd_status ptadd_set_precision(ptadd_ctx* ctx, ptadd_precision prec);
 
 /* Run the context's work on a caller-owned stream (a cudaStream_t passed as
@@ -449,7 +452,8 @@ ptadd_status ptadd_dissipation_projection_dev(int64_t n_points, const double* T6
  * the context across networks and batches (ptadd_forces_noalloc computes
  * forces only).  PTADD_ERR_ARG for another value; PTADD_ERR_STATE for
  * consistent = 1 while junctions are on, single or batched (they hold nodes
- * at rest by the lumped form's rule). */
+ * at rest by the lumped form's rule).  The system's rows (80 bytes per node)
+ * are made when they are first needed: PTADD_ERR_NOMEM leaves the setting. */
 ptadd_status ptadd_set_mobility(ptadd_ctx* ctx, int32_t consistent);
 
 /* Junctions and thermally activated breaking in the burst (Sec. 2.2).

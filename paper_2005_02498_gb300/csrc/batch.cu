@@ -106,7 +106,7 @@ struct DevBatch {
     bool graph_cons = false;
     bool consistent = false;          // consistent mobility in this burst (the context's setting)
     int64_t* d_loop_off = nullptr;    // [n_loops + 1] (consistent mobility)
-    double* cm_scratch = nullptr;     // [10 n] (consistent mobility)
+    double* cm_scratch = nullptr;     // [10 n] (consistent mobility; made at its first burst)
     DevBatchJunctions* junc = nullptr;  // junctions (ptadd_batch_set_junctions), NULL: off
     double dt_s = 0.0;                  // the step of the current burst, s (the junction clock)
     double time_scale = 0.0;            // mu / B: internal time -> s
@@ -333,6 +333,10 @@ ptadd_status apply_config(DevBatch& B, const BatchConfig& cfg, int prec, cudaStr
         const ptadd_status sp = bd_alloc(&B.fpart, need);
         if (sp != PTADD_OK) return sp;
         B.fpart_cap = need;
+    }
+    if (prec != (int)PTADD_MIXED && !B.srcdf) {  // (192 bytes per node that only FP64 reads)
+        const ptadd_status sp = bd_alloc(&B.srcdf, SRCDF_STRIDE * B.n);
+        if (sp != PTADD_OK) return sp;
     }
     if (B.d_items) cudaFree(B.d_items);
     B.d_items = nullptr;
@@ -703,7 +707,6 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     BALLOC(B.pinned, n);
     BALLOC(B.src, SRC_STRIDE * n);
     BALLOC(B.src32, SRC32_STRIDE * n);
-    BALLOC(B.srcdf, SRCDF_STRIDE * n);
     BALLOC(B.vel, 3 * n);
     BALLOC(B.force, 3 * n);
     BALLOC(B.part, 16 * (int64_t)B.n_grp);
@@ -721,7 +724,6 @@ ptadd_status ptadd_batch_set(ptadd_ctx* ctx, int32_t R, const int64_t* node_off,
     BALLOC(B.staging, 3 * n);
     BALLOC(B.k64, 4);
     BALLOC(B.d_loop_off, n_loops + 1);
-    BALLOC(B.cm_scratch, 10 * n);
 #undef BALLOC
     if (st != PTADD_OK) {
         free_batch(B);
@@ -807,6 +809,10 @@ ptadd_status ptadd_batch_advance(ptadd_ctx* ctx, int64_t n_steps, double dt, dou
     B.time_scale = ctx->mat.mu / ctx->mat.B;
     const bool junc = B.junc != nullptr;
     B.consistent = ctx->consistent_mass;
+    if (B.consistent && !B.cm_scratch) {
+        const ptadd_status st = bd_alloc(&B.cm_scratch, 10 * B.n);
+        if (st != PTADD_OK) return st;
+    }
     int64_t left = n_steps;
     if (n_steps > 0) {
         launch_batch_prep(B, prec, c, s);

@@ -56,6 +56,37 @@ static void free_network(DevNetwork& n)
     n = DevNetwork{};
 }
 
+// What only one precision uses, made for the one in use (ptadd_set_network) and when
+// another is switched to (ptadd_set_precision): its source records, 64 or 192 bytes per node, and
+// partial forces for the most chunks it splits the sources into.  A failure leaves what there was.
+static ptadd_status need_precision(DevNetwork& net, int prec)
+{
+    const int64_t n = net.n_nodes;
+    ptadd_status st = PTADD_OK;
+    if (prec == (int)PTADD_MIXED) {
+        if (!net.src32) st = dalloc(&net.src32, SRC32_STRIDE * n);
+    } else {
+        if (!net.srcdf) st = dalloc(&net.srcdf, SRCDF_STRIDE * n);
+    }
+    int chunks = 1;
+    for (int64_t nt : {net.n_tgt_burst, n}) chunks = std::max(chunks, choose_chunks(nt, n, network_max_chunks(n), prec));
+    if (st == PTADD_OK && chunks > net.max_chunks) {
+        double* more = nullptr;
+        st = dalloc(&more, (size_t)chunks * 6 * n);
+        if (st == PTADD_OK) {
+            if (net.fpart) cudaFree(net.fpart);  // (waits for the device)
+            net.fpart = more;
+            net.max_chunks = chunks;
+        }
+    }
+    return st;
+}
+// The rows of the consistent mobility's system, 80 bytes per node.
+static ptadd_status need_consistent(DevNetwork& net)
+{
+    return net.cm_scratch ? PTADD_OK : dalloc(&net.cm_scratch, 10 * net.n_nodes);
+}
+
 static Consts make_consts(const ptadd_ctx* ctx) { return make_consts(ctx->mat.a / ctx->len_unit, ctx->mat.nu); }
 
 }  // namespace ptadd
@@ -126,6 +157,11 @@ ptadd_status ptadd_set_precision(ptadd_ctx* ctx, ptadd_precision prec)
 {
     if (!ctx) return arg_error("null context");
     if (prec != PTADD_FP64 && prec != PTADD_MIXED) return arg_error("unknown precision");
+    if (ctx->have_net && prec != ctx->prec) {
+        PTADD_CUDA(cudaSetDevice(ctx->device));
+        const ptadd_status st = need_precision(ctx->net, (int)prec);
+        if (st != PTADD_OK) return st;
+    }
     ctx->prec = prec;
     return PTADD_OK;
 }
@@ -207,11 +243,6 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
         if (!(pinned && pinned[i] && pinned[nxt[i]])) tb.push_back((int32_t)i);
     }
     net.n_tgt_burst = (int64_t)tb.size();
-    // the most chunks any evaluation of this network splits its sources into
-    net.max_chunks = 1;
-    for (int prec : {(int)PTADD_FP64, (int)PTADD_MIXED})
-        for (int64_t nt : {net.n_tgt_burst, n})
-            net.max_chunks = std::max(net.max_chunks, choose_chunks(nt, n, network_max_chunks(n), prec));
     const int64_t node_off[2] = {0, n};
     const StepGroups grp = step_groups(n_loops, loop_off, 1, node_off);
     net.n_grp = grp.real_grp[1];
@@ -231,7 +262,6 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     ALLOC(net.tgt_burst, tb.size());
     ALLOC(net.tgt_all, n);
     ALLOC(net.src, SRC_STRIDE * n);
-    ALLOC(net.fpart, (size_t)net.max_chunks * 6 * n);
     ALLOC(net.vel, 3 * n);
     ALLOC(net.force, 3 * n);
     ALLOC(net.part, (size_t)net.n_grp * 16);
@@ -240,13 +270,12 @@ ptadd_status ptadd_set_network(ptadd_ctx* ctx, int64_t n_nodes, const double* xy
     ALLOC(net.acc, 16);
     ALLOC(net.flag, 1);
     ALLOC(net.staging, 3 * n);
-    ALLOC(net.src32, SRC32_STRIDE * n);
-    ALLOC(net.srcdf, SRCDF_STRIDE * n);
     ALLOC(net.near_count, 1);
     ALLOC(net.k64, 4);
     ALLOC(net.loop_off, n_loops + 1);
-    ALLOC(net.cm_scratch, 10 * n);
 #undef ALLOC
+    if (st == PTADD_OK) st = need_precision(net, (int)ctx->prec);
+    if (st == PTADD_OK && ctx->consistent_mass) st = need_consistent(net);
     if (st != PTADD_OK) {
         free_network(net);
         return st;
@@ -415,6 +444,10 @@ ptadd_status ptadd_set_mobility(ptadd_ctx* ctx, int32_t consistent)
     if (consistent && (ctx->junc || batch_has_junctions(ctx))) {
         set_error("ptadd_set_mobility: the consistent mobility does not combine with junctions (switch them off first)");
         return PTADD_ERR_STATE;
+    }
+    if (consistent && ctx->have_net) {
+        const ptadd_status st = need_consistent(ctx->net);
+        if (st != PTADD_OK) return st;
     }
     ctx->consistent_mass = consistent == 1;
     return PTADD_OK;

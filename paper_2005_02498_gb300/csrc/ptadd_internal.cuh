@@ -75,8 +75,8 @@ struct DevNetwork {
     int64_t n_tgt_burst = 0;
     int32_t* tgt_all = nullptr;    // every segment
     double* src = nullptr;         // [n*SRC_STRIDE]
-    float* src32 = nullptr;        // [n*SRC32_STRIDE] FP32 records of the mixed path
-    float* srcdf = nullptr;        // [n*SRCDF_STRIDE] double-float records of the FP64 path
+    float* src32 = nullptr;        // [n*SRC32_STRIDE] FP32 records of the mixed path (null until it is used)
+    float* srcdf = nullptr;        // [n*SRCDF_STRIDE] double-float records of the FP64 path (null until it is used)
     double origin[3] = {0, 0, 0};  // integer-valued origin of the FP32 records
     bool origin_node0 = false;     // instead: node 0's position rounded (read on the device)
     unsigned long long* near_count = nullptr;  // FP64 point-pairs of the mixed path
@@ -96,7 +96,7 @@ struct DevNetwork {
     int* flag = nullptr;           // non-finite flag
     double* staging = nullptr;     // [3*n] AoS SI positions in / out
     int64_t* loop_off = nullptr;   // [n_loops + 1] first node of each loop (consistent mobility)
-    double* cm_scratch = nullptr;  // [10*n] rows of the consistent mobility's system
+    double* cm_scratch = nullptr;  // [10*n] rows of the consistent mobility's system (null until it is used)
     double volume = 0;             // m^3
 };
 
