@@ -43,6 +43,21 @@ struct TileArgs {
 // ---------------------------------------------------------------- records
 constexpr double DF_NEAR = 32.0;      // in core widths a
 constexpr double DF_FAR = 2097152.0;  // 2^21 units
+// No product of the double-float path may leave FP32's range (a close pair's are formed too, and
+// then not used: an infinity would turn its 0 into NaN).  Far pairs are at least 1/16 unit apart
+// (farther for any core width of 1/512 unit or more).  A segment's pairs are all evaluated in
+// FP64 where its Burgers vector is outside 2^-20 to 2^20 units; where the core is below 2^-30; and
+// where the core is below 2^-12 and the segment below 2^-8: then 1/rho is below 2^40, 1/(rho1 rho2)^2 below 2^116.
+constexpr float DF_NEAR_MIN = 1.0f / (16 << -DF_SCALE);
+constexpr float DF_B_MIN = 1.0f / 1048576.0f, DF_B_MAX = 1048576.0f;
+constexpr float DF_L_MIN = 1.0f / (256 << -DF_SCALE);
+__device__ __forceinline__ bool df_unfit(const DF1& l, double a2, double bt, double be, const DF1& fbt, const DF1& fbe)
+{
+    const int ea = (__double2hiint(a2) >> 20) - 1023;  // exponent of a^2
+    if (ea < -60 || (ea < -24 && l.h < DF_L_MIN)) return true;
+    const float bm = fmaxf(fabsf(fbt.h), fabsf(fbe.h));
+    return !(bm >= DF_B_MIN && bm <= DF_B_MAX) && (bt != 0.0 || be != 0.0);
+}
 // The three FP32 parts of x - o (o an integer), scaled; NaN outside their range.
 __device__ __forceinline__ void df_parts(double x, double o, float* f)
 {
@@ -146,7 +161,15 @@ __device__ __forceinline__ void seg_records(const double x1[3], const double x2[
         f[32] = fb.l;
         f[33] = fe.h;
         f[34] = fe.l;
-        f[35] = fmaxf((float)(DF_NEAR * DF_NEAR * SC * SC * a2), ll.h * (1.0f / 256.0f));
+        f[35] = fmaxf(fmaxf((float)(DF_NEAR * DF_NEAR * SC * SC * a2), DF_NEAR_MIN * DF_NEAR_MIN), ll.h * (1.0f / 256.0f));
+        if (df_unfit(l, a2, bt, be, fb, fe)) {
+            // every pair of this segment in FP64: as a source by its length, as a target by its near limit
+            const float inf = __int_as_float(0x7f800000);
+            f[27] = inf;
+            f[35] = inf;
+#pragma unroll
+            for (int k = 36; k < 48; ++k) f[k] = 0.0f;
+        }
         float4* out = reinterpret_cast<float4*>(fdf);
 #pragma unroll
         for (int k = 0; k < SRCDF_STRIDE / 4; ++k) out[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
@@ -297,8 +320,8 @@ __device__ __forceinline__ void near_shift(uint2* q, int cnt)
 // chains of Gauss points then share one copy of the code, which must fit the
 // instruction cache) and are added to FP64 sums when the group closes.
 // Coordinates enter as three FP32 parts (srcdf records), so that x_a - x1 is
-// exact to 2^-48 units; a pair outside their range, or with a distance or a
-// length of DF_FAR or more, is evaluated in FP64.  A tile is one warp's: no lane waits for
+// exact to 2^-48 units; a pair outside their range, with a distance or a
+// length of DF_FAR or more, or with a segment that df_unfit() names, is evaluated in FP64.  A tile is one warp's: no lane waits for
 // another warp, and a small network gives as many tiles as it has warps.
 constexpr int DF_REC = 64;            // floats of a staged source record
 constexpr int DF_TILE = 12;           // sources per staged tile (16 blocks of 13 KB fit one SM)
@@ -325,12 +348,13 @@ __device__ __forceinline__ void pair_tile_fp64(const TileArgs& a, const Consts& 
     float xt[9], lim_t;
     DF1 D[3];
     DF2 bt[3];
-    bool wide = false;  // a target too long for the double-float range
+    bool wide;  // a target too long, or otherwise unfit, for the double-float range
     {
         const float* fr = a.srcdf + (int64_t)SRCDF_STRIDE * seg;
 #pragma unroll
         for (int k = 0; k < 9; ++k) xt[k] = fr[k];
         lim_t = fr[35];
+        wide = !(lim_t < __int_as_float(0x7f800000));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             D[k] = DF1{fr[36 + k], fr[39 + k]};

@@ -53,7 +53,8 @@ constexpr int SRC32_STRIDE = 16;
 //   [0..8] x1 - origin per coordinate as an integer, a multiple of 2^-23 below
 //   1/2 and the rest   [9..11] t high parts [12..14] t low parts   [15..20] e, the
 //   same   [21..26] n = t x e   [27..28] L   [29..30] L^2   [31..32] b.t   [33..34] b.e
-//   [35] squared near limit of the segment (df_field.cuh has the frame t, e, n);
+//   [35] squared near limit of the segment (df_field.cuh has the frame t, e, n); infinite, as [27] is,
+//   where the path cannot take the segment;
 //   for the segment as a target: [36..41] D = x2 - x1, [42..47] b (high parts, low parts)
 constexpr int SRCDF_STRIDE = 48;
 // Near field of the mixed path: point-to-segment distance below 10 a, with a
