@@ -226,9 +226,16 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
     };
     // The operands have been issued: wait for them (the `other` bytes of A in buffer b from other CTAs too),
     // multiply, wait for the product.  A wait that gives up leaves the rest of the tile's
-    // products out; every barrier is still met.
+    // products out; every barrier is still met, and the pieces that arrive all the same are
+    // counted for a last wait: they may not land in the shared memory of a CTA that has left.
+    uint32_t late = 0, owed[2] = {0, 0};  // thread 0: bit b: the wait on xbar[b] gave up; bytes not waited for since
     auto multiply = [&](int b, uint32_t other, int steps, uint32_t a_sbo, int N) {
-        if (tid == 0 && other) mbar_expect_tx(ux + 8 * b, other);
+        if (tid == 0 && other) {
+            if (ok)
+                mbar_expect_tx(ux + 8 * b, other);
+            else
+                owed[b] += other;
+        }
         cp_wait_all();
         fence_async_smem();
         tc_fence_before();
@@ -238,9 +245,11 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
                 tc_fence_after();
                 issue_mma<FB_N>(tmem, uA + b * FB_A, 2, PIECE, a_sbo, uB, steps, idesc_bf16_f32(128, N), false);
                 tc_commit(mb);
+            } else {
+                late |= 1u << b;
             }
         }
-        if (other) xph ^= 1u << b;
+        if (other && ok) xph ^= 1u << b;
         bool w = true;
         if (ok) w = mbar_wait_bounded(mb, phase, MBAR_WAIT_LIMIT);
         phase ^= 1u;
@@ -335,6 +344,15 @@ __global__ void __cluster_dims__(1, FB_CL, 1) __launch_bounds__(FB_T, 1) mlp_fb_
         // a last bounded chance for the tensor core before its memory is freed
         mbar_wait_bounded(mb, 0u, MBAR_WAIT_LIMIT);
         mbar_wait_bounded(mb, 1u, MBAR_WAIT_LIMIT);
+        // and for the pieces on their way here, if a phase that gave up completes at all
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const uint32_t next = (xph >> b) & 1u;
+            if (((late >> b) & 1u) && !mbar_wait_bounded(ux + 8 * b, next ^ 1u, MBAR_WAIT_LIMIT)) continue;
+            if (owed[b] == 0u) continue;
+            mbar_expect_tx(ux + 8 * b, owed[b]);
+            mbar_wait_bounded(ux + 8 * b, next, MBAR_WAIT_LIMIT);
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -481,6 +499,8 @@ __global__ void __launch_bounds__(DW_T, 1) mlp_dw_kernel(TrainArgs g)
         }
     } else if (tid == 0) {
         atomicExch(g.err, 1);
+        // a last bounded chance for the copies in flight and the tensor core
+        mbar_wait_bounded(uf, phase ^ 1u, MBAR_WAIT_LIMIT);
         mbar_wait_bounded(mb, phase ^ 1u, MBAR_WAIT_LIMIT);
     }
     tc_fence_before();
