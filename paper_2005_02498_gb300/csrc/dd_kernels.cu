@@ -138,6 +138,13 @@ static void pair_slots(int& sms, int& per_sm)
     }
 }
 
+int device_sms()
+{
+    int sms, per_sm;
+    pair_slots(sms, per_sm);
+    return sms;
+}
+
 int64_t fp64_slots()
 {
     int sms, per_sm;

@@ -124,6 +124,7 @@ cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& 
 // pair stage: writes fpart[chunk][6][seg] for the listed targets
 cudaError_t launch_pair(const DevNetwork& net, const int32_t* tgt, int64_t n_tgt, int chunks,
                         int precision, const Consts& c, const double sig_hat[6], cudaStream_t st, bool chained = false);
+int device_sms();
 // one-warp FP64 target tiles that run at a time
 int64_t fp64_slots();
 int choose_chunks(int64_t n_tgt, int64_t n_src, int max_chunks, int precision);

@@ -327,9 +327,13 @@ cudaError_t launch_step(const StepArgs& a, int n_groups, bool whole, int max_chu
 {
     if (a.n == 0) return cudaSuccess;
     auto go = [&](int w) {
-        // 16 rows where few blocks sum many chunks (a small network); 4 leave room for more blocks
+        // 16 rows where at most one block per SM sums many chunks: its rows shorten the chain of
+        // sums.  With more blocks than SMs, or few chunks, 4 rows: the others would
+        // only take part in barriers.  us a step with 16 / 4 rows: 64 groups 134.8 / 137.8 (mixed), 459.6 / 466.8
+        // (FP64); 128 groups equal; 192 groups 600.6 / 593.0, 3635 / 3625; 256 groups 971 / 966, 6244 / 6238; 16 groups of 2
+        // chunks 74.7 / 74.2.
         *launches += 1;
-        const bool tall = max_chunks > 16 && n_groups <= 304;
+        const bool tall = max_chunks > 16 && n_groups <= device_sms();
         if (chained)
             return tall ? launch_chained(step_kernel<16>, n_groups, 512, 0, st, a, w)
                         : launch_chained(step_kernel<4>, n_groups, 128, 0, st, a, w);
