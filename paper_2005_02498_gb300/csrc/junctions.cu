@@ -207,7 +207,6 @@ __global__ void __launch_bounds__(32) junction_event_kernel(int n_groups, const 
     chain_next();
     const double len = step_length(n_groups, part);
     if (threadIdx.x != 0) return;
-    acc[11] = len;
     const double t1 = __dadd_rn(clock[0], dt_s);
     const double vmax = sqrt(__longlong_as_double((long long)red[0]));
     const double tmin = __longlong_as_double((long long)red[1]);

@@ -91,9 +91,9 @@ struct DevNetwork {
     int n_grp = 0;
     bool grp_whole = true;
     double* part = nullptr;        // [16*n_grp] their sums
-    double* acc = nullptr;         // [16]: 0..8 sum Lp dt, 9 sum rho dt, 11 line length of the last
-                                   // step, 12 time jumped over while stuck (junctions), 13..15 sum
-                                   // (sum_s L vbar) dt (polar velocity)
+    double* acc = nullptr;         // [16]: 0..8 sum Lp dt, 9 sum rho dt, 12 time jumped over
+                                   // while stuck (junctions), 13..15 sum (sum_s L vbar) dt (polar
+                                   // velocity); in a batch 11 the line length of the last step
     int* flag = nullptr;           // non-finite flag
     double* staging = nullptr;     // [3*n] AoS SI positions in / out
     int64_t* loop_off = nullptr;   // [n_loops + 1] first node of each loop (consistent mobility)
