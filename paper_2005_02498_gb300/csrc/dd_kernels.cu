@@ -62,16 +62,17 @@ cudaError_t launch_seg_prep(const DevNetwork& net, int precision, const Consts& 
 constexpr int MIX_TPB = 32;
 constexpr int MIX_MAX_CHUNKS = 64;
 constexpr int MIX_TILE = 192;  // sources per tile (one plain FP32 sum), staged 32 at a time
-// One-warp blocks, 16 per SM.  Bound by the FP32 pipe (183 packed instructions per
-// source and warp, two cycles each); 16 warps at 128 registers (16 bytes spilled
+// One-warp blocks, 16 per SM.  Bound by the FP32 pipe (177 packed instructions per
+// source and warp, two cycles each, and 12 plain ones; 69 % of the active cycles, the rest being the
+// latency of the formula's chain to the four warps of a scheduler); 16 warps at 128 registers (16 bytes spilled
 // outside the loop's arithmetic) keep it busier than 12 at 160.  32 768 / 8192 segments:
 // 13.28 / 0.947 ms per launch, blocks of two warps 13.38 / 0.948, of four 13.41 / 0.987
 // (the tail is a warp's tile long, not a block's), three blocks of four warps 13.82 / 1.066.
 constexpr int MIX_MINB = 16;
 
-// FP64 path.  Bound by the FP32 pipe: about 1550 packed FP32 instructions per
-// source and warp, two pipe cycles each (3100 of the 3650 cycles that a source
-// takes on a full scheduler).  32 768 segments: 96.5 ms per evaluation (1.11e10
+// FP64 path.  Bound by the FP32 pipe: 1475 packed FP32 instructions per
+// source and warp, two pipe cycles each, and 33 plain ones: 3000 of the 3650 cycles that a source
+// takes on a full scheduler.  32 768 segments: 96.5 ms per evaluation (1.11e10
 // pairs/s), 826 ms when every pair ran on the FP64 pipe; 512 segments: 51
 // against 560 us per launch.  A tile's set-up and its closing stay off the FP64
 // pipe (64 cycles per warp instruction): the targets' D and b' come split from

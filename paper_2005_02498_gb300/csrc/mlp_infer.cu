@@ -103,7 +103,7 @@ constexpr int NV_XM = 0, NV_XR = NV_XM + NF, NV_YM = NV_XR + NF, NV_YS = NV_YM +
               NV_HI = NV_LO + NF, NV_THR = NV_HI + NF, NV_S2 = NV_THR + 1, NV_B4 = NV_S2 + 1, NV_COUNT = NV_B4 + 16;
 constexpr int NV_BYTES = (NV_COUNT * 4 + 127) / 128 * 128;
 // what stays in shared memory, laid out in global memory as it is there, one block per
-// CTA of a pair: two bulk copies (what layer 1 needs, then W2 and W3)
+// CTA of a pair: three bulk copies (what layer 1 needs, then W2, then W3)
 constexpr int R_W1 = 0;
 constexpr int R_LH = R_W1 + W1_BYTES;
 constexpr int R_LL = R_LH + LI_BYTES;
@@ -327,7 +327,9 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t mbar, uint32_t parity, vo
 // (the FP64 pipe is slow on this part).  Every rounding is written out, because a
 // last-bit difference here can flip the operand's FP16 rounding: the product by log10(2) is
 // rounded before the subtraction, except in columns 6 and 7 of each 8, where the two
-// are one fused operation.
+// are one fused operation.  That split has no reason in the mathematics; it is kept because the
+// trust-region flags depend on it: with every column fused 2 to 9 of 10^6 flags change (8 sets
+// of inputs), and the rates by 6e-5.
 __device__ __forceinline__ float standardise(double v, int k, float mean, float rdev)
 {
     constexpr float LOG10_2 = 0.30102999566398120f;

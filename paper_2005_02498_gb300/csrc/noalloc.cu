@@ -32,7 +32,7 @@ namespace {
 constexpr int64_t NA_MAX = PTADD_NOALLOC_MAX_SEGMENTS;
 constexpr int NA_CHUNKS = 4;  // source chunks at NA_MAX segments (smaller networks: more, in the same space)
 // doubles per segment: positions 3, source record 16, double-float record 24
-// (48 floats), partial forces 6 per chunk, force 3, velocity 3, Burgers vector 3, normal 3; then four int32
+// (48 floats), partial forces 6 per chunk, force 3, Burgers vector 3; then four int32
 // tables (loop index, target list, checked nxt and prv copies) and the error
 // word packed into the same array.
 constexpr int64_t NA_DOUBLES_PER_SEG = 3 + SRC_STRIDE + SRCDF_STRIDE / 2 + 6 * NA_CHUNKS + 3 + 3;

@@ -54,7 +54,11 @@ struct StepArgs {
 
 // Groups of consecutive nodes, a block each: whole loops of one realisation, up
 // to 32 nodes together, as long as no loop has more than STEP_LOOP_MAX nodes (a block walks a
-// longer loop 32 nodes at a time); otherwise 32 nodes wherever the loops end.
+// longer loop 32 nodes at a time); otherwise 32 nodes wherever the loops end, and a launch per
+// phase: two a step, eight with the consistent mobility.  us a step in whole loops / split, two loops of n nodes
+// in FP64: lumped, n = 64 47 / 38, 128 105 / 54, 256 160 / 84, 400 313 / 135; consistent 64 54 / 64,
+// 128 114 / 80, 256 174 / 111, 400 337 / 170.  Eight loops of 256 in mixed precision: lumped 247 / 198,
+// consistent 260 / 224.  The line could lie lower: a block's walk of a long loop is the chain.
 constexpr int STEP_LOOP_MAX = 256;
 struct StepGroups {
     std::vector<int32_t> off;       // [groups + 1]
