@@ -49,18 +49,26 @@ static ptadd_status dalloc(T** p, size_t count)
 static void free_network(DevNetwork& n)
 {
     void* ptrs[] = {n.pos[0], n.pos[1], n.nxt,   n.prv,   n.loop_of, n.loop_b,  n.loop_n, n.pinned, n.tgt_burst,
-                    n.tgt_all, n.src,    n.fpart, n.vel,   n.force,   n.part,   n.grp_off, n.real_grp, n.acc,    n.flag,   n.staging,
+                    n.tgt_all, n.src,    n.parts[0], n.parts[1], n.vel,   n.force,   n.part,   n.grp_off, n.real_grp, n.acc,    n.flag,   n.staging,
                     n.src32,   n.srcdf, n.near_count, n.k64, n.loop_off, n.cm_scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     n = DevNetwork{};
 }
 
+// Device allocations are allowed while the calling thread captures a stream: they are not part of the graph.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 // What only one precision uses, made for the one in use (ptadd_set_network) and when
 // another is switched to (ptadd_set_precision): its source records, 64 or 192 bytes per node, and
-// partial forces for the most chunks it splits the sources into.  A failure leaves what there was.
+// partial forces for the most chunks it splits the sources into.  Each stays where it is until the next
+// network, as a graph that a caller has captured holds its address.  A failure leaves what there was.
 static ptadd_status need_precision(DevNetwork& net, int prec)
 {
+    const RelaxedCapture relaxed;
     const int64_t n = net.n_nodes;
     ptadd_status st = PTADD_OK;
     if (prec == (int)PTADD_MIXED) {
@@ -68,16 +76,17 @@ static ptadd_status need_precision(DevNetwork& net, int prec)
     } else {
         if (!net.srcdf) st = dalloc(&net.srcdf, SRCDF_STRIDE * n);
     }
-    int chunks = 1;
-    for (int64_t nt : {net.n_tgt_burst, n}) chunks = std::max(chunks, choose_chunks(nt, n, network_max_chunks(n), prec));
-    if (st == PTADD_OK && chunks > net.max_chunks) {
-        double* more = nullptr;
-        st = dalloc(&more, (size_t)chunks * 6 * n);
-        if (st == PTADD_OK) {
-            if (net.fpart) cudaFree(net.fpart);  // (waits for the device)
-            net.fpart = more;
-            net.max_chunks = chunks;
-        }
+    const int k = prec == (int)PTADD_MIXED ? 1 : 0;
+    if (st == PTADD_OK && !net.parts[k]) {
+        int chunks = 1;
+        for (int64_t nt : {net.n_tgt_burst, n})
+            chunks = std::max(chunks, choose_chunks(nt, n, network_max_chunks(n), prec));
+        st = dalloc(&net.parts[k], (size_t)chunks * 6 * n);
+        if (st == PTADD_OK) net.parts_chunks[k] = chunks;
+    }
+    if (st == PTADD_OK) {
+        net.fpart = net.parts[k];
+        net.max_chunks = net.parts_chunks[k];
     }
     return st;
 }

@@ -82,7 +82,9 @@ struct DevNetwork {
     bool origin_node0 = false;     // instead: node 0's position rounded (read on the device)
     unsigned long long* near_count = nullptr;  // FP64 point-pairs of the mixed path
     double* k64 = nullptr;         // {a2, c1, c2} for the near-field path of the mixed kernel
-    double* fpart = nullptr;       // [max_chunks*6*n] partial nodal-force parts (targets' entries only are written)
+    double* parts[2] = {nullptr, nullptr};  // partial nodal-force parts of the FP64 and of the mixed path (null
+    int parts_chunks[2] = {0, 0};           // until it is used), and the chunks they hold
+    double* fpart = nullptr;       // those of the precision in use: [max_chunks*6*n] (targets' entries only are written)
     int max_chunks = 0;
     double* vel = nullptr;         // SoA [3*n]
     double* force = nullptr;       // SoA [3*n] (last evaluated nodal force)

@@ -80,3 +80,37 @@ def test_results_across_switches(order):
                 assert relmax(c.get_forces(), Fo) <= (1e-4 if mixed else 1e-11)
                 Lp, _ = c.advance(2, DT)
                 assert relmax(Lp, ref["Lp_avg"]) <= (1e-2 if mixed else 1e-9)
+
+
+def test_switch_inside_a_capture_and_replay_after_switches():
+    """Forces in both precisions captured into one graph, the switch (and its buffers) inside the capture; the graph
+    gives the same after the context has been switched on."""
+    sig = np.array([20e6, -35e6, 50e6, 10e6, -5e6, 25e6])
+    net = W.loop_ensemble(19, 5, 0.6e-6, sig, nodes_per_loop=24)
+    with ptadd.Context(MAT, ptadd.PTADD_MIXED, 0) as w:  # the kernels of both are loaded
+        w.set_network(net)
+        want = {}
+        for prec in (ptadd.PTADD_MIXED, ptadd.PTADD_FP64):
+            w.set_precision(prec)
+            want[prec] = w.get_forces()
+    out = {p: torch.zeros((net.n_nodes, 3), dtype=torch.float64, device="cuda") for p in want}
+    stream = torch.cuda.Stream()
+    with ptadd.Context(MAT, ptadd.PTADD_MIXED, 0) as c:
+        c.set_stream(stream.cuda_stream)
+        c.set_network(net)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for prec in (ptadd.PTADD_MIXED, ptadd.PTADD_FP64):
+                c.set_precision(prec)
+                c.get_forces_dev(out[prec].data_ptr())
+        for prec in (ptadd.PTADD_MIXED, ptadd.PTADD_FP64, ptadd.PTADD_MIXED):
+            c.set_precision(prec)
+            for o in out.values():
+                o.zero_()
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            for p, o in out.items():
+                assert np.array_equal(o.cpu().numpy(), want[p])
+        del graph
