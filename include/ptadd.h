@@ -79,8 +79,9 @@ typedef struct {
 
 typedef enum {
     PTADD_FP64 = 0, /* FP64 results: pairs nearer than 32a (or 1/16 of a segment's     *
-                     * length) in FP64, the others in double-float arithmetic (two     *
-                     * FP32 parts, 48 bits) on the FP32 pipe.  A far pair is reduced   *
+                     * length), and any that FP32's range cannot hold, in FP64, the    *
+                     * others in double-float arithmetic (two FP32 parts, 48 bits) on  *
+                     * the FP32 pipe.  A far pair is reduced                           *
                      * precision: 2e-14 of itself off in the median, 2e-13 in 99 of    *
                      * 100 (FP64: 4e-16, 1e-14).  Measured against 80-bit numbers on   *
                      * networks of 42 to 2125 segments, the forces are 1.7e-12 to      *
